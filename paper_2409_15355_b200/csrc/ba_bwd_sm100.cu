@@ -9,18 +9,23 @@
 // atomics, so results are run-to-run identical:
 //   * ba_bwd_dkv_kernel: one CTA owns 128 keys of one block and one KV head and walks over every
 //     query tile that sees them (all heads of the group).  It forms the scores transposed, S^T = K Q^T
-//     and dP^T = V dO^T (keys on the tensor-memory lanes, query rows on the columns), so that its 128
-//     threads -- one per key -- write P^T and dS^T back to tensor memory as bf16, where they are the A
+//     and dP^T = V dO^T (keys on the tensor-memory lanes, query rows on the columns), so that its
+//     threads -- two per key -- write P^T and dS^T back to tensor memory as bf16, where they are the A
 //     operands of dV += P^T dO and dK += dS^T Q (nothing goes through shared memory, nothing is transposed).
 //   * ba_bwd_dq_kernel: one CTA owns one query tile (tokens x heads of one KV group, as in the
 //     forward kernel) and walks over the key tiles it sees: S = Q K^T, dP = dO V^T (query rows on the
 //     lanes), dS written to tensor memory, dQ += dS K.
 // The tiles a CTA walks over (Q and dO there, K and V here) are double-buffered in shared memory, so the
-// loads of the next tile run under the current one.  Both kernels work in steps of 64 columns of S and dP with
-// two buffers of each in tensor memory (2 x 2 x 64 columns beside the accumulators): while the threads turn
-// one step's scores into P and dS, the tensor core forms the next step's scores and multiplies the previous
-// step's P and dS.
+// loads of the next tile run under the current one.
+//
+// Both are bound by the chain scores -> threads -> gradient products rather than by the tensor core alone, so both are
+// laid out to keep the tensor core busy while threads work: the dK/dV kernel hands P^T over before it touches dP^T, so that
+// dV and the next tile's S^T run under the formation of dS^T, and dK and the next dP^T under the next P^T; the dQ kernel
+// runs two CTAs per SM.  The dK/dV score products take 128 columns at a time: a 64-column product reads as much of its A
+// operand from shared memory as a 128-column one.  8 x 16384 ragged tokens, 32/8 heads of 128, one B200: dK/dV 6.49 -> 5.28 ms, dQ
+// 6.04 -> 4.15 ms against kernels that worked in steps of 64 columns with one CTA per SM.
 #include <math.h>
+#include <type_traits>
 
 #include "ba_common.cuh"
 #include "ba_sm100.cuh"
@@ -31,13 +36,15 @@ int ba_heads_per_tile(const ba_config &c);
 
 namespace {
 
-// warps 0-7: two threads per tile row (tensor-memory lane = tid & 127), warps w and w + 4 share a lane quarter and
-// take one half of every step's 64 columns each, so that every SM sub-partition has two warps to hide the
-// latency of tensor-memory loads, shared-memory reads and exponentials; warp 8: loads and MMA issue
-constexpr int kBwdThreads = 288;
-constexpr int kRowThreads = 256;
-constexpr int kCtlWarp = 8;
+// dK/dV kernel: eight row warps, two threads per key (tensor-memory lane), each with one half of a tile's 128 query
+// rows; warp 8 issues the products, warp 9 the loads.
+constexpr int kDkvThreads = 320;
+constexpr int kDkvMmaWarp = 8, kDkvLoadWarp = 9;
+// dQ kernel: one group of four row warps, a product warp and a load warp; two CTAs share an SM.
+constexpr int kDqThreads = 192;
+constexpr int kDqMmaWarp = 4, kDqLoadWarp = 5;
 constexpr int kTile = 128;
+constexpr int kStep = 64;              // keys a step of the dQ kernel works on
 
 struct BwdParams {
   const float *lse;          // [T, Hq] natural-log softmax denominators of the forward pass
@@ -52,24 +59,51 @@ struct BwdParams {
   ba_segments seg;
 };
 
+// Shared memory of the dK/dV kernel: K and V tiles that stay, two buffers of (Q, dO) tiles it walks over, and what
+// every key has to know about a query row -- -lse * log2 e, -dO . O * scale, visible keys of the tile --, two buffers of each.
 template <int D>
-struct BwdLayout {
+struct DkvLayout {
   static constexpr int kChunks = D / 64;
   static constexpr int kRegion = 128 * 128;              // 128 rows x 128 bytes
   static constexpr int kTileBytes = 128 * D * 2;
-  // two tiles that stay for the whole CTA (K, V in the dK/dV kernel; Q, dO in the dQ kernel) and two
-  // buffers of two tiles each for the ones it walks over
   static constexpr int kFix0 = 0, kFix1 = kTileBytes;
   static constexpr int kWalk = 2 * kTileBytes;            // buffer b: tiles at kWalk + b * 2 * kTileBytes, + kTileBytes
-  static constexpr int kStats = 6 * kTileBytes;           // dK/dV kernel: per query row lse * log2 e, dO . O * scale, visible keys; two buffers of each
-  static constexpr int kCtrl = kStats + 2 * 128 * 16;
+  static constexpr int kStats = 6 * kTileBytes;           // [buffer][3][128]
+  static constexpr int kCtrl = kStats + 2 * 3 * 128 * 4;
   static constexpr int kBytes = kCtrl + 256;
 };
 
-struct BwdCtrl {
+struct DkvCtrl {
   uint64_t fix_full, walk_full[2], walk_free[2];
-  uint64_t sd_full[2], rows_done[2];     // per buffer of S / dP in tensor memory
+  uint64_t s_full, dp_full;              // S^T / dP^T of the tile are in tensor memory
+  uint64_t p_done, ds_done;              // P^T / dS^T of the tile are in tensor memory
   uint64_t fin;                          // every product of the CTA has completed
+  uint32_t tmem_base;
+  int abort_flag;
+};
+
+// Shared memory of the dQ kernel: Q and dO tiles that stay, two 64-key tiles of K and one of V.  At head_dim 128 this is
+// 112 KB + 1 KB: exactly half of what an SM has for two CTAs, so the base must be 1024-byte aligned as it is.
+template <int D>
+struct DqLayout {
+  static constexpr int kChunks = D / 64;
+  static constexpr int kRegion = 128 * 128;
+  static constexpr int kTileBytes = 128 * D * 2;
+  static constexpr int kKeyRegion = kStep * 128;          // 64 rows x 128 bytes
+  static constexpr int kKeyBytes = kStep * D * 2;
+  static constexpr int kQ = 0, kDo = kTileBytes;
+  static constexpr int kK = 2 * kTileBytes;               // K of step i at kK + (i & 1) * kKeyBytes
+  static constexpr int kV = kK + 2 * kKeyBytes;
+  static constexpr int kCtrl = kV + kKeyBytes;
+  static constexpr int kBytes = kCtrl + 1024;
+};
+
+struct DqCtrl {
+  uint64_t fix_full, k_full[2], k_free[2], v_full, v_free;
+  uint64_t sd_full;                      // S and dP of the step are in tensor memory
+  uint64_t s_read;                       // the row threads hold S in registers: the next step's S may overwrite it
+  uint64_t rows_done;                    // dS of the step is in tensor memory
+  uint64_t fin;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -82,7 +116,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
-__device__ __forceinline__ void named_barrier_rows() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void row_warps_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 __device__ __forceinline__ int upper_bound_dev(const int32_t *a, int n, int x) {
   int lo = 0, hi = n;
@@ -93,33 +127,26 @@ __device__ __forceinline__ int upper_bound_dev(const int32_t *a, int n, int x) {
   return lo;
 }
 
-// The kernels work in steps of 64 columns of S and dP: tensor memory then holds two buffers of each next to the
-// accumulators, so the threads turn one step's scores into P / dS while the tensor core forms the next step's
-// scores and multiplies the previous step's P / dS.
-//
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t *>(&v);
+}
 
-// The arithmetic of both helpers is packed fp32x2: for a pair of columns, x = s * scale_log2 - lse_log2 (one FMA),
+// The arithmetic of these helpers is packed fp32x2: for a pair of columns, x = s * scale_log2 - lse_log2 (one FMA),
 // p = exp2(x) (two), t = dp * scale - delta * scale (one FMA), ds = p * t (one multiply).  kMasked = false is for
 // steps in which every (row, key) pair is visible: no comparison at all.
 //
-// dQ kernel, one query row (= lane) against 64 keys: the thread takes chunk `c` (32 columns) of the step's S and
-// dP and writes dS back over the first 16 dP columns it has read, as bf16 (two per column): the A operand of
-// dQ += dS K.  `n_ok`: columns 0 .. n_ok - 1 of the step are visible to this row (0: none).
+// dQ kernel, one query row (= lane) against 32 keys: dS as bf16, two per register.  Keys 0 .. n_ok - 1 are visible.
 template <bool kMasked>
-__device__ __forceinline__ void bwd_row_ds(uint32_t tS, uint32_t tDP, int c, int n_ok, float scale_log2, float lse_log2,
-                                           float delta_scaled, float scale) {
-  uint32_t s[32], dp[32];
-  tmem_ld_32x32b_x32(tS + c * 32, s);
-  tmem_ld_32x32b_x32(tDP + c * 32, dp);
-  tmem_wait_ld();
-  const uint64_t sl2 = pack2(scale_log2, scale_log2), nl2 = pack2(-lse_log2, -lse_log2);
-  const uint64_t sc2 = pack2(scale, scale), nd2 = pack2(-delta_scaled, -delta_scaled);
-  uint32_t dw[16];
+__device__ __forceinline__ void bwd_row_ds(const uint32_t *s, const uint32_t *dp, uint32_t (&dw)[16], int n_ok, float scale_log2,
+                                           float neg_lse_log2, float neg_delta_scaled, float scale) {
+  const uint64_t sl2 = pack2(scale_log2, scale_log2), nl2 = pack2(neg_lse_log2, neg_lse_log2);
+  const uint64_t sc2 = pack2(scale, scale), nd2 = pack2(neg_delta_scaled, neg_delta_scaled);
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const uint64_t x2 = fma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), sl2, nl2);
@@ -127,46 +154,31 @@ __device__ __forceinline__ void bwd_row_ds(uint32_t tS, uint32_t tDP, int c, int
     unpack2(x2, x0, x1);
     float p0 = ex2(x0), p1 = ex2(x1);
     if (kMasked) {
-      const int e0 = c * 32 + 2 * i;
-      if (e0 >= n_ok) p0 = 0.f;
-      if (e0 + 1 >= n_ok) p1 = 0.f;
+      if (2 * i >= n_ok) p0 = 0.f;
+      if (2 * i + 1 >= n_ok) p1 = 0.f;
     }
     const uint64_t t2 = fma2(pack2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])), sc2, nd2);
     float d0, d1;
     unpack2(mul2(pack2(p0, p1), t2), d0, d1);
-    __nv_bfloat162 dv = __floats2bfloat162_rn(d0, d1);
-    dw[i] = *reinterpret_cast<uint32_t *>(&dv);
+    dw[i] = bf16_pair(d0, d1);
   }
-  tmem_st16(tDP + c * 32, dw);
-  tmem_wait_st();
 }
 
-// dK/dV kernel, one key (= lane `j`) against 64 query rows of a tile (= columns): the thread takes chunk `c`
-// (32 columns) of the step's S^T and dP^T; the per-row values -- lse * log2 e, dO . O * scale, and the number of
-// keys of this tile the row sees -- are read from shared memory, the same address by every thread.  P^T goes back
-// over the S^T columns and dS^T over the dP^T columns as bf16 -- each thread over columns it has read itself,
-// because the other thread of the lane works on its own 32 columns at its own pace.
+// dK/dV kernel, one key (= lane `j`) against 32 query rows (= columns).  The per-row values come from shared memory,
+// the same address for every thread; lim = number of keys of this tile the row sees.  First P^T: fp32 in place of s
+// (the second half of the step needs it), bf16 in pw.
 template <bool kMasked>
-__device__ __forceinline__ void bwd_key_p_ds(uint32_t tST, uint32_t tDPT, int c, int j, const float *lse2, const float *dls,
-                                             const int *lim, float scale_log2, float scale) {
-  uint32_t s[32], dp[32];
-  tmem_ld_32x32b_x32(tST + c * 32, s);
-  tmem_ld_32x32b_x32(tDPT + c * 32, dp);
-  tmem_wait_ld();
-  const uint64_t sl2 = pack2(scale_log2, scale_log2), sc2 = pack2(scale, scale);
-  uint32_t pw[16], dw[16];
+__device__ __forceinline__ void dkv_p(uint32_t *s, uint32_t (&pw)[16], int j, const float *neg_lse2, const int *lim, float scale_log2) {
+  const uint64_t sl2 = pack2(scale_log2, scale_log2);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {                          // four columns at a time: one 16-byte read of each per-row array
-    const float4 l4 = *reinterpret_cast<const float4 *>(lse2 + c * 32 + 4 * q);
-    const float4 d4 = *reinterpret_cast<const float4 *>(dls + c * 32 + 4 * q);
+    const ulonglong2 l4 = *reinterpret_cast<const ulonglong2 *>(neg_lse2 + 4 * q);
     int4 m4 = make_int4(0, 0, 0, 0);
-    if (kMasked) m4 = *reinterpret_cast<const int4 *>(lim + c * 32 + 4 * q);
+    if (kMasked) m4 = *reinterpret_cast<const int4 *>(lim + 4 * q);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const int i = 2 * q + e;
-      const uint64_t nl2 = e ? pack2(-l4.z, -l4.w) : pack2(-l4.x, -l4.y);
-      const uint64_t nd2 = e ? pack2(-d4.z, -d4.w) : pack2(-d4.x, -d4.y);
-      const uint64_t x2 = fma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), sl2, nl2);
+      const uint64_t x2 = fma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), sl2, e ? l4.y : l4.x);
       float x0, x1;
       unpack2(x2, x0, x1);
       float p0 = ex2(x0), p1 = ex2(x1);
@@ -174,27 +186,33 @@ __device__ __forceinline__ void bwd_key_p_ds(uint32_t tST, uint32_t tDPT, int c,
         if (j >= (e ? m4.z : m4.x)) p0 = 0.f;
         if (j >= (e ? m4.w : m4.y)) p1 = 0.f;
       }
-      const uint64_t t2 = fma2(pack2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])), sc2, nd2);
-      float d0, d1;
-      unpack2(mul2(pack2(p0, p1), t2), d0, d1);
-      __nv_bfloat162 pv = __floats2bfloat162_rn(p0, p1), dv = __floats2bfloat162_rn(d0, d1);
-      pw[i] = *reinterpret_cast<uint32_t *>(&pv);
-      dw[i] = *reinterpret_cast<uint32_t *>(&dv);
+      s[2 * i] = __float_as_uint(p0); s[2 * i + 1] = __float_as_uint(p1);
+      pw[i] = bf16_pair(p0, p1);
     }
   }
-  tmem_st16(tST + c * 32, pw);
-  tmem_st16(tDPT + c * 32, dw);
-  tmem_wait_st();
+}
+// Then dS^T = P^T (dP^T - dO . O) scale.
+__device__ __forceinline__ void dkv_ds(const uint32_t *p, const uint32_t *dp, uint32_t (&dw)[16], const float *neg_dls, float scale) {
+  const uint64_t sc2 = pack2(scale, scale);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const ulonglong2 d4 = *reinterpret_cast<const ulonglong2 *>(neg_dls + 4 * q);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int i = 2 * q + e;
+      const uint64_t t2 = fma2(pack2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])), sc2, e ? d4.y : d4.x);
+      float d0, d1;
+      unpack2(mul2(pack2(__uint_as_float(p[2 * i]), __uint_as_float(p[2 * i + 1])), t2), d0, d1);
+      dw[i] = bf16_pair(d0, d1);
+    }
+  }
 }
 
 // Writes one accumulator row (D fp32 columns of tensor memory, lane = row) to global memory.
-// The two threads of a row take alternate chunks of 32 columns (`half` = 0 or 1).
 template <int D>
-__device__ __forceinline__ void store_acc_row(uint32_t tAcc, void *dst_base, size_t elem_off, int out_f32, bool valid,
-                                              int half) {
+__device__ __forceinline__ void store_acc_row(uint32_t tAcc, void *dst_base, size_t elem_off, int out_f32, bool valid) {
 #pragma unroll
-  for (int cc = 0; cc < D / 64; ++cc) {
-    const int c = 2 * cc + half;
+  for (int c = 0; c < D / 32; ++c) {
     uint32_t a[32];
     tmem_ld_32x32b_x32(tAcc + c * 32, a);
     tmem_wait_ld();
@@ -225,14 +243,14 @@ __device__ __forceinline__ void store_acc_row(uint32_t tAcc, void *dst_base, siz
 // dK, dV: CTA = (128-key tile of one block, KV head)
 // ---------------------------------------------------------------------------------------------
 template <int D>
-__global__ void __launch_bounds__(kBwdThreads, 1)
+__global__ void __launch_bounds__(kDkvThreads, 1)
 ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_do,
                   const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
                   const BwdParams p) {
-  using L = BwdLayout<D>;
+  using L = DkvLayout<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  BwdCtrl *ctrl = reinterpret_cast<BwdCtrl *>(smem + L::kCtrl);
+  DkvCtrl *ctrl = reinterpret_cast<DkvCtrl *>(smem + L::kCtrl);
   const int tid = threadIdx.x, warp = tid >> 5;
   const ba_segments &sg = p.seg;
   if (__ldg(sg.totals + 7) != BA_TABLES_VALID) return;
@@ -267,31 +285,32 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
 
   if (tid == 0) {
     mbar_init(&ctrl->fix_full, 1); mbar_init(&ctrl->fin, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&ctrl->walk_full[i], 1); mbar_init(&ctrl->walk_free[i], 1);
-      mbar_init(&ctrl->sd_full[i], 1); mbar_init(&ctrl->rows_done[i], kRowThreads);
-    }
+    for (int i = 0; i < 2; ++i) { mbar_init(&ctrl->walk_full[i], 1); mbar_init(&ctrl->walk_free[i], 1); }
+    mbar_init(&ctrl->s_full, 1); mbar_init(&ctrl->dp_full, 1);
+    mbar_init(&ctrl->p_done, 256); mbar_init(&ctrl->ds_done, 256);
     ctrl->abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == kCtlWarp) { tmem_alloc(&ctrl->tmem_base, 512); tmem_relinquish(); }
+  if (warp == kDkvMmaWarp) { tmem_alloc(&ctrl->tmem_base, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctrl->tmem_base;
   volatile int *abort_flag = &ctrl->abort_flag;
-  // tensor memory: S^T buffers at columns 0 and 64, dP^T buffers at 128 and 192 (64 query rows each), dV, dK
   const uint32_t tST = tmem, tDPT = tmem + 128, tDV = tmem + 256, tDK = tmem + 384;
-  const int n_steps = 2 * n_iter;                        // step i: query rows 64 (i & 1) .. + 63 of tile i >> 1
 
-  if (warp == kCtlWarp) {
+  if (warp == kDkvLoadWarp) {
     if (elect_one()) {
-      constexpr uint32_t idesc_nt = make_idesc_bf16(128, 64, 0);                // both operands K-major, 64 query rows
-      constexpr uint32_t idesc_tn = make_idesc_bf16(128, D, 1);                 // A from tensor memory, B MN-major
-      const uint64_t k_desc = make_smem_desc(smem_u32(smem + L::kFix0), 16, 1024);
-      const uint64_t v_desc = make_smem_desc(smem_u32(smem + L::kFix1), 16, 1024);
+      mbar_arrive_expect_tx(&ctrl->fix_full, 2 * L::kTileBytes);
+      for (int c = 0; c < L::kChunks; ++c) {
+        tma_load_3d(smem + L::kFix0 + c * L::kRegion, &tmap_k, &ctrl->fix_full, c * 64, g, k0);
+        tma_load_3d(smem + L::kFix1 + c * L::kRegion, &tmap_v, &ctrl->fix_full, c * 64, g, k0);
+      }
       bool ok = true;
-      auto load_walk = [&](int it) {                     // Q and dO tiles of tile `it` into buffer it & 1
+      int it = 0;
+      for (; it < n_iter; ++it) {                        // Q and dO tiles of tile `it` into buffer it & 1
+        ok = mbar_wait(&ctrl->walk_free[it & 1], ((it >> 1) & 1) ^ 1, abort_flag);
+        if (!ok) break;
         int row0, row_end, head0; bool causal;
         iter_rows(it, row0, row_end, causal, head0);
         uint8_t *dst = smem + L::kWalk + (it & 1) * 2 * L::kTileBytes;
@@ -300,154 +319,175 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
           tma_load_3d(dst + c * L::kRegion, &tmap_q, &ctrl->walk_full[it & 1], c * 64, head0, row0);
           tma_load_3d(dst + L::kTileBytes + c * L::kRegion, &tmap_do, &ctrl->walk_full[it & 1], c * 64, head0, row0);
         }
-      };
-      // S^T = K Q^T and dP^T = V dO^T for the 64 query rows of step i.  They follow the gradient products of step
-      // i - 2 (same buffers) on the tensor pipe in issue order, so those have read P^T and dS^T before.
-      auto issue_scores = [&](int i) -> bool {
-        const int it = i >> 1, h = i & 1;
-        if (h == 0) {
-          if (!mbar_wait(&ctrl->walk_full[it & 1], (it >> 1) & 1, abort_flag)) return false;
-          tc_fence_after();
-        }
-        const uint32_t walk = smem_u32(smem + L::kWalk + (it & 1) * 2 * L::kTileBytes) + h * 64 * 128;   // rows 64 h ..
-        const uint64_t q_desc = make_smem_desc(walk, 16, 1024);
-        const uint64_t do_desc = make_smem_desc(walk + L::kTileBytes, 16, 1024);
-#pragma unroll
-        for (int k = 0; k < D / 16; ++k) {
-          const uint64_t off = (uint64_t)(((k >> 2) * L::kRegion + (k & 3) * 32) >> 4);
-          mma_ss(tST + (i & 1) * 64, k_desc + off, q_desc + off, idesc_nt, k > 0);
-        }
-#pragma unroll
-        for (int k = 0; k < D / 16; ++k) {
-          const uint64_t off = (uint64_t)(((k >> 2) * L::kRegion + (k & 3) * 32) >> 4);
-          mma_ss(tDPT + (i & 1) * 64, v_desc + off, do_desc + off, idesc_nt, k > 0);
-        }
-        mma_commit(&ctrl->sd_full[i & 1]);
-        return true;
-      };
-      // dV += P^T dO, dK += dS^T Q over the 64 query rows of step i (16 at a time)
-      auto issue_grads = [&](int i) -> bool {
-        const int it = i >> 1, h = i & 1;
-        if (!mbar_wait(&ctrl->rows_done[i & 1], (i >> 1) & 1, abort_flag)) return false;
-        tc_fence_after();
-        const uint32_t walk = smem_u32(smem + L::kWalk + (it & 1) * 2 * L::kTileBytes);
-        const uint64_t q_mn = make_smem_desc(walk, L::kRegion, 1024);
-        const uint64_t do_mn = make_smem_desc(walk + L::kTileBytes, L::kRegion, 1024);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_ts(tDV, tST + (i & 1) * 64 + (k >> 1) * 32 + (k & 1) * 8, do_mn + (uint64_t)(((h * 64 + k * 16) * 128) >> 4), idesc_tn,
-                 (i > 0 || k > 0) ? 1u : 0u);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_ts(tDK, tDPT + (i & 1) * 64 + (k >> 1) * 32 + (k & 1) * 8, q_mn + (uint64_t)(((h * 64 + k * 16) * 128) >> 4), idesc_tn,
-                 (i > 0 || k > 0) ? 1u : 0u);
-        if (h == 1) mma_commit(&ctrl->walk_free[it & 1]);   // the tile's Q and dO have been read for the last time
-        return true;
-      };
-      mbar_arrive_expect_tx(&ctrl->fix_full, 2 * L::kTileBytes);
-      for (int c = 0; c < L::kChunks; ++c) {
-        tma_load_3d(smem + L::kFix0 + c * L::kRegion, &tmap_k, &ctrl->fix_full, c * 64, g, k0);
-        tma_load_3d(smem + L::kFix1 + c * L::kRegion, &tmap_v, &ctrl->fix_full, c * 64, g, k0);
       }
-      if (n_iter > 0) load_walk(0);
-      if (n_iter > 1) load_walk(1);
-      ok = mbar_wait(&ctrl->fix_full, 0, abort_flag);
-      int reload = -1;                                   // tile whose buffer is refilled once its products have completed
-      for (int i = 0; i <= n_steps && ok; ++i) {
-        if (i < n_steps) ok = issue_scores(i);
-        if (ok && reload >= 0) {
-          if (reload + 2 < n_iter) {
-            ok = mbar_wait(&ctrl->walk_free[reload & 1], (reload >> 1) & 1, abort_flag);
-            if (ok) load_walk(reload + 2);
-          }
-          reload = -1;
+      if (!ok) {                                         // leave no copy in flight: wait (bounded) for those already requested
+        for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(&ctrl->fix_full, 0); ++spin) { }
+        for (int k = max(0, it - 2); k < it; ++k)
+          for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(&ctrl->walk_full[k & 1], (k >> 1) & 1); ++spin) { }
+      }
+    }
+  } else if (warp == kDkvMmaWarp) {
+    if (elect_one()) {
+      constexpr uint32_t idesc_nt = make_idesc_bf16(128, kTile, 0);             // both operands K-major
+      constexpr uint32_t idesc_tn = make_idesc_bf16(128, D, 1);                 // A from tensor memory, B MN-major
+      const uint64_t k_desc = make_smem_desc(smem_u32(smem + L::kFix0), 16, 1024);
+      const uint64_t v_desc = make_smem_desc(smem_u32(smem + L::kFix1), 16, 1024);
+      // scores of the tile in walk buffer `buf`: S^T = K Q^T (which = 0) or dP^T = V dO^T (1)
+      auto issue_scores = [&](int buf, int which) {
+        const uint64_t a_desc = which ? v_desc : k_desc;
+        const uint64_t b_desc = make_smem_desc(smem_u32(smem + L::kWalk + (buf * 2 + which) * L::kTileBytes), 16, 1024);
+#pragma unroll
+        for (int k = 0; k < D / 16; ++k) {
+          const uint64_t off = (uint64_t)(((k >> 2) * L::kRegion + (k & 3) * 32) >> 4);
+          mma_ss(which ? tDPT : tST, a_desc + off, b_desc + off, idesc_nt, k > 0);
         }
-        if (ok && i > 0) {
-          ok = issue_grads(i - 1);
-          if ((i - 1) & 1) reload = (i - 1) >> 1;
+        mma_commit(which ? &ctrl->dp_full : &ctrl->s_full);
+      };
+      // gradients: dV += P^T dO (which = 0) or dK += dS^T Q (1), 16 query rows at a time
+      auto issue_grads = [&](int buf, int which, bool first) {
+        const uint64_t b_mn = make_smem_desc(smem_u32(smem + L::kWalk + (buf * 2 + (which ^ 1)) * L::kTileBytes), L::kRegion, 1024);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          mma_ts(which ? tDK : tDV, (which ? tDPT : tST) + (k >> 2) * 64 + (k & 3) * 8, b_mn + (uint64_t)((k * 16 * 128) >> 4), idesc_tn,
+                 (!first || k > 0) ? 1u : 0u);
+      };
+      bool ok = mbar_wait(&ctrl->fix_full, 0, abort_flag);
+      if (ok && n_iter > 0) ok = mbar_wait(&ctrl->walk_full[0], 0, abort_flag);
+      if (ok && n_iter > 0) { tc_fence_after(); issue_scores(0, 0); issue_scores(0, 1); }
+      for (int it = 0; it < n_iter && ok; ++it) {
+        const int buf = it & 1;
+        const bool more = it + 1 < n_iter;
+        // the next tile's S^T follows dV on the tensor pipe (P^T has been read then) and runs while the threads form dS^T;
+        // its dP^T follows dK and runs while they form the next P^T
+        ok = mbar_wait(&ctrl->p_done, it & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        issue_grads(buf, 0, it == 0);
+        if (more) {
+          ok = mbar_wait(&ctrl->walk_full[buf ^ 1], ((it + 1) >> 1) & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          issue_scores(buf ^ 1, 0);
         }
+        ok = mbar_wait(&ctrl->ds_done, it & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        issue_grads(buf, 1, it == 0);
+        mma_commit(&ctrl->walk_free[buf]);
+        if (more) issue_scores(buf ^ 1, 1);
       }
       if (ok) mma_commit(&ctrl->fin);
     }
   } else {
     const int j = tid & 127;                             // key of the tile = tensor-memory lane
-    const int ch = tid >> 7;                             // which 32 of a step's 64 columns this thread takes
+    const int h = warp >> 2;                             // this thread's half of every tile: query rows 64 h .. + 63
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-    // per query row of the tile, two buffers: lse * log2 e [128], dO . O * scale [128], visible keys [128]
-    float *st_lse = reinterpret_cast<float *>(smem + L::kStats);
-    float *st_dls = st_lse + 2 * 128;
-    int *st_lim = reinterpret_cast<int *>(st_dls + 2 * 128);
-    bool ok = true;
-    for (int i = 0; i < n_steps; ++i) {
-      const int it = i >> 1, h = i & 1;
+    float *stats = reinterpret_cast<float *>(smem + L::kStats);
+    // thread tid < 128 fetches what the keys need to know about query row `tid`, one tile ahead
+    float n_lse = 0.f, n_dls = 0.f; int n_lim = 0;
+    auto fetch_stats = [&](int it) {
       int row0, row_end, head0; bool causal;
       iter_rows(it, row0, row_end, causal, head0);
-      if (h == 0) {
-        if (tid < 128) {
-          // this thread also prepares what every key thread needs to know about query row `tid` of the tile
-          const int tok_i = row0 + (tid >> p.hpt_log2);
-          const int head = head0 + (tid & (p.hpt - 1));
-          float l2 = 0.f, dl = 0.f; int lm = 0;
-          if (tok_i < row_end) {
-            l2 = __ldg(p.lse + (size_t)tok_i * p.Hq + head) * 1.4426950408889634f;
-            dl = __ldg(p.delta + (size_t)tok_i * p.Hq + head) * p.scale;
-            lm = causal ? max(0, min(n_keys, tok_i - k0 + 1)) : n_keys;      // keys 0 .. lm - 1 of the tile are visible
-          }
-          st_lse[(it & 1) * 128 + tid] = l2; st_dls[(it & 1) * 128 + tid] = dl; st_lim[(it & 1) * 128 + tid] = lm;
-        }
-        named_barrier_rows();
+      const int tok_i = row0 + (tid >> p.hpt_log2);
+      const int head = head0 + (tid & (p.hpt - 1));
+      n_lse = 0.f; n_dls = 0.f; n_lim = 0;
+      if (tok_i < row_end) {
+        n_lse = __ldg(p.lse + (size_t)tok_i * p.Hq + head);                    // (used a tile later: nothing waits for them here)
+        n_dls = __ldg(p.delta + (size_t)tok_i * p.Hq + head);
+        n_lim = causal ? max(0, min(n_keys, tok_i - k0 + 1)) : n_keys;         // keys 0 .. n_lim - 1 of the tile are visible
       }
-      // every pair of this step visible?  (all 128 keys exist, the step's rows exist and, in the causal range,
-      // already its first row sees the tile's last key)
+    };
+    if (tid < 128 && n_iter > 0) fetch_stats(0);
+    bool ok = true;
+    for (int it = 0; it < n_iter; ++it) {
+      float *st = stats + (it & 1) * 3 * 128;
+      if (tid < 128) {
+        st[tid] = n_lse * -1.4426950408889634f; st[128 + tid] = -n_dls * p.scale; reinterpret_cast<int *>(st)[256 + tid] = n_lim;
+        if (it + 1 < n_iter) fetch_stats(it + 1);
+      }
+      row_warps_barrier();
+      int row0, row_end, head0; bool causal;
+      iter_rows(it, row0, row_end, causal, head0);
+      // every pair of this thread's half visible?  (all 128 keys exist, the rows exist and, in the causal range,
+      // already the first one sees the tile's last key)
       const int tok_first = row0 + ((h * 64) >> p.hpt_log2), tok_last = row0 + ((h * 64 + 63) >> p.hpt_log2);
       const bool all_visible = n_keys == kTile && tok_last < row_end && (!causal || tok_first - k0 + 1 >= kTile);
-      ok = mbar_wait(&ctrl->sd_full[i & 1], (i >> 1) & 1, abort_flag);
+      const uint32_t a = tST + h * 64 + lane_off, d = tDPT + h * 64 + lane_off;
+      const float *lse = st + h * 64, *dls = st + 128 + h * 64;
+      const int *lim = reinterpret_cast<const int *>(st) + 256 + h * 64;
+      uint32_t s[64], w[16];
+      ok = mbar_wait(&ctrl->s_full, it & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
-      const int so = (it & 1) * 128 + h * 64;
-      if (all_visible)
-        bwd_key_p_ds<false>(tST + (i & 1) * 64 + lane_off, tDPT + (i & 1) * 64 + lane_off, ch, j, st_lse + so, st_dls + so,
-                            st_lim + so, p.scale_log2, p.scale);
-      else
-        bwd_key_p_ds<true>(tST + (i & 1) * 64 + lane_off, tDPT + (i & 1) * 64 + lane_off, ch, j, st_lse + so, st_dls + so,
-                           st_lim + so, p.scale_log2, p.scale);
+      // P^T as bf16 over the S^T columns the thread has read, two per column: the A operand of dV
+      auto form_p = [&](auto masked) {
+        constexpr bool kMasked = decltype(masked)::value;
+        tmem_ld_32x32b_x32(a, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+        tmem_wait_ld();
+        tmem_ld_32x32b_x32(a + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+        dkv_p<kMasked>(s, w, j, lse, lim, p.scale_log2);
+        tmem_st16(a, w);
+        tmem_wait_ld();
+        dkv_p<kMasked>(s + 32, w, j, lse + 32, lim + 32, p.scale_log2);
+        tmem_st16(a + 16, w);
+        tmem_wait_st();
+      };
+      if (all_visible) form_p(std::false_type{});
+      else form_p(std::true_type{});
       tc_fence_before();
-      mbar_arrive(&ctrl->rows_done[i & 1]);
+      mbar_arrive(&ctrl->p_done);
+      ok = mbar_wait(&ctrl->dp_full, it & 1, abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t d0[32], d1[32];
+      tmem_ld_32x32b_x32(d, d0);
+      tmem_wait_ld();
+      tmem_ld_32x32b_x32(d + 32, d1);
+      dkv_ds(s, d0, w, dls, p.scale);
+      tmem_st16(d, w);
+      tmem_wait_ld();
+      dkv_ds(s + 32, d1, w, dls + 32, p.scale);
+      tmem_st16(d + 16, w);
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive(&ctrl->ds_done);
     }
-    // accumulators: lane = key row of the tile
+    // accumulators: lane = key row of the tile; one thread of a key writes dV, the other dK
     if (ok && n_iter > 0) ok = mbar_wait(&ctrl->fin, 0, abort_flag);
     if (ok && n_iter > 0) {
       tc_fence_after();
-      const bool valid = j < n_keys;
-      const size_t off = ((size_t)(k0 + j) * p.Hkv + g) * D;
-      store_acc_row<D>(tDV + lane_off, p.dv, off, p.out_f32, valid, ch);
-      store_acc_row<D>(tDK + lane_off, p.dk, off, p.out_f32, valid, ch);
+      store_acc_row<D>((h ? tDK : tDV) + lane_off, h ? p.dk : p.dv, ((size_t)(k0 + j) * p.Hkv + g) * D, p.out_f32, j < n_keys);
     }
   }
   tc_fence_before();
   __syncthreads();
   if (tid == 0 && ctrl->abort_flag) ba_record_status(p.status, BA_ERR_TIMEOUT);
-  if (warp == kCtlWarp) tmem_dealloc(tmem, 512);
+  if (warp == kDkvMmaWarp) tmem_dealloc(tmem, 512);
 }
 
 // ---------------------------------------------------------------------------------------------
 // dQ: CTA = (query tile of `tok` tokens x `hpt` heads, head chunk)
 // ---------------------------------------------------------------------------------------------
+// Two CTAs share an SM (half of the shared memory and 256 of the 512 tensor-memory columns each): while the threads of
+// one turn scores into dS, the tensor core works for the other, and one's start-up and write-out hide under the
+// other's products.
 template <int D>
-__global__ void __launch_bounds__(kBwdThreads, 1)
+__global__ void __launch_bounds__(kDqThreads, 2)
 ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_do,
                  const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
-                 const BwdParams p) {
-  using L = BwdLayout<D>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  BwdCtrl *ctrl = reinterpret_cast<BwdCtrl *>(smem + L::kCtrl);
+                 const BwdParams p, int n_tiles_upper, int n_head_chunks) {
+  using L = DqLayout<D>;
+  extern __shared__ __align__(1024) uint8_t smem_dq[];
+  uint8_t *smem = smem_dq;
+  DqCtrl *ctrl = reinterpret_cast<DqCtrl *>(smem + L::kCtrl);
   const int tid = threadIdx.x, warp = tid >> 5;
   const ba_segments &sg = p.seg;
   if (__ldg(sg.totals + 7) != BA_TABLES_VALID) return;
 
-  // query tile: half `blockIdx.x & 1` of query-tile pair `blockIdx.x >> 1` (the pairs of the forward kernel)
-  const int pair = blockIdx.x >> 1, half = blockIdx.x & 1;
+  // query tile: one half of a query-tile pair of the forward kernel.  Tiles are taken from the end of the list (within a
+  // sequence the last ones see the most keys), all head chunks of a tile side by side.
+  const int qt = n_tiles_upper - 1 - (int)blockIdx.x / n_head_chunks;
+  const int pair = qt >> 1, half = qt & 1;
   if (pair >= __ldg(sg.totals + 2)) return;
   const int b = upper_bound_dev(sg.cu_qtile, sg.n_blocks + 1, pair) - 1;
   const int blk0 = __ldg(sg.cu_block + b), blk1 = __ldg(sg.cu_block + b + 1);
@@ -455,140 +495,163 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
   if (q0 >= blk1) return;
   const int q_end = min(q0 + p.tok, blk1);                // rows q0 .. q_end - 1
   const int kv0 = __ldg(sg.block_kv_begin + b);           // row i sees keys kv0 .. i
-  const int head0 = blockIdx.y * p.hpt, g = head0 / p.G;
-  const int n_iter = (q_end - kv0 + kTile - 1) / kTile;   // key tiles kv0 + 128 j
-  const int n_steps = (q_end - kv0 + 63) / 64;            // step i: keys kv0 + 64 i .. + 63 (half of tile i >> 1)
+  const int head0 = ((int)blockIdx.x % n_head_chunks) * p.hpt, g = head0 / p.G;
+  const int n_steps = (q_end - kv0 + kStep - 1) / kStep;  // step i: keys kv0 + 64 i .. + 63
 
   if (tid == 0) {
     mbar_init(&ctrl->fix_full, 1); mbar_init(&ctrl->fin, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&ctrl->walk_full[i], 1); mbar_init(&ctrl->walk_free[i], 1);
-      mbar_init(&ctrl->sd_full[i], 1); mbar_init(&ctrl->rows_done[i], kRowThreads);
-    }
+    for (int i = 0; i < 2; ++i) { mbar_init(&ctrl->k_full[i], 1); mbar_init(&ctrl->k_free[i], 1); }
+    mbar_init(&ctrl->v_full, 1); mbar_init(&ctrl->v_free, 1);
+    mbar_init(&ctrl->sd_full, 1); mbar_init(&ctrl->s_read, 128); mbar_init(&ctrl->rows_done, 128);
     ctrl->abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == kCtlWarp) { tmem_alloc(&ctrl->tmem_base, 512); tmem_relinquish(); }
+  if (warp == kDqMmaWarp) { tmem_alloc(&ctrl->tmem_base, 256); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctrl->tmem_base;
   volatile int *abort_flag = &ctrl->abort_flag;
-  // tensor memory: S buffers at columns 0 and 64, dP buffers at 128 and 192 (64 keys each), dQ
-  const uint32_t tS = tmem, tDP = tmem + 128, tDQ = tmem + 256;
+  const uint32_t tS = tmem, tDP = tmem + 64, tDQ = tmem + 128;   // S and dP of one step (64 keys each), dQ
 
-  if (warp == kCtlWarp) {
+  if (warp == kDqLoadWarp) {
     if (elect_one()) {
-      constexpr uint32_t idesc_nt = make_idesc_bf16(128, 64, 0);
-      constexpr uint32_t idesc_nn = make_idesc_bf16(128, D, 1);                 // A from tensor memory (dS), B MN-major (K)
-      const uint64_t q_desc = make_smem_desc(smem_u32(smem + L::kFix0), 16, 1024);
-      const uint64_t do_desc = make_smem_desc(smem_u32(smem + L::kFix1), 16, 1024);
-      bool ok = true;
-      auto load_walk = [&](int it) {                     // K and V tiles of key tile `it` into buffer it & 1
-        uint8_t *dst = smem + L::kWalk + (it & 1) * 2 * L::kTileBytes;
-        mbar_arrive_expect_tx(&ctrl->walk_full[it & 1], 2 * L::kTileBytes);
-        for (int c = 0; c < L::kChunks; ++c) {
-          tma_load_3d(dst + c * L::kRegion, &tmap_k, &ctrl->walk_full[it & 1], c * 64, g, kv0 + it * kTile);
-          tma_load_3d(dst + L::kTileBytes + c * L::kRegion, &tmap_v, &ctrl->walk_full[it & 1], c * 64, g, kv0 + it * kTile);
-        }
-      };
-      auto issue_scores = [&](int i) -> bool {           // S = Q K^T, dP = dO V^T for the 64 keys of step i
-        const int it = i >> 1, h = i & 1;
-        if (h == 0) {
-          if (!mbar_wait(&ctrl->walk_full[it & 1], (it >> 1) & 1, abort_flag)) return false;
-          tc_fence_after();
-        }
-        const uint32_t walk = smem_u32(smem + L::kWalk + (it & 1) * 2 * L::kTileBytes) + h * 64 * 128;   // keys 64 h ..
-        const uint64_t k_desc = make_smem_desc(walk, 16, 1024);
-        const uint64_t v_desc = make_smem_desc(walk + L::kTileBytes, 16, 1024);
-#pragma unroll
-        for (int k = 0; k < D / 16; ++k) {
-          const uint64_t off = (uint64_t)(((k >> 2) * L::kRegion + (k & 3) * 32) >> 4);
-          mma_ss(tS + (i & 1) * 64, q_desc + off, k_desc + off, idesc_nt, k > 0);
-        }
-#pragma unroll
-        for (int k = 0; k < D / 16; ++k) {
-          const uint64_t off = (uint64_t)(((k >> 2) * L::kRegion + (k & 3) * 32) >> 4);
-          mma_ss(tDP + (i & 1) * 64, do_desc + off, v_desc + off, idesc_nt, k > 0);
-        }
-        mma_commit(&ctrl->sd_full[i & 1]);
-        return true;
-      };
-      auto issue_grads = [&](int i) -> bool {            // dQ += dS K over the 64 keys of step i (16 at a time)
-        const int it = i >> 1, h = i & 1;
-        if (!mbar_wait(&ctrl->rows_done[i & 1], (i >> 1) & 1, abort_flag)) return false;
-        tc_fence_after();
-        const uint64_t k_mn = make_smem_desc(smem_u32(smem + L::kWalk + (it & 1) * 2 * L::kTileBytes), L::kRegion, 1024);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_ts(tDQ, tDP + (i & 1) * 64 + (k >> 1) * 32 + (k & 1) * 8, k_mn + (uint64_t)(((h * 64 + k * 16) * 128) >> 4), idesc_nn,
-                 (i > 0 || k > 0) ? 1u : 0u);
-        if (h == 1 || i + 1 == n_steps) mma_commit(&ctrl->walk_free[it & 1]);   // last use of the tile's K and V
-        return true;
-      };
       mbar_arrive_expect_tx(&ctrl->fix_full, 2 * L::kTileBytes);
       for (int c = 0; c < L::kChunks; ++c) {
-        tma_load_3d(smem + L::kFix0 + c * L::kRegion, &tmap_q, &ctrl->fix_full, c * 64, head0, q0);
-        tma_load_3d(smem + L::kFix1 + c * L::kRegion, &tmap_do, &ctrl->fix_full, c * 64, head0, q0);
+        tma_load_3d(smem + L::kQ + c * L::kRegion, &tmap_q, &ctrl->fix_full, c * 64, head0, q0);
+        tma_load_3d(smem + L::kDo + c * L::kRegion, &tmap_do, &ctrl->fix_full, c * 64, head0, q0);
       }
-      if (n_iter > 0) load_walk(0);
-      if (n_iter > 1) load_walk(1);
-      ok = mbar_wait(&ctrl->fix_full, 0, abort_flag);
-      int reload = -1;                                   // key tile whose buffer is refilled once its products have completed
-      for (int i = 0; i <= n_steps && ok; ++i) {
-        if (i < n_steps) ok = issue_scores(i);
-        if (ok && reload >= 0) {
-          if (reload + 2 < n_iter) {
-            ok = mbar_wait(&ctrl->walk_free[reload & 1], (reload >> 1) & 1, abort_flag);
-            if (ok) load_walk(reload + 2);
-          }
-          reload = -1;
+      bool ok = true;
+      int nk = 0, nv = 0;                                // tiles of K and V requested so far
+      for (int i = 0; i < n_steps; ++i) {
+        ok = mbar_wait(&ctrl->k_free[i & 1], ((i >> 1) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        mbar_arrive_expect_tx(&ctrl->k_full[i & 1], L::kKeyBytes);
+        for (int c = 0; c < L::kChunks; ++c)
+          tma_load_3d(smem + L::kK + (i & 1) * L::kKeyBytes + c * L::kKeyRegion, &tmap_k, &ctrl->k_full[i & 1], c * 64, g, kv0 + i * kStep);
+        ++nk;
+        ok = mbar_wait(&ctrl->v_free, (i & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        mbar_arrive_expect_tx(&ctrl->v_full, L::kKeyBytes);
+        for (int c = 0; c < L::kChunks; ++c)
+          tma_load_3d(smem + L::kV + c * L::kKeyRegion, &tmap_v, &ctrl->v_full, c * 64, g, kv0 + i * kStep);
+        ++nv;
+      }
+      if (!ok) {                                         // leave no copy in flight: wait (bounded) for those already requested
+        for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(&ctrl->fix_full, 0); ++spin) { }
+        for (int k = max(0, nk - 2); k < nk; ++k)
+          for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(&ctrl->k_full[k & 1], (k >> 1) & 1); ++spin) { }
+        if (nv > 0)
+          for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(&ctrl->v_full, (nv - 1) & 1); ++spin) { }
+      }
+    }
+  } else if (warp == kDqMmaWarp) {
+    if (elect_one()) {
+      constexpr uint32_t idesc_nt = make_idesc_bf16(128, kStep, 0);
+      constexpr uint32_t idesc_nn = make_idesc_bf16(128, D, 1);                 // A from tensor memory (dS), B MN-major (K)
+      const uint64_t q_desc = make_smem_desc(smem_u32(smem + L::kQ), 16, 1024);
+      const uint64_t do_desc = make_smem_desc(smem_u32(smem + L::kDo), 16, 1024);
+      const uint64_t v_desc = make_smem_desc(smem_u32(smem + L::kV), 16, 1024);
+      auto issue_s = [&](int i) -> bool {                // S = Q K^T for the 64 keys of step i
+        if (!mbar_wait(&ctrl->k_full[i & 1], (i >> 1) & 1, abort_flag)) return false;
+        tc_fence_after();
+        const uint64_t k_desc = make_smem_desc(smem_u32(smem + L::kK + (i & 1) * L::kKeyBytes), 16, 1024);
+#pragma unroll
+        for (int k = 0; k < D / 16; ++k) {
+          const uint64_t qo = (uint64_t)(((k >> 2) * L::kRegion + (k & 3) * 32) >> 4);
+          const uint64_t ko = (uint64_t)(((k >> 2) * L::kKeyRegion + (k & 3) * 32) >> 4);
+          mma_ss(tS, q_desc + qo, k_desc + ko, idesc_nt, k > 0);
         }
-        if (ok && i > 0) {
-          ok = issue_grads(i - 1);
-          if ((i - 1) & 1) reload = (i - 1) >> 1;
+        return true;
+      };
+      auto issue_dp = [&](int i) -> bool {               // dP = dO V^T
+        if (!mbar_wait(&ctrl->v_full, i & 1, abort_flag)) return false;
+        tc_fence_after();
+#pragma unroll
+        for (int k = 0; k < D / 16; ++k) {
+          const uint64_t qo = (uint64_t)(((k >> 2) * L::kRegion + (k & 3) * 32) >> 4);
+          const uint64_t vo = (uint64_t)(((k >> 2) * L::kKeyRegion + (k & 3) * 32) >> 4);
+          mma_ss(tDP, do_desc + qo, v_desc + vo, idesc_nt, k > 0);
         }
+        mma_commit(&ctrl->sd_full);
+        mma_commit(&ctrl->v_free);
+        return true;
+      };
+      bool ok = mbar_wait(&ctrl->fix_full, 0, abort_flag);
+      if (ok && n_steps > 0) ok = issue_s(0) && issue_dp(0);
+      for (int i = 0; i < n_steps && ok; ++i) {
+        // the next step's S is formed while the threads still work on this step: they hold S in registers
+        if (i + 1 < n_steps) {
+          ok = mbar_wait(&ctrl->s_read, i & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          ok = issue_s(i + 1);
+          if (!ok) break;
+        }
+        ok = mbar_wait(&ctrl->rows_done, i & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t k_mn = make_smem_desc(smem_u32(smem + L::kK + (i & 1) * L::kKeyBytes), L::kKeyRegion, 1024);
+#pragma unroll
+        for (int k = 0; k < kStep / 16; ++k)             // dQ += dS K, 16 keys at a time
+          mma_ts(tDQ, tDP + k * 8, k_mn + (uint64_t)((k * 16 * 128) >> 4), idesc_nn, (i > 0 || k > 0) ? 1u : 0u);
+        mma_commit(&ctrl->k_free[i & 1]);
+        if (i + 1 < n_steps) ok = issue_dp(i + 1);       // (behind dQ on the tensor pipe: dS has been read)
       }
       if (ok) mma_commit(&ctrl->fin);
     }
   } else {
-    const int r = tid & 127;                             // row of the query tile = tensor-memory lane
-    const int ch = tid >> 7;                             // which 32 of a step's 64 columns this thread takes
-    const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
+    const int r = tid;                                   // row of the query tile = tensor-memory lane
+    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
     const int tok_i = q0 + (r >> p.hpt_log2);
     const int head = head0 + (r & (p.hpt - 1));
     const bool row_ok = tok_i < q_end;
-    float lse2 = 0.f, dl = 0.f;
+    float nlse = 0.f, ndl = 0.f;
     if (row_ok) {
-      lse2 = __ldg(p.lse + (size_t)tok_i * p.Hq + head) * 1.4426950408889634f;
-      dl = __ldg(p.delta + (size_t)tok_i * p.Hq + head) * p.scale;
+      nlse = __ldg(p.lse + (size_t)tok_i * p.Hq + head) * -1.4426950408889634f;
+      ndl = -__ldg(p.delta + (size_t)tok_i * p.Hq + head) * p.scale;
     }
     bool ok = true;
     for (int i = 0; i < n_steps; ++i) {
-      const int kr = kv0 + i * 64;
-      const int n_ok = row_ok ? max(0, min(64, tok_i - kr + 1)) : 0;
+      const int kr = kv0 + i * kStep;
+      const int n_ok = row_ok ? max(0, min(kStep, tok_i - kr + 1)) : 0;
       // every pair of this step visible?  (every row of the tile exists and already the first one sees the step's last key)
-      const bool all_visible = q0 + p.tok <= q_end && q0 - kr + 1 >= 64;
-      ok = mbar_wait(&ctrl->sd_full[i & 1], (i >> 1) & 1, abort_flag);
+      const bool all_visible = q0 + p.tok <= q_end && q0 - kr + 1 >= kStep;
+      ok = mbar_wait(&ctrl->sd_full, i & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
-      if (all_visible)
-        bwd_row_ds<false>(tS + (i & 1) * 64 + lane_off, tDP + (i & 1) * 64 + lane_off, ch, n_ok, p.scale_log2, lse2, dl, p.scale);
-      else
-        bwd_row_ds<true>(tS + (i & 1) * 64 + lane_off, tDP + (i & 1) * 64 + lane_off, ch, n_ok, p.scale_log2, lse2, dl, p.scale);
+      auto step = [&](auto masked) {
+        constexpr bool kMasked = decltype(masked)::value;
+        uint32_t s[64], d0[32], d1[32], dw[16];
+        tmem_ld_32x32b_x32(tS + lane_off, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+        tmem_ld_32x32b_x32(tS + lane_off + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+        tmem_ld_32x32b_x32(tDP + lane_off, d0);
+        tmem_wait_ld();
+        tc_fence_before();
+        mbar_arrive(&ctrl->s_read);
+        tmem_ld_32x32b_x32(tDP + lane_off + 32, d1);
+        bwd_row_ds<kMasked>(s, d0, dw, n_ok, p.scale_log2, nlse, ndl, p.scale);
+        tmem_st16(tDP + lane_off, dw);                   // dS as bf16 over the dP columns that have been read
+        tmem_wait_ld();
+        bwd_row_ds<kMasked>(s + 32, d1, dw, n_ok - 32, p.scale_log2, nlse, ndl, p.scale);
+        tmem_st16(tDP + lane_off + 16, dw);
+        tmem_wait_st();
+      };
+      if (all_visible) step(std::false_type{});
+      else step(std::true_type{});
       tc_fence_before();
-      mbar_arrive(&ctrl->rows_done[i & 1]);
+      mbar_arrive(&ctrl->rows_done);
     }
     if (ok && n_steps > 0) ok = mbar_wait(&ctrl->fin, 0, abort_flag);
     if (ok && n_steps > 0) {
       tc_fence_after();
-      store_acc_row<D>(tDQ + lane_off, p.dq, ((size_t)tok_i * p.Hq + head) * D, p.out_f32, row_ok, ch);
+      store_acc_row<D>(tDQ + lane_off, p.dq, ((size_t)tok_i * p.Hq + head) * D, p.out_f32, row_ok);
     }
   }
   tc_fence_before();
   __syncthreads();
   if (tid == 0 && ctrl->abort_flag) ba_record_status(p.status, BA_ERR_TIMEOUT);
-  if (warp == kCtlWarp) tmem_dealloc(tmem, 512);
+  if (warp == kDqMmaWarp) tmem_dealloc(tmem, 256);
 }
 
 // delta[row, head] = dO . O: D / 8 threads per (row, head), each with one 16-byte vector of both operands
@@ -640,13 +703,14 @@ bool bwd_make_map(CUtensorMap *m, const void *ptr, int D, int heads, long long r
 }
 
 template <int D>
-ba_status launch_bwd(ba_ctx *ctx, const BwdParams &p, const CUtensorMap &tq, const CUtensorMap &tdo,
-                     const CUtensorMap &tk, const CUtensorMap &tv, int n_ktiles_upper, int n_pairs_upper,
+ba_status launch_bwd(ba_ctx *ctx, const BwdParams &p, const CUtensorMap &tq, const CUtensorMap &tdo, const CUtensorMap &tk,
+                     const CUtensorMap &tv, const CUtensorMap &tk64, const CUtensorMap &tv64, int n_ktiles_upper, int n_pairs_upper,
                      cudaStream_t stream) {
-  const int smem = BwdLayout<D>::kBytes + 1024;
-  ba_bwd_dkv_kernel<D><<<dim3((unsigned)n_ktiles_upper, (unsigned)p.Hkv), kBwdThreads, smem, stream>>>(tq, tdo, tk, tv, p);
+  ba_bwd_dkv_kernel<D><<<dim3((unsigned)n_ktiles_upper, (unsigned)p.Hkv), kDkvThreads, DkvLayout<D>::kBytes + 1024, stream>>>(tq, tdo, tk, tv, p);
   BA_CUDA_TRY(cudaGetLastError());
-  ba_bwd_dq_kernel<D><<<dim3((unsigned)(2 * n_pairs_upper), (unsigned)(p.Hq / p.hpt)), kBwdThreads, smem, stream>>>(tq, tdo, tk, tv, p);
+  const int n_head_chunks = p.Hq / p.hpt;
+  ba_bwd_dq_kernel<D><<<(unsigned)(2 * n_pairs_upper) * n_head_chunks, kDqThreads, DqLayout<D>::kBytes, stream>>>(
+      tq, tdo, tk64, tv64, p, 2 * n_pairs_upper, n_head_chunks);
   BA_CUDA_TRY(cudaGetLastError());
   ctx->launches += 2;
   return BA_OK;
@@ -656,10 +720,10 @@ ba_status launch_bwd(ba_ctx *ctx, const BwdParams &p, const CUtensorMap &tq, con
 
 // Per-context set-up (device current): the kernels' shared-memory limit is raised once.
 ba_status ba_bwd_sm100_setup(ba_ctx *) {
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dkv_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdLayout<128>::kBytes + 1024));
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dq_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdLayout<128>::kBytes + 1024));
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dkv_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdLayout<64>::kBytes + 1024));
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dq_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdLayout<64>::kBytes + 1024));
+  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dkv_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DkvLayout<128>::kBytes + 1024));
+  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dq_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqLayout<128>::kBytes));
+  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dkv_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DkvLayout<64>::kBytes + 1024));
+  BA_CUDA_TRY(cudaFuncSetAttribute(ba_bwd_dq_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqLayout<64>::kBytes));
   return BA_OK;
 }
 
@@ -693,12 +757,13 @@ ba_status ba_bwd_sm100_launch(ba_ctx *ctx, const void *q, const void *k, const v
         (const __nv_bfloat16 *)o, (const __nv_bfloat16 *)d_o, delta, n_rh);
   BA_CUDA_TRY(cudaGetLastError());
   ctx->launches += 1;
-  CUtensorMap tq, tdo, tk, tv;
+  CUtensorMap tq, tdo, tk, tv, tk64, tv64;
   if (!bwd_make_map(&tq, q, D, Hq, T, p.hpt, p.tok) || !bwd_make_map(&tdo, d_o, D, Hq, T, p.hpt, p.tok) ||
-      !bwd_make_map(&tk, k, D, Hkv, T, 1, kTile) || !bwd_make_map(&tv, v, D, Hkv, T, 1, kTile))
+      !bwd_make_map(&tk, k, D, Hkv, T, 1, kTile) || !bwd_make_map(&tv, v, D, Hkv, T, 1, kTile) ||
+      !bwd_make_map(&tk64, k, D, Hkv, T, 1, kStep) || !bwd_make_map(&tv64, v, D, Hkv, T, 1, kStep))
     return BA_ERR_CUDA;
   const int n_ktiles_upper = T / kTile + seg->n_blocks;
   const int n_pairs_upper = seg->n_prompt_items > 0 ? seg->n_prompt_items : T / (2 * p.tok) + seg->n_blocks;
-  if (D == 128) return launch_bwd<128>(ctx, p, tq, tdo, tk, tv, n_ktiles_upper, n_pairs_upper, stream);
-  return launch_bwd<64>(ctx, p, tq, tdo, tk, tv, n_ktiles_upper, n_pairs_upper, stream);
+  if (D == 128) return launch_bwd<128>(ctx, p, tq, tdo, tk, tv, tk64, tv64, n_ktiles_upper, n_pairs_upper, stream);
+  return launch_bwd<64>(ctx, p, tq, tdo, tk, tv, tk64, tv64, n_ktiles_upper, n_pairs_upper, stream);
 }
