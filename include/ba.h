@@ -123,6 +123,12 @@ typedef struct {
   /* rotation of every cached block, used by ba_final_attend_fused: (cos, sin)(cache_delta[c] * theta_m),
    * fp32 from fp64 angles, [Bc][head_dim / 2][2] */
   float *cache_rope;
+  /* work items of the attention kernels (not part of the bit-exact contract), 8 ints each: first query row, query rows,
+   * first own key row, first cached row, cached rows, first cached block, its first key tile, cached key tiles */
+  int32_t *prompt_items;   /* [totals[2]] items of ba_block_prefill */
+  int32_t *final_items;    /* [totals[3]] items of ba_final_attend */
+  int32_t *cu_stream;      /* [2][batch+1] prefix sums over sequences of the key tiles the items of its final block see:
+                            * cached keys packed, then block by block */
 } ba_segments;
 
 /* Create a context on CUDA device `device` and allocate `workspace_bytes` of

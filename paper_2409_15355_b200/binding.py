@@ -45,7 +45,7 @@ class ba_segments(C.Structure):
             "cu_seq", "cu_cache_seq", "cu_final_seq", "cu_seq_block", "cu_block", "block_delta",
             "block_seq", "block_kv_begin", "block_part_off", "block_is_final", "cache_block",
             "cache_cu", "cache_delta", "tok_block", "tok_pos", "tok_pos_local", "cu_qtile",
-            "cu_ftile", "cache_tile_cu", "cu_ktile", "totals", "cache_rope")]
+            "cu_ftile", "cache_tile_cu", "cu_ktile", "totals", "cache_rope", "prompt_items", "final_items", "cu_stream")]
 
 
 class ba_page_table(C.Structure):
@@ -64,6 +64,7 @@ class BaError(RuntimeError):
 
 
 _lib = None
+_raw_stream = _raw_device = None
 
 
 def load_library(path: Optional[str] = None) -> C.CDLL:
@@ -138,9 +139,19 @@ def _ptr(t) -> Optional[int]:
 
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
+        return _current_raw_stream()
     return stream.cuda_stream or None
+
+
+def _current_raw_stream() -> Optional[int]:
+    """Handle of torch's current stream.  torch.cuda.current_stream() builds a stream object, 3.4 us a call; the raw query
+    takes 0.1 us."""
+    global _raw_stream, _raw_device
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()                        # initialises CUDA in torch
+        _raw_stream, _raw_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    return _raw_stream(_raw_device()) or None
 
 
 # ---------------------------------------------------------------------------

@@ -46,7 +46,7 @@ int q_tile_tokens(const ba_config &c) { return 2 * 128 / ba_heads_per_tile(c); }
 size_t stage_bytes_for(int32_t max_blocks) { return ba_align_up((size_t)(2 * (size_t)max_blocks + 64) * 4, 256); }
 
 struct TableLayout {
-  size_t off[24];
+  size_t off[28];
   size_t bytes;
 };
 
@@ -70,6 +70,9 @@ TableLayout table_layout(int32_t batch, int32_t B, int32_t T) {
   take((size_t)(B + 1) * 4);                                  // cu_ktile
   take(8 * 4);                                                // totals
   take((size_t)B * 64 * 8);                                   // cache_rope: at most 64 rotary pairs per block
+  take(((size_t)T / 64 + B) * 32);                            // prompt_items: at least 64 tokens each, one remainder per block
+  take(((size_t)T / 64 + batch) * 32);                        // final_items
+  take((size_t)(batch + 1) * 8);                              // cu_stream
   L.bytes = cur;
   return L;
 }
@@ -242,6 +245,9 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
     if (!ctx->workspace || need > ctx->workspace_bytes ||
         (ctx->workspace_bytes >= ba_scratch_offset(ctx) && need > ba_scratch_offset(ctx) - 256))
       return BA_ERR_WORKSPACE;
+  }
+  const bool inline_lengths = host_lens && n_blocks + batch <= BA_SEGMENT_INLINE;
+  if (host_lens && !inline_lengths) {
     int32_t *stage = (int32_t *)ctx->workspace;
     BA_CUDA_TRY(cudaMemcpyAsync(stage, block_lens, (size_t)n_blocks * 4, cudaMemcpyHostToDevice, s));
     BA_CUDA_TRY(cudaMemcpyAsync(stage + n_blocks, seq_nblocks, (size_t)batch * 4, cudaMemcpyHostToDevice, s));
@@ -295,6 +301,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
   out->cu_qtile = next(); out->cu_ftile = next(); out->cache_tile_cu = next(); out->cu_ktile = next();
   out->totals = next();
   out->cache_rope = (float *)next();
+  out->prompt_items = next(); out->final_items = next(); out->cu_stream = next();
   ctx->seg_delta = nullptr; ctx->seg_rope = nullptr; ctx->seg_rope_blocks = 0; ctx->seg_gen = nullptr;
   // Every call stamps its tables (totals[6]) with a value that differs from call to call and from
   // context to context: a later re-encoding that wants to reuse the rotation table stored with the
@@ -302,11 +309,9 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
   ctx->seg_counter += 1;
   const int32_t gen = (int32_t)((((uint32_t)((uintptr_t)ctx >> 6)) * 0x9E3779B1u +
                                  (uint32_t)ctx->seg_counter * 0x85EBCA6Bu) | 1u);
-  ba_status st = ba_segment_launch(ctx, d_lens, d_nb, batch, n_blocks, n_tokens, mode, gen, out, s);
-  if (st != BA_OK || out->n_cached_blocks == 0) return st;
-  // rotations of the cached blocks (the same angle table ba_reencode_k builds), once per prompt
-  st = ba_reencode_table_launch(ctx, out->cache_delta, out->n_cached_blocks, (float2 *)out->cache_rope, s);
-  if (st == BA_OK) {
+  // (the rotations of the cached blocks -- the same angle table ba_reencode_k builds -- are part of the tables)
+  ba_status st = ba_segment_launch(ctx, d_lens, d_nb, inline_lengths, batch, n_blocks, n_tokens, mode, gen, out, s);
+  if (st == BA_OK && out->n_cached_blocks > 0) {
     ctx->seg_delta = out->cache_delta; ctx->seg_rope = (const float2 *)out->cache_rope;
     ctx->seg_rope_blocks = out->n_cached_blocks;
     ctx->seg_gen = out->totals + 6; ctx->seg_gen_value = gen;

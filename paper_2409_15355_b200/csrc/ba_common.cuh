@@ -140,7 +140,8 @@ __device__ __forceinline__ void ba_record_status(int32_t *status, int32_t code) 
 }
 
 // Entry points implemented in the individual .cu files.
-ba_status ba_segment_launch(ba_ctx *ctx, const int32_t *d_block_lens, const int32_t *d_seq_nblocks,
+constexpr int BA_SEGMENT_INLINE = 960;    // host-side lengths passed as kernel arguments, up to this many values
+ba_status ba_segment_launch(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_nblocks, bool inline_lengths,
                             int32_t batch, int32_t n_blocks, int32_t n_tokens, int mode, int32_t gen,
                             const ba_segments *seg, cudaStream_t stream);
 

@@ -25,3 +25,48 @@ def test_backward_tile_edges(lens, heads):
         dq, dk, dv, q, k, v, g = run_forward_backward(w, mode)
         rq, rk, rv = ob.block_prefill_backward(q, k, v, g, w.block_lens, w.seq_nblocks, mode)
         check_grad("dq", dq, rq); check_grad("dk", dk, rk); check_grad("dv", dv, rv)
+
+def _ragged_lens(n_blocks, seed):
+    return [int(v) for v in np.random.default_rng(seed).integers(1, 9, n_blocks)]
+
+
+# ba_segment: one launch with the lengths as kernel arguments (two sizes of them), one launch from a staged copy, two launches
+@pytest.mark.parametrize("n_blocks,batch", [(1, 1), (127, 1), (126, 2), (127, 2), (256, 256), (257, 3), (955, 5), (956, 5), (1024, 7), (1025, 7), (1500, 1100)])
+def test_segment_launch_variants(n_blocks, batch):
+    counts = [n_blocks // batch + (1 if i < n_blocks % batch else 0) for i in range(batch)]
+    lens = _ragged_lens(n_blocks, n_blocks)
+    lens[-1] = 700                                           # a final block of several work items
+    c = R.Context(8, 2, 64, 1e4)
+    tables = []
+    for host in (True, False):
+        a, b = np.asarray(lens, dtype=np.int32), np.asarray(counts, dtype=np.int32)
+        if not host:
+            a, b = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+        seg, buf = c.segment(a, b, B.BA_MODE_BLOCK, n_tokens=sum(lens))
+        got = R.read_tables(seg, buf)
+        base, raw = buf.data_ptr(), buf.cpu().numpy()
+        rope = raw[seg.cache_rope - base:][:seg.n_cached_blocks * 32 * 8].view(np.float32).reshape(-1, 32, 2)
+        items = raw[seg.final_items - base:][:int(got["totals"][3]) * 32].view(np.int32).reshape(-1, 8)
+        stream = raw[seg.cu_stream - base:][:(batch + 1) * 8].view(np.int32).reshape(2, -1)
+        tables.append((got, rope.copy(), items.copy(), stream.copy()))
+    assert c.device_status() == B.BA_OK
+    ref = ob.segment_tables(lens, counts, B.BA_MODE_BLOCK)
+    for got, rope, items, stream in tables:
+        for k in ("cu_block", "block_delta", "block_kv_begin", "cache_cu", "cache_delta", "tok_block", "tok_pos", "cu_final_seq"):
+            assert got[k].tolist() == ref[k].tolist(), k
+        angle = ref["cache_delta"].astype(np.float64)[:, None] * 1e4 ** (-2.0 * np.arange(32) / 64)
+        assert np.abs(rope[..., 0] - np.cos(angle)).max(initial=0) < 1e-6 and np.abs(rope[..., 1] - np.sin(angle)).max(initial=0) < 1e-6
+        want, sums, b0 = [], [[0], [0]], 0
+        for s, n in enumerate(counts):
+            seq = lens[b0:b0 + n]
+            f0, cached0 = int(ref["cu_final_seq"][s]), int(ref["cu_seq"][s]) - int(ref["cu_final_seq"][s])
+            walked, cached, per = sum(-(-v // 128) for v in seq[:-1]), sum(seq[:-1]), [0, 0]
+            for q in range(0, seq[-1], seg.q_tile_tokens):
+                rows = min(seg.q_tile_tokens, seq[-1] - q)
+                want.append([f0 + q, rows, f0, cached0, cached, b0 - s, int(got["cache_tile_cu"][b0 - s]), walked])
+                own = -(-(q + rows) // 128)
+                per = [per[0] + -(-cached // 128) + own, per[1] + walked + own]
+            sums[0].append(sums[0][-1] + per[0]); sums[1].append(sums[1][-1] + per[1])
+            b0 += n
+        assert items.tolist() == want and stream.tolist() == sums
+    c.close()
