@@ -99,6 +99,7 @@ struct AttnParams {
   ba_reencode_job bg;             // bg.n_rows > 0: a re-encoding job the two spare warps carry out meanwhile
   int bg_rows_per_chunk;
   ba_segments seg;
+  const int32_t *items;           // work items of this call (seg.final_items or seg.prompt_items)
   const int32_t *k_src_off;       // non-null: keys of cached block c start at pool row k_src_off[c] (fused path only)
   int walk;                       // cached keys are walked block by block (a tile never spans two blocks)
   // paged pool: cached block c owns the pages page_idx[page_cu[c] .. page_cu[c+1]) of 1 << page_lg rows each;
@@ -128,7 +129,6 @@ struct Layout {
 // What the scheduling thread publishes to the other roles of its CTA.
 struct WorkEntry {
   int pair;            // item (index into the list of query tile pairs); < 0: no more work
-  int unit;            // the sequence (final attend) or block (prefill) of the item
   int chunk;           // head chunk
   int tile0, n_tiles;  // key tiles [tile0, tile0 + n_tiles) of the item
   int split;           // slot of the partial results this entry writes
@@ -139,7 +139,7 @@ struct Ctrl {
   // [buffer pair][query tile].  Plain path without a background job: the query tiles of successive entries
   // alternate between two pairs of buffers, so the next entry's queries are fetched while the current one runs.
   uint64_t q_full[2][2];
-  uint64_t q_empty[2];            // every QK^T of the entry that used this buffer pair has completed: it may be reloaded
+  uint64_t q_empty[2][2];         // the softmax warps have written the entry's rows out (they pass through this buffer): it may be reloaded
   uint64_t kv_full[kStages];
   uint64_t kv_empty[kStages];
   uint64_t s_full[2];
@@ -176,59 +176,30 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
-__device__ __forceinline__ int upper_bound_tbl(const int32_t *a, int n, int x) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (__ldg(a + mid) <= x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
+// The thread index, read where it is used: addresses that depend on it alone would otherwise be computed once and kept in
+// registers through the softmax loop, which spills.
+__device__ __forceinline__ int thread_index_anew() {
+  int i;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(i));
+  return i;
 }
 
-// The sequence (final attend) or block (prefill) that item `pair` belongs to; -1 past the end of the list.
-__device__ __forceinline__ int find_unit(const AttnParams &p, int pair) {
-  const ba_segments &sg = p.seg;
-  if (p.final_only) {
-    if (pair >= __ldg(sg.totals + 3)) return -1;
-    if (sg.batch == 1) return 0;
-    return upper_bound_tbl(sg.cu_ftile, sg.batch + 1, pair) - 1;
-  }
-  if (pair >= __ldg(sg.totals + 2)) return -1;
-  return upper_bound_tbl(sg.cu_qtile, sg.n_blocks + 1, pair) - 1;
+// Work items of the call, as ba_segment left them (0 when the tables are not valid).
+__device__ __forceinline__ int count_items(const AttnParams &p) {
+  if (__ldg(p.seg.totals + 7) != BA_TABLES_VALID) return 0;
+  return __ldg(p.seg.totals + (p.final_only ? 3 : 2));
 }
 
-// Item `pair` of sequence / block `unit`.  The table look-ups are independent of one another (the search for the
-// unit, a chain of dependent loads, is done once by the scheduling thread and published with the entry).
-__device__ __forceinline__ bool resolve_item(const AttnParams &p, int pair, int unit, Item &it) {
-  const ba_segments &sg = p.seg;
-  const int pair_tok = 2 * p.tok;
-  if (unit < 0) return false;
-  if (p.final_only) {
-    const int s = unit;
-    int f0 = __ldg(sg.cu_final_seq + s), f1 = __ldg(sg.cu_final_seq + s + 1);
-    it.q_row0 = f0 + (pair - __ldg(sg.cu_ftile + s)) * pair_tok;
-    it.q_rows = min(pair_tok, f1 - it.q_row0);
-    it.cache_row0 = __ldg(sg.cu_cache_seq + s);
-    it.cache_len = __ldg(sg.cu_cache_seq + s + 1) - it.cache_row0;
-    it.own_row0 = f0;
-    it.cb0 = __ldg(sg.cu_seq_block + s) - s;           // every earlier sequence has one final block
-    it.ctile0 = p.walk ? __ldg(sg.cache_tile_cu + it.cb0) : 0;
-    it.n_cache_tiles = p.walk ? __ldg(sg.cache_tile_cu + (__ldg(sg.cu_seq_block + s + 1) - s - 1)) - it.ctile0
-                                   : (it.cache_len + kBlockN - 1) / kBlockN;
-  } else {
-    const int b = unit;
-    int b0 = __ldg(sg.cu_block + b), b1 = __ldg(sg.cu_block + b + 1);
-    it.q_row0 = b0 + (pair - __ldg(sg.cu_qtile + b)) * pair_tok;
-    it.q_rows = min(pair_tok, b1 - it.q_row0);
-    it.cache_row0 = 0;
-    it.cache_len = 0;
-    it.own_row0 = __ldg(sg.block_kv_begin + b);
-    it.cb0 = 0; it.ctile0 = 0; it.n_cache_tiles = 0;
-  }
-  if (it.q_rows < 1) return false;
+// Item `idx`: independent loads of one line of the table ba_segment built, instead of a search for the item's sequence or
+// block and look-ups that depend on it.  (Four-byte loads: 16-byte ones tie up groups of four registers, and the softmax
+// loop of the fused path spills.)
+__device__ __forceinline__ void load_item(const AttnParams &p, int idx, Item &it) {
+  const int32_t *x = p.items + 8 * (size_t)idx;
+  it.q_row0 = __ldg(x); it.q_rows = __ldg(x + 1); it.own_row0 = __ldg(x + 2); it.cache_row0 = __ldg(x + 3);
+  it.cache_len = __ldg(x + 4); it.cb0 = __ldg(x + 5); it.ctile0 = __ldg(x + 6);
+  it.n_cache_tiles = p.walk ? __ldg(x + 7) : (it.cache_len + kBlockN - 1) / kBlockN;
   it.n_qt = it.q_rows > p.tok ? 2 : 1;
   it.n_tiles = it.n_cache_tiles + (it.q_row0 + it.q_rows - it.own_row0 + kBlockN - 1) / kBlockN;
-  return true;
 }
 
 // One entry of a CTA's work list: an item, the heads it covers and its share of the key tiles.
@@ -236,7 +207,6 @@ struct Work {
   Item it;
   int head0, kv_head;
   int tile0, n_tiles;   // key tiles [tile0, tile0 + n_tiles) of the item (split-KV share)
-  int split, fill;
 };
 
 // Entry w of the global work list (equal shares of every item's key tiles).  pair < 0 past the end.
@@ -245,13 +215,12 @@ struct Work {
 //  Final attend: all items cost about the same, so the pair index varies fastest instead: the
 //  CTAs running at the same time then work on the same (KV head, key range) for different query
 //  tiles and each K/V tile comes from HBM once and from L2 for the others.
-__device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int w) {
-  WorkEntry e = {-1, -1, 0, 0, 0, 0, 0};
+__device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int total_pairs, int w) {
+  WorkEntry e = {-1, 0, 0, 0, 0, 0};
   const int per_pair = p.n_chunks * p.n_splits;
-  const int total_pairs = __ldg(p.seg.totals + (p.final_only ? 3 : 2));
   int rank, rem;
+  if (total_pairs <= 0) return e;
   if (p.final_only) {
-    if (total_pairs <= 0) return e;
     rem = w / total_pairs; rank = w - rem * total_pairs;
     if (rem >= per_pair) return e;
   } else {
@@ -259,9 +228,8 @@ __device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int w) {
     if (rank >= total_pairs) return e;
   }
   Item it;
-  e.unit = find_unit(p, total_pairs - 1 - rank);
-  if (!resolve_item(p, total_pairs - 1 - rank, e.unit, it)) return e;
   e.pair = total_pairs - 1 - rank;
+  load_item(p, e.pair, it);
   e.chunk = rem / p.n_splits;
   e.split = rem - e.chunk * p.n_splits;
   e.fill = p.n_splits;
@@ -272,13 +240,12 @@ __device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int w) {
 
 // A published entry, decoded by the role that reads it.  Returns false at the end of the work.
 __device__ __forceinline__ bool load_work(const AttnParams &p, const WorkEntry &e, Work &wk) {
-  if (e.pair < 0 || !resolve_item(p, e.pair, e.unit, wk.it)) return false;
+  if (e.pair < 0) return false;
+  load_item(p, e.pair, wk.it);
   wk.head0 = e.chunk * p.hpt;
   wk.kv_head = wk.head0 / p.G;
   wk.tile0 = e.tile0;
   wk.n_tiles = e.n_tiles;
-  wk.split = e.split;
-  wk.fill = e.fill;
   return true;
 }
 
@@ -379,12 +346,11 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   Ctrl *ctrl = reinterpret_cast<Ctrl *>(smem + L::kCtrl);
 
-  // inconsistent tables: no attention work is taken, a background job still runs
-  const bool tables_ok = __ldg(p.seg.totals + 7) == BA_TABLES_VALID;
   const int tid = threadIdx.x, warp = tid >> 5;
 
   if (tid == 0) {
-    for (int b = 0; b < 2; ++b) { mbar_init(&ctrl->q_full[b][0], 1); mbar_init(&ctrl->q_full[b][1], 1); mbar_init(&ctrl->q_empty[b], 1); }
+    for (int b = 0; b < 2; ++b)
+      for (int t = 0; t < 2; ++t) { mbar_init(&ctrl->q_full[b][t], 1); mbar_init(&ctrl->q_empty[b][t], 4); }
     for (int s = 0; s < kStages; ++s) { mbar_init(&ctrl->kv_full[s], 1); mbar_init(&ctrl->kv_empty[s], 1); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(&ctrl->s_full[t], 1); mbar_init(&ctrl->p_full[t][0], 128); mbar_init(&ctrl->p_full[t][1], 128);
@@ -397,6 +363,14 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     fence_barrier_init();
   }
   if (warp == 9) { tmem_alloc(&ctrl->tmem_base, 512); tmem_relinquish(); }
+  // The CTA's first entry is known from its index: the scheduling warp looks it up while the others set the CTA up.
+  // Inconsistent tables: no attention work is taken, a background job still runs.
+  int n_items = 0;
+  WorkEntry first = {-1, 0, 0, 0, 0, 0};
+  if (warp == 8) {
+    n_items = count_items(p);
+    if (!p.balanced) first = list_entry(p, n_items, (int)blockIdx.x);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -415,8 +389,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     // same for every head chunk), one item per lane, kept in shared memory for the scheduling thread
     int *bal_cu = reinterpret_cast<int *>(smem + L::kCtrl + kBalTableOff);
     int bal_np = 0;
-    if (p.balanced && tables_ok) {
-      bal_np = __ldg(p.seg.totals + 3);
+    if (p.balanced && n_items > 0) {
+      bal_np = n_items;
       if (bal_np < 1 || bal_np > kBalMaxPairs || bal_np * p.n_chunks != p.balanced) {
         ba_record_status(p.status, BA_ERR_SHAPE);          // the tables describe another launch than the host sized
         bal_np = 0;
@@ -426,8 +400,11 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         for (int base = 0; base < bal_np; base += 32) {
           const int i = base + lane;
           int x = 0;
-          Item it;
-          if (i < bal_np && resolve_item(p, bal_np - 1 - i, find_unit(p, bal_np - 1 - i), it)) x = max(0, it.n_tiles - p.bal_len);
+          if (i < bal_np) {
+            Item it;
+            load_item(p, bal_np - 1 - i, it);
+            x = max(0, it.n_tiles - p.bal_len);
+          }
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -455,15 +432,14 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         bal_end = (int)(bal_all * (j + 1) / bal_nh);
       }
       auto balanced_entry = [&](int n_done) -> WorkEntry {
-        WorkEntry e = {-1, -1, 0, 0, 0, 0, 0};
+        WorkEntry e = {-1, 0, 0, 0, 0, 0};
         if (bal_np == 0) return e;
         const int b = (int)blockIdx.x;
         if (b < p.balanced) {                              // the last bal_len key tiles of item b
           if (n_done > 0) return e;
           Item it;
           const int pair = bal_np - 1 - b % bal_np;
-          e.unit = find_unit(p, pair);
-          if (!resolve_item(p, pair, e.unit, it)) return e;
+          load_item(p, pair, it);
           e.pair = pair; e.chunk = b / bal_np;
           e.tile0 = max(0, it.n_tiles - p.bal_len);
           e.n_tiles = it.n_tiles - e.tile0;
@@ -484,14 +460,14 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         e.split = 1 + ((int)blockIdx.x - p.balanced) - j_first;
         if (e.split >= p.n_splits) { ba_record_status(p.status, BA_ERR_SHAPE); return e; }
         e.pair = bal_np - 1 - i; e.chunk = chunk;
-        e.unit = find_unit(p, e.pair);
         e.tile0 = r - bal_cu[i]; e.n_tiles = n;
         e.fill = bal_pos + n == front_end ? e.split + 1 : p.n_splits;
         bal_pos += n;
         return e;
       };
       int gidx = 0;                       // K/V tiles requested so far (ring position)
-      int n_items = 0;                    // items with at least one tile so far
+      int n_loaded = 0;                   // entries whose queries have been requested so far
+      int uses1[2] = {0, 0};              // of those in buffer pair b, the ones with a second query tile
       bool ok = true;
       Work wk;
       int n_work = 0;                    // work entries published so far
@@ -502,12 +478,10 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (!ok) break;
         // balanced launch: the next piece of this CTA's share; persistent launch: next entry of the global list;
         // one-item launch: this CTA's own entry, then stop
-        WorkEntry e = {-1, -1, 0, 0, 0, 0, 0};
-        if (tables_ok) {
-          if (p.balanced) e = balanced_entry(n_work);
-          else if (p.persistent) e = list_entry(p, atomicAdd(p.counters, 1));
-          else if (n_work == 0) e = list_entry(p, (int)blockIdx.x);
-        }
+        WorkEntry e = {-1, 0, 0, 0, 0, 0};
+        if (p.balanced) e = balanced_entry(n_work);
+        else if (n_work == 0) e = first;
+        else if (p.persistent) e = list_entry(p, n_items, (int)gridDim.x + atomicAdd(p.counters, 1));
         const bool more = load_work(p, e, wk);
         if (!more) e.pair = -1;
         ctrl->work_ring[slot] = e;
@@ -517,12 +491,14 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (wk.n_tiles == 0) continue;
         const Item &it = wk.it;
         if (!kFused) {      // (on the fused path the softmax warps fetch the query tiles themselves)
-          // the Q buffers are free once every QK^T of the previous item has completed
-          const int qb = p.q_double ? (n_items & 1) : 0;           // buffer pair of this entry
-          const int q_use = p.q_double ? (n_items >> 1) : n_items;  // earlier entries that used it
-          ok = mbar_wait(&ctrl->q_empty[qb], (q_use & 1) ^ 1, abort_flag);
+          // a Q buffer is free once the rows of the entry that used it have been written out
+          const int qb = p.q_double ? (n_loaded & 1) : 0;            // buffer pair of this entry
+          const int q_use = p.q_double ? (n_loaded >> 1) : n_loaded;  // earlier entries that used it
+          ok = mbar_wait(&ctrl->q_empty[qb][0], (q_use & 1) ^ 1, abort_flag);
+          if (ok && it.n_qt == 2) ok = mbar_wait(&ctrl->q_empty[qb][1], ((qb ? uses1[1] : uses1[0]) & 1) ^ 1, abort_flag);
           if (!ok) break;
-          ++n_items;
+          ++n_loaded;
+          if (it.n_qt == 2) { if (qb) ++uses1[1]; else ++uses1[0]; }
           for (int t = 0; t < 2; ++t) {
             if (t >= it.n_qt) { mbar_arrive(&ctrl->q_full[qb][t]); continue; }   // (every entry moves both barriers on)
             mbar_arrive_expect_tx(&ctrl->q_full[qb][t], L::kTileBytes);
@@ -724,7 +700,6 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           if (t < n_qt && ok) ok = issue_qk(t, 0, gidx);
         if (!ok) break;
         mma_commit(&ctrl->kv_empty[gidx % kStages]);
-        if (n_tiles == 1) mma_commit(&ctrl->q_empty[q_buf]);
         for (int j = 0; j < n_tiles && ok; ++j) {
           const bool last = j + 1 == n_tiles;
           const int iv = gidx + 2 * j + 1, ik = gidx + 2 * j + 2;   // ring positions of V_j and K_(j+1)
@@ -757,10 +732,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               ok = issue_qk(t, j + 1, ik);
               if (!ok) continue;
               BA_TR(2, j, t * 4 + 3);
-              if (t + 1 == n_qt) {
-                mma_commit(&ctrl->kv_empty[ik % kStages]);
-                if (j + 2 == n_tiles) mma_commit(&ctrl->q_empty[q_buf]);   // that was the item's last QK^T
-              }
+              if (t + 1 == n_qt) mma_commit(&ctrl->kv_empty[ik % kStages]);
             }
           }
         }
@@ -797,6 +769,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     int n_staged = 0;                     // fused: (cos, sin) rows staged so far by this group
     int n_made = 0;                       // fused: versions of this query tile prepared so far
     int tiles_before = 0;                 // key tiles of all earlier items (the producer counts the same way)
+    int n_loaded = 0;                     // entries with key tiles so far (the producer counts the same way)
     bool ok = true;
     Work wk;
     int n_work = 0;
@@ -813,14 +786,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       const int n_tiles = wk.n_tiles, tile0 = wk.tile0, head0 = wk.head0;
       const bool half_last = last_tile_is_half(wk);
       if (t < it.n_qt) {
-      const int q_last = it.q_row0 + it.q_rows - 1;
-      const int row_tok = it.q_row0 + t * p.tok + (r >> p.hpt_log2);
-      // a row is stored only if it belongs to the item and lies inside the caller's tensors; tables that
-      // describe more rows than the caller gave are reported, nothing is written past the end
-      const bool row_valid = row_tok <= q_last && row_tok < p.n_q_rows;
-      if (row_tok <= q_last && row_tok >= p.n_q_rows) ba_record_status(p.status, BA_ERR_SHAPE);
-      const int tok_c = min(row_tok, q_last);               // rows past the block behave like its last row
-      const int head = head0 + (r & (p.hpt - 1));
+      // rows past the block behave like its last row
+      const int tok_c = min(it.q_row0 + t * p.tok + (r >> p.hpt_log2), it.q_row0 + it.q_rows - 1);
       float m_used = -INFINITY, l = 0.f;
 
       // fused path: this thread prepares row r of every version of query tile t (see the MMA warp):
@@ -855,7 +822,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           if (r < D / 2) { cs_stage[r] = cs_next; mbar_arrive(&ctrl->cs_full[t]); }
           if (!mbar_wait(&ctrl->cs_full[t], n_staged & 1, abort_flag)) return false;
           ++n_staged;
-          rotate_q_row<D>(ver_buf(n_made), ver_buf(n_made), cs_stage, p.rope_layout, r);
+          rotate_q_row<D>(ver_buf(n_made), ver_buf(n_made), cs_stage, p.rope_layout, thread_index_anew() & 127);
         }
         fence_proxy_async();                               // the tensor core reads through the async proxy
         __syncwarp();
@@ -991,8 +958,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           const bool due = tile0 + j + 1 == next_start;    // the next tile is the first to need it
           const bool next_cached = next_start < cached_end;
           if (r == 0) BA_TR(t, j, 6);
-          if (prep == 0) { begin_version(); prep = 1; if (due) { ok = finish_version(next_cached); prep = 2; } }
-          else if (prep == 1) { ok = finish_version(next_cached); prep = 2; }
+          const bool finish = prep == 1 || (prep == 0 && due);
+          if (prep == 0) { begin_version(); prep = 1; }
+          if (finish) { ok = finish_version(next_cached); prep = 2; }
           if (!ok) break;
           if (r == 0) BA_TR(t, j, 7);
           if (due) { if (next_cached) ++f_pc; plan_next(next_cached ? f_pc : -1); }
@@ -1003,72 +971,104 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         l += ((sum[0] + sum[1]) + (sum[2] + sum[3])) + ((sum[4] + sum[5]) + (sum[6] + sum[7]));
       }
 
+      // (the item is looked up again for the write-out: its rows need not be kept in registers through the loop)
+      int q_row0, q_rows;
+      asm volatile("ld.global.nc.v2.s32 {%0, %1}, [%2];" : "=r"(q_row0), "=r"(q_rows) : "l"(p.items + 8 * (size_t)e.pair));
       if (ok && n_tiles > 0) { ok = mbar_wait(&ctrl->o_done[t], o_uses & 1, abort_flag); ++o_uses; }
       if (ok) {
         tc_fence_after();
         const float inv = l > 0.f ? 1.f / l : 0.f;
         const float lse_val = l > 0.f ? (m_used * sl + log2f(l)) * 0.6931471805599453f : -INFINITY;
-        const size_t orow = ((size_t)row_tok * p.Hq + head) * D;
         const bool partial = p.n_splits > 1;
-        float *part = partial ? p.o_part + (size_t)wk.split * p.n_q_rows * p.Hq * D + orow : nullptr;
+        // Rows leave through shared memory -- the warp's quarter of the entry's own query tile, which every product has
+        // read by now -- so that a store instruction writes whole rows: stores straight from the row each thread owns touch
+        // 32 rows at a time and took 5000-7000 cycles a tile (seven edited blocks, 312 entries: 34.9 -> 27 us a layer).
+        const int thread = thread_index_anew();
+        const int lane = thread & 31, quarter = (thread >> 5) & 3;
+        const int q_last = q_row0 + q_rows - 1, out_head0 = e.chunk * p.hpt;
+        // a row is stored only if it belongs to the item and lies inside the caller's tensors; tables that
+        // describe more rows than the caller gave are reported, nothing is written past the end
+        const int row_tok = q_row0 + t * p.tok + ((quarter * 32 + lane) >> p.hpt_log2), head = out_head0 + (lane & (p.hpt - 1));
+        const bool row_valid = row_tok <= q_last && row_tok < p.n_q_rows;
+        if (row_tok <= q_last && row_tok >= p.n_q_rows) ba_record_status(p.status, BA_ERR_SHAPE);
+        uint8_t *stage = (kFused ? ver_buf(n_made - 1)
+                                 : smem + ((p.q_double && (n_loaded & 1)) ? L::kBg + t * L::kTileBytes : (t ? L::kQ1 : L::kQ0))) +
+                         quarter * (32 * D * 2);
+        auto store_rows = [&](auto &&address) {                      // address(output row) of the D * 2 bytes staged for it
+          constexpr int kRowChunks = D / 8;
+          __syncwarp();
+#pragma unroll 4
+          for (int i = 0; i < kRowChunks; ++i) {
+            const int lr = (i * 32 + lane) / kRowChunks, c = lane % kRowChunks;
+            const uint4 x = *reinterpret_cast<const uint4 *>(stage + lr * (kRowChunks * 16) + ((c ^ (lr & 7)) << 4));
+            const int rr = quarter * 32 + lr;
+            const int tk = q_row0 + t * p.tok + (rr >> p.hpt_log2);
+            if (tk <= q_last && tk < p.n_q_rows)
+              *reinterpret_cast<uint4 *>(address((size_t)tk * p.Hq + out_head0 + (rr & (p.hpt - 1))) + c * 16) = x;
+          }
+          __syncwarp();
+        };
+        if (n_tiles > 0) {
+          if (partial || p.out_f32) {
+            uint8_t *base = partial ? reinterpret_cast<uint8_t *>(p.o_part + (size_t)e.split * p.n_q_rows * p.Hq * D)
+                                    : reinterpret_cast<uint8_t *>(p.o);
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-          uint32_t o[32];
-          if (n_tiles > 0) {
-            tmem_ld_32x32b_x32(tO + c * 32, o);
-            tmem_wait_ld();
+            for (int h = 0; h < 2; ++h) {                            // half of every row at a time: as many bytes as a bf16 row
+#pragma unroll
+              for (int q = 0; q < D / 64; ++q) {
+                uint32_t o[32];
+                tmem_ld_32x32b_x32(tO + h * (D / 2) + q * 32, o);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                  *reinterpret_cast<float4 *>(stage + lane * (D * 2) + (((q * 8 + i) ^ (lane & 7)) << 4)) =
+                      make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
+                                  __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
+              }
+              store_rows([&](size_t row) { return base + (row * D + h * (D / 2)) * 4; });
+            }
           } else {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] = 0u;
-          }
-          if (row_valid) {
-            if (partial) {
-              // 32-byte stores (the workspace is aligned for them): a thread owns a row, so each fills a whole sector
-              float *dst = part + c * 32;
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                float v[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(o[8 * i + e]) * inv;
-                st_global_v8(dst + 8 * i, v);
-              }
-            } else if (p.out_f32) {
-              float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.o) + orow + c * 32);
-#pragma unroll
-              for (int i = 0; i < 8; ++i)
-                dst[i] = make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
-                                     __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
-            } else {
-              uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.o) + orow + c * 32);
+            for (int c = 0; c < D / 32; ++c) {
+              uint32_t o[32];
+              tmem_ld_32x32b_x32(tO + c * 32, o);
+              tmem_wait_ld();
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
                 uint32_t w[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * e]) * inv,
-                                                           __uint_as_float(o[8 * i + 2 * e + 1]) * inv);
-                  w[e] = *reinterpret_cast<uint32_t *>(&v);
+                for (int e2 = 0; e2 < 4; ++e2) {
+                  __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * e2]) * inv,
+                                                           __uint_as_float(o[8 * i + 2 * e2 + 1]) * inv);
+                  w[e2] = *reinterpret_cast<uint32_t *>(&v);
                 }
-                dst[i] = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4 *>(stage + lane * (D * 2) + (((c * 4 + i) ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
               }
             }
+            store_rows([&](size_t row) { return reinterpret_cast<uint8_t *>(p.o) + row * D * 2; });
           }
         }
         if (n_tiles > 0) {
           // O_t has been read out of tensor memory: the next item's first PV may overwrite it
           tc_fence_before();
           mbar_arrive(&ctrl->o_free[t]);
+          if (!kFused) {
+            fence_proxy_async();                           // the copy engine writes the buffer next
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctrl->q_empty[p.q_double ? (n_loaded & 1) : 0][t]);
+          }
         }
         if (row_valid) {
           if (partial) {
-            p.lse_part[((size_t)wk.split * p.n_q_rows + row_tok) * p.Hq + head] = lse_val;
-            for (int s = wk.fill; s < p.n_splits; ++s)      // slots no entry of this item writes: empty
+            p.lse_part[((size_t)e.split * p.n_q_rows + row_tok) * p.Hq + head] = lse_val;
+            for (int s = e.fill; s < p.n_splits; ++s)      // slots no entry of this item writes: empty
               p.lse_part[((size_t)s * p.n_q_rows + row_tok) * p.Hq + head] = -INFINITY;
           } else if (p.lse) p.lse[(size_t)row_tok * p.Hq + head] = lse_val;
         }
       }
       }
       tiles_before += n_tiles;
+      if (n_tiles > 0) ++n_loaded;
     }
   }
 
@@ -1292,6 +1292,8 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   if (p.fused && !p.q_rope) return BA_ERR_INVALID_ARG;
   p.n_q_rows = a.n_q_rows;
   p.seg = *seg;
+  p.items = a.final_only ? seg->final_items : seg->prompt_items;
+  if (!p.items) return BA_ERR_INVALID_ARG;
   if (seg->q_tile_tokens != 2 * p.tok) return BA_ERR_INVALID_ARG;
 
   // Split the keys of each work item over several CTAs when the items alone cannot fill the
@@ -1327,7 +1329,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   // over a long cache: about two, the write-out of a CTA's first entry overlaps the start of its second).
   // Shorter lists are launched one CTA per entry.
   const long long work_upper = (long long)pairs_upper * (Hq / p.hpt) * n_splits;
-  p.persistent = !p.balanced && items * n_splits > (a.final_only ? 1LL : 2LL) * ctx->sm_count;
+  p.persistent = !p.balanced && work_upper > ctx->sm_count;
   // the counters live in the last 256 bytes below the scratch area: zeroed by ba_create, left at zero by every launch
   int32_t *counters = nullptr;
   if (ctx->workspace && ctx->workspace_bytes >= ba_scratch_offset(ctx))
