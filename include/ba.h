@@ -94,6 +94,8 @@ typedef struct {
    * sum, minimum and maximum over the items, [0..2] with the cached keys of a sequence packed in one run,
    * [3..5] with every cached block starting a tile of its own (pools, fused path).  Used to balance the launch. */
   int32_t final_key_tiles[6];
+  int32_t prompt_key_tiles; /* sum over the work items of ba_block_prefill in block mode, lengths on the host (else 0) */
+  int32_t reserved;
   /* per sequence, [batch + 1] */
   int32_t *cu_seq;         /* first row of the sequence, prompt packing */
   int32_t *cu_cache_seq;   /* first row of the sequence, cache packing */
@@ -125,10 +127,12 @@ typedef struct {
   float *cache_rope;
   /* work items of the attention kernels (not part of the bit-exact contract), 8 ints each: first query row, query rows,
    * first own key row, first cached row, cached rows, first cached block, its first key tile, cached key tiles */
-  int32_t *prompt_items;   /* [totals[2]] items of ba_block_prefill */
+  int32_t *prompt_items;   /* [totals[2]] items of ba_block_prefill, those of the final blocks last; [5] of these:
+                            * place of the first query row among the rows of final blocks */
   int32_t *final_items;    /* [totals[3]] items of ba_final_attend */
   int32_t *cu_stream;      /* [2][batch+1] prefix sums over sequences of the key tiles the items of its final block see:
                             * cached keys packed, then block by block */
+  int32_t *cache_tile_block; /* [cache_tile_cu[Bc]] cached block a key tile of cache_tile_cu belongs to */
 } ba_segments;
 
 /* Create a context on CUDA device `device` and allocate `workspace_bytes` of

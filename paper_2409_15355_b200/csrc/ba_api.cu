@@ -73,6 +73,7 @@ TableLayout table_layout(int32_t batch, int32_t B, int32_t T) {
   take(((size_t)T / 64 + B) * 32);                            // prompt_items: at least 64 tokens each, one remainder per block
   take(((size_t)T / 64 + batch) * 32);                        // final_items
   take((size_t)(batch + 1) * 8);                              // cu_stream
+  take(((size_t)T / 128 + B) * 4);                            // cache_tile_block
   L.bytes = cur;
   return L;
 }
@@ -268,6 +269,16 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
     for (int b = 0; b < n_blocks; ++b) items += (block_lens[b] + tt - 1) / tt;
     for (int q = 0, b = 0; q < batch; ++q) { b += seq_nblocks[q]; fitems += (block_lens[b - 1] + tt - 1) / tt; }
     out->n_prompt_items = (int32_t)items; out->n_final_items = (int32_t)fitems;
+    long long prompt_tiles = 0;                          // key tiles the items of ba_block_prefill see in block mode
+    for (int q = 0, b = 0; q < batch; ++q) {
+      long long seq_rows = 0;
+      for (int c = 0; c < seq_nblocks[q]; ++c, ++b) {
+        const long long before = c + 1 == seq_nblocks[q] ? seq_rows : 0;
+        for (int r0 = 0; r0 < block_lens[b]; r0 += tt) prompt_tiles += (before + std::min(block_lens[b], r0 + tt) + 127) / 128;
+        seq_rows += block_lens[b];
+      }
+    }
+    out->prompt_key_tiles = prompt_tiles <= INT32_MAX ? (int32_t)prompt_tiles : 0;
     // key tiles per item of the final blocks (the counting of the attention kernel, done here on the host)
     long long sum[2] = {0, 0}, mn[2] = {INT32_MAX, INT32_MAX}, mx[2] = {0, 0};
     for (int q = 0, b = 0; q < batch; ++q) {
@@ -301,7 +312,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
   out->cu_qtile = next(); out->cu_ftile = next(); out->cache_tile_cu = next(); out->cu_ktile = next();
   out->totals = next();
   out->cache_rope = (float *)next();
-  out->prompt_items = next(); out->final_items = next(); out->cu_stream = next();
+  out->prompt_items = next(); out->final_items = next(); out->cu_stream = next(); out->cache_tile_block = next();
   ctx->seg_delta = nullptr; ctx->seg_rope = nullptr; ctx->seg_rope_blocks = 0; ctx->seg_gen = nullptr;
   // Every call stamps its tables (totals[6]) with a value that differs from call to call and from
   // context to context: a later re-encoding that wants to reuse the rotation table stored with the
@@ -420,6 +431,7 @@ ba_status ba_block_prefill(ba_ctx *ctx, const void *q, const void *k, const void
   a.o = o; a.lse = lse; a.n_q_rows = seg->n_tokens; a.n_kv_rows = seg->n_tokens;
   a.out_f32 = out_dtype == BA_OUT_F32;
   a.final_only = 0;
+  a.mode = (int)mode;
   return ba_attend_launch(ctx, a, seg, (cudaStream_t)stream);
 }
 

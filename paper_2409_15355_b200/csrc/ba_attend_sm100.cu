@@ -59,7 +59,15 @@ namespace {
 
 constexpr int kThreads = 384;
 constexpr int kBlockN = 128;      // keys per tile
-constexpr int kStages = 3;           // ring of K/V tiles (K_j, V_j, K_j+1, ...)
+// Variants of the kernel, so that each carries only its own code.  The ring of K/V tiles (K_j, V_j, K_j+1, ...) has three
+// stages; the rest of the shared memory is a second pair of query buffers (or the background job's staging area).  In
+// kDeepRing it is a fourth stage and a staging area for the write-out: a tile that comes from HBM while every SM streams
+// takes 2000-4500 cycles, three stages cover 2700 (64-token query over 32K cached keys: 800-1900 cycles of waiting in a
+// period of 4000-4900), and with the write-out elsewhere the one pair of query buffers is reloaded as soon as its last
+// product is done.
+constexpr int kPlain = 0, kFusedPath = 1, kDeepRing = 2;
+constexpr int ring_stages(int variant) { return variant == kDeepRing ? 4 : 3; }
+constexpr int kMaxStages = 4;
 constexpr float kRescaleThreshold = 8.0f;
 constexpr int kBgStageBytes = 16384; // two spare warps x two stages of source rows
 constexpr int kWorkSlots = 4;      // ring of published work entries (power of two)
@@ -83,9 +91,15 @@ struct AttnParams {
   int final_only;
   int n_q_rows;
   int n_chunks;                   // head chunks per token (Hq / hpt)
-  int n_splits;                   // > 1: the key tiles of an item are divided among n_splits work entries, combined later
-  float *o_part;                  // [n_splits, n_q_rows, Hq, D] fp32, each normalised by its own denominator
-  float *lse_part;                // [n_splits, n_q_rows, Hq] natural-log denominators (-inf: split saw no key)
+  int n_splits;                   // > 1: the key tiles of an item are divided among several work entries, combined later
+                                  // (prefill: of the items of final blocks only)
+  float *o_part;                  // [n_splits, n_part_rows, Hq, D] fp32, each normalised by its own denominator
+  float *lse_part;                // [n_splits, n_part_rows, Hq] natural-log denominators (-inf: split saw no key)
+  int n_part_rows;
+  // stream = 1: the key tiles of all (item, head chunk) are laid end to end and cut into one run per CTA
+  int stream;
+  // cluster > 1: the CTAs of a cluster share one item's key tiles and merge their results in shared memory
+  int cluster;
   const int32_t *v_src_off;       // non-null: values of cached block c start at pool row v_src_off[c]
   int persistent;                 // 1: CTAs draw work from counters[0]; 0: CTA b handles entry b only
   // balanced > 0 (final block over a long cache, fewer items than CTAs): the first `balanced` CTAs each take the
@@ -120,18 +134,22 @@ struct Layout {
   static constexpr int kQ0 = 0;
   static constexpr int kQ1 = kTileBytes;
   static constexpr int kRing = 2 * kTileBytes;
-  static constexpr int kCtrl = kRing + kStages * kTileBytes;   // 2 KB: Ctrl, then two ba_bg_smem
-  static constexpr int kBg = kCtrl + 2048;                     // staging of the background re-encoding, or (fused
-                                                               // path) the second pair of query tile buffers
-  static constexpr int kBytes = kBg + 4 * kBgStageBytes;
+  static constexpr int kBg = kRing + 3 * kTileBytes;           // staging of the background re-encoding, the second pair
+                                                               // of query tile buffers, or a fourth stage and staging rows
+  static constexpr int kCtrl = kBg + 4 * kBgStageBytes;        // 2 KB: Ctrl, then two ba_bg_smem
+  static constexpr int kBytes = kCtrl + 2048;
+  static_assert(2 * kTileBytes <= 4 * kBgStageBytes, "two tiles fit the staging area");
 };
+
+// In lse_part (stream launch): the row needed no partial results, its output is written.  A NaN no arithmetic produces.
+constexpr uint32_t kRowIsComplete = 0xffc0ba11u;
 
 // What the scheduling thread publishes to the other roles of its CTA.
 struct WorkEntry {
   int pair;            // item (index into the list of query tile pairs); < 0: no more work
   int chunk;           // head chunk
   int tile0, n_tiles;  // key tiles [tile0, tile0 + n_tiles) of the item
-  int split;           // slot of the partial results this entry writes
+  int split;           // slot of the partial results this entry writes; < 0: it covers the whole item, rows go to the output
   int fill;            // slots fill .. n_splits - 1 of the item stay unused: this entry marks them empty
 };
 
@@ -139,9 +157,11 @@ struct Ctrl {
   // [buffer pair][query tile].  Plain path without a background job: the query tiles of successive entries
   // alternate between two pairs of buffers, so the next entry's queries are fetched while the current one runs.
   uint64_t q_full[2][2];
-  uint64_t q_empty[2][2];         // the softmax warps have written the entry's rows out (they pass through this buffer): it may be reloaded
-  uint64_t kv_full[kStages];
-  uint64_t kv_empty[kStages];
+  // the buffer may be reloaded: the softmax warps have written the entry's rows out, which pass through it (kDeepRing: every
+  // QK^T of the entry has completed, [0][0] only)
+  uint64_t q_empty[2][2];
+  uint64_t kv_full[kMaxStages];
+  uint64_t kv_empty[kMaxStages];
   uint64_t s_full[2];
   uint64_t p_full[2][2];          // [query tile][half of the P tile]
   uint64_t o_done[2];
@@ -210,31 +230,42 @@ struct Work {
 };
 
 // Entry w of the global work list (equal shares of every item's key tiles).  pair < 0 past the end.
-//  Prefill: items heaviest-first (descending pair index: within a sequence an item's cost grows
-//  with its index, the final block comes last), then head chunk, then split.
+//  Prefill: items heaviest-first (descending index: the table ends with the items of the final blocks, and within a
+//  sequence an item's cost grows with its index), then head chunk, then split (final blocks only).
 //  Final attend: all items cost about the same, so the pair index varies fastest instead: the
 //  CTAs running at the same time then work on the same (KV head, key range) for different query
 //  tiles and each K/V tile comes from HBM once and from L2 for the others.
 __device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int total_pairs, int w) {
-  WorkEntry e = {-1, 0, 0, 0, 0, 0};
-  const int per_pair = p.n_chunks * p.n_splits;
-  int rank, rem;
+  WorkEntry e = {-1, 0, 0, 0, -1, 0};
+  int n_splits = p.n_splits, per_pair = p.n_chunks * n_splits, rank, rem;
   if (total_pairs <= 0) return e;
-  if (p.final_only) {
+  if (p.cluster > 1) {
+    n_splits = p.cluster;
+    const int member = w % n_splits, i = w / n_splits;
+    rem = i / total_pairs; rank = i - rem * total_pairs;
+    if (rem >= p.n_chunks) return e;
+    rem = rem * n_splits + member;
+  } else if (p.final_only) {
     rem = w / total_pairs; rank = w - rem * total_pairs;
     if (rem >= per_pair) return e;
   } else {
-    rank = w / per_pair; rem = w - rank * per_pair;
+    rank = 0;
+    if (n_splits > 1) {                                    // first the items of final blocks, in pieces
+      const int n_final = __ldg(p.seg.totals + 3);
+      if (w >= n_final * per_pair) { w -= n_final * per_pair; rank = n_final; n_splits = 1; per_pair = p.n_chunks; }
+    }
+    rank += w / per_pair; rem = w % per_pair;
     if (rank >= total_pairs) return e;
   }
   Item it;
   e.pair = total_pairs - 1 - rank;
   load_item(p, e.pair, it);
-  e.chunk = rem / p.n_splits;
-  e.split = rem - e.chunk * p.n_splits;
-  e.fill = p.n_splits;
-  e.tile0 = (int)(((long long)it.n_tiles * e.split) / p.n_splits);
-  e.n_tiles = (int)(((long long)it.n_tiles * (e.split + 1)) / p.n_splits) - e.tile0;
+  e.chunk = rem / n_splits;
+  const int k = rem - e.chunk * n_splits;
+  e.split = p.cluster > 1 || n_splits > 1 ? k : -1;
+  e.fill = n_splits;
+  e.tile0 = (int)(((long long)it.n_tiles * k) / n_splits);
+  e.n_tiles = (int)(((long long)it.n_tiles * (k + 1)) / n_splits) - e.tile0;
   return e;
 }
 
@@ -249,6 +280,94 @@ __device__ __forceinline__ bool load_work(const AttnParams &p, const WorkEntry &
   return true;
 }
 
+// Stream launch.  The key tiles of all (sequence, head chunk, item), in that order, are laid end to end and cut into one
+// run per CTA, so that every SM gets the same number of tiles whatever the items' number and sizes.  A cut within
+// kStreamSnap tiles of an item's edge is moved to the edge: a sliver of an item costs more than its tiles.
+constexpr int kStreamSnap = 2;
+struct StreamState {
+  int pos, end;              // tiles left to this CTA: [pos, end)
+  int seq, chunk, i;         // item i of sequence seq that holds pos, its first tile g0
+  int g0, cached_tiles, final_rows, n_items, item0;
+  int total;
+};
+__device__ __forceinline__ void stream_sequence(const AttnParams &p, StreamState &s) {
+  const int32_t *ft = p.seg.cu_ftile + s.seq, *fs = p.seg.cu_final_seq + s.seq;
+  s.item0 = __ldg(ft); s.n_items = __ldg(ft + 1) - s.item0;
+  s.final_rows = __ldg(fs + 1) - __ldg(fs);
+  Item it;
+  load_item(p, s.item0, it);
+  s.cached_tiles = it.n_cache_tiles;
+}
+__device__ __forceinline__ int stream_item_tiles(const AttnParams &p, const StreamState &s) {
+  return s.cached_tiles + (min((s.i + 1) * 2 * p.tok, s.final_rows) + kBlockN - 1) / kBlockN;
+}
+// The item that holds tile x.
+__device__ __forceinline__ void stream_locate(const AttnParams &p, StreamState &s, int x) {
+  const int32_t *cu = p.seg.cu_stream + (p.walk ? p.seg.batch + 1 : 0);
+  int lo = 0, hi = p.seg.batch - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(cu + mid) * p.n_chunks <= x) lo = mid; else hi = mid - 1;
+  }
+  s.seq = lo;
+  const int first = __ldg(cu + lo), per_chunk = __ldg(cu + lo + 1) - first;
+  int r = x - first * p.n_chunks;
+  s.chunk = r / per_chunk;
+  r -= s.chunk * per_chunk;
+  s.g0 = x - r;
+  stream_sequence(p, s);
+  s.i = 0;
+  for (int n; r >= (n = stream_item_tiles(p, s)) && s.i + 1 < s.n_items; ++s.i) { r -= n; s.g0 += n; }
+}
+// This CTA's run (all lanes of a warp).
+__device__ __forceinline__ void stream_start(const AttnParams &p, StreamState &s) {
+  s.total = __ldg(p.seg.cu_stream + (p.walk ? p.seg.batch + 1 : 0) + p.seg.batch) * p.n_chunks;
+  const int lane = threadIdx.x & 31;
+  const int x = (int)((long long)s.total * ((int)blockIdx.x + (lane & 1)) / (int)gridDim.x);   // lane 0: begin, lane 1: end
+  int cut = x;
+  if (x < s.total) {
+    stream_locate(p, s, x);
+    const int n = stream_item_tiles(p, s);
+    if (x - s.g0 <= kStreamSnap) cut = s.g0;
+    else if (s.g0 + n - x <= kStreamSnap) cut = s.g0 + n;
+  }
+  s.pos = __shfl_sync(0xffffffffu, cut, 0); s.end = __shfl_sync(0xffffffffu, cut, 1);
+  s.seq = __shfl_sync(0xffffffffu, s.seq, 0); s.chunk = __shfl_sync(0xffffffffu, s.chunk, 0);
+  s.i = __shfl_sync(0xffffffffu, s.i, 0); s.g0 = __shfl_sync(0xffffffffu, s.g0, 0);
+  s.cached_tiles = __shfl_sync(0xffffffffu, s.cached_tiles, 0); s.final_rows = __shfl_sync(0xffffffffu, s.final_rows, 0);
+  s.n_items = __shfl_sync(0xffffffffu, s.n_items, 0); s.item0 = __shfl_sync(0xffffffffu, s.item0, 0);
+}
+// The next piece of the run.
+__device__ __forceinline__ WorkEntry stream_next(const AttnParams &p, StreamState &s) {
+  WorkEntry e = {-1, 0, 0, 0, -1, 0};
+  if (s.pos >= s.end) return e;
+  int n = stream_item_tiles(p, s);
+  while (s.pos >= s.g0 + n) {
+    s.g0 += n;
+    if (++s.i == s.n_items) {
+      s.i = 0;
+      if (++s.chunk == p.n_chunks) { s.chunk = 0; ++s.seq; stream_sequence(p, s); }
+    }
+    n = stream_item_tiles(p, s);
+  }
+  e.pair = s.item0 + s.i; e.chunk = s.chunk;
+  e.tile0 = s.pos - s.g0;
+  e.n_tiles = min(s.end, s.g0 + n) - s.pos;
+  s.pos += e.n_tiles;
+  // the CTAs that share the item: the last one whose run begins at or before its first tile .. the last one whose run
+  // begins inside it (cuts near the edges moved as above)
+  const int g = (int)gridDim.x;
+  auto last_cut_up_to = [&](int x) { return min(g - 1, (int)((((long long)x + 1) * g - 1) / s.total)); };
+  const int j0 = last_cut_up_to(s.g0 + min(kStreamSnap, n - 1));
+  const int j1 = max(j0, last_cut_up_to(s.g0 + n - kStreamSnap - 1));
+  if (j1 > j0) {
+    e.split = (int)blockIdx.x - j0;
+    e.fill = (int)blockIdx.x == j1 ? e.split + 1 : p.n_splits;
+    if (e.split < 0 || j1 - j0 >= p.n_splits) { ba_record_status(p.status, BA_ERR_SHAPE); e.pair = -1; }
+  }
+  return e;
+}
+
 // The last own key tile of an item covers the diagonal of the causal range.  When every row of the item
 // ends in the tile's first 64 keys (true for every other item: items are 64-token aligned, key tiles 128),
 // its second half is masked for all of them: the products and the exponentials of that half are skipped.
@@ -260,15 +379,8 @@ __device__ __forceinline__ bool last_tile_is_half(const Work &wk) {
 }
 
 // Block-by-block walk of the cached keys: index (cache order) of the block that holds key tile
-// `target` (counted over the whole batch); the sequence's blocks follow cb0.
-__device__ __forceinline__ int find_cache_block(const AttnParams &p, const Item &it, int target) {
-  int lo = it.cb0, hi = p.seg.n_cached_blocks;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(p.seg.cache_tile_cu + mid) <= target) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
+// `target` (counted over the whole batch).
+__device__ __forceinline__ int find_cache_block(const AttnParams &p, int target) { return __ldg(p.seg.cache_tile_block + target); }
 
 // Counter-rotation of query rows [row_begin, row_end) of one tile (fused warm path): dst = R(-delta) src,
 // with cs = (cos, sin)(delta * theta_m) of the current cached block.  Both tiles are in the 128-byte
@@ -331,13 +443,14 @@ __device__ __forceinline__ void rotate_q_row(const uint8_t *__restrict__ src, ui
   for (int i = 0; i < kVec; ++i) *reinterpret_cast<uint4 *>(dst + off[i]) = v[i];
 }
 
-// kFused selects the fused warm path at compile time, so that the plain path carries none of its code.
-template <int D, bool kFused>
+template <int D, int kVariant>
 __global__ void __launch_bounds__(kThreads, 1)
 ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                        const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_kc,
                        const __grid_constant__ CUtensorMap tmap_vc, const AttnParams p) {
   using L = Layout<D>;
+  constexpr bool kFused = kVariant == kFusedPath;
+  constexpr int kStages = ring_stages(kVariant);
   // setmaxnreg is a warpgroup-wide instruction: the four service warps (8-11) must ask for the same count
   constexpr int kServiceRegs = kFused ? kServiceRegsFused : kServiceRegsPlain;
   constexpr int kSoftmaxRegs = kFused ? kSoftmaxRegsFused : kSoftmaxRegsPlain;
@@ -350,7 +463,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
 
   if (tid == 0) {
     for (int b = 0; b < 2; ++b)
-      for (int t = 0; t < 2; ++t) { mbar_init(&ctrl->q_full[b][t], 1); mbar_init(&ctrl->q_empty[b][t], 4); }
+      for (int t = 0; t < 2; ++t) { mbar_init(&ctrl->q_full[b][t], 1); mbar_init(&ctrl->q_empty[b][t], kVariant == kDeepRing ? 1 : 4); }
     for (int s = 0; s < kStages; ++s) { mbar_init(&ctrl->kv_full[s], 1); mbar_init(&ctrl->kv_empty[s], 1); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(&ctrl->s_full[t], 1); mbar_init(&ctrl->p_full[t][0], 128); mbar_init(&ctrl->p_full[t][1], 128);
@@ -363,13 +476,16 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     fence_barrier_init();
   }
   if (warp == 9) { tmem_alloc(&ctrl->tmem_base, 512); tmem_relinquish(); }
+  if (warp == 10 && elect_one()) {
+    prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_kc); prefetch_tmap(&tmap_vc);
+  }
   // The CTA's first entry is known from its index: the scheduling warp looks it up while the others set the CTA up.
   // Inconsistent tables: no attention work is taken, a background job still runs.
   int n_items = 0;
-  WorkEntry first = {-1, 0, 0, 0, 0, 0};
+  WorkEntry first = {-1, 0, 0, 0, -1, 0};
   if (warp == 8) {
     n_items = count_items(p);
-    if (!p.balanced) first = list_entry(p, n_items, (int)blockIdx.x);
+    if (!p.balanced && !p.stream) first = list_entry(p, n_items, (int)blockIdx.x);
   }
   tc_fence_before();
   __syncthreads();
@@ -417,9 +533,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         __syncwarp();
       }
     }
+    StreamState ss = {};
+    if (p.stream && n_items > 0) stream_start(p, ss);
     if (elect_one()) {
-      prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v);
-      prefetch_tmap(&tmap_kc); prefetch_tmap(&tmap_vc);
       // balanced launch: run [bal_pos, bal_end) of the front tiles of all (chunk, item), bal_hm of them per chunk
       int bal_pos = 0, bal_end = 0, bal_hm = 0, bal_nh = 0;
       long long bal_all = 0;
@@ -432,7 +548,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         bal_end = (int)(bal_all * (j + 1) / bal_nh);
       }
       auto balanced_entry = [&](int n_done) -> WorkEntry {
-        WorkEntry e = {-1, 0, 0, 0, 0, 0};
+        WorkEntry e = {-1, 0, 0, 0, -1, 0};
         if (bal_np == 0) return e;
         const int b = (int)blockIdx.x;
         if (b < p.balanced) {                              // the last bal_len key tiles of item b
@@ -478,8 +594,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (!ok) break;
         // balanced launch: the next piece of this CTA's share; persistent launch: next entry of the global list;
         // one-item launch: this CTA's own entry, then stop
-        WorkEntry e = {-1, 0, 0, 0, 0, 0};
+        WorkEntry e = {-1, 0, 0, 0, -1, 0};
         if (p.balanced) e = balanced_entry(n_work);
+        else if (p.stream) e = stream_next(p, ss);
         else if (n_work == 0) e = first;
         else if (p.persistent) e = list_entry(p, n_items, (int)gridDim.x + atomicAdd(p.counters, 1));
         const bool more = load_work(p, e, wk);
@@ -495,7 +612,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           const int qb = p.q_double ? (n_loaded & 1) : 0;            // buffer pair of this entry
           const int q_use = p.q_double ? (n_loaded >> 1) : n_loaded;  // earlier entries that used it
           ok = mbar_wait(&ctrl->q_empty[qb][0], (q_use & 1) ^ 1, abort_flag);
-          if (ok && it.n_qt == 2) ok = mbar_wait(&ctrl->q_empty[qb][1], ((qb ? uses1[1] : uses1[0]) & 1) ^ 1, abort_flag);
+          if (kVariant != kDeepRing && ok && it.n_qt == 2) ok = mbar_wait(&ctrl->q_empty[qb][1], ((qb ? uses1[1] : uses1[0]) & 1) ^ 1, abort_flag);
           if (!ok) break;
           ++n_loaded;
           if (it.n_qt == 2) { if (qb) ++uses1[1]; else ++uses1[0]; }
@@ -524,7 +641,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         };
         if (p.walk && wk.tile0 < it.n_cache_tiles) {
           const int target = it.ctile0 + wk.tile0;
-          pc = find_cache_block(p, it, target);
+          pc = find_cache_block(p, target);
           poff = (target - __ldg(p.seg.cache_tile_cu + pc)) * kBlockN;
           load_block(pc, c_len, k_base, v_base);
           load_block(pc + 1, n_len, n_kbase, n_vbase);
@@ -651,7 +768,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (jt < cached_end) {
           const int g = wk.it.ctile0 + jt;
           if (g >= ver_end[t]) {                           // first key tile of another cached block
-            if (walk_end < 0) { walk_pc = find_cache_block(p, wk.it, g); walk_end = __ldg(p.seg.cache_tile_cu + walk_pc + 1); }
+            if (walk_end < 0) { walk_pc = find_cache_block(p, g); walk_end = __ldg(p.seg.cache_tile_cu + walk_pc + 1); }
             while (g >= walk_end) { ++walk_pc; walk_end = __ldg(p.seg.cache_tile_cu + walk_pc + 1); }
             ver_end[t] = walk_end;
             change = true;
@@ -700,6 +817,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           if (t < n_qt && ok) ok = issue_qk(t, 0, gidx);
         if (!ok) break;
         mma_commit(&ctrl->kv_empty[gidx % kStages]);
+        if (kVariant == kDeepRing && n_tiles == 1) mma_commit(&ctrl->q_empty[0][0]);
         for (int j = 0; j < n_tiles && ok; ++j) {
           const bool last = j + 1 == n_tiles;
           const int iv = gidx + 2 * j + 1, ik = gidx + 2 * j + 2;   // ring positions of V_j and K_(j+1)
@@ -732,7 +850,10 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               ok = issue_qk(t, j + 1, ik);
               if (!ok) continue;
               BA_TR(2, j, t * 4 + 3);
-              if (t + 1 == n_qt) mma_commit(&ctrl->kv_empty[ik % kStages]);
+              if (t + 1 == n_qt) {
+                mma_commit(&ctrl->kv_empty[ik % kStages]);
+                if (kVariant == kDeepRing && j + 2 == n_tiles) mma_commit(&ctrl->q_empty[0][0]);   // that was the entry's last QK^T
+              }
             }
           }
         }
@@ -842,7 +963,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       };
       if (kFused && n_tiles > 0) {
         const bool first_cached = tile0 < cached_end;
-        if (first_cached) { f_pc = find_cache_block(p, it, it.ctile0 + tile0); fetch_cs(f_pc); }
+        if (first_cached) { f_pc = find_cache_block(p, it.ctile0 + tile0); fetch_cs(f_pc); }
         begin_version();
         ok = finish_version(first_cached);
         if (!ok) break;
@@ -972,14 +1093,15 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       }
 
       // (the item is looked up again for the write-out: its rows need not be kept in registers through the loop)
-      int q_row0, q_rows;
-      asm volatile("ld.global.nc.v2.s32 {%0, %1}, [%2];" : "=r"(q_row0), "=r"(q_rows) : "l"(p.items + 8 * (size_t)e.pair));
+      int q_row0, q_rows, part_row0;
+      asm volatile("ld.global.nc.v2.s32 {%0, %1}, [%3];\n\tld.global.nc.s32 %2, [%3 + 20];"
+                   : "=&r"(q_row0), "=&r"(q_rows), "=r"(part_row0) : "l"(p.items + 8 * (size_t)e.pair));
       if (ok && n_tiles > 0) { ok = mbar_wait(&ctrl->o_done[t], o_uses & 1, abort_flag); ++o_uses; }
       if (ok) {
         tc_fence_after();
         const float inv = l > 0.f ? 1.f / l : 0.f;
         const float lse_val = l > 0.f ? (m_used * sl + log2f(l)) * 0.6931471805599453f : -INFINITY;
-        const bool partial = p.n_splits > 1;
+        const bool partial = e.split >= 0 && p.cluster <= 1;
         // Rows leave through shared memory -- the warp's quarter of the entry's own query tile, which every product has
         // read by now -- so that a store instruction writes whole rows: stores straight from the row each thread owns touch
         // 32 rows at a time and took 5000-7000 cycles a tile (seven edited blocks, 312 entries: 34.9 -> 27 us a layer).
@@ -991,79 +1113,93 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         const int row_tok = q_row0 + t * p.tok + ((quarter * 32 + lane) >> p.hpt_log2), head = out_head0 + (lane & (p.hpt - 1));
         const bool row_valid = row_tok <= q_last && row_tok < p.n_q_rows;
         if (row_tok <= q_last && row_tok >= p.n_q_rows) ba_record_status(p.status, BA_ERR_SHAPE);
-        uint8_t *stage = (kFused ? ver_buf(n_made - 1)
-                                 : smem + ((p.q_double && (n_loaded & 1)) ? L::kBg + t * L::kTileBytes : (t ? L::kQ1 : L::kQ0))) +
-                         quarter * (32 * D * 2);
-        auto store_rows = [&](auto &&address) {                      // address(output row) of the D * 2 bytes staged for it
-          constexpr int kRowChunks = D / 8;
+        // (kDeepRing: through rows of its own, 128 bytes at a time)
+        constexpr int kStageRow = kVariant == kDeepRing ? 128 : 2 * D;
+        uint8_t *stage = (kVariant == kDeepRing ? smem + L::kBg + L::kTileBytes + t * (128 * kStageRow)
+                          : kFused              ? ver_buf(n_made - 1)
+                                                : smem + ((p.q_double && (n_loaded & 1)) ? L::kBg + t * L::kTileBytes : (t ? L::kQ1 : L::kQ0))) +
+                         quarter * (32 * kStageRow);
+        // partial results of a prefill are indexed by the row's place among the rows of final blocks
+        const int part_shift = partial && !p.final_only ? part_row0 - q_row0 : 0;
+        const int tile_row0 = q_row0 + t * p.tok, tile_rows = min(q_last + 1, p.n_q_rows) - tile_row0;   // tokens stored
+        const size_t out_row0 = (size_t)(tile_row0 + part_shift) * p.Hq + out_head0;
+        // dst: where the staged bytes of the tile's first row go; row_bytes: from one (token, head) row to the next
+        auto store_rows = [&](uint8_t *dst, int row_bytes) {
+          constexpr int kRowChunks = kStageRow / 16;
+          const int c = lane % kRowChunks;
+          dst += c * 16;
           __syncwarp();
-#pragma unroll 4
+#pragma unroll 8
           for (int i = 0; i < kRowChunks; ++i) {
-            const int lr = (i * 32 + lane) / kRowChunks, c = lane % kRowChunks;
+            const int lr = i * (32 / kRowChunks) + lane / kRowChunks, rr = quarter * 32 + lr, tk = rr >> p.hpt_log2;
             const uint4 x = *reinterpret_cast<const uint4 *>(stage + lr * (kRowChunks * 16) + ((c ^ (lr & 7)) << 4));
-            const int rr = quarter * 32 + lr;
-            const int tk = q_row0 + t * p.tok + (rr >> p.hpt_log2);
-            if (tk <= q_last && tk < p.n_q_rows)
-              *reinterpret_cast<uint4 *>(address((size_t)tk * p.Hq + out_head0 + (rr & (p.hpt - 1))) + c * 16) = x;
+            if (tk < tile_rows) *reinterpret_cast<uint4 *>(dst + (tk * p.Hq + (rr & (p.hpt - 1))) * row_bytes) = x;
           }
           __syncwarp();
         };
         if (n_tiles > 0) {
           if (partial || p.out_f32) {
-            uint8_t *base = partial ? reinterpret_cast<uint8_t *>(p.o_part + (size_t)e.split * p.n_q_rows * p.Hq * D)
+            uint8_t *base = partial ? reinterpret_cast<uint8_t *>(p.o_part + (size_t)e.split * p.n_part_rows * p.Hq * D)
                                     : reinterpret_cast<uint8_t *>(p.o);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {                            // half of every row at a time: as many bytes as a bf16 row
+            for (int h = 0; h < 4 * D / kStageRow; ++h) {            // kStageRow bytes of every row at a time
 #pragma unroll
-              for (int q = 0; q < D / 64; ++q) {
+              for (int q = 0; q < kStageRow / 128; ++q) {
                 uint32_t o[32];
-                tmem_ld_32x32b_x32(tO + h * (D / 2) + q * 32, o);
+                tmem_ld_32x32b_x32(tO + h * (kStageRow / 4) + q * 32, o);
                 tmem_wait_ld();
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                  *reinterpret_cast<float4 *>(stage + lane * (D * 2) + (((q * 8 + i) ^ (lane & 7)) << 4)) =
+                  *reinterpret_cast<float4 *>(stage + lane * kStageRow + (((q * 8 + i) ^ (lane & 7)) << 4)) =
                       make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
                                   __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
               }
-              store_rows([&](size_t row) { return base + (row * D + h * (D / 2)) * 4; });
+              store_rows(base + out_row0 * D * 4 + h * kStageRow, D * 4);
             }
           } else {
 #pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-              uint32_t o[32];
-              tmem_ld_32x32b_x32(tO + c * 32, o);
-              tmem_wait_ld();
+            for (int h = 0; h < 2 * D / kStageRow; ++h) {
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                uint32_t w[4];
+              for (int c = 0; c < kStageRow / 64; ++c) {
+                uint32_t o[32];
+                tmem_ld_32x32b_x32(tO + h * (kStageRow / 2) + c * 32, o);
+                tmem_wait_ld();
 #pragma unroll
-                for (int e2 = 0; e2 < 4; ++e2) {
-                  __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * e2]) * inv,
-                                                           __uint_as_float(o[8 * i + 2 * e2 + 1]) * inv);
-                  w[e2] = *reinterpret_cast<uint32_t *>(&v);
+                for (int i = 0; i < 4; ++i) {
+                  uint32_t w[4];
+#pragma unroll
+                  for (int e2 = 0; e2 < 4; ++e2) {
+                    __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * e2]) * inv,
+                                                             __uint_as_float(o[8 * i + 2 * e2 + 1]) * inv);
+                    w[e2] = *reinterpret_cast<uint32_t *>(&v);
+                  }
+                  *reinterpret_cast<uint4 *>(stage + lane * kStageRow + (((c * 4 + i) ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
-                *reinterpret_cast<uint4 *>(stage + lane * (D * 2) + (((c * 4 + i) ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
               }
+              store_rows(reinterpret_cast<uint8_t *>(p.o) + out_row0 * D * 2 + h * kStageRow, D * 2);
             }
-            store_rows([&](size_t row) { return reinterpret_cast<uint8_t *>(p.o) + row * D * 2; });
           }
         }
         if (n_tiles > 0) {
           // O_t has been read out of tensor memory: the next item's first PV may overwrite it
           tc_fence_before();
           mbar_arrive(&ctrl->o_free[t]);
-          if (!kFused) {
+          if (kVariant == kPlain) {
             fence_proxy_async();                           // the copy engine writes the buffer next
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctrl->q_empty[p.q_double ? (n_loaded & 1) : 0][t]);
           }
         }
         if (row_valid) {
+          float *lp = p.lse_part + (size_t)(row_tok + part_shift) * p.Hq + head;
           if (partial) {
-            p.lse_part[((size_t)e.split * p.n_q_rows + row_tok) * p.Hq + head] = lse_val;
+            lp[(size_t)e.split * p.n_part_rows * p.Hq] = lse_val;
             for (int s = e.fill; s < p.n_splits; ++s)      // slots no entry of this item writes: empty
-              p.lse_part[((size_t)s * p.n_q_rows + row_tok) * p.Hq + head] = -INFINITY;
-          } else if (p.lse) p.lse[(size_t)row_tok * p.Hq + head] = lse_val;
+              lp[(size_t)s * p.n_part_rows * p.Hq] = -INFINITY;
+          } else {
+            if (p.lse) p.lse[(size_t)row_tok * p.Hq + head] = lse_val;
+            if (p.stream && p.n_splits > 1) *lp = __uint_as_float(kRowIsComplete);
+          }
         }
       }
       }
@@ -1090,56 +1226,66 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
 }
 
 // Merge of split-KV partial results: o = sum_s w_s o_s / sum_s w_s with w_s = exp(lse_s - max lse).
-// One thread per 4 output columns; the order of the sum is fixed, so results are run-to-run stable.
-// kNS > 0: the number of splits is known at compile time and every load is issued before the first use.
-template <int D, int kNS>
+// blockIdx.y is a work item, blockIdx.x a head chunk and a part of the 256 (token, head) rows it has; one thread per 4
+// columns of a row; the order of the sum is fixed, so results are run-to-run stable.  Bound by latency: the log-sum-exps of all slots are loaded before the first use, and the partial rows kBatch at
+// a time (one by one, ten slots of 64 rows took 5.9 us).  In a stream launch many items need nothing and
+// their CTAs leave after one load: with many items a CTA takes 32 rows (16 requests: 18 us with a CTA for every 8 rows), with
+// few 8 rows at once.
+struct CombineParams {
+  const float *o_part, *lse_part;
+  void *o;
+  float *lse;
+  const int32_t *items, *totals;
+  int final_only, Hq, hpt, hpt_log2, parts_log2, n_part_rows, n_q_rows, n_splits, out_f32;
+};
+template <int D, int kMax>
 __global__ void __launch_bounds__(256)
-ba_combine_splits_kernel(const float *__restrict__ o_part, const float *__restrict__ lse_part, void *o, float *lse,
-                         int n_rows_heads, int n_splits, int out_f32) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  constexpr int kVec = D / 4;
-  const int rh = idx / kVec, v = idx - rh * kVec;
-  if (rh >= n_rows_heads) return;
-  float den = 0.f, mx = -INFINITY;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (kNS > 0) {
-    float ls[kNS > 0 ? kNS : 1];
-    float4 x[kNS > 0 ? kNS : 1];
+ba_combine_splits_kernel(const CombineParams p) {
+  constexpr int kVec = D / 4, kBatch = kMax < 8 ? kMax : 8;
+  const int n_final = __ldg(p.totals + 3);
+  if ((int)blockIdx.y >= n_final) return;
+  const int32_t *line = p.items + 8 * ((p.final_only ? 0 : __ldg(p.totals + 2) - n_final) + blockIdx.y);
+  const int q_row0 = __ldg(line), q_rows = min(__ldg(line + 1), p.n_q_rows - q_row0);
+  const int part0 = p.final_only ? q_row0 : __ldg(line + 5), head0 = (blockIdx.x >> p.parts_log2) * p.hpt;
+  const size_t slot = (size_t)p.n_part_rows * p.Hq;
+  const int v = threadIdx.x % kVec;
+  const int rows = 256 >> p.parts_log2, part_row0 = (blockIdx.x & ((1 << p.parts_log2) - 1)) * rows;
+  for (int r = threadIdx.x / kVec; r < rows; r += 256 / kVec) {          // head r % hpt of token r / hpt
+    const int row = (part_row0 + r) >> p.hpt_log2, h = head0 + (r & (p.hpt - 1));
+    if (row >= q_rows) return;
+    const size_t at = (size_t)(part0 + row) * p.Hq + h, out = (size_t)(q_row0 + row) * p.Hq + h;
+    float ls[kMax], mx = -INFINITY, den = 0.f;
 #pragma unroll
-    for (int s = 0; s < kNS; ++s) {
-      ls[s] = __ldg(lse_part + (size_t)s * n_rows_heads + rh);
-      x[s] = __ldcs(reinterpret_cast<const float4 *>(o_part + ((size_t)s * n_rows_heads + rh) * D) + v);
-    }
+    for (int s = 0; s < kMax; ++s) ls[s] = s < p.n_splits ? __ldg(p.lse_part + s * slot + at) : -INFINITY;
+    if (__float_as_uint(ls[0]) == kRowIsComplete) return;                // (the whole item is)
 #pragma unroll
-    for (int s = 0; s < kNS; ++s) mx = fmaxf(mx, ls[s]);
+    for (int s = 0; s < kMax; ++s) mx = fmaxf(mx, ls[s]);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int s = 0; s < kNS; ++s) {
-      const float w = (ls[s] == -INFINITY) ? 0.f : __expf(ls[s] - mx);
-      if (w == 0.f) x[s] = make_float4(0.f, 0.f, 0.f, 0.f);   // an empty slot holds no values at all
-      den += w;
-      acc.x = fmaf(w, x[s].x, acc.x); acc.y = fmaf(w, x[s].y, acc.y); acc.z = fmaf(w, x[s].z, acc.z); acc.w = fmaf(w, x[s].w, acc.w);
+    for (int s0 = 0; s0 < kMax; s0 += kBatch) {
+      float4 x[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i)                       // an empty slot holds no values at all
+        x[i] = ls[s0 + i] == -INFINITY ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                       : __ldcs(reinterpret_cast<const float4 *>(p.o_part + ((s0 + i) * slot + at) * D) + v);
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const float w = ls[s0 + i] == -INFINITY ? 0.f : __expf(ls[s0 + i] - mx);
+        den += w;
+        acc.x = fmaf(w, x[i].x, acc.x); acc.y = fmaf(w, x[i].y, acc.y); acc.z = fmaf(w, x[i].z, acc.z); acc.w = fmaf(w, x[i].w, acc.w);
+      }
     }
-  } else {
-    for (int s = 0; s < n_splits; ++s) mx = fmaxf(mx, __ldg(lse_part + (size_t)s * n_rows_heads + rh));
-    for (int s = 0; s < n_splits; ++s) {
-      const float ls = __ldg(lse_part + (size_t)s * n_rows_heads + rh);
-      const float w = (ls == -INFINITY) ? 0.f : __expf(ls - mx);
-      float4 x = __ldg(reinterpret_cast<const float4 *>(o_part + ((size_t)s * n_rows_heads + rh) * D) + v);
-      if (w == 0.f) x = make_float4(0.f, 0.f, 0.f, 0.f);
-      den += w;
-      acc.x = fmaf(w, x.x, acc.x); acc.y = fmaf(w, x.y, acc.y); acc.z = fmaf(w, x.z, acc.z); acc.w = fmaf(w, x.w, acc.w);
+    const float inv = 1.f / den;
+    acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+    if (p.out_f32) {
+      reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.o) + out * D)[v] = acc;
+    } else {
+      __nv_bfloat162 a = __floats2bfloat162_rn(acc.x, acc.y), b = __floats2bfloat162_rn(acc.z, acc.w);
+      uint2 w2 = make_uint2(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b));
+      reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(p.o) + out * D)[v] = w2;
     }
+    if (p.lse && v == 0) p.lse[out] = mx + logf(den);
   }
-  const float inv = 1.f / den;
-  acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
-  if (out_f32) {
-    reinterpret_cast<float4 *>(reinterpret_cast<float *>(o) + (size_t)rh * D)[v] = acc;
-  } else {
-    __nv_bfloat162 a = __floats2bfloat162_rn(acc.x, acc.y), b = __floats2bfloat162_rn(acc.z, acc.w);
-    uint2 w2 = make_uint2(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b));
-    reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(o) + (size_t)rh * D)[v] = w2;
-  }
-  if (lse && v == 0) lse[rh] = mx + logf(den);
 }
 
 // ------------------------------------------------------------------ host side
@@ -1215,14 +1361,13 @@ constexpr int attend_smem_bytes() {
 // Per-context set-up of the attention path, with the context's device current: the kernels' shared-memory
 // limit is raised once here instead of on every launch, and the tensor-map table is created.
 ba_status ba_attend_sm100_setup(ba_ctx *ctx) {
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_attend_sm100_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   attend_smem_bytes<128>()));
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_attend_sm100_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   attend_smem_bytes<128>()));
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_attend_sm100_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   attend_smem_bytes<64>()));
-  BA_CUDA_TRY(cudaFuncSetAttribute(ba_attend_sm100_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   attend_smem_bytes<64>()));
+  auto raise = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kPlain>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedPath>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>()));
   ctx->maps = new (std::nothrow) ba_map_cache();
   if (!ctx->maps) return BA_ERR_CUDA;
   for (auto &sl : ctx->maps->slot) sl.ptr = nullptr;
@@ -1304,9 +1449,11 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   // work items: the exact count when ba_segment() saw the lengths on the host, else an upper bound
   const int pairs_known = a.final_only ? seg->n_final_items : seg->n_prompt_items;
   const unsigned pairs_upper = pairs_known > 0 ? (unsigned)pairs_known : (unsigned)(a.n_q_rows / pair_tok + n_units);
-  const long long items = (long long)((a.n_q_rows + pair_tok - 1) / pair_tok) * (Hq / p.hpt);
-  int n_splits = 1;
-  if (a.final_only && items < 2LL * ctx->sm_count) {
+  const long long items = (a.final_only && seg->n_final_items > 0 ? (long long)seg->n_final_items
+                                                                  : (long long)((a.n_q_rows + pair_tok - 1) / pair_tok)) * (Hq / p.hpt);
+  int n_splits = 1, stream_ctas = 0;
+  p.stream = 0; p.cluster = 0;
+  if (a.final_only) {
     // key tiles of an average item: counted by ba_segment() when it saw the lengths, else estimated
     const int32_t *ft = seg->final_key_tiles + (p.walk ? 3 : 0);
     const long long avg_tiles = (ft[0] > 0 && seg->n_final_items > 0)
@@ -1321,6 +1468,19 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     // equal splits or the balanced launch (ba_plan_splits, above the kernels' common declarations)
     const ba_split_plan plan = ba_plan_splits(ctx->sm_count, items, seg->n_final_items, Hq / p.hpt, avg_tiles, ft, cap);
     n_splits = plan.n_splits; p.balanced = plan.balanced; p.bal_len = plan.bal_len;
+    if (!p.balanced && ft[0] > 0 && cap > 0) {
+      const ba_stream_plan stream = ba_plan_stream(ctx->sm_count, Hq / p.hpt, ft, cap);
+      if (stream.n_ctas > 0 && stream.cost < ba_equal_splits_cost(ctx->sm_count, items, ft[2], n_splits)) {
+        p.stream = 1; stream_ctas = stream.n_ctas; n_splits = stream.n_slots;
+      }
+    }
+  } else if (!a.final_only && a.mode == BA_MODE_BLOCK && seg->n_final_items > 0 && seg->prompt_key_tiles > 0) {
+    // The items of final blocks see the whole prompt: with few of them the launch would end on one CTA each.
+    const size_t per_split = (size_t)seg->n_final_items * pair_tok * Hq * (D + 1) * sizeof(float);
+    const size_t taken = ba_scratch_offset(ctx) + ctx->pending_table_bytes;
+    const size_t avail = ctx->workspace_bytes > taken ? ctx->workspace_bytes - taken : 0;
+    n_splits = ba_plan_final_splits(ctx->sm_count, Hq / p.hpt, seg->n_prompt_items, seg->prompt_key_tiles,
+                                    seg->final_key_tiles[2], (int)min((size_t)16, avail / per_split));
   }
   p.n_splits = n_splits;
   p.n_chunks = Hq / p.hpt;
@@ -1328,8 +1488,9 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   // entry's start-up and write-out behind its neighbours (cold prefill: many entries per SM; final block
   // over a long cache: about two, the write-out of a CTA's first entry overlaps the start of its second).
   // Shorter lists are launched one CTA per entry.
-  const long long work_upper = (long long)pairs_upper * (Hq / p.hpt) * n_splits;
-  p.persistent = !p.balanced && work_upper > ctx->sm_count;
+  const long long work_upper = ((long long)pairs_upper * (a.final_only ? n_splits : 1) +
+                                (a.final_only ? 0 : (long long)seg->n_final_items * (n_splits - 1))) * (Hq / p.hpt);
+  p.persistent = !p.balanced && !p.stream && work_upper > ctx->sm_count;
   // the counters live in the last 256 bytes below the scratch area: zeroed by ba_create, left at zero by every launch
   int32_t *counters = nullptr;
   if (ctx->workspace && ctx->workspace_bytes >= ba_scratch_offset(ctx))
@@ -1338,9 +1499,10 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   if (p.persistent && !counters) p.persistent = 0;   // a context without workspace: one CTA per entry, however many
   if (p.persistent) p.counters = counters;
   p.o_part = nullptr; p.lse_part = nullptr;
+  p.n_part_rows = a.final_only ? a.n_q_rows : seg->n_final_items * pair_tok;
   if (n_splits > 1) {
     p.o_part = reinterpret_cast<float *>(reinterpret_cast<char *>(ctx->workspace) + ba_scratch_offset(ctx));
-    p.lse_part = p.o_part + (size_t)n_splits * a.n_q_rows * Hq * D;
+    p.lse_part = p.o_part + (size_t)n_splits * p.n_part_rows * Hq * D;
   }
 
   const CUtensorMap *mq = cached_map(ctx, a.q, D, Hq, a.n_q_rows, p.hpt, p.tok);
@@ -1359,7 +1521,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     if (!mvc) return BA_ERR_CUDA;
     tvc = *mvc;
   }
-  dim3 grid((unsigned)((p.persistent || p.balanced) ? ctx->sm_count : work_upper));
+  dim3 grid((unsigned)(p.stream ? stream_ctas : (p.persistent || p.balanced) ? ctx->sm_count : work_upper));
   // a queued re-encoding job rides along in the spare warps; a job whose rows do not fit the
   // staging buffers is run on its own first
   p.bg.n_rows = 0; p.bg_rows_per_chunk = 0;
@@ -1376,7 +1538,12 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
       if (fs != BA_OK) return fs;
     }
   }
-  p.q_double = (!p.fused && p.bg.n_rows == 0) ? 1 : 0;     // the staging area is free: second pair of query buffers
+  // The staging area is free on the plain path without a background job: a deeper ring where the keys and
+  // values are streamed once or twice (final blocks over their caches; in the balanced launch a tile is read by many CTAs
+  // and comes from L2), a second pair of query buffers elsewhere.
+  const bool free_area = !p.fused && p.bg.n_rows == 0;
+  const bool deep_ring = free_area && a.final_only && a.n_cache_rows > 0 && !p.balanced;
+  p.q_double = free_area && !deep_ring;
   // Side output of the fused call: the re-encoded keys, written by the stand-alone re-encoding kernel on the
   // context's side stream beside the attention launch (which cannot share an SM with anything and leaves
   // some SMs idle in its last wave); the caller's stream continues only when both are done.  (Measured
@@ -1394,12 +1561,15 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     if (rs != BA_OK) return rs;
     BA_CUDA_TRY(cudaEventRecord(ctx->ev_join, ctx->side_stream));
   }
+  auto launch_attend = [&](auto kern, int smem) { kern<<<grid, kThreads, smem, stream>>>(tq, tk, tv, tkc, tvc, p); };
   if (D == 128) {
-    auto kern = p.fused ? ba_attend_sm100_kernel<128, true> : ba_attend_sm100_kernel<128, false>;
-    kern<<<grid, kThreads, attend_smem_bytes<128>(), stream>>>(tq, tk, tv, tkc, tvc, p);
+    if (p.fused) launch_attend(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>());
+    else if (deep_ring) launch_attend(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>());
+    else launch_attend(ba_attend_sm100_kernel<128, kPlain>, attend_smem_bytes<128>());
   } else {
-    auto kern = p.fused ? ba_attend_sm100_kernel<64, true> : ba_attend_sm100_kernel<64, false>;
-    kern<<<grid, kThreads, attend_smem_bytes<64>(), stream>>>(tq, tk, tv, tkc, tvc, p);
+    if (p.fused) launch_attend(ba_attend_sm100_kernel<64, kFusedPath>, attend_smem_bytes<64>());
+    else if (deep_ring) launch_attend(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>());
+    else launch_attend(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>());
   }
   BA_CUDA_TRY(cudaGetLastError());
   ctx->launches += 1;
@@ -1407,22 +1577,20 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   ctx->last_attend[2] = p.balanced; ctx->last_attend[3] = p.bal_len;
   if (side_job) BA_CUDA_TRY(cudaStreamWaitEvent(stream, ctx->ev_join, 0));
   if (n_splits > 1) {
-    const int n_rh = a.n_q_rows * Hq;
-    const long long threads = (long long)n_rh * (D / 4);
-    const unsigned cgrid = (unsigned)((threads + 255) / 256);
-    auto launch = [&](auto kern) {
-      kern<<<cgrid, 256, 0, stream>>>(p.o_part, p.lse_part, a.o, a.lse, n_rh, n_splits, a.out_f32);
-    };
+    const unsigned n_merge_items = a.final_only && seg->n_final_items == 0 ? pairs_upper : (unsigned)seg->n_final_items;
+    const int parts_log2 = n_merge_items * p.n_chunks <= 64 ? 5 : 3;
+    CombineParams c = {p.o_part, p.lse_part, a.o, a.lse, p.items, seg->totals, a.final_only, Hq, p.hpt, p.hpt_log2, parts_log2, p.n_part_rows,
+                       a.n_q_rows, n_splits, a.out_f32};
+    const dim3 cgrid((unsigned)(p.n_chunks << parts_log2), n_merge_items);
+    auto launch = [&](auto kern) { kern<<<cgrid, 256, 0, stream>>>(c); };
     if (D == 128) {
-      if (n_splits == 2) launch(ba_combine_splits_kernel<128, 2>);
-      else if (n_splits == 3) launch(ba_combine_splits_kernel<128, 3>);
-      else if (n_splits == 4) launch(ba_combine_splits_kernel<128, 4>);
-      else launch(ba_combine_splits_kernel<128, 0>);
+      if (n_splits <= 4) launch(ba_combine_splits_kernel<128, 4>);
+      else if (n_splits <= 8) launch(ba_combine_splits_kernel<128, 8>);
+      else launch(ba_combine_splits_kernel<128, 32>);
     } else {
-      if (n_splits == 2) launch(ba_combine_splits_kernel<64, 2>);
-      else if (n_splits == 3) launch(ba_combine_splits_kernel<64, 3>);
-      else if (n_splits == 4) launch(ba_combine_splits_kernel<64, 4>);
-      else launch(ba_combine_splits_kernel<64, 0>);
+      if (n_splits <= 4) launch(ba_combine_splits_kernel<64, 4>);
+      else if (n_splits <= 8) launch(ba_combine_splits_kernel<64, 8>);
+      else launch(ba_combine_splits_kernel<64, 32>);
     }
     BA_CUDA_TRY(cudaGetLastError());
     ctx->launches += 1;

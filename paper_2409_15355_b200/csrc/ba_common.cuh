@@ -134,6 +134,39 @@ static inline ba_split_plan ba_plan_splits(int sm_count, long long items, int n_
   return plan;
 }
 
+// Time of equal splits in key tiles (an entry's start-up and write-out count as 3, the merging kernel as 3); every wave is
+// as long as its longest entry.
+static inline long long ba_equal_splits_cost(int sm_count, long long items, long long max_tiles, int n_splits) {
+  const long long waves = (items * n_splits + sm_count - 1) / sm_count;
+  return waves * ((max_tiles + n_splits - 1) / n_splits + 3) + (n_splits > 1 ? 3 : 0);
+}
+
+// Stream launch of ba_final_attend: the key tiles of all items, end to end, in one run per CTA.  Each CTA works on about
+// 1 + run / item pieces of items; a piece that is not a whole item costs a partial result.  key_tiles: sum, minimum, maximum
+// over the items of one head chunk.  cap: the most partial results per row.
+struct ba_stream_plan { int n_ctas, n_slots; long long cost; };
+static inline ba_stream_plan ba_plan_stream(int sm_count, int n_chunks, const int32_t *key_tiles, int cap) {
+  ba_stream_plan plan = {0, 0, 0};
+  const long long total = (long long)key_tiles[0] * n_chunks, n_max = key_tiles[2];
+  if (total <= 0 || total > 0x3fffffff) return plan;
+  const long long g = total < 2LL * sm_count ? (total + 1) / 2 : sm_count;
+  const long long run = (total + g - 1) / g, run_min = total / g;
+  const long long slots = (n_max - 1) / run_min + 2;           // runs an item of n_max tiles can touch
+  if (slots > cap) return plan;
+  const long long pieces = 1 + (run + n_max - 1) / n_max;
+  plan.n_ctas = (int)g; plan.n_slots = (int)slots; plan.cost = run + 2 + 2 * pieces + 3;
+  return plan;
+}
+
+// ba_block_prefill in block mode: into how many pieces the key tiles of a final block's items are cut, so that no entry is
+// longer than half of what an SM gets altogether (an entry's start-up and write-out count as one tile in a full list).
+static inline int ba_plan_final_splits(int sm_count, int n_chunks, int n_items, int n_tiles, int longest, int cap) {
+  const long long share = ((long long)n_tiles + n_items) * n_chunks / sm_count;
+  const long long piece = share / 2 > 6 ? share / 2 : 6;
+  const long long want = (longest + piece - 1) / piece;
+  return (int)(want < 1 || cap < 2 ? 1 : want < cap ? want : cap);
+}
+
 // Records the first device-side problem; later ones are dropped.
 __device__ __forceinline__ void ba_record_status(int32_t *status, int32_t code) {
   atomicCAS(status, 0, code);
@@ -184,6 +217,7 @@ struct ba_attend_args {
   int32_t page_rows;
   const int32_t *page_cu, *page_idx;
   int final_only;  // 1: ba_final_attend, 0: ba_block_prefill
+  int mode;        // ba_mode
 };
 
 ba_status ba_attend_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_segments *seg,

@@ -252,12 +252,18 @@ __device__ __forceinline__ void segment_rows(const SegmentArgs &a, const BlockTa
   // work items, 32 bytes each: first query row, query rows, first own key row, first cached row, cached rows, first cached
   // block, its first key tile and the sequence's key tiles when the cached keys are walked block by block
   int4 *items = reinterpret_cast<int4 *>(seg.prompt_items);
-  for (int i = at; i < t.cu_qtile[B]; i += step) {
-    const int b = upper_bound(t.cu_qtile, B + 1, i) - 1;
-    const int q0 = t.cu_block[b] + (i - t.cu_qtile[b]) * tt;
-    items[2 * i] = make_int4(q0, min(tt, t.cu_block[b + 1] - q0), t.kv_begin[b], 0);
-    items[2 * i + 1] = make_int4(0, 0, 0, 0);
+  const int n_final = t.cu_ftile[batch], n_other = t.cu_qtile[B] - n_final;
+  for (int i = at; i < n_other + n_final; i += step) {
+    const int b = upper_bound(t.cu_qtile, B + 1, i) - 1, k = i - t.cu_qtile[b];
+    const int s = upper_bound(t.cu_seq_block, batch + 1, b) - 1;
+    const bool fin = b == t.cu_seq_block[s + 1] - 1;
+    const int q0 = t.cu_block[b] + k * tt;
+    // final blocks last, the others closed up (cu_ftile[s] items of final blocks come before block b)
+    const int j = fin ? n_other + t.cu_ftile[s] + k : i - t.cu_ftile[s];
+    items[2 * j] = make_int4(q0, min(tt, t.cu_block[b + 1] - q0), t.kv_begin[b], 0);
+    items[2 * j + 1] = make_int4(0, fin ? t.cu_final_seq[s] + k * tt : 0, 0, 0);
   }
+  for (int i = at; i < t.cache_tile_cu[B - batch]; i += step) seg.cache_tile_block[i] = upper_bound(t.cache_tile_cu, B - batch + 1, i) - 1;
   items = reinterpret_cast<int4 *>(seg.final_items);
   for (int i = at; i < t.cu_ftile[batch]; i += step) {
     const int s = upper_bound(t.cu_ftile, batch + 1, i) - 1;

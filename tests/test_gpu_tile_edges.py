@@ -10,6 +10,7 @@ from paper_2409_15355_b200 import binding as B
 from paper_2409_15355_b200 import runtime as R
 from paper_2409_15355_b200 import workloads as W
 from tests.test_gpu_backward import check_grad, run_forward_backward
+from tests.test_gpu_parity import check_attention, run_prefill, run_warm
 
 pytestmark = pytest.mark.gpu
 
@@ -69,4 +70,56 @@ def test_segment_launch_variants(n_blocks, batch):
             sums[0].append(sums[0][-1] + per[0]); sums[1].append(sums[1][-1] + per[1])
             b0 += n
         assert items.tolist() == want and stream.tolist() == sums
+    c.close()
+
+
+def _requests(name, n, seed, cached, final, heads=(8, 2, 128), pool=False):
+    """n requests of cached[0] blocks of cached[1]..cached[2] tokens and a final block of final[0]..final[1]."""
+    rng = np.random.default_rng(seed)
+    lens, counts, pool_lens, idx = [], [], None, None
+    if pool:
+        pool_lens, idx = [int(v) for v in rng.integers(cached[1], cached[2] + 1, 20)], []
+    for _ in range(n):
+        if pool:
+            idx.append([int(v) for v in rng.integers(0, 20, cached[0])])
+            seq = [pool_lens[i] for i in idx[-1]]
+        else:
+            seq = [int(v) for v in rng.integers(cached[1], cached[2] + 1, cached[0])]
+        lens += seq + [int(rng.integers(final[0], final[1] + 1))]
+        counts.append(len(seq) + 1)
+    return W.Workload(name, *heads, 1e4, lens, counts, seed=seed, pool_lens=pool_lens, request_pool_idx=idx)
+
+
+STREAM_CASES = [_requests("more_items_than_sms", 40, 91, (4, 100, 300), (60, 200)),      # most items whole, some cut once
+                _requests("fewer_items", 9, 92, (5, 1, 400), (1, 130)),                  # every item cut several times
+                _requests("one_long_among_short", 30, 93, (1, 1, 2500), (64, 65)),
+                _requests("two_chunks_a_group", 7, 94, (4, 90, 300), (40, 140), heads=(8, 1, 64)),
+                _requests("pool", 24, 95, (5, 20, 290), (33, 129), pool=True)]
+
+
+@pytest.mark.parametrize("w", STREAM_CASES, ids=lambda w: w.name)
+@pytest.mark.parametrize("fused", [False, True], ids=["reencode_then_attend", "fused"])
+def test_stream_launch(w, fused):
+    shapes = []
+    o, lse, o_ref, lse_ref = run_warm(w, B.BA_MODE_BLOCK, fused=fused, shape_out=shapes)
+    assert shapes[0]["ctas"] <= 148 and shapes[0]["partials"] > 1 and shapes[0]["balanced_tails"] == 0
+    check_attention(o, o_ref, lse, lse_ref)
+    again = run_warm(w, B.BA_MODE_BLOCK, fused=fused)
+    assert np.array_equal(o, again[0]) and np.array_equal(lse, again[1])
+
+
+# The key tiles of the final blocks' items split in a prefill: one sequence and several, bf16 and fp32 stores
+@pytest.mark.parametrize("w", [_requests("one", 1, 96, (9, 150, 400), (65, 65)), _requests("three", 3, 97, (7, 64, 300), (1, 200)),
+                               _requests("half_head", 2, 98, (8, 100, 300), (129, 129), heads=(6, 2, 64))], ids=lambda w: w.name)
+def test_prefill_with_split_final_blocks(w):
+    o, lse, o_ref, lse_ref = run_prefill(w, B.BA_MODE_BLOCK)
+    check_attention(o, o_ref, lse, lse_ref)
+    o, lse, _, _ = run_prefill(w, B.BA_MODE_BLOCK, out_dtype=B.BA_OUT_BF16)
+    check_attention(o, o_ref, lse, lse_ref, bf16_store=True)
+    c = R.Context.for_workload(w)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    x = torch.zeros(w.n_tokens, w.n_q_heads, w.head_dim, dtype=torch.bfloat16, device="cuda")
+    kv = torch.zeros(w.n_tokens, w.n_kv_heads, w.head_dim, dtype=torch.bfloat16, device="cuda")
+    B.ba_block_prefill(c.ctx, x, kv, kv, x, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_BF16)
+    assert c.last_attend_shape()["partials"] > 1
     c.close()
