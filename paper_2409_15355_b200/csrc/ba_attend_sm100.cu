@@ -479,6 +479,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   if (warp == 10 && elect_one()) {
     prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); prefetch_tmap(&tmap_kc); prefetch_tmap(&tmap_vc);
   }
+  ba_pdl_wait();
   // The CTA's first entry is known from its index: the scheduling warp looks it up while the others set the CTA up.
   // Inconsistent tables: no attention work is taken, a background job still runs.
   int n_items = 0;
@@ -492,6 +493,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   tc_fence_after();
   const uint32_t tmem = ctrl->tmem_base;
   volatile int *abort_flag = &ctrl->abort_flag;
+  ba_pdl_trigger();
 
   // The CTA is persistent: its producer thread draws entries of the global work list from an
   // atomic counter (heaviest items first, whichever SM is free takes the next) and publishes them
@@ -1242,6 +1244,8 @@ template <int D, int kMax>
 __global__ void __launch_bounds__(256)
 ba_combine_splits_kernel(const CombineParams p) {
   constexpr int kVec = D / 4, kBatch = kMax < 8 ? kMax : 8;
+  ba_pdl_wait();
+  ba_pdl_trigger();
   const int n_final = __ldg(p.totals + 3);
   if ((int)blockIdx.y >= n_final) return;
   const int32_t *line = p.items + 8 * ((p.final_only ? 0 : __ldg(p.totals + 2) - n_final) + blockIdx.y);
@@ -1561,7 +1565,11 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     if (rs != BA_OK) return rs;
     BA_CUDA_TRY(cudaEventRecord(ctx->ev_join, ctx->side_stream));
   }
-  auto launch_attend = [&](auto kern, int smem) { kern<<<grid, kThreads, smem, stream>>>(tq, tk, tv, tkc, tvc, p); };
+  // (The balanced launch fills the GPU for hundreds of microseconds, and a re-encode on another stream fills the SMs it leaves
+  // at its end: early CTAs of the next kernel would only take those.)
+  const bool early = !p.balanced;
+  cudaError_t launched = cudaSuccess;
+  auto launch_attend = [&](auto kern, int smem) { launched = ba_launch(kern, grid, kThreads, smem, stream, early, tq, tk, tv, tkc, tvc, p); };
   if (D == 128) {
     if (p.fused) launch_attend(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>());
     else if (deep_ring) launch_attend(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>());
@@ -1571,7 +1579,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     else if (deep_ring) launch_attend(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>());
     else launch_attend(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>());
   }
-  BA_CUDA_TRY(cudaGetLastError());
+  BA_CUDA_TRY(launched);
   ctx->launches += 1;
   ctx->last_attend[0] = (int32_t)grid.x; ctx->last_attend[1] = n_splits;
   ctx->last_attend[2] = p.balanced; ctx->last_attend[3] = p.bal_len;
@@ -1582,7 +1590,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     CombineParams c = {p.o_part, p.lse_part, a.o, a.lse, p.items, seg->totals, a.final_only, Hq, p.hpt, p.hpt_log2, parts_log2, p.n_part_rows,
                        a.n_q_rows, n_splits, a.out_f32};
     const dim3 cgrid((unsigned)(p.n_chunks << parts_log2), n_merge_items);
-    auto launch = [&](auto kern) { kern<<<cgrid, 256, 0, stream>>>(c); };
+    auto launch = [&](auto kern) { launched = ba_launch(kern, cgrid, 256, 0, stream, early, c); };
     if (D == 128) {
       if (n_splits <= 4) launch(ba_combine_splits_kernel<128, 4>);
       else if (n_splits <= 8) launch(ba_combine_splits_kernel<128, 8>);
@@ -1592,7 +1600,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
       else if (n_splits <= 8) launch(ba_combine_splits_kernel<64, 8>);
       else launch(ba_combine_splits_kernel<64, 32>);
     }
-    BA_CUDA_TRY(cudaGetLastError());
+    BA_CUDA_TRY(launched);
     ctx->launches += 1;
   }
   return BA_OK;

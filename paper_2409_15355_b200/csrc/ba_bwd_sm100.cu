@@ -253,6 +253,7 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
   DkvCtrl *ctrl = reinterpret_cast<DkvCtrl *>(smem + L::kCtrl);
   const int tid = threadIdx.x, warp = tid >> 5;
   const ba_segments &sg = p.seg;
+  ba_pdl_wait();
   if (__ldg(sg.totals + 7) != BA_TABLES_VALID) return;
 
   // which keys: tile `kt` of the batch (a tile never spans two blocks), KV head `g`
@@ -297,6 +298,7 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
   tc_fence_after();
   const uint32_t tmem = ctrl->tmem_base;
   volatile int *abort_flag = &ctrl->abort_flag;
+  ba_pdl_trigger();
   const uint32_t tST = tmem, tDPT = tmem + 128, tDV = tmem + 256, tDK = tmem + 384;
 
   if (warp == kDkvLoadWarp) {
@@ -482,6 +484,9 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
   DqCtrl *ctrl = reinterpret_cast<DqCtrl *>(smem + L::kCtrl);
   const int tid = threadIdx.x, warp = tid >> 5;
   const ba_segments &sg = p.seg;
+  // This kernel needs dO . O, which was complete before the dK/dV kernel triggered, and nothing of the dK/dV kernel itself:
+  // it starts on the SMs that one leaves and waits for it only before it ends.
+  struct WaitAtExit { __device__ ~WaitAtExit() { ba_pdl_wait(); } } wait_at_exit;
   if (__ldg(sg.totals + 7) != BA_TABLES_VALID) return;
 
   // query tile: one half of a query-tile pair of the forward kernel.  Tiles are taken from the end of the list (within a
@@ -512,6 +517,7 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
   tc_fence_after();
   const uint32_t tmem = ctrl->tmem_base;
   volatile int *abort_flag = &ctrl->abort_flag;
+  ba_pdl_trigger();
   const uint32_t tS = tmem, tDP = tmem + 64, tDQ = tmem + 128;   // S and dP of one step (64 keys each), dQ
 
   if (warp == kDqLoadWarp) {
@@ -659,6 +665,8 @@ template <int D>
 __global__ void __launch_bounds__(256)
 ba_bwd_delta_kernel(const __nv_bfloat16 *__restrict__ o, const __nv_bfloat16 *__restrict__ d_o, float *__restrict__ delta,
                     int n_rows_heads) {
+  ba_pdl_wait();
+  ba_pdl_trigger();
   constexpr int kLanes = D / 8;                          // 8 or 16 threads per row
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long rh = t / kLanes;
@@ -706,12 +714,11 @@ template <int D>
 ba_status launch_bwd(ba_ctx *ctx, const BwdParams &p, const CUtensorMap &tq, const CUtensorMap &tdo, const CUtensorMap &tk,
                      const CUtensorMap &tv, const CUtensorMap &tk64, const CUtensorMap &tv64, int n_ktiles_upper, int n_pairs_upper,
                      cudaStream_t stream) {
-  ba_bwd_dkv_kernel<D><<<dim3((unsigned)n_ktiles_upper, (unsigned)p.Hkv), kDkvThreads, DkvLayout<D>::kBytes + 1024, stream>>>(tq, tdo, tk, tv, p);
-  BA_CUDA_TRY(cudaGetLastError());
+  BA_CUDA_TRY(ba_launch(ba_bwd_dkv_kernel<D>, dim3((unsigned)n_ktiles_upper, (unsigned)p.Hkv), kDkvThreads, DkvLayout<D>::kBytes + 1024,
+                        stream, true, tq, tdo, tk, tv, p));
   const int n_head_chunks = p.Hq / p.hpt;
-  ba_bwd_dq_kernel<D><<<(unsigned)(2 * n_pairs_upper) * n_head_chunks, kDqThreads, DqLayout<D>::kBytes, stream>>>(
-      tq, tdo, tk64, tv64, p, 2 * n_pairs_upper, n_head_chunks);
-  BA_CUDA_TRY(cudaGetLastError());
+  BA_CUDA_TRY(ba_launch(ba_bwd_dq_kernel<D>, dim3((unsigned)(2 * n_pairs_upper) * n_head_chunks), kDqThreads, DqLayout<D>::kBytes, stream,
+                        true, tq, tdo, tk64, tv64, p, 2 * n_pairs_upper, n_head_chunks));
   ctx->launches += 2;
   return BA_OK;
 }
@@ -749,13 +756,8 @@ ba_status ba_bwd_sm100_launch(ba_ctx *ctx, const void *q, const void *k, const v
   p.delta = delta;
   const int n_rh = T * Hq;
   const long long threads = (long long)n_rh * (D / 8);
-  if (D == 128)
-    ba_bwd_delta_kernel<128><<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(
-        (const __nv_bfloat16 *)o, (const __nv_bfloat16 *)d_o, delta, n_rh);
-  else
-    ba_bwd_delta_kernel<64><<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(
-        (const __nv_bfloat16 *)o, (const __nv_bfloat16 *)d_o, delta, n_rh);
-  BA_CUDA_TRY(cudaGetLastError());
+  BA_CUDA_TRY(ba_launch(D == 128 ? ba_bwd_delta_kernel<128> : ba_bwd_delta_kernel<64>, dim3((unsigned)((threads + 255) / 256)), 256, 0,
+                        stream, true, (const __nv_bfloat16 *)o, (const __nv_bfloat16 *)d_o, delta, n_rh));
   ctx->launches += 1;
   CUtensorMap tq, tdo, tk, tv, tk64, tv64;
   if (!bwd_make_map(&tq, q, D, Hq, T, p.hpt, p.tok) || !bwd_make_map(&tdo, d_o, D, Hq, T, p.hpt, p.tok) ||

@@ -16,6 +16,29 @@
     if (_e != cudaSuccess) { cudaGetLastError(); return BA_ERR_CUDA; } \
   } while (0)
 
+// Programmatic dependent launch.  A call is a chain of short kernels (tables, re-encode, attention, merge), and between two
+// of them the GPU idles for 1-2 us (a 32-layer retrieval prompt, 96 kernels: 1010 -> 897 us; forward and backward of three small
+// prompts: 91 -> 66 us).  Kernels launched with ba_launch may be scheduled as soon as every CTA of the kernel
+// before them in the stream has said ba_pdl_trigger() or exited: their set-up runs beside that kernel's tail.
+//  * ba_pdl_wait() returns when the kernel before has completed and its writes are visible; every thread calls it before it
+//    touches global memory, on every path to an exit, so that a kernel's completion implies that of all before it.
+//  * A kernel that allocates tensor memory triggers after its allocation: a CTA of the next kernel on the same SM must
+//    never hold columns that a CTA of this one still waits for.
+// A kernel launched in the ordinary way, before or after, behaves as usual.
+__device__ __forceinline__ void ba_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void ba_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+static inline cudaError_t ba_launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, bool early,
+                                    A &&...args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cfg.attrs = &attr; cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Value of ba_segments::totals[7] once ba_segment's kernel has found the lengths consistent.
 #define BA_TABLES_VALID 0x600D
 

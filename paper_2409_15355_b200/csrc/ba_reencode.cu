@@ -20,6 +20,8 @@ namespace {
 __global__ void __launch_bounds__(128)
 ba_rope_table_kernel(const int32_t *__restrict__ delta, int n_blocks, int half_dim,
                      double neg2_over_d_log2_base, float2 *__restrict__ table) {
+  ba_pdl_wait();
+  ba_pdl_trigger();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_blocks * half_dim) return;
   int c = i / half_dim, m = i - c * half_dim;
@@ -37,6 +39,8 @@ ba_rope_table_kernel(const int32_t *__restrict__ delta, int n_blocks, int half_d
 template <int kLayout, int kRows, int kPasses>
 __global__ void __launch_bounds__(512)
 ba_reencode_kernel(const ba_reencode_job job, int units_shift, int32_t *status) {
+  ba_pdl_wait();
+  ba_pdl_trigger();
   // units per row is a power of two for every head count that is one (units_shift >= 0): shifts, no divisions
   const int units_per_row = (kLayout == BA_ROPE_ADJACENT) ? job.row_vecs : (job.row_vecs >> 1);
   const int row_step = units_shift >= 0 ? (int)(blockDim.x >> units_shift) : (int)(blockDim.x / units_per_row);
@@ -76,8 +80,7 @@ ba_status ba_reencode_table_launch(ba_ctx *ctx, const int32_t *delta, int32_t n_
   const int D = ctx->cfg.head_dim, half = D / 2;
   const double k = -2.0 / (double)D * log2(ctx->cfg.rope_theta);
   const int n = n_blocks * half;
-  ba_rope_table_kernel<<<(n + 127) / 128, 128, 0, stream>>>(delta, n_blocks, half, k, table);
-  BA_CUDA_TRY(cudaGetLastError());
+  BA_CUDA_TRY(ba_launch(ba_rope_table_kernel, dim3((n + 127) / 128), 128, 0, stream, true, delta, n_blocks, half, k, table));
   ctx->launches += 1;
   return BA_OK;
 }
@@ -107,11 +110,8 @@ ba_status ba_reencode_main_launch(ba_ctx *ctx, const ba_reencode_job &job, cudaS
   constexpr int kPasses = 4;                // consecutive row groups per CTA
   const int rows_per_cta = (threads / units) * kRows * kPasses;
   const int grid = (job.n_rows + rows_per_cta - 1) / rows_per_cta;
-  if (adjacent)
-    ba_reencode_kernel<BA_ROPE_ADJACENT, kRows, kPasses><<<grid, threads, 0, stream>>>(job, units_shift, ctx->dev_status);
-  else
-    ba_reencode_kernel<BA_ROPE_HALF, kRows, kPasses><<<grid, threads, 0, stream>>>(job, units_shift, ctx->dev_status);
-  BA_CUDA_TRY(cudaGetLastError());
+  BA_CUDA_TRY(ba_launch(adjacent ? ba_reencode_kernel<BA_ROPE_ADJACENT, kRows, kPasses> : ba_reencode_kernel<BA_ROPE_HALF, kRows, kPasses>,
+                        dim3(grid), (unsigned)threads, 0, stream, true, job, units_shift, ctx->dev_status));
   ctx->launches += 1;
   return BA_OK;
 }

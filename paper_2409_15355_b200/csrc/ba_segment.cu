@@ -294,6 +294,8 @@ ba_segment_kernel(const SegmentArgs a, const int32_t *__restrict__ lens, const i
     __syncthreads();
   }
   const double theta = thread_theta(a);                  // (independent of the lengths: in front of the scans)
+  ba_pdl_wait();
+  ba_pdl_trigger();
   const BlockTables t = {tab[0], tab[1], tab[2], tab[3], tab[4], tab[5], tab[6], tab[7], tab[8], tab[9]};
   if (!segment_blocks<true>(a, lens, seq_nblocks, t, blockIdx.x == 0, scan_smem, &bad)) {
     if (blockIdx.x == 0 && threadIdx.x == 0) ba_record_status(a.status, BA_ERR_INVALID_ARG);
@@ -325,7 +327,7 @@ void launch_inline(const SegmentArgs &a, const int32_t *lens, const int32_t *nb,
   InlineLengths<N> in;
   for (int i = 0; i < a.B; ++i) in.v[i] = lens[i];
   for (int i = 0; i < a.batch; ++i) in.v[a.B + i] = nb[i];
-  ba_segment_kernel<N, kThreads><<<grid, kThreads, 0, stream>>>(a, nullptr, nullptr, in);
+  ba_launch(ba_segment_kernel<N, kThreads>, dim3(grid), kThreads, 0, stream, true, a, nullptr, nullptr, in);
 }
 
 }  // namespace
