@@ -166,6 +166,8 @@ struct Ctrl {
   uint64_t p_full[2][2];          // [query tile][half of the P tile]
   uint64_t o_done[2];
   uint64_t o_free[2];             // the softmax warps have read O_t out of tensor memory
+  uint64_t out_staged[2];         // every row of the output tile is in shared memory
+  int n_staged_out[2];            // output tiles handed to the copy engine so far
   uint64_t work_full[kWorkSlots];  // work entry published by the scheduler (producer thread)
   uint64_t work_empty[kWorkSlots]; // entry read by the MMA thread and the 8 softmax warps
   WorkEntry work_ring[kWorkSlots];
@@ -447,7 +449,7 @@ template <int D, int kVariant>
 __global__ void __launch_bounds__(kThreads, 1)
 ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                        const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_kc,
-                       const __grid_constant__ CUtensorMap tmap_vc, const AttnParams p) {
+                       const __grid_constant__ CUtensorMap tmap_vc, const __grid_constant__ CUtensorMap tmap_o, const AttnParams p) {
   using L = Layout<D>;
   constexpr bool kFused = kVariant == kFusedPath;
   constexpr int kStages = ring_stages(kVariant);
@@ -467,12 +469,12 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     for (int s = 0; s < kStages; ++s) { mbar_init(&ctrl->kv_full[s], 1); mbar_init(&ctrl->kv_empty[s], 1); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(&ctrl->s_full[t], 1); mbar_init(&ctrl->p_full[t][0], 128); mbar_init(&ctrl->p_full[t][1], 128);
-      mbar_init(&ctrl->o_done[t], 1); mbar_init(&ctrl->o_free[t], 128);
+      mbar_init(&ctrl->o_done[t], 1); mbar_init(&ctrl->o_free[t], 128); mbar_init(&ctrl->out_staged[t], 128);
       mbar_init(&ctrl->qr_full[t][0], 4); mbar_init(&ctrl->qr_full[t][1], 4); mbar_init(&ctrl->cs_full[t], D / 2);
       mbar_init(&ctrl->qraw_full[t], 1);
     }
     for (int k = 0; k < kWorkSlots; ++k) { mbar_init(&ctrl->work_full[k], 1); mbar_init(&ctrl->work_empty[k], 9); }
-    ctrl->abort_flag = 0;
+    ctrl->abort_flag = 0; ctrl->n_staged_out[0] = 0; ctrl->n_staged_out[1] = 0;
     fence_barrier_init();
   }
   if (warp == 9) { tmem_alloc(&ctrl->tmem_base, 512); tmem_relinquish(); }
@@ -893,6 +895,15 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     int n_made = 0;                       // fused: versions of this query tile prepared so far
     int tiles_before = 0;                 // key tiles of all earlier items (the producer counts the same way)
     int n_loaded = 0;                     // entries with key tiles so far (the producer counts the same way)
+    int out_pending = -1;                 // query buffer pair the copy engine may still be reading (thread 0 of the group)
+    auto release_out = [&]() {
+      if (kVariant == kPlain && out_pending >= 0) {
+        bulk_wait_read();
+        mbar_arrive_n(&ctrl->q_empty[out_pending][t], 4);
+        out_pending = -1;
+      }
+      __syncwarp();
+    };
     bool ok = true;
     Work wk;
     int n_work = 0;
@@ -908,6 +919,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       const Item &it = wk.it;
       const int n_tiles = wk.n_tiles, tile0 = wk.tile0, head0 = wk.head0;
       const bool half_last = last_tile_is_half(wk);
+      release_out();
       if (t < it.n_qt) {
       // rows past the block behave like its last row
       const int tok_c = min(it.q_row0 + t * p.tok + (r >> p.hpt_log2), it.q_row0 + it.q_rows - 1);
@@ -1139,7 +1151,44 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           }
           __syncwarp();
         };
-        if (n_tiles > 0) {
+        // A whole tile of bf16 rows leaves as one copy, laid out in the query tile's place the way the query tile was: the
+        // threads only fill shared memory (row by row as below a tile takes about 3500 cycles).
+        const bool whole_tile = kVariant == kPlain && n_tiles > 0 && !partial && !p.out_f32 && tile_rows >= p.tok;
+        if (whole_tile) {
+          uint8_t *tile = smem + ((p.q_double && (n_loaded & 1)) ? L::kBg + t * L::kTileBytes : (t ? L::kQ1 : L::kQ0));
+          uint8_t *row = tile + (thread & 127) * 128;
+#pragma unroll
+          for (int c = 0; c < D / 32; ++c) {
+            uint32_t o[32];
+            tmem_ld_32x32b_x32(tO + c * 32, o);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              uint32_t w[4];
+#pragma unroll
+              for (int e2 = 0; e2 < 4; ++e2) {
+                __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * e2]) * inv,
+                                                         __uint_as_float(o[8 * i + 2 * e2 + 1]) * inv);
+                w[e2] = *reinterpret_cast<uint32_t *>(&v);
+              }
+              *reinterpret_cast<uint4 *>(row + (c >> 1) * L::kRegionBytes + ((((c & 1) * 4 + i) ^ (lane & 7)) << 4)) =
+                  make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          }
+          fence_proxy_async();
+          mbar_arrive(&ctrl->out_staged[t]);
+          if ((thread & 127) == 0) {
+            ok = mbar_wait(&ctrl->out_staged[t], ctrl->n_staged_out[t] & 1, abort_flag);
+            ctrl->n_staged_out[t] += 1;
+            if (ok) {
+              for (int c = 0; c < L::kChunks; ++c) tma_store_3d(&tmap_o, tile + c * L::kRegionBytes, c * 64, out_head0, tile_row0);
+              bulk_commit_group();
+              out_pending = p.q_double ? (n_loaded & 1) : 0;
+            }
+          }
+          __syncwarp();
+          if (!p.q_double) release_out();                  // the next entry's queries want the same place
+        } else if (n_tiles > 0) {
           if (partial || p.out_f32) {
             uint8_t *base = partial ? reinterpret_cast<uint8_t *>(p.o_part + (size_t)e.split * p.n_part_rows * p.Hq * D)
                                     : reinterpret_cast<uint8_t *>(p.o);
@@ -1186,7 +1235,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           // O_t has been read out of tensor memory: the next item's first PV may overwrite it
           tc_fence_before();
           mbar_arrive(&ctrl->o_free[t]);
-          if (kVariant == kPlain) {
+          if (kVariant == kPlain && !whole_tile) {
             fence_proxy_async();                           // the copy engine writes the buffer next
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctrl->q_empty[p.q_double ? (n_loaded & 1) : 0][t]);
@@ -1208,6 +1257,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       tiles_before += n_tiles;
       if (n_tiles > 0) ++n_loaded;
     }
+    release_out();                        // no copy reads this CTA's memory when it ends
   }
 
   tc_fence_before();
@@ -1513,7 +1563,12 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   const CUtensorMap *mk = cached_map(ctx, a.k, D, Hkv, a.n_kv_rows, 1, kBlockN);
   const CUtensorMap *mv = cached_map(ctx, a.v, D, Hkv, a.n_kv_rows, 1, kBlockN);
   if (!mq || !mk || !mv) return BA_ERR_CUDA;
-  CUtensorMap tq = *mq, tk = *mk, tv = *mv, tkc = *mk, tvc = *mv;   // (a slot may be reused by a later look-up)
+  CUtensorMap tq = *mq, tk = *mk, tv = *mv, tkc = *mk, tvc = *mv, to = *mq;   // (a slot may be reused by a later look-up)
+  if (!a.out_f32) {
+    const CUtensorMap *mo = cached_map(ctx, a.o, D, Hq, a.n_q_rows, p.hpt, p.tok);
+    if (!mo) return BA_ERR_CUDA;
+    to = *mo;
+  }
   if (a.final_only && a.n_cache_rows > 0) {
     const int page_box = p.v_paged ? min(kBlockN, a.page_rows) : kBlockN;
     const CUtensorMap *mkc = cached_map(ctx, a.k_cache, D, Hkv, p.fused ? a.n_k_rows : a.n_cache_rows, 1,
@@ -1569,7 +1624,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   // at its end: early CTAs of the next kernel would only take those.)
   const bool early = !p.balanced;
   cudaError_t launched = cudaSuccess;
-  auto launch_attend = [&](auto kern, int smem) { launched = ba_launch(kern, grid, kThreads, smem, stream, early, tq, tk, tv, tkc, tvc, p); };
+  auto launch_attend = [&](auto kern, int smem) { launched = ba_launch(kern, grid, kThreads, smem, stream, early, tq, tk, tv, tkc, tvc, to, p); };
   if (D == 128) {
     if (p.fused) launch_attend(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>());
     else if (deep_ring) launch_attend(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>());

@@ -123,3 +123,28 @@ def test_prefill_with_split_final_blocks(w):
     B.ba_block_prefill(c.ctx, x, kv, kv, x, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_BF16)
     assert c.last_attend_shape()["partials"] > 1
     c.close()
+
+
+# bf16 rows leave as whole tiles (one copy) where a query tile is full and row by row where it is not: full, partly filled
+# and missing second tiles, many entries per CTA, a background job (one pair of query buffers), 1 / 2 / 4 heads per tile
+@pytest.mark.parametrize("heads", [(32, 8, 128), (8, 4, 64), (6, 2, 64)], ids=str)
+@pytest.mark.parametrize("background", [False, True], ids=["plain", "background_job"])
+def test_prefill_bf16_rows_full_and_ragged_tiles(heads, background):
+    rng = np.random.default_rng(101)
+    lens = [64, 32, 33, 1, 128, 96, 256, 65, 160] + [int(v) for v in rng.integers(1, 300, 60)]
+    w = W.Workload("rows", *heads, 1e4, lens, [20, 30, 19], seed=101)
+    x = [R.bits_to_device(b) for b in W.prefill_inputs(w)]
+    o32 = torch.full((w.n_tokens, heads[0], heads[2]), float("nan"), dtype=torch.float32, device="cuda")
+    o16 = torch.full_like(o32, float("nan"), dtype=torch.bfloat16)
+    c = R.Context.for_workload(w)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    B.ba_block_prefill(c.ctx, *x, o32, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    k_re = torch.empty(w.n_tokens - sum(w.final_lens()), heads[1], heads[2], dtype=torch.bfloat16, device="cuda")
+    for _ in range(3):
+        o16.fill_(float("nan"))
+        if background:
+            B.ba_reencode_k_deferred(c.ctx, x[1], None, w.n_tokens, k_re, seg.cache_cu, seg.cache_delta, seg.n_cached_blocks, len(k_re))
+        B.ba_block_prefill(c.ctx, *x, o16, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_BF16)
+        assert torch.equal(o16, o32.to(torch.bfloat16))      # the same fp32 rows, rounded to nearest even
+    assert c.device_status() == B.BA_OK
+    c.close()
