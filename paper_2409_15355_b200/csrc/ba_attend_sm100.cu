@@ -32,6 +32,7 @@
 // so the QK^T products switch buffers without a pause.  The cached keys are never rewritten or
 // re-read, and a key tile never spans two blocks.
 #include <math.h>
+#include <atomic>
 #include <new>
 #include <type_traits>
 
@@ -65,8 +66,10 @@ constexpr int kBlockN = 128;      // keys per tile
 // takes 2000-4500 cycles, three stages cover 2700 (64-token query over 32K cached keys: 800-1900 cycles of waiting in a
 // period of 4000-4900), and with the write-out elsewhere the one pair of query buffers is reloaded as soon as its last
 // product is done.
-constexpr int kPlain = 0, kFusedPath = 1, kDeepRing = 2;
-constexpr int ring_stages(int variant) { return variant == kDeepRing ? 4 : 3; }
+// The cluster forms of the last two merge the results of a cluster's CTAs in shared memory.
+constexpr int kPlain = 0, kFusedPath = 1, kDeepRing = 2, kFusedCluster = 3, kDeepCluster = 4;
+constexpr bool is_fused(int variant) { return variant == kFusedPath || variant == kFusedCluster; }
+constexpr bool is_deep(int variant) { return variant == kDeepRing || variant == kDeepCluster; }
 constexpr int kMaxStages = 4;
 constexpr float kRescaleThreshold = 8.0f;
 constexpr int kBgStageBytes = 16384; // two spare warps x two stages of source rows
@@ -445,14 +448,66 @@ __device__ __forceinline__ void rotate_q_row(const uint8_t *__restrict__ src, ui
   for (int i = 0; i < kVec; ++i) *reinterpret_cast<uint4 *>(dst + off[i]) = v[i];
 }
 
+// Cluster launch: the rows of an item are shared out among the CTAs of the cluster (a warp takes whole rows), each row is the
+// sum of every CTA's normalised row, weighted by its denominator -- the arithmetic of ba_combine_splits_kernel, through
+// distributed shared memory.  rows: fp32 [128][D] of this CTA for query tile 0 (at rows0) and 1 (rows1), 16-byte chunk c of row
+// r at chunk position c ^ (r & 7); lse: [2][128].
+template <int D>
+__device__ __forceinline__ void cluster_merge_rows(const AttnParams &p, const WorkEntry &e, int warp, uint32_t rows0, uint32_t rows1,
+                                                   uint32_t lse) {
+  constexpr int kLanes = D / 4, kRows = 32 / kLanes;      // lanes per row, rows a warp takes at a time
+  const int lane = threadIdx.x & 31, c = lane % kLanes;
+  const int n = p.cluster, rank = (int)cluster_rank();
+  Item it;
+  load_item(p, e.pair, it);
+  const int q_end = min(it.q_row0 + it.q_rows, p.n_q_rows);
+  for (int rr = (rank * 8 + warp) * kRows + lane / kLanes; rr < it.n_qt * 128; rr += n * 8 * kRows) {
+    const int t = rr >> 7, r = rr & 127;
+    const int tk = it.q_row0 + t * p.tok + (r >> p.hpt_log2), head = e.chunk * p.hpt + (r & (p.hpt - 1));
+    if (tk >= q_end) continue;
+    const uint32_t at = (t ? rows1 : rows0) + r * (D * 4) + ((c ^ (r & 7)) << 4);
+    float ls[kMaxCluster], mx = -INFINITY, den = 0.f;
+    float4 x[kMaxCluster], acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int s = 0; s < kMaxCluster; ++s) {
+      ls[s] = -INFINITY;
+      if (s < n) {
+        ls[s] = cluster_ld_f32(cluster_map(lse + rr * 4, s));
+        x[s] = cluster_ld_v4(cluster_map(at, s));
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < kMaxCluster; ++s) mx = fmaxf(mx, ls[s]);
+#pragma unroll
+    for (int s = 0; s < kMaxCluster; ++s) {
+      if (ls[s] == -INFINITY) continue;                   // that CTA saw no key: it holds no row at all
+      const float w = __expf(ls[s] - mx);
+      den += w;
+      acc.x = fmaf(w, x[s].x, acc.x); acc.y = fmaf(w, x[s].y, acc.y); acc.z = fmaf(w, x[s].z, acc.z); acc.w = fmaf(w, x[s].w, acc.w);
+    }
+    const float inv = 1.f / den;
+    acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+    const size_t row = (size_t)tk * p.Hq + head;
+    if (p.out_f32) {
+      reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.o) + row * D)[c] = acc;
+    } else {
+      __nv_bfloat162 a = __floats2bfloat162_rn(acc.x, acc.y), b = __floats2bfloat162_rn(acc.z, acc.w);
+      uint2 w2 = make_uint2(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b));
+      reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(p.o) + row * D)[c] = w2;
+    }
+    if (p.lse && c == 0) p.lse[row] = mx + logf(den);
+  }
+}
+
 template <int D, int kVariant>
 __global__ void __launch_bounds__(kThreads, 1)
 ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                        const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_kc,
                        const __grid_constant__ CUtensorMap tmap_vc, const __grid_constant__ CUtensorMap tmap_o, const AttnParams p) {
   using L = Layout<D>;
-  constexpr bool kFused = kVariant == kFusedPath;
-  constexpr int kStages = ring_stages(kVariant);
+  constexpr bool kFused = is_fused(kVariant), kDeep = is_deep(kVariant);
+  constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster;
+  constexpr int kStages = kDeep ? 4 : 3;
   // setmaxnreg is a warpgroup-wide instruction: the four service warps (8-11) must ask for the same count
   constexpr int kServiceRegs = kFused ? kServiceRegsFused : kServiceRegsPlain;
   constexpr int kSoftmaxRegs = kFused ? kSoftmaxRegsFused : kSoftmaxRegsPlain;
@@ -465,7 +520,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
 
   if (tid == 0) {
     for (int b = 0; b < 2; ++b)
-      for (int t = 0; t < 2; ++t) { mbar_init(&ctrl->q_full[b][t], 1); mbar_init(&ctrl->q_empty[b][t], kVariant == kDeepRing ? 1 : 4); }
+      for (int t = 0; t < 2; ++t) { mbar_init(&ctrl->q_full[b][t], 1); mbar_init(&ctrl->q_empty[b][t], kDeep ? 1 : 4); }
     for (int s = 0; s < kStages; ++s) { mbar_init(&ctrl->kv_full[s], 1); mbar_init(&ctrl->kv_empty[s], 1); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(&ctrl->s_full[t], 1); mbar_init(&ctrl->p_full[t][0], 128); mbar_init(&ctrl->p_full[t][1], 128);
@@ -474,6 +529,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       mbar_init(&ctrl->qraw_full[t], 1);
     }
     for (int k = 0; k < kWorkSlots; ++k) { mbar_init(&ctrl->work_full[k], 1); mbar_init(&ctrl->work_empty[k], 9); }
+    if (kClustered) ctrl->work_ring[0].pair = -1;
     ctrl->abort_flag = 0; ctrl->n_staged_out[0] = 0; ctrl->n_staged_out[1] = 0;
     fence_barrier_init();
   }
@@ -616,7 +672,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           const int qb = p.q_double ? (n_loaded & 1) : 0;            // buffer pair of this entry
           const int q_use = p.q_double ? (n_loaded >> 1) : n_loaded;  // earlier entries that used it
           ok = mbar_wait(&ctrl->q_empty[qb][0], (q_use & 1) ^ 1, abort_flag);
-          if (kVariant != kDeepRing && ok && it.n_qt == 2) ok = mbar_wait(&ctrl->q_empty[qb][1], ((qb ? uses1[1] : uses1[0]) & 1) ^ 1, abort_flag);
+          if (!kDeep && ok && it.n_qt == 2) ok = mbar_wait(&ctrl->q_empty[qb][1], ((qb ? uses1[1] : uses1[0]) & 1) ^ 1, abort_flag);
           if (!ok) break;
           ++n_loaded;
           if (it.n_qt == 2) { if (qb) ++uses1[1]; else ++uses1[0]; }
@@ -711,6 +767,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
             if (mbar_try_wait(&ctrl->kv_full[idx % kStages], (idx / kStages) & 1)) break;
       }
     }
+    if (kClustered) { __syncwarp(); cluster_sync(); }      // (the softmax warps merge between this one and the next)
   } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issuer
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMmaRegs));
@@ -821,7 +878,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           if (t < n_qt && ok) ok = issue_qk(t, 0, gidx);
         if (!ok) break;
         mma_commit(&ctrl->kv_empty[gidx % kStages]);
-        if (kVariant == kDeepRing && n_tiles == 1) mma_commit(&ctrl->q_empty[0][0]);
+        if (kDeep && n_tiles == 1) mma_commit(&ctrl->q_empty[0][0]);
         for (int j = 0; j < n_tiles && ok; ++j) {
           const bool last = j + 1 == n_tiles;
           const int iv = gidx + 2 * j + 1, ik = gidx + 2 * j + 2;   // ring positions of V_j and K_(j+1)
@@ -856,7 +913,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               BA_TR(2, j, t * 4 + 3);
               if (t + 1 == n_qt) {
                 mma_commit(&ctrl->kv_empty[ik % kStages]);
-                if (kVariant == kDeepRing && j + 2 == n_tiles) mma_commit(&ctrl->q_empty[0][0]);   // that was the entry's last QK^T
+                if (kDeep && j + 2 == n_tiles) mma_commit(&ctrl->q_empty[0][0]);   // that was the entry's last QK^T
               }
             }
           }
@@ -867,6 +924,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           if (t < n_qt) ++q_uses[t];
       }
     }
+    if (kClustered) { __syncwarp(); cluster_sync(); }
   } else if (warp >= 10) {
     // ------------------------------------------------------------ spare warps: background re-encoding
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kSpareRegs));
@@ -880,6 +938,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       ba_reencode_background(p.bg, p.counters + 1, smem + L::kBg + bw * 2 * kBgStageBytes, bsm, p.bg_rows_per_chunk,
                              p.status, [&](uint64_t *bar, uint32_t parity) { return mbar_wait(bar, parity, abort_flag); });
     }
+    if (kClustered) { __syncwarp(); cluster_sync(); }
   } else {
     // ------------------------------------------------------------ softmax, one thread per tile row
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
@@ -1115,7 +1174,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         tc_fence_after();
         const float inv = l > 0.f ? 1.f / l : 0.f;
         const float lse_val = l > 0.f ? (m_used * sl + log2f(l)) * 0.6931471805599453f : -INFINITY;
-        const bool partial = e.split >= 0 && p.cluster <= 1;
+        const bool partial = !kClustered && e.split >= 0;
         // Rows leave through shared memory -- the warp's quarter of the entry's own query tile, which every product has
         // read by now -- so that a store instruction writes whole rows: stores straight from the row each thread owns touch
         // 32 rows at a time and took 5000-7000 cycles a tile (seven edited blocks, 312 entries: 34.9 -> 27 us a layer).
@@ -1128,8 +1187,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         const bool row_valid = row_tok <= q_last && row_tok < p.n_q_rows;
         if (row_tok <= q_last && row_tok >= p.n_q_rows) ba_record_status(p.status, BA_ERR_SHAPE);
         // (kDeepRing: through rows of its own, 128 bytes at a time)
-        constexpr int kStageRow = kVariant == kDeepRing ? 128 : 2 * D;
-        uint8_t *stage = (kVariant == kDeepRing ? smem + L::kBg + L::kTileBytes + t * (128 * kStageRow)
+        constexpr int kStageRow = kDeep ? 128 : 2 * D;
+        uint8_t *stage = (kDeep ? smem + L::kBg + L::kTileBytes + t * (128 * kStageRow)
                           : kFused              ? ver_buf(n_made - 1)
                                                 : smem + ((p.q_double && (n_loaded & 1)) ? L::kBg + t * L::kTileBytes : (t ? L::kQ1 : L::kQ0))) +
                          quarter * (32 * kStageRow);
@@ -1188,6 +1247,24 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           }
           __syncwarp();
           if (!p.q_double) release_out();                  // the next entry's queries want the same place
+        } else if (kClustered) {
+          // fp32 rows stay here for the other CTAs of the cluster: tile 0 over both query tiles, tile 1 over the ring (every
+          // product that reads them has completed)
+          if (n_tiles > 0) {
+            uint8_t *row = smem + (t ? L::kRing : L::kQ0) + (thread & 127) * (D * 4);
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+              uint32_t o[32];
+              tmem_ld_32x32b_x32(tO + c * 32, o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<float4 *>(row + (((c * 8 + i) ^ (lane & 7)) << 4)) =
+                    make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
+                                __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
+            }
+          }
+          reinterpret_cast<float *>(smem + L::kCtrl + 1024)[t * 128 + (thread & 127)] = lse_val;
         } else if (n_tiles > 0) {
           if (partial || p.out_f32) {
             uint8_t *base = partial ? reinterpret_cast<uint8_t *>(p.o_part + (size_t)e.split * p.n_part_rows * p.Hq * D)
@@ -1241,7 +1318,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
             if (lane == 0) mbar_arrive(&ctrl->q_empty[p.q_double ? (n_loaded & 1) : 0][t]);
           }
         }
-        if (row_valid) {
+        if (row_valid && !kClustered) {
           float *lp = p.lse_part + (size_t)(row_tok + part_shift) * p.Hq + head;
           if (partial) {
             lp[(size_t)e.split * p.n_part_rows * p.Hq] = lse_val;
@@ -1258,8 +1335,16 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       if (n_tiles > 0) ++n_loaded;
     }
     release_out();                        // no copy reads this CTA's memory when it ends
+    if (kClustered) {
+      __syncwarp();
+      cluster_sync();
+      const WorkEntry e = ctrl->work_ring[0];
+      if (e.pair >= 0) cluster_merge_rows<D>(p, e, warp, smem_u32(smem + L::kQ0), smem_u32(smem + L::kRing), smem_u32(smem + L::kCtrl + 1024));
+      __syncwarp();
+    }
   }
 
+  if (kClustered) { __syncwarp(); cluster_sync(); }       // no CTA leaves while another reads its rows
   tc_fence_before();
   __syncthreads();
   if (tid == 0) {
@@ -1419,9 +1504,13 @@ ba_status ba_attend_sm100_setup(ba_ctx *ctx) {
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kPlain>, attend_smem_bytes<128>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedCluster>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepCluster>, attend_smem_bytes<128>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedPath>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedCluster>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepCluster>, attend_smem_bytes<64>()));
   ctx->maps = new (std::nothrow) ba_map_cache();
   if (!ctx->maps) return BA_ERR_CUDA;
   for (auto &sl : ctx->maps->slot) sl.ptr = nullptr;
@@ -1453,6 +1542,26 @@ extern "C" ba_status ba_selftest_wait_expiry(ba_ctx *ctx, void *stream) {
   BA_CUDA_TRY(cudaGetLastError());
   ctx->launches += 1;
   return BA_OK;
+}
+
+// Clusters of n attention CTAs (one per SM) the device runs at a time; asked once per process, device and size.
+static int max_clusters(ba_ctx *ctx, int n) {
+  static std::atomic<int> known[64][kMaxCluster + 1];
+  std::atomic<int> &slot = known[ctx->device & 63][n];
+  int v = slot.load(std::memory_order_relaxed);
+  if (v == 0) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)n; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ctx->sm_count / n * n)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = attend_smem_bytes<128>();
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    int got = 0;
+    if (cudaOccupancyMaxActiveClusters(&got, ba_attend_sm100_kernel<128, kDeepCluster>, &cfg) != cudaSuccess) { cudaGetLastError(); got = 0; }
+    v = got + 1;
+    slot.store(v, std::memory_order_relaxed);
+  }
+  return v - 1;
 }
 
 // Heads of one KV group packed into a query tile: the largest of 4, 2, 1 that divides the group size.
@@ -1524,8 +1633,13 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     n_splits = plan.n_splits; p.balanced = plan.balanced; p.bal_len = plan.bal_len;
     if (!p.balanced && ft[0] > 0 && cap > 0) {
       const ba_stream_plan stream = ba_plan_stream(ctx->sm_count, Hq / p.hpt, ft, cap);
-      if (stream.n_ctas > 0 && stream.cost < ba_equal_splits_cost(ctx->sm_count, items, ft[2], n_splits)) {
+      const long long equal_cost = ba_equal_splits_cost(ctx->sm_count, items, ft[2], n_splits);
+      if (stream.n_ctas > 0 && stream.cost < equal_cost) {
         p.stream = 1; stream_ctas = stream.n_ctas; n_splits = stream.n_slots;
+      }
+      if (a.n_cache_rows > 0 && !ctx->has_pending) {
+        const ba_cluster_plan cl = ba_plan_cluster(items, ft[2], [&](int n) { return max_clusters(ctx, n); });
+        if (cl.size > 0 && cl.cost < (double)(p.stream ? stream.cost : equal_cost)) { p.cluster = cl.size; p.stream = 0; n_splits = 1; }
       }
     }
   } else if (!a.final_only && a.mode == BA_MODE_BLOCK && seg->n_final_items > 0 && seg->prompt_key_tiles > 0) {
@@ -1544,7 +1658,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   // Shorter lists are launched one CTA per entry.
   const long long work_upper = ((long long)pairs_upper * (a.final_only ? n_splits : 1) +
                                 (a.final_only ? 0 : (long long)seg->n_final_items * (n_splits - 1))) * (Hq / p.hpt);
-  p.persistent = !p.balanced && !p.stream && work_upper > ctx->sm_count;
+  p.persistent = !p.balanced && !p.stream && p.cluster <= 1 && work_upper > ctx->sm_count;
   // the counters live in the last 256 bytes below the scratch area: zeroed by ba_create, left at zero by every launch
   int32_t *counters = nullptr;
   if (ctx->workspace && ctx->workspace_bytes >= ba_scratch_offset(ctx))
@@ -1580,7 +1694,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     if (!mvc) return BA_ERR_CUDA;
     tvc = *mvc;
   }
-  dim3 grid((unsigned)(p.stream ? stream_ctas : (p.persistent || p.balanced) ? ctx->sm_count : work_upper));
+  dim3 grid((unsigned)(p.cluster > 1 ? items * p.cluster : p.stream ? stream_ctas : (p.persistent || p.balanced) ? ctx->sm_count : work_upper));
   // a queued re-encoding job rides along in the spare warps; a job whose rows do not fit the
   // staging buffers is run on its own first
   p.bg.n_rows = 0; p.bg_rows_per_chunk = 0;
@@ -1624,16 +1738,20 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   // at its end: early CTAs of the next kernel would only take those.)
   const bool early = !p.balanced;
   cudaError_t launched = cudaSuccess;
-  auto launch_attend = [&](auto kern, int smem) { launched = ba_launch(kern, grid, kThreads, smem, stream, early, tq, tk, tv, tkc, tvc, to, p); };
-  if (D == 128) {
-    if (p.fused) launch_attend(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>());
-    else if (deep_ring) launch_attend(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>());
-    else launch_attend(ba_attend_sm100_kernel<128, kPlain>, attend_smem_bytes<128>());
-  } else {
-    if (p.fused) launch_attend(ba_attend_sm100_kernel<64, kFusedPath>, attend_smem_bytes<64>());
-    else if (deep_ring) launch_attend(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>());
-    else launch_attend(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>());
-  }
+  auto launch_attend = [&](auto kern, int smem) { launched = ba_launch_clusters(kern, p.cluster, grid, kThreads, smem, stream, early, tq, tk, tv, tkc, tvc, to, p); };
+  const int variant = p.fused ? (p.cluster > 1 ? kFusedCluster : kFusedPath) : deep_ring ? (p.cluster > 1 ? kDeepCluster : kDeepRing) : kPlain;
+  auto pick = [&](auto d_tag) {
+    constexpr int kD = decltype(d_tag)::value, kSmem = attend_smem_bytes<kD>();
+    switch (variant) {
+      case kFusedPath: launch_attend(ba_attend_sm100_kernel<kD, kFusedPath>, kSmem); break;
+      case kFusedCluster: launch_attend(ba_attend_sm100_kernel<kD, kFusedCluster>, kSmem); break;
+      case kDeepRing: launch_attend(ba_attend_sm100_kernel<kD, kDeepRing>, kSmem); break;
+      case kDeepCluster: launch_attend(ba_attend_sm100_kernel<kD, kDeepCluster>, kSmem); break;
+      default: launch_attend(ba_attend_sm100_kernel<kD, kPlain>, kSmem);
+    }
+  };
+  if (D == 128) pick(std::integral_constant<int, 128>{});
+  else pick(std::integral_constant<int, 64>{});
   BA_CUDA_TRY(launched);
   ctx->launches += 1;
   ctx->last_attend[0] = (int32_t)grid.x; ctx->last_attend[1] = n_splits;

@@ -28,15 +28,27 @@
 __device__ __forceinline__ void ba_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void ba_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
-static inline cudaError_t ba_launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, bool early,
-                                    A &&...args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+static inline cudaError_t ba_launch_clusters(void (*kernel)(P...), int cluster, dim3 grid, unsigned threads, size_t smem,
+                                             cudaStream_t stream, bool early, A &&...args) {
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (early) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-  cfg.attrs = &attr; cfg.numAttrs = early ? 1 : 0;
+  cfg.attrs = attr; cfg.numAttrs = (unsigned)n;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+static inline cudaError_t ba_launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, bool early,
+                                    A &&...args) {
+  return ba_launch_clusters(kernel, 1, grid, threads, smem, stream, early, static_cast<A &&>(args)...);
 }
 
 // Value of ba_segments::totals[7] once ba_segment's kernel has found the lengths consistent.
@@ -157,11 +169,11 @@ static inline ba_split_plan ba_plan_splits(int sm_count, long long items, int n_
   return plan;
 }
 
-// Time of equal splits in key tiles (an entry's start-up and write-out count as 3, the merging kernel as 3); every wave is
+// Time of equal splits in key tiles (an entry's start-up and write-out count as 3, the merging kernel as 5); every wave is
 // as long as its longest entry.
 static inline long long ba_equal_splits_cost(int sm_count, long long items, long long max_tiles, int n_splits) {
   const long long waves = (items * n_splits + sm_count - 1) / sm_count;
-  return waves * ((max_tiles + n_splits - 1) / n_splits + 3) + (n_splits > 1 ? 3 : 0);
+  return waves * ((max_tiles + n_splits - 1) / n_splits + 3) + (n_splits > 1 ? 5 : 0);
 }
 
 // Stream launch of ba_final_attend: the key tiles of all items, end to end, in one run per CTA.  Each CTA works on about
@@ -177,7 +189,24 @@ static inline ba_stream_plan ba_plan_stream(int sm_count, int n_chunks, const in
   const long long slots = (n_max - 1) / run_min + 2;           // runs an item of n_max tiles can touch
   if (slots > cap) return plan;
   const long long pieces = 1 + (run + n_max - 1) / n_max;
-  plan.n_ctas = (int)g; plan.n_slots = (int)slots; plan.cost = run + 2 + 2 * pieces + 3;
+  plan.n_ctas = (int)g; plan.n_slots = (int)slots; plan.cost = run + 2 + 2 * pieces + 5;
+  return plan;
+}
+
+// Cluster launch of ba_final_attend: the `size` CTAs of a cluster share one item's key tiles and merge their results in
+// shared memory, which costs about as much as 1.5 tiles and saves the partial results' way through memory and the merging
+// kernel.  fits(size): clusters of that size the GPU runs at a time (0: none).
+constexpr int kMaxCluster = 8;
+struct ba_cluster_plan { int size; double cost; };
+template <class Fits>
+static inline ba_cluster_plan ba_plan_cluster(long long items, long long max_tiles, Fits fits) {
+  ba_cluster_plan plan = {0, 0.};
+  for (int n = 2; n <= kMaxCluster && n <= max_tiles; ++n) {
+    const long long at_a_time = items <= 8 * (kMaxCluster + 1 - n) ? items : fits(n);   // (a few clusters always fit)
+    if (at_a_time < 1) continue;
+    const double cost = (double)((items + at_a_time - 1) / at_a_time) * ((max_tiles + n - 1) / n + 3) + 1.5;
+    if (!plan.size || cost < plan.cost) { plan.size = n; plan.cost = cost; }
+  }
   return plan;
 }
 
