@@ -1,4 +1,4 @@
-"""ctypes binding of the C ABI declared in include/ba.h.
+"""Binding of the C ABI declared in include/ba.h: ctypes, and for the calls a layer makes a small extension.
 
 Argument marshalling only: every step of the path runs in the CUDA library.
 Tensors are torch CUDA tensors (torch is used for device memory and streams);
@@ -65,12 +65,13 @@ class BaError(RuntimeError):
 
 
 _lib = None
+_marshal = None
 _raw_stream = _raw_device = None
 
 
 def load_library(path: Optional[str] = None) -> C.CDLL:
     """dlopen libba.so (building it first if its sources changed) and declare prototypes."""
-    global _lib
+    global _lib, _marshal
     if _lib is not None and path is None:
         return _lib
     if path is None:
@@ -114,8 +115,30 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
             raise RuntimeError(f"{name}: prototype not declared")
         if name not in ("ba_status_string", "ba_launch_count"):
             getattr(lib, name).restype = C.c_int
+    _marshal = _load_marshal()
+    _marshal.bind(lib._handle)
     _lib = lib
     return lib
+
+
+def _load_marshal():
+    """The extension that marshals the arguments of the hot calls (csrc/ba_marshal.c)."""
+    import importlib.util
+    spec = importlib.util.spec_from_file_location("ba_marshal", _build.build_marshal())
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    return mod
+
+
+def _calls():
+    if _marshal is None:
+        load_library()
+    return _marshal
+
+
+def _address(x):
+    """Host arrays are passed as addresses, as the library tells host from device memory by them."""
+    return x if x is None or isinstance(x, int) or hasattr(x, "data_ptr") else x.ctypes.data
 
 
 def status_string(status: int) -> str:
@@ -210,16 +233,14 @@ def ba_segment(ctx, block_lens, seq_nblocks, batch, n_blocks, n_tokens, mode, ta
     """block_lens / seq_nblocks: int32 numpy arrays (host) or torch CUDA tensors.
     table_buf: torch uint8 CUDA tensor of at least ba_segments_bytes() bytes.  Returns ba_segments."""
     seg = ba_segments()
-    _check(load_library().ba_segment(ctx, _ptr(block_lens), _ptr(seq_nblocks), batch, n_blocks, n_tokens,
-                                     mode, _ptr(table_buf), table_buf.numel() * table_buf.element_size(),
-                                     C.byref(seg), _stream_ptr(stream)), "ba_segment")
+    _check(_calls().segment(ctx, _address(block_lens), _address(seq_nblocks), batch, n_blocks, n_tokens, mode, table_buf,
+                            table_buf.numel() * table_buf.element_size(), seg, _stream_ptr(stream)), "ba_segment")
     return seg
 
 
 def ba_reencode_k(ctx, k_src, src_off, n_src_rows, k_dst, cu, delta, n_blocks, n_rows, stream=None):
     """cu / delta / src_off: device addresses (ints, e.g. seg.cache_cu) or torch int32 CUDA tensors."""
-    _check(load_library().ba_reencode_k(ctx, _ptr(k_src), _ptr(src_off), n_src_rows, _ptr(k_dst),
-                                        _ptr(cu), _ptr(delta), n_blocks, n_rows, _stream_ptr(stream)),
+    _check(_calls().reencode_k(ctx, k_src, src_off, n_src_rows, k_dst, cu, delta, n_blocks, n_rows, _stream_ptr(stream)),
            "ba_reencode_k")
 
 
@@ -248,50 +269,39 @@ def ba_selftest_wait_expiry(ctx, stream=None) -> None:
 
 
 def ba_block_prefill(ctx, q, k, v, o, lse, seg, mode, out_dtype, stream=None):
-    _check(load_library().ba_block_prefill(ctx, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
-                                           C.byref(seg), mode, out_dtype, _stream_ptr(stream)),
-           "ba_block_prefill")
+    _check(_calls().block_prefill(ctx, q, k, v, o, lse, seg, mode, out_dtype, _stream_ptr(stream)), "ba_block_prefill")
 
 
 def ba_final_attend_fused(ctx, q_f, k_f, v_f, n_final_rows, k_src, v_src, n_src_rows, src_off,
                           n_cache_rows, o, lse, seg, mode, out_dtype, stream=None, k_out=None):
     """k_out: optional bf16 tensor [n_cache_rows, n_kv_heads, head_dim] that receives the re-encoded keys."""
-    _check(load_library().ba_final_attend_fused(ctx, _ptr(q_f), _ptr(k_f), _ptr(v_f), n_final_rows,
-                                                _ptr(k_src), _ptr(v_src), n_src_rows, _ptr(src_off),
-                                                n_cache_rows, _ptr(k_out), _ptr(o), _ptr(lse), C.byref(seg), mode,
-                                                out_dtype, _stream_ptr(stream)), "ba_final_attend_fused")
+    _check(_calls().final_attend_fused(ctx, q_f, k_f, v_f, n_final_rows, k_src, v_src, n_src_rows, src_off, n_cache_rows, k_out, o,
+                                       lse, seg, mode, out_dtype, _stream_ptr(stream)), "ba_final_attend_fused")
 
 
 def ba_final_attend(ctx, q_f, k_f, v_f, n_final_rows, k_cache, v_cache, n_cache_rows, v_src_off,
                     n_v_rows, o, lse, seg, mode, out_dtype, stream=None):
-    _check(load_library().ba_final_attend(ctx, _ptr(q_f), _ptr(k_f), _ptr(v_f), n_final_rows,
-                                          _ptr(k_cache), _ptr(v_cache), n_cache_rows, _ptr(v_src_off),
-                                          n_v_rows, _ptr(o), _ptr(lse), C.byref(seg), mode, out_dtype,
-                                          _stream_ptr(stream)), "ba_final_attend")
+    _check(_calls().final_attend(ctx, q_f, k_f, v_f, n_final_rows, k_cache, v_cache, n_cache_rows, v_src_off, n_v_rows, o, lse, seg,
+                                 mode, out_dtype, _stream_ptr(stream)), "ba_final_attend")
 
 
 def ba_reencode_k_paged(ctx, k_pool, pages, k_dst, cu, delta, n_blocks, n_rows, stream=None):
-    _check(load_library().ba_reencode_k_paged(ctx, _ptr(k_pool), C.byref(pages), _ptr(k_dst), _ptr(cu), _ptr(delta),
-                                              n_blocks, n_rows, _stream_ptr(stream)), "ba_reencode_k_paged")
+    _check(_calls().reencode_k_paged(ctx, k_pool, pages, k_dst, cu, delta, n_blocks, n_rows, _stream_ptr(stream)),
+           "ba_reencode_k_paged")
 
 
 def ba_final_attend_paged(ctx, q_f, k_f, v_f, n_final_rows, k_cache, n_cache_rows, v_pool, pages, o, lse, seg,
                           mode, out_dtype, stream=None):
-    _check(load_library().ba_final_attend_paged(ctx, _ptr(q_f), _ptr(k_f), _ptr(v_f), n_final_rows, _ptr(k_cache),
-                                                n_cache_rows, _ptr(v_pool), C.byref(pages), _ptr(o), _ptr(lse),
-                                                C.byref(seg), mode, out_dtype, _stream_ptr(stream)),
-           "ba_final_attend_paged")
+    _check(_calls().final_attend_paged(ctx, q_f, k_f, v_f, n_final_rows, k_cache, n_cache_rows, v_pool, pages, o, lse, seg, mode,
+                                       out_dtype, _stream_ptr(stream)), "ba_final_attend_paged")
 
 
 def ba_final_attend_fused_paged(ctx, q_f, k_f, v_f, n_final_rows, k_pool, v_pool, pages, n_cache_rows, o, lse, seg,
                                 mode, out_dtype, stream=None, k_out=None):
-    _check(load_library().ba_final_attend_fused_paged(ctx, _ptr(q_f), _ptr(k_f), _ptr(v_f), n_final_rows,
-                                                      _ptr(k_pool), _ptr(v_pool), C.byref(pages), n_cache_rows,
-                                                      _ptr(k_out), _ptr(o), _ptr(lse), C.byref(seg), mode, out_dtype,
-                                                      _stream_ptr(stream)), "ba_final_attend_fused_paged")
+    _check(_calls().final_attend_fused_paged(ctx, q_f, k_f, v_f, n_final_rows, k_pool, v_pool, pages, n_cache_rows, k_out, o, lse, seg,
+                                             mode, out_dtype, _stream_ptr(stream)), "ba_final_attend_fused_paged")
 
 
 def ba_block_prefill_bwd(ctx, q, k, v, o, lse, d_o, dq, dk, dv, seg, mode, grad_dtype, stream=None):
-    _check(load_library().ba_block_prefill_bwd(ctx, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(d_o),
-                                               _ptr(dq), _ptr(dk), _ptr(dv), C.byref(seg), mode, grad_dtype,
-                                               _stream_ptr(stream)), "ba_block_prefill_bwd")
+    _check(_calls().block_prefill_bwd(ctx, q, k, v, o, lse, d_o, dq, dk, dv, seg, mode, grad_dtype, _stream_ptr(stream)),
+           "ba_block_prefill_bwd")

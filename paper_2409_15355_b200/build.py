@@ -1,7 +1,7 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a.
+"""Builds the CUDA library in-tree with nvcc for sm_100a, and the Python extension that marshals its arguments.
 
-The shared object is written next to this file (libba.so).  A sidecar file
-stores a hash of the sources and flags so that an up-to-date build is reused.
+The shared objects are written next to this file (libba.so, ba_marshal.so).  Sidecar files
+store a hash of the sources and flags so that an up-to-date build is reused.
 """
 from __future__ import annotations
 
@@ -9,6 +9,7 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -61,5 +62,23 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_marshal(force: bool = False) -> str:
+    """Compile csrc/ba_marshal.c into ba_marshal.so (if needed) and return its path."""
+    out, src, header = os.path.join(HERE, "ba_marshal.so"), os.path.join(CSRC, "ba_marshal.c"), os.path.join(INCLUDE, "ba.h")
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-fPIC", "-shared", "-Wall", "-Werror",
+           "-I", sysconfig.get_paths()["include"], "-I", INCLUDE, src, "-o", out]
+    digest = hashlib.sha256(" ".join(cmd + [sys.version]).encode() + open(src, "rb").read() + open(header, "rb").read()).hexdigest()
+    stamp = out + ".hash"
+    if not force and os.path.exists(out) and os.path.exists(stamp) and open(stamp).read().strip() == digest:
+        return out
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("the argument marshalling extension failed to build:\n" + res.stdout + res.stderr)
+    with open(stamp, "w") as fh:
+        fh.write(digest)
+    return out
+
+
 if __name__ == "__main__":
+    build_marshal(force="--force" in sys.argv)
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
