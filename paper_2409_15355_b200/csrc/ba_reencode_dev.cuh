@@ -60,6 +60,38 @@ __device__ __forceinline__ void ba_reencode_state_init(const ba_reencode_job &jo
   st.t_blk = -1; st.t_delta = 0;
 }
 
+// The rotation of one vector (ADJACENT) or one pair of vectors (HALF) in place.
+template <int kLayout>
+__device__ __forceinline__ void ba_reencode_rotate(const float4 (&tcs)[4], uint4 &x, uint4 &y) {
+  if (kLayout == BA_ROPE_ADJACENT) {
+    const float4 a = tcs[0], b = tcs[1];                      // two (cos,sin) pairs per float4
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+    const float2 cs[4] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y), make_float2(b.z, b.w)};
+    uint32_t o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float xo, yo;
+      rot2(bf16_lo(w[j]), bf16_hi(w[j]), cs[j], xo, yo);
+      o[j] = pack_bf16x2(xo, yo);
+    }
+    x = make_uint4(o[0], o[1], o[2], o[3]);
+  } else {
+    const uint32_t wx[4] = {x.x, x.y, x.z, x.w}, wy[4] = {y.x, y.y, y.z, y.w};
+    uint32_t ox[4], oy[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 cs = tcs[j];                               // pairs m0+2j, m0+2j+1
+      float x0, y0, x1, y1;
+      rot2(bf16_lo(wx[j]), bf16_lo(wy[j]), make_float2(cs.x, cs.y), x0, y0);
+      rot2(bf16_hi(wx[j]), bf16_hi(wy[j]), make_float2(cs.z, cs.w), x1, y1);
+      ox[j] = pack_bf16x2(x0, x1);
+      oy[j] = pack_bf16x2(y0, y1);
+    }
+    x = make_uint4(ox[0], ox[1], ox[2], ox[3]);
+    y = make_uint4(oy[0], oy[1], oy[2], oy[3]);
+  }
+}
+
 // Rows row0, row0 + row_step, ... (kRows of them, those below total_rows), all loads first.
 template <int kLayout, int kRows>
 __device__ __forceinline__ void ba_reencode_rows(const ba_reencode_job &job, ba_reencode_state &st, int row0,
@@ -123,39 +155,45 @@ __device__ __forceinline__ void ba_reencode_rows(const ba_reencode_job &job, ba_
       st.tcs[0] = __ldg(t4); st.tcs[1] = __ldg(t4 + 1);
       if (kLayout == BA_ROPE_HALF) { st.tcs[2] = __ldg(t4 + 2); st.tcs[3] = __ldg(t4 + 3); }
     }
-    if (st.t_delta == 0) {                       // identity: copy bit-exactly
-      q[vec_x] = x[i];
-      if (kLayout == BA_ROPE_HALF) q[vec_y] = y[i];
-      continue;
-    }
-    if (kLayout == BA_ROPE_ADJACENT) {
-      const float4 a = st.tcs[0], b = st.tcs[1];              // two (cos,sin) pairs per float4
-      uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
-      float2 cs[4] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y), make_float2(b.z, b.w)};
-      uint32_t o[4];
+    if (st.t_delta != 0) ba_reencode_rotate<kLayout>(st.tcs, x[i], y[i]);   // delta 0 copies bit-exactly
+    q[vec_x] = x[i];
+    if (kLayout == BA_ROPE_HALF) q[vec_y] = y[i];
+  }
+}
+
+// Rows row0, row0 + row_step, ... (kRows of them, those below end), all of the block in `st`: no look-up but the page
+// numbers, all loads first.
+template <int kLayout, int kRows>
+__device__ __forceinline__ void ba_reencode_block_rows(const ba_reencode_job &job, const ba_reencode_state &st, int row0, int row_step,
+                                                       int end, int32_t *status) {
+  const int row_vecs = job.row_vecs;
+  uint4 x[kRows], y[kRows];
+  bool live[kRows];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float xo, yo;
-        rot2(bf16_lo(w[j]), bf16_hi(w[j]), cs[j], xo, yo);
-        o[j] = pack_bf16x2(xo, yo);
-      }
-      q[vec_x] = make_uint4(o[0], o[1], o[2], o[3]);
+  for (int i = 0; i < kRows; ++i) {
+    const int r = row0 + i * row_step;
+    live[i] = r < end;
+    if (!live[i]) continue;
+    long long sr = r + st.shift;
+    if (job.page_cu) {
+      const int t = r - st.c_begin, page = __ldg(job.page_idx + st.page0 + (t >> job.page_lg));
+      sr = page < 0 ? -1 : ((long long)page << job.page_lg) + (t & ((1 << job.page_lg) - 1));
+    }
+    if (sr < 0 || sr >= job.n_src_rows) {
+      ba_record_status(status, BA_ERR_INVALID_ARG);
+      live[i] = false;
     } else {
-      uint32_t wx[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
-      uint32_t wy[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
-      uint32_t ox[4], oy[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 cs = st.tcs[j];                          // pairs m0+2j, m0+2j+1
-        float x0, y0, x1, y1;
-        rot2(bf16_lo(wx[j]), bf16_lo(wy[j]), make_float2(cs.x, cs.y), x0, y0);
-        rot2(bf16_hi(wx[j]), bf16_hi(wy[j]), make_float2(cs.z, cs.w), x1, y1);
-        ox[j] = pack_bf16x2(x0, x1);
-        oy[j] = pack_bf16x2(y0, y1);
-      }
-      q[vec_x] = make_uint4(ox[0], ox[1], ox[2], ox[3]);
-      q[vec_y] = make_uint4(oy[0], oy[1], oy[2], oy[3]);
+      x[i] = __ldcs(job.src + sr * row_vecs + st.vec_x);
+      if (kLayout == BA_ROPE_HALF) y[i] = __ldcs(job.src + sr * row_vecs + st.vec_y);
     }
+  }
+#pragma unroll
+  for (int i = 0; i < kRows; ++i) {
+    if (!live[i]) continue;
+    uint4 *q = job.dst + (long long)(row0 + i * row_step) * row_vecs;
+    if (st.t_delta != 0) ba_reencode_rotate<kLayout>(st.tcs, x[i], y[i]);   // delta 0 copies bit-exactly
+    q[st.vec_x] = x[i];
+    if (kLayout == BA_ROPE_HALF) q[st.vec_y] = y[i];
   }
 }
 
