@@ -1570,8 +1570,39 @@ int ba_heads_per_tile(const ba_config &c) {
   return (G % 4 == 0) ? 4 : (G % 2 == 0) ? 2 : 1;
 }
 
+// The fused call in two steps: re-encode the cached keys into k_out, or the end of the workspace, and attend them.  The fused
+// kernel rotates every query tile once per cached block and cannot let a key tile span two blocks; with one pair of query
+// tiles per sequence that costs less than a pass over the cached keys, with two it no longer does (8 requests, 29000 cached
+// tokens in blocks of 37-611, final blocks of 64 / 101 / 256 tokens: fused 81 / 121 / 244 us, two steps 74 / 95 / 163; one
+// request, 32 x 1000 cached: 66 / 94 / 161 and 74 / 98 / 166).  The choice depends on the lengths alone, so that a call gives
+// the same result with k_out and without.
+static bool fused_in_two_steps(const ba_ctx *ctx, const ba_attend_args &a, const ba_segments *seg, size_t *scratch) {
+  if (!a.fused || !a.final_only || a.n_cache_rows < 1 || !seg->cache_rope) return false;
+  if (seg->n_final_items < 1 || 2LL * seg->n_final_items < 3LL * seg->batch) return false;
+  *scratch = ba_align_up((size_t)a.n_cache_rows * ctx->cfg.n_kv_heads * ctx->cfg.head_dim * 2, 256);
+  return ctx->workspace && ctx->workspace_bytes > ba_scratch_offset(ctx) && *scratch <= (ctx->workspace_bytes - ba_scratch_offset(ctx)) / 2;
+}
+
 ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_segments *seg,
                                  cudaStream_t stream) {
+  size_t scratch = 0;
+  if (fused_in_two_steps(ctx, a, seg, &scratch)) {
+    ba_status st = ba_flush_pending(ctx, stream);
+    if (st != BA_OK) return st;
+    ba_attend_args b = a;
+    b.fused = 0; b.k_src_off = nullptr; b.k_out = nullptr;
+    b.reserved_bytes = a.k_out ? 0 : scratch;
+    void *keys = a.k_out ? a.k_out : (char *)ctx->workspace + (ctx->workspace_bytes - scratch) / 256 * 256;
+    b.k_cache = (const __nv_bfloat16 *)keys;
+    ba_reencode_job job = ba_make_reencode_job(ctx, a.k_cache, a.k_src_off, a.n_k_rows, keys, seg->cache_cu, seg->cache_delta,
+                                               seg->n_cached_blocks, a.n_cache_rows, reinterpret_cast<const float2 *>(seg->cache_rope));
+    if (a.page_rows > 0) {
+      job.src_off = nullptr; job.page_cu = a.page_cu; job.page_idx = a.page_idx;
+      while ((1 << job.page_lg) < a.page_rows) ++job.page_lg;
+    }
+    st = ba_reencode_main_launch(ctx, job, stream);
+    return st == BA_OK ? ba_attend_sm100_launch(ctx, b, seg, stream) : st;
+  }
   const int D = ctx->cfg.head_dim, Hq = ctx->cfg.n_q_heads, Hkv = ctx->cfg.n_kv_heads;
   AttnParams p;
   p.o = a.o; p.lse = a.lse; p.status = ctx->dev_status; p.out_f32 = a.out_f32;
@@ -1625,7 +1656,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     const size_t per_split = (size_t)a.n_q_rows * Hq * (D + 1) * sizeof(float);
     // the angle table of a queued re-encoding job sits at the end of the workspace and is read by
     // this very launch: the partial results must stay below it
-    const size_t taken = ba_scratch_offset(ctx) + ctx->pending_table_bytes;
+    const size_t taken = ba_scratch_offset(ctx) + ctx->pending_table_bytes + (a.reserved_bytes ? a.reserved_bytes + 256 : 0);
     const size_t avail = ctx->workspace_bytes > taken ? ctx->workspace_bytes - taken : 0;
     const int cap = (int)min((size_t)32, per_split ? avail / per_split : 0);
     // equal splits or the balanced launch (ba_plan_splits, above the kernels' common declarations)

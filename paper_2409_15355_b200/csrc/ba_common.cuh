@@ -202,7 +202,7 @@ template <class Fits>
 static inline ba_cluster_plan ba_plan_cluster(long long items, long long max_tiles, Fits fits) {
   ba_cluster_plan plan = {0, 0.};
   for (int n = 2; n <= kMaxCluster && n <= max_tiles; ++n) {
-    const long long at_a_time = items <= 8 * (kMaxCluster + 1 - n) ? items : fits(n);   // (a few clusters always fit)
+    const long long at_a_time = items == 1 ? 1 : fits(n);
     if (at_a_time < 1) continue;
     const double cost = (double)((items + at_a_time - 1) / at_a_time) * ((max_tiles + n - 1) / n + 3) + 1.5;
     if (!plan.size || cost < plan.cost) { plan.size = n; plan.cost = cost; }
@@ -270,6 +270,7 @@ struct ba_attend_args {
   const int32_t *page_cu, *page_idx;
   int final_only;  // 1: ba_final_attend, 0: ba_block_prefill
   int mode;        // ba_mode
+  size_t reserved_bytes;   // of the end of the workspace, in use during this call
 };
 
 ba_status ba_attend_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_segments *seg,

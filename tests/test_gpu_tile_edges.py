@@ -10,7 +10,7 @@ from paper_2409_15355_b200 import binding as B
 from paper_2409_15355_b200 import runtime as R
 from paper_2409_15355_b200 import workloads as W
 from tests.test_gpu_backward import check_grad, run_forward_backward
-from tests.test_gpu_parity import check_attention, run_prefill, run_warm
+from tests.test_gpu_parity import check_attention, check_reencoded, run_prefill, run_warm
 
 pytestmark = pytest.mark.gpu
 
@@ -172,3 +172,57 @@ def test_cluster_launch(w, fused):
 def _hpt(w):
     g = w.n_q_heads // w.n_kv_heads
     return 4 if g % 4 == 0 else 2 if g % 2 == 0 else 1
+
+
+# ba_reencode_k: CTAs whose rows lie in one block and CTAs that cross blocks, both rotary layouts, all sources
+@pytest.mark.parametrize("layout", [B.BA_ROPE_ADJACENT, B.BA_ROPE_HALF], ids=["adjacent", "half"])
+@pytest.mark.parametrize("heads", [(8, 8, 128), (2, 1, 64), (6, 3, 64)], ids=str)
+def test_reencode_rows_in_one_block_and_across(layout, heads):
+    lens = [1, 2, 3, 4, 5, 7, 8, 9, 31, 32, 33, 100, 1, 1, 64, 17]
+    w = W.Workload("rows", *heads, 1e4, lens + [5], [len(lens) + 1], seed=121)
+    c = R.Context(*heads, 1e4, rope_layout=layout)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    t = ob.segment_tables(w.block_lens, w.seq_nblocks)
+    packed = W.normal_bf16(122, (sum(lens), heads[1], heads[2]))
+    want = ob.reencode_blocks(W.bf16_bits_to_f64(packed), None, t["cache_cu"], t["cache_delta"], 1e4, layout)
+    src = R.bits_to_device(packed)
+    out = torch.full_like(src, float("nan"))
+    B.ba_reencode_k(c.ctx, src, None, len(src), out, seg.cache_cu, seg.cache_delta, len(lens), len(src))
+    assert c.device_status() == B.BA_OK
+    check_reencoded(R.device_to_bits(out), want)
+    pool, page_cu, page_idx, n_pages = W.scatter_into_pages(packed, lens, 16, 123)
+    keep = [R.bits_to_device(pool), torch.from_numpy(page_cu).cuda(), torch.from_numpy(page_idx).cuda()]
+    paged = torch.full_like(src, float("nan"))
+    B.ba_reencode_k_paged(c.ctx, keep[0], B.make_page_table(16, n_pages, keep[1], keep[2]), paged, seg.cache_cu, seg.cache_delta,
+                          len(lens), len(src))
+    assert c.device_status() == B.BA_OK and torch.equal(paged, out)
+    c.close()
+
+
+# The fused call over final blocks of several query tiles: in two steps through the workspace, through k_out, and (a workspace
+# without room for the keys) in one
+@pytest.mark.parametrize("w", [_requests("one", 1, 131, (6, 50, 300), (200, 200)), _requests("pool", 5, 132, (4, 20, 290), (70, 129), pool=True)],
+                         ids=lambda w: w.name)
+def test_fused_call_in_two_steps(w):
+    o, lse, o_ref, lse_ref = run_warm(w, B.BA_MODE_BLOCK, fused=True)
+    check_attention(o, o_ref, lse, lse_ref)
+    x, t = W.warm_inputs(w), ob.segment_tables(w.block_lens, w.seq_nblocks)
+    k_src, v_src = (R.bits_to_device(x[n]) for n in (("k_pool", "v_pool") if w.pool_lens else ("k_cache", "v_cache")))
+    off = torch.from_numpy(x["src_off"]).cuda() if w.pool_lens else None
+    q, k, v = (R.bits_to_device(x[n]) for n in ("q_f", "k_f", "v_f"))
+    cfg = B.ba_config(w.n_q_heads, w.n_kv_heads, w.head_dim, 0, w.rope_theta, 0.0, 0)
+    Tc, Tf = t["n_cached_tokens"], t["n_final_tokens"]
+    for room in (B.ba_workspace_bytes(cfg, 64, 4096), 64 * 1024 + 4096):
+        ctx = B.ba_create(cfg, 0, room)
+        tb = torch.empty(B.ba_segments_bytes(w.batch, w.n_blocks, w.n_tokens), dtype=torch.uint8, device="cuda")
+        seg = B.ba_segment(ctx, np.asarray(w.block_lens, dtype=np.int32), np.asarray(w.seq_nblocks, dtype=np.int32), w.batch, w.n_blocks,
+                           w.n_tokens, B.BA_MODE_BLOCK, tb)
+        out, keys = torch.empty(Tf, w.n_q_heads, w.head_dim, device="cuda"), torch.empty(Tc, w.n_kv_heads, w.head_dim, dtype=torch.bfloat16, device="cuda")
+        for k_out in (None, keys):
+            B.ba_final_attend_fused(ctx, q, k, v, Tf, k_src, v_src, len(k_src), off, Tc, out, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32, k_out=k_out)
+            assert B.ba_last_device_status(ctx) == B.BA_OK
+            check_attention(out.cpu().numpy(), o_ref)
+        ref = torch.empty_like(keys)
+        B.ba_reencode_k(ctx, k_src, off, len(k_src), ref, seg.cache_cu, seg.cache_delta, seg.n_cached_blocks, Tc)
+        assert torch.equal(keys, ref)
+        B.ba_destroy(ctx)
