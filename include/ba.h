@@ -322,11 +322,9 @@ ba_status ba_final_attend(ba_ctx *ctx, const void *q_f, const void *k_f, const v
  * so the query tiles are rotated once per cached block on chip and the cached keys are neither
  * rewritten nor read twice.  The result equals ba_reencode_k followed by ba_final_attend up to
  * the rounding of the rotated operand to bf16 (queries here, keys there).  The re-encoded keys
- * themselves -- what the rest of generation reads -- are written as a side output when k_out is
- * given (final blocks of several query tiles are attended in two steps inside the call instead, the keys going to k_out or the
- * workspace): the call then also runs the re-encoding kernel, on a stream of the context's own beside the
- * attention launch (which leaves SMs idle in its last wave), and joins it back into `stream`; k_out is
- * bit-identical to ba_reencode_k's output and complete, in stream order, when the call is.
+ * themselves -- what the rest of generation reads -- are written as well when k_out is given, bit-identical to
+ * ba_reencode_k's output.  Where the two steps are quicker (k_out given, final blocks of several query tiles, small caches) the
+ * call takes them one after the other, the keys going to k_out or the workspace.
  *   q_f, k_f, v_f   as for ba_final_attend
  *   k_src, v_src    bf16 [n_src_rows, n_kv_heads, head_dim]: cached block c (cache order, as in
  *                   seg->cache_cu) occupies rows src_off[c] .. src_off[c] + length - 1 of both, or

@@ -141,7 +141,6 @@ ba_status ba_create(ba_ctx **out, const ba_config *cfg, int device, size_t works
   ctx->seg_delta = nullptr; ctx->seg_rope = nullptr; ctx->seg_rope_blocks = 0;
   ctx->seg_gen = nullptr; ctx->seg_gen_value = 0; ctx->seg_counter = 0;
   ctx->maps = nullptr;
-  ctx->side_stream = nullptr; ctx->ev_fork = nullptr; ctx->ev_join = nullptr;
   ctx->workspace = nullptr;
   ctx->dev_status = nullptr;
   if (cudaMalloc(&ctx->dev_status, 256) != cudaSuccess ||
@@ -150,15 +149,9 @@ ba_status ba_create(ba_ctx **out, const ba_config *cfg, int device, size_t works
       // launch counters of the attention kernels (below the scratch area): zero once, every launch leaves them zero
       (workspace_bytes >= ba_scratch_offset(ctx) &&
        cudaMemset((char *)ctx->workspace + ba_scratch_offset(ctx) - 256, 0, 256) != cudaSuccess) ||
-      cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       ba_attend_sm100_setup(ctx) != BA_OK || ba_bwd_sm100_setup(ctx) != BA_OK) {
     cudaGetLastError();
     ba_attend_sm100_teardown(ctx);
-    if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
-    if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
     if (ctx->workspace) cudaFree(ctx->workspace);
     if (ctx->dev_status) cudaFree(ctx->dev_status);
     delete ctx;
@@ -173,9 +166,6 @@ ba_status ba_destroy(ba_ctx *ctx) {
   cudaSetDevice(ctx->device);
   if (ctx->has_pending) ba_flush_pending(ctx, ctx->pending_stream);   // a queued job is not dropped
   cudaDeviceSynchronize();
-  if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
-  if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
   if (ctx->workspace) cudaFree(ctx->workspace);
   if (ctx->dev_status) cudaFree(ctx->dev_status);
   ba_attend_sm100_teardown(ctx);

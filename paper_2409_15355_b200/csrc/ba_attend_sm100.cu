@@ -506,6 +506,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
                        const __grid_constant__ CUtensorMap tmap_vc, const __grid_constant__ CUtensorMap tmap_o, const AttnParams p) {
   using L = Layout<D>;
   constexpr bool kFused = is_fused(kVariant), kDeep = is_deep(kVariant);
+  // Half tiles at the ends of cached blocks, values walked in a pool: 16 requests over 20 blocks of 50-500 tokens 1401 -> 1377 us
+  // (four layers).  Not on the fused path: the flags cost its product thread more than the halves save.
+  constexpr bool kWalks = kDeep;
   constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster;
   constexpr int kStages = kDeep ? 4 : 3;
   // setmaxnreg is a warpgroup-wide instruction: the four service warps (8-11) must ask for the same count
@@ -785,11 +788,16 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       const uint64_t q_desc[2] = {make_smem_desc(q_addr[0], 16, 1024), make_smem_desc(q_addr[1], 16, 1024)};
       const uint64_t k_desc0 = make_smem_desc(ring, 16, 1024);
       const uint64_t v_desc0 = make_smem_desc(ring, L::kRegionBytes, 1024);
+      Work wk = {};
       bool half_last = false;              // the entry's last key tile is used in its first 64 keys only
       int entry_tiles = 0;
+      // a cached tile whose block ends in its first 64 keys (walk mode; the producer's word comes with the tile)
+      auto cached_half = [&](int jrel, int idx) -> bool {
+        return kWalks && p.walk && wk.tile0 + jrel < wk.it.n_cache_tiles && ctrl->tile_valid[(idx >> 1) & 7] <= kBlockN / 2;
+      };
       auto issue_qk_with = [&](int t, int jrel, int idx, uint64_t qd) {
         const uint64_t kd = k_desc0 + (uint64_t)(((idx % kStages) * L::kTileBytes) >> 4);
-        const uint32_t idesc = (half_last && jrel + 1 == entry_tiles) ? idesc_qk_half : idesc_qk;
+        const uint32_t idesc = ((half_last && jrel + 1 == entry_tiles) || cached_half(jrel, idx)) ? idesc_qk_half : idesc_qk;
 #pragma unroll
         for (int k = 0; k < D / 16; ++k) {
           const uint64_t off = (uint64_t)(((k >> 2) * L::kRegionBytes + (k & 3) * 32) >> 4);
@@ -807,7 +815,6 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       int gidx = 0;                        // K/V tiles consumed so far (ring position)
       int q_uses[2] = {0, 0};              // items in which query tile t was loaded
       int p_uses[2] = {0, 0};              // P tiles of query tile t consumed
-      Work wk = {};
       int n_work = 0;
       // Every loop over the query tile t below is unrolled, so that t is a constant and the small
       // per-tile arrays live in registers: this thread's issue latency is on the critical path.
@@ -902,7 +909,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
             ok = mbar_wait(&ctrl->p_full[t][1], p_uses[t] & 1, abort_flag);
             if (!ok) continue;
             tc_fence_after();
-            if (!(last && half_last)) issue_pv(t, iv, j == 0, 1);
+            if (!(last && half_last) && !cached_half(j, iv)) issue_pv(t, iv, j == 0, 1);
             ++p_uses[t];
             BA_TR(2, j, t * 4 + 2);
             if (last) mma_commit(&ctrl->o_done[t]);
@@ -1053,8 +1060,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         // visible columns of this tile for this row: 0 .. lim
         int lim;
         const int jt = tile0 + j;
-        if (jt < it.n_cache_tiles) lim = p.walk ? ctrl->tile_valid[(tiles_before + j) & 7] - 1
-                                                     : it.cache_len - jt * kBlockN - 1;
+        const bool walked = p.walk && jt < it.n_cache_tiles;
+        if (jt < it.n_cache_tiles) lim = walked ? ctrl->tile_valid[(tiles_before + j) & 7] - 1 : it.cache_len - jt * kBlockN - 1;
         else lim = tok_c - (it.own_row0 + (jt - it.n_cache_tiles) * kBlockN);
         uint64_t sum2[4] = {0ull, 0ull, 0ull, 0ull};       // packed (0.f, 0.f)
         // One tile of softmax for this row over kCols key columns: 128, or 64 for a half tile (only the first
@@ -1145,7 +1152,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           mbar_arrive(&ctrl->p_full[t][1]);               // (half tile: nothing to hand over, that product is skipped)
           if (r == 0) BA_TR(t, j, 5);
         };
-        if (half_last && j + 1 == n_tiles) tile_softmax(std::integral_constant<int, kBlockN / 2>{});
+        if ((half_last && j + 1 == n_tiles) || (kWalks && walked && lim < kBlockN / 2)) tile_softmax(std::integral_constant<int, kBlockN / 2>{});
         else tile_softmax(std::integral_constant<int, kBlockN>{});
         // P of this tile is with the tensor core: time to work on the next version of the query row
         if (kFused && next_start < tile_end) {
@@ -1571,15 +1578,19 @@ int ba_heads_per_tile(const ba_config &c) {
 }
 
 // The fused call in two steps: re-encode the cached keys into k_out, or the end of the workspace, and attend them.  The fused
-// kernel rotates every query tile once per cached block and cannot let a key tile span two blocks; with one pair of query
-// tiles per sequence that costs less than a pass over the cached keys, with two it no longer does (8 requests, 29000 cached
-// tokens in blocks of 37-611, final blocks of 64 / 101 / 256 tokens: fused 81 / 121 / 244 us, two steps 74 / 95 / 163; one
-// request, 32 x 1000 cached: 66 / 94 / 161 and 74 / 98 / 166).  The choice depends on the lengths alone, so that a call gives
-// the same result with k_out and without.
+// kernel rotates every query tile once per cached block and cannot let a key tile span two blocks.  Taken
+//  * when k_out is wanted: the keys are read twice otherwise (32 x 1000 cached tokens and a final block of 1 / 64 / 128: 76 / 88 /
+//    119 us with the re-encoding beside the fused kernel, 67 / 73 / 100 in two steps; paged 79 / 92 / 125 and 72 / 80 / 109);
+//  * with more than one pair of query tiles per sequence (8 requests, 29000 cached tokens in blocks of 37-611, final blocks of
+//    64 / 101 / 256 tokens: fused 81 / 121 / 244 us, two steps 74 / 95 / 163);
+//  * for caches a re-encoding pass takes only a few microseconds over (10 x 128-384 and 32: 23.5 and 19.9).
+// What is left to the fused kernel: short final blocks over long caches (32 x 1000 and 1 / 32 / 64: 53 / 55 / 66 us, two steps
+// 67 / 68 / 73).
 static bool fused_in_two_steps(const ba_ctx *ctx, const ba_attend_args &a, const ba_segments *seg, size_t *scratch) {
   if (!a.fused || !a.final_only || a.n_cache_rows < 1 || !seg->cache_rope) return false;
-  if (seg->n_final_items < 1 || 2LL * seg->n_final_items < 3LL * seg->batch) return false;
+  if (a.k_out) return true;
   *scratch = ba_align_up((size_t)a.n_cache_rows * ctx->cfg.n_kv_heads * ctx->cfg.head_dim * 2, 256);
+  if (*scratch > (16u << 20) && (seg->n_final_items < 1 || 2LL * seg->n_final_items < 3LL * seg->batch)) return false;
   return ctx->workspace && ctx->workspace_bytes > ba_scratch_offset(ctx) && *scratch <= (ctx->workspace_bytes - ba_scratch_offset(ctx)) / 2;
 }
 
@@ -1748,23 +1759,6 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   const bool free_area = !p.fused && p.bg.n_rows == 0;
   const bool deep_ring = free_area && a.final_only && a.n_cache_rows > 0 && !p.balanced;
   p.q_double = free_area && !deep_ring;
-  // Side output of the fused call: the re-encoded keys, written by the stand-alone re-encoding kernel on the
-  // context's side stream beside the attention launch (which cannot share an SM with anything and leaves
-  // some SMs idle in its last wave); the caller's stream continues only when both are done.  (Measured
-  // alternative: the spare warps of the attention CTAs moving the rows cost 50 us per layer at 32K context,
-  // more than the kernel alone takes.)
-  const bool side_job = p.fused && a.k_out;
-  if (side_job) {
-    ba_reencode_job job = ba_make_reencode_job(ctx, a.k_cache, a.k_src_off, a.n_k_rows, a.k_out, seg->cache_cu,
-                                               seg->cache_delta, seg->n_cached_blocks, a.n_cache_rows,
-                                               reinterpret_cast<const float2 *>(seg->cache_rope));
-    if (p.k_paged) { job.src_off = nullptr; job.page_cu = a.page_cu; job.page_idx = a.page_idx; job.page_lg = p.page_lg; }
-    BA_CUDA_TRY(cudaEventRecord(ctx->ev_fork, stream));
-    BA_CUDA_TRY(cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0));
-    ba_status rs = ba_reencode_main_launch(ctx, job, ctx->side_stream);
-    if (rs != BA_OK) return rs;
-    BA_CUDA_TRY(cudaEventRecord(ctx->ev_join, ctx->side_stream));
-  }
   // (The balanced launch fills the GPU for hundreds of microseconds, and a re-encode on another stream fills the SMs it leaves
   // at its end: early CTAs of the next kernel would only take those.)
   const bool early = !p.balanced;
@@ -1787,7 +1781,6 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   ctx->launches += 1;
   ctx->last_attend[0] = (int32_t)grid.x; ctx->last_attend[1] = n_splits;
   ctx->last_attend[2] = p.balanced; ctx->last_attend[3] = p.bal_len;
-  if (side_job) BA_CUDA_TRY(cudaStreamWaitEvent(stream, ctx->ev_join, 0));
   if (n_splits > 1) {
     const unsigned n_merge_items = a.final_only && seg->n_final_items == 0 ? pairs_upper : (unsigned)seg->n_final_items;
     const int parts_log2 = n_merge_items * p.n_chunks <= 64 ? 5 : 3;

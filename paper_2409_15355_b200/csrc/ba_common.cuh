@@ -113,9 +113,6 @@ struct ba_ctx {
   int32_t seg_counter;      // ba_segment calls so far on this context
   // tensor maps of recently used tensors (attention launches re-use a handful of buffers)
   struct ba_map_cache *maps;
-  // side stream of the fused call's key write-back (forked from and joined to the caller's stream by events)
-  cudaStream_t side_stream;
-  cudaEvent_t ev_fork, ev_join;
 };
 
 static inline size_t ba_align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -263,7 +260,7 @@ struct ba_attend_args {
   int fused;
   const int32_t *k_src_off;
   int32_t n_k_rows;
-  void *k_out;     // fused warm path: non-null -> the re-encoded keys are also written here (cache packing)
+  void *k_out;     // fused call: non-null -> the re-encoded keys are written here (cache packing)
   // paged pool (page_rows > 0): the cached values -- and on the fused path the cached keys -- are read
   // through a page table instead of v_src_off / k_src_off
   int32_t page_rows;

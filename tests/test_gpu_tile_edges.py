@@ -226,3 +226,50 @@ def test_fused_call_in_two_steps(w):
         B.ba_reencode_k(ctx, k_src, off, len(k_src), ref, seg.cache_cu, seg.cache_delta, seg.n_cached_blocks, Tc)
         assert torch.equal(keys, ref)
         B.ba_destroy(ctx)
+
+
+def _fused_kernel_cases():
+    big = [_requests("stream_pool", 60, 95, (5, 20, 290), (33, 129), pool=True), _requests("stream_chunks", 60, 94, (4, 90, 300), (40, 140), heads=(8, 1, 64)),
+           _requests("cluster", 1, 115, (9, 200, 340), (64, 64), heads=(32, 8, 128)), _requests("cluster_ragged", 5, 114, (3, 1, 500), (1, 70), heads=(8, 1, 64))]
+    return big + [W.config1(), W.config2(), W.random_ragged(31, 3, 5, 200, 4, 2, 64), W.random_ragged(33, 3, 5, 200, 16, 2, 128),
+                  _requests("odd_group", 2, 116, (6, 100, 300), (100, 140), heads=(6, 2, 64)), W.config5(4, 64, 6, 32)]
+
+
+# The fused kernel itself, on caches that the call would take in two steps: a workspace without room for the keys leaves it
+# no choice
+@pytest.mark.parametrize("w", _fused_kernel_cases(), ids=lambda w: w.name)
+@pytest.mark.parametrize("layout", [B.BA_ROPE_ADJACENT, B.BA_ROPE_HALF], ids=["adjacent", "half"])
+def test_fused_kernel(w, layout):
+    x, t = W.warm_inputs(w), ob.segment_tables(w.block_lens, w.seq_nblocks)
+    k_src, v_src = (x[n] for n in (("k_pool", "v_pool") if w.pool_lens else ("k_cache", "v_cache")))
+    off = x["src_off"] if w.pool_lens else None
+    Tc, Tf = t["n_cached_tokens"], t["n_final_tokens"]
+    lens = np.diff(t["cache_cu"])
+    rows = np.concatenate([np.arange(o, o + n) for o, n in zip(off if off is not None else t["cache_cu"], lens)])
+    f64 = W.bf16_bits_to_f64
+    k_ref = ob.reencode_blocks(f64(k_src), off, t["cache_cu"], t["cache_delta"], w.rope_theta, layout)
+    o_ref, lse_ref = ob.final_attend(f64(x["q_f"]), f64(x["k_f"]), f64(x["v_f"]), k_ref, f64(v_src)[rows], w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    cfg = B.ba_config(w.n_q_heads, w.n_kv_heads, w.head_dim, layout, w.rope_theta, 0.0, 0)
+    ctx = B.ba_create(cfg, 0, 64 * 1024 + Tc * w.n_kv_heads * w.head_dim * 3)
+    tb = torch.empty(B.ba_segments_bytes(w.batch, w.n_blocks, w.n_tokens), dtype=torch.uint8, device="cuda")
+    seg = B.ba_segment(ctx, np.asarray(w.block_lens, dtype=np.int32), np.asarray(w.seq_nblocks, dtype=np.int32), w.batch, w.n_blocks, w.n_tokens,
+                       B.BA_MODE_BLOCK, tb)
+    n0 = B.ba_launch_count(ctx)
+    q, k, v, ks, vs = (R.bits_to_device(b) for b in (x["q_f"], x["k_f"], x["v_f"], k_src, v_src))
+    d_off = torch.from_numpy(off).cuda() if off is not None else None
+    o = torch.empty(Tf, w.n_q_heads, w.head_dim, device="cuda")
+    lse = torch.empty(Tf, w.n_q_heads, device="cuda")
+    B.ba_final_attend_fused(ctx, q, k, v, Tf, ks, vs, len(ks), d_off, Tc, o, lse, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    assert B.ba_last_device_status(ctx) == B.BA_OK
+    assert B.ba_launch_count(ctx) - n0 == (1 if B.ba_last_attend_shape(ctx)["partials"] == 1 else 2)     # no re-encoding pass
+    check_attention(o.cpu().numpy(), o_ref, lse.cpu().numpy(), lse_ref)
+    # the same pool in pages of 16 rows
+    if w.pool_lens is None:
+        (kp, page_cu, page_idx, n_pages), vp = W.scatter_into_pages(k_src, lens, 16, 7), W.scatter_into_pages(v_src, lens, 16, 7)[0]
+        keep = [R.bits_to_device(kp), R.bits_to_device(vp), torch.from_numpy(page_cu).cuda(), torch.from_numpy(page_idx).cuda()]
+        o.fill_(float("nan"))
+        B.ba_final_attend_fused_paged(ctx, q, k, v, Tf, keep[0], keep[1], B.make_page_table(16, n_pages, keep[2], keep[3]), Tc, o, lse, seg,
+                                      B.BA_MODE_BLOCK, B.BA_OUT_F32)
+        assert B.ba_last_device_status(ctx) == B.BA_OK
+        check_attention(o.cpu().numpy(), o_ref, lse.cpu().numpy(), lse_ref)
+    B.ba_destroy(ctx)
