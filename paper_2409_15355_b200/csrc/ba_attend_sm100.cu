@@ -1481,18 +1481,18 @@ struct ba_map_cache {
 
 namespace {
 
-const CUtensorMap *cached_map(ba_ctx *ctx, const void *ptr, int D, int heads, long long rows, int box_heads,
-                              int box_rows) {
+// (by value: two tensors of one call can share a slot)
+bool cached_map(ba_ctx *ctx, CUtensorMap *out, const void *ptr, int D, int heads, long long rows, int box_heads, int box_rows) {
   uint64_t h = (uint64_t)(uintptr_t)ptr * 0x9E3779B97F4A7C15ull;
   h ^= (uint64_t)rows * 0xC2B2AE3D27D4EB4Full + (uint64_t)(box_heads * 131 + box_rows);
   ba_map_cache::Slot &sl = ctx->maps->slot[(h >> 40) & (ba_map_cache::kSlots - 1)];
-  if (sl.ptr == ptr && sl.rows == rows && sl.D == D && sl.heads == heads && sl.box_heads == box_heads &&
-      sl.box_rows == box_rows)
-    return &sl.map;
-  sl.ptr = nullptr;
-  if (!make_map(&sl.map, ptr, D, heads, rows, box_heads, box_rows)) return nullptr;
-  sl.ptr = ptr; sl.rows = rows; sl.D = D; sl.heads = heads; sl.box_heads = box_heads; sl.box_rows = box_rows;
-  return &sl.map;
+  if (sl.ptr != ptr || sl.rows != rows || sl.D != D || sl.heads != heads || sl.box_heads != box_heads || sl.box_rows != box_rows) {
+    sl.ptr = nullptr;
+    if (!make_map(&sl.map, ptr, D, heads, rows, box_heads, box_rows)) return false;
+    sl.ptr = ptr; sl.rows = rows; sl.D = D; sl.heads = heads; sl.box_heads = box_heads; sl.box_rows = box_rows;
+  }
+  *out = sl.map;
+  return true;
 }
 
 template <int D>
@@ -1715,26 +1715,17 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     p.lse_part = p.o_part + (size_t)n_splits * p.n_part_rows * Hq * D;
   }
 
-  const CUtensorMap *mq = cached_map(ctx, a.q, D, Hq, a.n_q_rows, p.hpt, p.tok);
-  const CUtensorMap *mk = cached_map(ctx, a.k, D, Hkv, a.n_kv_rows, 1, kBlockN);
-  const CUtensorMap *mv = cached_map(ctx, a.v, D, Hkv, a.n_kv_rows, 1, kBlockN);
-  if (!mq || !mk || !mv) return BA_ERR_CUDA;
-  CUtensorMap tq = *mq, tk = *mk, tv = *mv, tkc = *mk, tvc = *mv, to = *mq;   // (a slot may be reused by a later look-up)
-  if (!a.out_f32) {
-    const CUtensorMap *mo = cached_map(ctx, a.o, D, Hq, a.n_q_rows, p.hpt, p.tok);
-    if (!mo) return BA_ERR_CUDA;
-    to = *mo;
-  }
+  CUtensorMap tq, tk, tv;
+  if (!cached_map(ctx, &tq, a.q, D, Hq, a.n_q_rows, p.hpt, p.tok) || !cached_map(ctx, &tk, a.k, D, Hkv, a.n_kv_rows, 1, kBlockN) ||
+      !cached_map(ctx, &tv, a.v, D, Hkv, a.n_kv_rows, 1, kBlockN))
+    return BA_ERR_CUDA;
+  CUtensorMap tkc = tk, tvc = tv, to = tq;
+  if (!a.out_f32 && !cached_map(ctx, &to, a.o, D, Hq, a.n_q_rows, p.hpt, p.tok)) return BA_ERR_CUDA;
   if (a.final_only && a.n_cache_rows > 0) {
     const int page_box = p.v_paged ? min(kBlockN, a.page_rows) : kBlockN;
-    const CUtensorMap *mkc = cached_map(ctx, a.k_cache, D, Hkv, p.fused ? a.n_k_rows : a.n_cache_rows, 1,
-                                        p.k_paged ? page_box : kBlockN);
-    if (!mkc) return BA_ERR_CUDA;
-    tkc = *mkc;
-    const CUtensorMap *mvc = cached_map(ctx, a.v_cache, D, Hkv, (a.v_src_off || p.v_paged) ? a.n_v_rows : a.n_cache_rows, 1,
-                                        page_box);
-    if (!mvc) return BA_ERR_CUDA;
-    tvc = *mvc;
+    if (!cached_map(ctx, &tkc, a.k_cache, D, Hkv, p.fused ? a.n_k_rows : a.n_cache_rows, 1, p.k_paged ? page_box : kBlockN) ||
+        !cached_map(ctx, &tvc, a.v_cache, D, Hkv, (a.v_src_off || p.v_paged) ? a.n_v_rows : a.n_cache_rows, 1, page_box))
+      return BA_ERR_CUDA;
   }
   dim3 grid((unsigned)(p.cluster > 1 ? items * p.cluster : p.stream ? stream_ctas : (p.persistent || p.balanced) ? ctx->sm_count : work_upper));
   // a queued re-encoding job rides along in the spare warps; a job whose rows do not fit the

@@ -273,3 +273,28 @@ def test_fused_kernel(w, layout):
         assert B.ba_last_device_status(ctx) == B.BA_OK
         check_attention(o.cpu().numpy(), o_ref, lse.cpu().numpy(), lse_ref)
     B.ba_destroy(ctx)
+
+
+# Tensors of one call whose cached tensor maps fall on the same slot of the context's 512: with the keys at 4096 places the
+# map of the queries or of the values is met about 16 times.
+def test_tensor_maps_that_share_a_slot():
+    c = R.Context(4, 4, 64, 1e4)
+    rows, places = 24, 4096
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    q, k, v = (torch.randn(rows, 4, 64, generator=gen, device="cuda").bfloat16() for _ in range(3))
+    seg, buf = c.segment(np.asarray([rows], dtype=np.int32), np.asarray([1], dtype=np.int32), B.BA_MODE_BLOCK, rows)
+    room = torch.zeros(places * 128 + rows * 4 * 64, dtype=torch.bfloat16, device="cuda")
+    want, o = torch.empty(rows, 4, 64, device="cuda"), torch.empty(rows, 4, 64, device="cuda")
+    B.ba_block_prefill(c.ctx, q, k.float().bfloat16(), v, want, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    s = torch.einsum("ihd,jhd->hij", q.float(), k.float()) / 8.0
+    p = s.masked_fill(torch.ones(rows, rows, device="cuda").triu(1).bool(), float("-inf")).softmax(-1)
+    assert (want - torch.einsum("hij,jhd->ihd", p, v.float())).abs().max() < 1e-2
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for i in range(places):
+        at = room[i * 128:i * 128 + rows * 4 * 64].view(rows, 4, 64)
+        at.copy_(k)
+        B.ba_block_prefill(c.ctx, q, at, v, o, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+        wrong += (o != want).any()
+    assert int(wrong) == 0
+    assert c.device_status() == B.BA_OK
+    c.close()
