@@ -95,6 +95,7 @@ typedef struct {
    * [3..5] with every cached block starting a tile of its own (pools, fused path).  Used to balance the launch. */
   int32_t final_key_tiles[6];
   int32_t prompt_key_tiles; /* sum over the work items of ba_block_prefill in block mode, lengths on the host (else 0) */
+  int32_t final_key_tiles_odd[2]; /* final_key_tiles[0] and [3] over every second item (1, 3, ..) of a sequence only */
   int32_t reserved;
   /* per sequence, [batch + 1] */
   int32_t *cu_seq;         /* first row of the sequence, prompt packing */
@@ -130,8 +131,8 @@ typedef struct {
   int32_t *prompt_items;   /* [totals[2]] items of ba_block_prefill, those of the final blocks last; [5] of these:
                             * place of the first query row among the rows of final blocks */
   int32_t *final_items;    /* [totals[3]] items of ba_final_attend */
-  int32_t *cu_stream;      /* [2][batch+1] prefix sums over sequences of the key tiles the items of its final block see:
-                            * cached keys packed, then block by block */
+  int32_t *cu_stream;      /* [4][batch+1] prefix sums over sequences of the key tiles the items of its final block see:
+                            * cached keys packed, then block by block, then both over every second item (1, 3, ..) only */
   int32_t *cache_tile_block; /* [cache_tile_cu[Bc]] cached block a key tile of cache_tile_cu belongs to */
 } ba_segments;
 

@@ -72,7 +72,7 @@ TableLayout table_layout(int32_t batch, int32_t B, int32_t T) {
   take((size_t)B * 64 * 8);                                   // cache_rope: at most 64 rotary pairs per block
   take(((size_t)T / 64 + B) * 32);                            // prompt_items: at least 64 tokens each, one remainder per block
   take(((size_t)T / 64 + batch) * 32);                        // final_items
-  take((size_t)(batch + 1) * 8);                              // cu_stream
+  take((size_t)(batch + 1) * 16);                             // cu_stream
   take(((size_t)T / 128 + B) * 4);                            // cache_tile_block
   L.bytes = cur;
   return L;
@@ -270,7 +270,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
     }
     out->prompt_key_tiles = prompt_tiles <= INT32_MAX ? (int32_t)prompt_tiles : 0;
     // key tiles per item of the final blocks (the counting of the attention kernel, done here on the host)
-    long long sum[2] = {0, 0}, mn[2] = {INT32_MAX, INT32_MAX}, mx[2] = {0, 0};
+    long long sum[2] = {0, 0}, odd[2] = {0, 0}, mn[2] = {INT32_MAX, INT32_MAX}, mx[2] = {0, 0};
     for (int q = 0, b = 0; q < batch; ++q) {
       long long cached = 0, walked = 0;
       for (int c = 0; c + 1 < seq_nblocks[q]; ++c) { cached += block_lens[b + c]; walked += (block_lens[b + c] + 127) / 128; }
@@ -281,7 +281,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
         const long long own = (std::min(fin, r0 + tt) + 127) / 128;
         for (int k = 0; k < 2; ++k) {
           const long long n = ct[k] + own;
-          sum[k] += n; mn[k] = std::min(mn[k], n); mx[k] = std::max(mx[k], n);
+          sum[k] += n; odd[k] += (r0 / tt) & 1 ? n : 0; mn[k] = std::min(mn[k], n); mx[k] = std::max(mx[k], n);
         }
       }
     }
@@ -290,6 +290,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
       out->final_key_tiles[3 * k] = fits ? (int32_t)sum[k] : 0;
       out->final_key_tiles[3 * k + 1] = fits ? (int32_t)mn[k] : 0;
       out->final_key_tiles[3 * k + 2] = fits ? (int32_t)mx[k] : 0;
+      out->final_key_tiles_odd[k] = fits ? (int32_t)odd[k] : 0;
     }
   }
   auto next = [&]() { return (int32_t *)(base + L.off[i++]); };

@@ -174,19 +174,30 @@ static inline long long ba_equal_splits_cost(int sm_count, long long items, long
 }
 
 // Stream launch of ba_final_attend: the key tiles of all items, end to end, in one run per CTA.  Each CTA works on about
-// 1 + run / item pieces of items; a piece that is not a whole item costs a partial result.  key_tiles: sum, minimum, maximum
-// over the items of one head chunk.  cap: the most partial results per row.
-struct ba_stream_plan { int n_ctas, n_slots; long long cost; };
-static inline ba_stream_plan ba_plan_stream(int sm_count, int n_chunks, const int32_t *key_tiles, int cap) {
-  ba_stream_plan plan = {0, 0, 0};
-  const long long total = (long long)key_tiles[0] * n_chunks, n_max = key_tiles[2];
+// 1 + run / item pieces of items; a piece that is not a whole item costs a partial result.  There are two such streams, one
+// of every sequence's items 0, 2, .. and one of its items 1, 3, .. (n_odd of the CTAs).  key_tiles: sum, minimum, maximum
+// over the items of one head chunk, odd_tiles: sum over the second stream.  cap: the most partial results per row.
+struct ba_stream_plan { int n_ctas, n_odd, n_slots; long long cost; };
+static inline ba_stream_plan ba_plan_stream(int sm_count, int n_chunks, const int32_t *key_tiles, int odd_tiles, int cap) {
+  ba_stream_plan plan = {0, 0, 0, 0};
+  const long long total = (long long)key_tiles[0] * n_chunks, odd = (long long)odd_tiles * n_chunks, n_max = key_tiles[2];
   if (total <= 0 || total > 0x3fffffff) return plan;
   const long long g = total < 2LL * sm_count ? (total + 1) / 2 : sm_count;
-  const long long run = (total + g - 1) / g, run_min = total / g;
-  const long long slots = (n_max - 1) / run_min + 2;           // runs an item of n_max tiles can touch
+  // the division of the CTAs that leaves the shorter longest run; a stream in one run has no cuts
+  long long run = total, run_min = total, n_odd = 0;
+  for (long long n = odd * g / total; n <= odd * g / total + 1; ++n) {
+    if (n >= g || (n == 0) != (odd == 0)) continue;
+    const long long even = total - odd, e = g - n;
+    const long long longest = std::max((even + e - 1) / e, n ? (odd + n - 1) / n : 0);
+    if (longest >= run) continue;
+    run = longest; n_odd = n;
+    run_min = std::min(e > 1 ? even / e : total, n > 1 ? odd / n : total);
+  }
+  if (run >= total && g > 1) return plan;
+  const long long slots = (n_max - 1) / std::max(run_min, 1LL) + 2;   // runs an item of n_max tiles can touch
   if (slots > cap) return plan;
   const long long pieces = 1 + (run + n_max - 1) / n_max;
-  plan.n_ctas = (int)g; plan.n_slots = (int)slots; plan.cost = run + 2 + 2 * pieces + 5;
+  plan.n_ctas = (int)g; plan.n_odd = (int)n_odd; plan.n_slots = (int)slots; plan.cost = run + 2 + 2 * pieces + 5;
   return plan;
 }
 

@@ -89,6 +89,12 @@ __device__ __forceinline__ int own_tiles_sum(int fin, int tt) {
   return whole + (fin + 127) / 128;
 }
 
+// The same over every second item (1, 3, ..): whole ones end at 2 * tt, 4 * tt, .. rows, multiples of 128.
+__device__ __forceinline__ int own_tiles_sum_odd(int fin, int tt) {
+  const int n = (fin + tt - 1) / tt, cut = n % 2 == 0 && fin % tt != 0, whole = n / 2 - cut;
+  return (whole * (whole + 1) / 2) * (tt >> 6) + (cut ? (fin + 127) / 128 : 0);
+}
+
 // Prefix sums over blocks and sequences.  Returns false when the lengths are inconsistent.  `writer`: this CTA also
 // writes the caller's tables.
 template <bool kShared>
@@ -198,25 +204,31 @@ __device__ __forceinline__ bool segment_blocks(const SegmentArgs &a, const int32
       if (!fin) seg.cache_delta[b - s] = start - seq_start;
     }
   }
-  // --- key tiles of all work items of a sequence's final block, one head chunk (cached keys packed / block by block)
+  // --- key tiles of all work items of a sequence's final block, one head chunk (cached keys packed / block by block; all
+  // items, then every second one)
   if (writer) {
-    int d[2] = {0, 0};
+    int d[4] = {0, 0, 0, 0};
     for (int base = 0; base < batch; base += (int)blockDim.x) {
       const int s = base + tid;
-      int v[2] = {0, 0}, total[2];
+      int v[4] = {0, 0, 0, 0}, total[4];
       if (s < batch) {
         const int fin = t.cu_final_seq[s + 1] - t.cu_final_seq[s], cached = t.cu_seq[s + 1] - t.cu_seq[s] - fin;
         const int n_items = t.cu_ftile[s + 1] - t.cu_ftile[s], own = own_tiles_sum(fin, tt);
+        const int n_odd = n_items / 2, own_odd = own_tiles_sum_odd(fin, tt), packed = (cached + 127) / 128;
         const int walked = t.cache_tile_cu[t.cu_seq_block[s + 1] - s - 1] - t.cache_tile_cu[t.cu_seq_block[s] - s];
-        v[0] = n_items * ((cached + 127) / 128) + own;
-        v[1] = n_items * walked + own;
+        v[0] = n_items * packed + own; v[1] = n_items * walked + own;
+        v[2] = n_odd * packed + own_odd; v[3] = n_odd * walked + own_odd;
       }
-      cta_exclusive_scan<2>(v, total, scan_smem);
-      if (s < batch) { seg.cu_stream[s] = d[0] + v[0]; seg.cu_stream[batch + 1 + s] = d[1] + v[1]; }
-      d[0] += total[0]; d[1] += total[1];
+      cta_exclusive_scan<4>(v, total, scan_smem);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (s < batch) seg.cu_stream[k * (batch + 1) + s] = d[k] + v[k];
+        d[k] += total[k];
+      }
     }
     if (tid == 0) {
-      seg.cu_stream[batch] = d[0]; seg.cu_stream[2 * batch + 1] = d[1];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) seg.cu_stream[k * (batch + 1) + batch] = d[k];
       seg.totals[7] = BA_TABLES_VALID;  // kernels that walk the tables check this word first
     }
   }

@@ -48,7 +48,7 @@ def test_segment_launch_variants(n_blocks, batch):
         base, raw = buf.data_ptr(), buf.cpu().numpy()
         rope = raw[seg.cache_rope - base:][:seg.n_cached_blocks * 32 * 8].view(np.float32).reshape(-1, 32, 2)
         items = raw[seg.final_items - base:][:int(got["totals"][3]) * 32].view(np.int32).reshape(-1, 8)
-        stream = raw[seg.cu_stream - base:][:(batch + 1) * 8].view(np.int32).reshape(2, -1)
+        stream = raw[seg.cu_stream - base:][:(batch + 1) * 16].view(np.int32).reshape(4, -1)
         tables.append((got, rope.copy(), items.copy(), stream.copy()))
     assert c.device_status() == B.BA_OK
     ref = ob.segment_tables(lens, counts, B.BA_MODE_BLOCK)
@@ -57,17 +57,21 @@ def test_segment_launch_variants(n_blocks, batch):
             assert got[k].tolist() == ref[k].tolist(), k
         angle = ref["cache_delta"].astype(np.float64)[:, None] * 1e4 ** (-2.0 * np.arange(32) / 64)
         assert np.abs(rope[..., 0] - np.cos(angle)).max(initial=0) < 1e-6 and np.abs(rope[..., 1] - np.sin(angle)).max(initial=0) < 1e-6
-        want, sums, b0 = [], [[0], [0]], 0
+        want, sums, b0 = [], [[0], [0], [0], [0]], 0
         for s, n in enumerate(counts):
             seq = lens[b0:b0 + n]
             f0, cached0 = int(ref["cu_final_seq"][s]), int(ref["cu_seq"][s]) - int(ref["cu_final_seq"][s])
-            walked, cached, per = sum(-(-v // 128) for v in seq[:-1]), sum(seq[:-1]), [0, 0]
+            walked, cached, per = sum(-(-v // 128) for v in seq[:-1]), sum(seq[:-1]), [0, 0, 0, 0]
             for q in range(0, seq[-1], seg.q_tile_tokens):
                 rows = min(seg.q_tile_tokens, seq[-1] - q)
                 want.append([f0 + q, rows, f0, cached0, cached, b0 - s, int(got["cache_tile_cu"][b0 - s]), walked])
                 own = -(-(q + rows) // 128)
-                per = [per[0] + -(-cached // 128) + own, per[1] + walked + own]
-            sums[0].append(sums[0][-1] + per[0]); sums[1].append(sums[1][-1] + per[1])
+                odd = q // seg.q_tile_tokens % 2
+                for k, tiles in enumerate((-(-cached // 128) + own, walked + own)):
+                    per[k] += tiles
+                    per[2 + k] += odd * tiles
+            for k in range(4):
+                sums[k].append(sums[k][-1] + per[k])
             b0 += n
         assert items.tolist() == want and stream.tolist() == sums
     c.close()
