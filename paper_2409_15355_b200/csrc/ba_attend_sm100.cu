@@ -292,7 +292,7 @@ __device__ __forceinline__ bool load_work(const AttnParams &p, const WorkEntry &
 // There are two streams, one of every sequence's items 0, 2, .. and one of its items 1, 3, .., each on CTAs of its own: two
 // successive items of a sequence read the same keys, and the two streams get to them at the same time, so that one of
 // them finds them in L2.  (In one stream the second item comes a whole item later, when every SM has read some 50 tiles
-// of 64 KB since.)  16 requests of 20 cached blocks of 50-500 tokens and 128 final tokens, four layers: 1333 -> 1284 us.
+// of 64 KB since: 16 requests of 20 cached blocks of 50-500 tokens, 128 final tokens, four layers, 1333 us, now 1284.)
 constexpr int kStreamSnap = 2;
 struct StreamState {
   int pos, end;              // tiles left to this CTA: [pos, end)
@@ -528,6 +528,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   // (four layers).  Not on the fused path: the flags cost its product thread more than the halves save.
   constexpr bool kWalks = kDeep;
   constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster;
+  // (layouts a variant is never launched with are not in its code: a short launch pays for every instruction it passes; a 32-layer
+  // prompt of 2500 cached tokens 824 -> 795 us)
+  const int balanced = kClustered || kDeep ? 0 : p.balanced, stream = kClustered ? 0 : p.stream, persistent = kClustered ? 0 : p.persistent;
   constexpr int kStages = kDeep ? 4 : 3;
   // setmaxnreg is a warpgroup-wide instruction: the four service warps (8-11) must ask for the same count
   constexpr int kServiceRegs = kFused ? kServiceRegsFused : kServiceRegsPlain;
@@ -565,7 +568,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   WorkEntry first = {-1, 0, 0, 0, -1, 0};
   if (warp == 8) {
     n_items = count_items(p);
-    if (!p.balanced && !p.stream) first = list_entry(p, n_items, (int)blockIdx.x);
+    if (!balanced && !stream) first = list_entry(p, n_items, (int)blockIdx.x);
   }
   tc_fence_before();
   __syncthreads();
@@ -586,12 +589,12 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     // same for every head chunk), one item per lane, kept in shared memory for the scheduling thread
     int *bal_cu = reinterpret_cast<int *>(smem + L::kCtrl + kBalTableOff);
     int bal_np = 0;
-    if (p.balanced && n_items > 0) {
+    if (balanced && n_items > 0) {
       bal_np = n_items;
-      if (bal_np < 1 || bal_np > kBalMaxPairs || bal_np * p.n_chunks != p.balanced) {
+      if (bal_np < 1 || bal_np > kBalMaxPairs || bal_np * p.n_chunks != balanced) {
         ba_record_status(p.status, BA_ERR_SHAPE);          // the tables describe another launch than the host sized
         bal_np = 0;
-      } else if ((int)blockIdx.x >= p.balanced) {
+      } else if ((int)blockIdx.x >= balanced) {
         const int lane = tid & 31;
         int carry = 0;
         for (int base = 0; base < bal_np; base += 32) {
@@ -615,16 +618,16 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       }
     }
     StreamState ss = {};
-    if (p.stream && n_items > 0) stream_start(p, ss);
+    if (stream && n_items > 0) stream_start(p, ss);
     if (elect_one()) {
       // balanced launch: run [bal_pos, bal_end) of the front tiles of all (chunk, item), bal_hm of them per chunk
       int bal_pos = 0, bal_end = 0, bal_hm = 0, bal_nh = 0;
       long long bal_all = 0;
-      if (bal_np > 0 && (int)blockIdx.x >= p.balanced) {
+      if (bal_np > 0 && (int)blockIdx.x >= balanced) {
         bal_hm = bal_cu[bal_np];
         bal_all = (long long)bal_hm * p.n_chunks;
-        bal_nh = (int)gridDim.x - p.balanced;
-        const int j = (int)blockIdx.x - p.balanced;
+        bal_nh = (int)gridDim.x - balanced;
+        const int j = (int)blockIdx.x - balanced;
         bal_pos = (int)(bal_all * j / bal_nh);
         bal_end = (int)(bal_all * (j + 1) / bal_nh);
       }
@@ -632,7 +635,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         WorkEntry e = {-1, 0, 0, 0, -1, 0};
         if (bal_np == 0) return e;
         const int b = (int)blockIdx.x;
-        if (b < p.balanced) {                              // the last bal_len key tiles of item b
+        if (b < balanced) {                              // the last bal_len key tiles of item b
           if (n_done > 0) return e;
           Item it;
           const int pair = bal_np - 1 - b % bal_np;
@@ -654,7 +657,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         // the slot counts the CTAs from the one that holds the first front tile of the item
         const long long g0 = (long long)chunk * bal_hm + bal_cu[i];
         const int j_first = (int)(((g0 + 1) * bal_nh - 1) / bal_all);
-        e.split = 1 + ((int)blockIdx.x - p.balanced) - j_first;
+        e.split = 1 + ((int)blockIdx.x - balanced) - j_first;
         if (e.split >= p.n_splits) { ba_record_status(p.status, BA_ERR_SHAPE); return e; }
         e.pair = bal_np - 1 - i; e.chunk = chunk;
         e.tile0 = r - bal_cu[i]; e.n_tiles = n;
@@ -676,10 +679,10 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         // balanced launch: the next piece of this CTA's share; persistent launch: next entry of the global list;
         // one-item launch: this CTA's own entry, then stop
         WorkEntry e = {-1, 0, 0, 0, -1, 0};
-        if (p.balanced) e = balanced_entry(n_work);
-        else if (p.stream) e = stream_next(p, ss);
+        if (balanced) e = balanced_entry(n_work);
+        else if (stream) e = stream_next(p, ss);
         else if (n_work == 0) e = first;
-        else if (p.persistent) e = list_entry(p, n_items, (int)gridDim.x + atomicAdd(p.counters, 1));
+        else if (persistent) e = list_entry(p, n_items, (int)gridDim.x + atomicAdd(p.counters, 1));
         const bool more = load_work(p, e, wk);
         if (!more) e.pair = -1;
         ctrl->work_ring[slot] = e;
@@ -1351,7 +1354,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               lp[(size_t)s * p.n_part_rows * p.Hq] = -INFINITY;
           } else {
             if (p.lse) p.lse[(size_t)row_tok * p.Hq + head] = lse_val;
-            if (p.stream && p.n_splits > 1) *lp = __uint_as_float(kRowIsComplete);
+            if (stream && p.n_splits > 1) *lp = __uint_as_float(kRowIsComplete);
           }
         }
       }
