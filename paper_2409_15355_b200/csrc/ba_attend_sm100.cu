@@ -102,8 +102,9 @@ struct AttnParams {
   // stream = 1: the key tiles of all (item, head chunk) are laid end to end and cut into one run per CTA, those of the
   // items 1, 3, .. of every sequence on the last n_odd CTAs
   int stream, n_odd;
-  // cluster > 1: the CTAs of a cluster share one item's key tiles and merge their results in shared memory
-  int cluster;
+  // cluster > 1: the CTAs of a cluster share one item's key tiles and merge their results in shared memory; single: one
+  // query tile of an item
+  int cluster, single;
   const int32_t *v_src_off;       // non-null: values of cached block c start at pool row v_src_off[c]
   int persistent;                 // 1: CTAs draw work from counters[0]; 0: CTA b handles entry b only
   // balanced > 0 (final block over a long cache, fewer items than CTAs): the first `balanced` CTAs each take the
@@ -154,7 +155,7 @@ struct WorkEntry {
   int chunk;           // head chunk
   int tile0, n_tiles;  // key tiles [tile0, tile0 + n_tiles) of the item
   int split;           // slot of the partial results this entry writes; < 0: it covers the whole item, rows go to the output
-  int fill;            // slots fill .. n_splits - 1 of the item stay unused: this entry marks them empty
+  int fill;            // slots fill .. n_splits - 1 of the item stay unused: this entry marks them empty (clusters: narrow_item)
 };
 
 struct Ctrl {
@@ -228,6 +229,16 @@ __device__ __forceinline__ void load_item(const AttnParams &p, int idx, Item &it
   it.n_tiles = it.n_cache_tiles + (it.q_row0 + it.q_rows - it.own_row0 + kBlockN - 1) / kBlockN;
 }
 
+// The part of its item that a cluster's entry covers (WorkEntry::fill: 1 + query tile, 0 the whole item).
+__device__ __forceinline__ void narrow_item(const AttnParams &p, int fill, Item &it) {
+  if (fill == 0) return;
+  const int skip = (fill - 1) * p.tok;
+  it.q_row0 += skip;
+  it.q_rows = min(it.q_rows - skip, p.tok);
+  it.n_qt = 1;
+  it.n_tiles = it.n_cache_tiles + (it.q_row0 + it.q_rows - it.own_row0 + kBlockN - 1) / kBlockN;
+}
+
 // One entry of a CTA's work list: an item, the heads it covers and its share of the key tiles.
 struct Work {
   Item it;
@@ -241,17 +252,28 @@ struct Work {
 //  Final attend: all items cost about the same, so the pair index varies fastest instead: the
 //  CTAs running at the same time then work on the same (KV head, key range) for different query
 //  tiles and each K/V tile comes from HBM once and from L2 for the others.
+//  Clusters: the CTAs of a cluster are the splits of one item (p.single: of one query tile of it).
+__device__ __forceinline__ WorkEntry cluster_entry(const AttnParams &p, int total_pairs) {
+  WorkEntry e = {-1, 0, 0, 0, -1, 0};
+  if (total_pairs <= 0) return e;
+  const unsigned units = (unsigned)total_pairs << p.single, i = cluster_index(), chunk = i / units, rank = i - chunk * units;
+  const unsigned k = cluster_rank(), n = (unsigned)p.cluster;
+  if ((int)chunk >= p.n_chunks) return e;
+  const int pair = total_pairs - 1 - (int)(rank >> p.single), fill = p.single ? 1 + (int)(rank & 1) : 0;
+  Item it;
+  load_item(p, pair, it);
+  if (fill == 2 && it.n_qt < 2) return e;                  // (every CTA of the cluster leaves)
+  narrow_item(p, fill, it);
+  e.pair = pair; e.chunk = (int)chunk; e.split = (int)k; e.fill = fill;
+  e.tile0 = (int)((unsigned)it.n_tiles * k / n);           // (at most 2^24 tiles, eight CTAs)
+  e.n_tiles = (int)((unsigned)it.n_tiles * (k + 1) / n) - e.tile0;
+  return e;
+}
 __device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int total_pairs, int w) {
   WorkEntry e = {-1, 0, 0, 0, -1, 0};
   int n_splits = p.n_splits, per_pair = p.n_chunks * n_splits, rank, rem;
   if (total_pairs <= 0) return e;
-  if (p.cluster > 1) {
-    n_splits = p.cluster;
-    const int member = w % n_splits, i = w / n_splits;
-    rem = i / total_pairs; rank = i - rem * total_pairs;
-    if (rem >= p.n_chunks) return e;
-    rem = rem * n_splits + member;
-  } else if (p.final_only) {
+  if (p.final_only) {
     rem = w / total_pairs; rank = w - rem * total_pairs;
     if (rem >= per_pair) return e;
   } else {
@@ -268,7 +290,7 @@ __device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int total_p
   load_item(p, e.pair, it);
   e.chunk = rem / n_splits;
   const int k = rem - e.chunk * n_splits;
-  e.split = p.cluster > 1 || n_splits > 1 ? k : -1;
+  e.split = n_splits > 1 ? k : -1;
   e.fill = n_splits;
   e.tile0 = (int)(((long long)it.n_tiles * k) / n_splits);
   e.n_tiles = (int)(((long long)it.n_tiles * (k + 1)) / n_splits) - e.tile0;
@@ -276,9 +298,11 @@ __device__ __forceinline__ WorkEntry list_entry(const AttnParams &p, int total_p
 }
 
 // A published entry, decoded by the role that reads it.  Returns false at the end of the work.
+template <bool kClustered>
 __device__ __forceinline__ bool load_work(const AttnParams &p, const WorkEntry &e, Work &wk) {
   if (e.pair < 0) return false;
   load_item(p, e.pair, wk.it);
+  if (kClustered) narrow_item(p, e.fill, wk.it);
   wk.head0 = e.chunk * p.hpt;
   wk.kv_head = wk.head0 / p.G;
   wk.tile0 = e.tile0;
@@ -478,6 +502,7 @@ __device__ __forceinline__ void cluster_merge_rows(const AttnParams &p, const Wo
   const int n = p.cluster, rank = (int)cluster_rank();
   Item it;
   load_item(p, e.pair, it);
+  narrow_item(p, e.fill, it);
   const int q_end = min(it.q_row0 + it.q_rows, p.n_q_rows);
   for (int rr = (rank * 8 + warp) * kRows + lane / kLanes; rr < it.n_qt * 128; rr += n * 8 * kRows) {
     const int t = rr >> 7, r = rr & 127;
@@ -568,7 +593,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   WorkEntry first = {-1, 0, 0, 0, -1, 0};
   if (warp == 8) {
     n_items = count_items(p);
-    if (!balanced && !stream) first = list_entry(p, n_items, (int)blockIdx.x);
+    if (kClustered) first = cluster_entry(p, n_items);
+    else if (!balanced && !stream) first = list_entry(p, n_items, (int)blockIdx.x);
   }
   tc_fence_before();
   __syncthreads();
@@ -683,7 +709,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         else if (stream) e = stream_next(p, ss);
         else if (n_work == 0) e = first;
         else if (persistent) e = list_entry(p, n_items, (int)gridDim.x + atomicAdd(p.counters, 1));
-        const bool more = load_work(p, e, wk);
+        const bool more = load_work<kClustered>(p, e, wk);
         if (!more) e.pair = -1;
         ctrl->work_ring[slot] = e;
         mbar_arrive(&ctrl->work_full[slot]);
@@ -783,6 +809,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
             ++gidx;
           }
         }
+        if (kClustered) break;
       }
       if (!ok) {
         // leave no copy in flight: wait (bounded) for the tiles already requested
@@ -882,7 +909,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (!ok) break;
         const WorkEntry e = ctrl->work_ring[slot];
         ++n_work;
-        if (!load_work(p, e, wk)) break;
+        if (!load_work<kClustered>(p, e, wk)) break;
         mbar_arrive(&ctrl->work_empty[slot]);          // the entry has been decoded into registers
         const int n_tiles = wk.n_tiles, n_qt = wk.it.n_qt;
         if (n_tiles == 0) continue;
@@ -950,6 +977,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
 #pragma unroll
         for (int t = 0; t < 2; ++t)
           if (t < n_qt) ++q_uses[t];
+        if (kClustered) break;                             // (one entry)
       }
     }
     if (kClustered) { __syncwarp(); cluster_sync(); }
@@ -1000,7 +1028,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       if (!ok) break;
       const WorkEntry e = ctrl->work_ring[slot];
       ++n_work;
-      if (!load_work(p, e, wk)) break;
+      if (!load_work<kClustered>(p, e, wk)) break;
       __syncwarp();
       if ((tid & 31) == 0) mbar_arrive(&ctrl->work_empty[slot]);   // one arrival per softmax warp
       const Item &it = wk.it;
@@ -1197,6 +1225,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       int q_row0, q_rows, part_row0;
       asm volatile("ld.global.nc.v2.s32 {%0, %1}, [%3];\n\tld.global.nc.s32 %2, [%3 + 20];"
                    : "=&r"(q_row0), "=&r"(q_rows), "=r"(part_row0) : "l"(p.items + 8 * (size_t)e.pair));
+      if (kClustered && e.fill == 2) { q_row0 += p.tok; q_rows -= p.tok; }
       if (ok && n_tiles > 0) { ok = mbar_wait(&ctrl->o_done[t], o_uses & 1, abort_flag); ++o_uses; }
       if (ok) {
         tc_fence_after();
@@ -1361,6 +1390,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       }
       tiles_before += n_tiles;
       if (n_tiles > 0) ++n_loaded;
+      if (kClustered) break;
     }
     release_out();                        // no copy reads this CTA's memory when it ends
     if (kClustered) {
@@ -1678,7 +1708,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   const long long items = (a.final_only && seg->n_final_items > 0 ? (long long)seg->n_final_items
                                                                   : (long long)((a.n_q_rows + pair_tok - 1) / pair_tok)) * (Hq / p.hpt);
   int n_splits = 1, stream_ctas = 0;
-  p.stream = 0; p.n_odd = 0; p.cluster = 0;
+  p.stream = 0; p.n_odd = 0; p.cluster = 0; p.single = 0;
   if (a.final_only) {
     // key tiles of an average item: counted by ba_segment() when it saw the lengths, else estimated
     const int32_t *ft = seg->final_key_tiles + (p.walk ? 3 : 0);
@@ -1701,8 +1731,8 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
         p.stream = 1; stream_ctas = stream.n_ctas; p.n_odd = stream.n_odd; n_splits = stream.n_slots;
       }
       if (a.n_cache_rows > 0 && !ctx->has_pending) {
-        const ba_cluster_plan cl = ba_plan_cluster(items, ft[2], [&](int n) { return max_clusters(ctx, n); });
-        if (cl.size > 0 && cl.cost < (double)(p.stream ? stream.cost : equal_cost)) { p.cluster = cl.size; p.stream = 0; n_splits = 1; }
+        const ba_cluster_plan cl = ba_plan_cluster(items, a.n_q_rows > (long long)p.tok * seg->n_final_items, ft[2], [&](int n) { return max_clusters(ctx, n); });
+        if (cl.size > 0 && cl.cost < (double)(p.stream ? stream.cost : equal_cost)) { p.cluster = cl.size; p.single = cl.single; p.stream = 0; n_splits = 1; }
       }
     }
   } else if (!a.final_only && a.mode == BA_MODE_BLOCK && seg->n_final_items > 0 && seg->prompt_key_tiles > 0) {
@@ -1748,7 +1778,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
         !cached_map(ctx, &tvc, a.v_cache, D, Hkv, (a.v_src_off || p.v_paged) ? a.n_v_rows : a.n_cache_rows, 1, page_box))
       return BA_ERR_CUDA;
   }
-  dim3 grid((unsigned)(p.cluster > 1 ? items * p.cluster : p.stream ? stream_ctas : (p.persistent || p.balanced) ? ctx->sm_count : work_upper));
+  dim3 grid((unsigned)(p.cluster > 1 ? (items << p.single) * p.cluster : p.stream ? stream_ctas : (p.persistent || p.balanced) ? ctx->sm_count : work_upper));
   // a queued re-encoding job rides along in the spare warps; a job whose rows do not fit the
   // staging buffers is run on its own first
   p.bg.n_rows = 0; p.bg_rows_per_chunk = 0;

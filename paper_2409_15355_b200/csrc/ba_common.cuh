@@ -203,18 +203,24 @@ static inline ba_stream_plan ba_plan_stream(int sm_count, int n_chunks, const in
 
 // Cluster launch of ba_final_attend: the `size` CTAs of a cluster share one item's key tiles and merge their results in
 // shared memory, which costs about as much as 1.5 tiles and saves the partial results' way through memory and the merging
-// kernel.  fits(size): clusters of that size the GPU runs at a time (0: none).
+// kernel.  single: a cluster takes one query tile of an item instead of two, where most items have two (`two_tiles`): a key
+// tile costs a little less and a CTA has half the rows to fetch, write out and collect from the others.  (32/8 heads of 128, us a
+// layer, whole items and single tiles, CTAs: 2500 cached tokens and 64 final ones, 56 and 80 CTAs: 23.9, 22.1; 6000, 64 and 96:
+// 32.7, 31.3; 128 final ones, 96 and 128 CTAs, 1000: 26.8, 27.3; 6000: 36.7, 37.7.)  fits(size): clusters of that size the GPU
+// runs at a time (0: none).
 constexpr int kMaxCluster = 8;
-struct ba_cluster_plan { int size; double cost; };
+struct ba_cluster_plan { int size, single; double cost; };
 template <class Fits>
-static inline ba_cluster_plan ba_plan_cluster(long long items, long long max_tiles, Fits fits) {
-  ba_cluster_plan plan = {0, 0.};
-  for (int n = 2; n <= kMaxCluster && n <= max_tiles; ++n) {
-    const long long at_a_time = items == 1 ? 1 : fits(n);
-    if (at_a_time < 1) continue;
-    const double cost = (double)((items + at_a_time - 1) / at_a_time) * ((max_tiles + n - 1) / n + 3) + 1.5;
-    if (!plan.size || cost < plan.cost) { plan.size = n; plan.cost = cost; }
-  }
+static inline ba_cluster_plan ba_plan_cluster(long long items, bool two_tiles, long long max_tiles, Fits fits) {
+  ba_cluster_plan plan = {0, 0, 0.};
+  for (int single = 0; single <= (two_tiles ? 1 : 0); ++single)
+    for (int n = 2; n <= kMaxCluster && n <= max_tiles; ++n) {
+      const long long units = items << single, at_a_time = units == 1 ? 1 : fits(n);
+      if (at_a_time < 1) continue;
+      const double tile = single ? 0.85 : 1.0, merge = single ? 0.25 : 1.5;
+      const double cost = (double)((units + at_a_time - 1) / at_a_time) * ((max_tiles + n - 1) / n * tile + 3) + merge;
+      if (!plan.size || cost < plan.cost) { plan.size = n; plan.single = single; plan.cost = cost; }
+    }
   return plan;
 }
 

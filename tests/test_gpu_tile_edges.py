@@ -155,19 +155,20 @@ def test_prefill_bf16_rows_full_and_ragged_tiles(heads, background):
 
 
 # A short final block over a cache of a few key tiles: the CTAs of a cluster share an item and merge in shared memory.
-# Cluster sizes 2 .. 8, one and two query tiles per item, both packings of heads, CTAs that get no tile, bf16 and fp32 rows.
+# Cluster sizes 2 .. 8, one and two query tiles per item, clusters of one query tile and of whole items, both packings of heads, CTAs that get no tile, bf16 and fp32 rows.
 @pytest.mark.parametrize("w", [_requests("two_tiles", 1, 111, (1, 120, 120), (3, 3), heads=(4, 2, 64)),
                                _requests("three_tiles", 2, 112, (3, 70, 90), (33, 64), heads=(8, 2, 128)),
                                _requests("five_tiles", 3, 113, (4, 20, 200), (1, 130), heads=(8, 8, 128)),
                                _requests("ragged_sizes", 5, 114, (3, 1, 500), (1, 70), heads=(8, 1, 64)),
                                _requests("twenty_tiles", 1, 115, (9, 200, 340), (64, 64), heads=(32, 8, 128)),
-                               _requests("odd_group", 2, 116, (6, 100, 300), (100, 140), heads=(6, 2, 64))], ids=lambda w: w.name)
+                               _requests("odd_group", 2, 116, (6, 100, 300), (100, 140), heads=(6, 2, 64)),
+                               _requests("one_and_two_query_tiles", 2, 117, (7, 100, 300), (65, 120), heads=(8, 2, 128))], ids=lambda w: w.name)
 @pytest.mark.parametrize("fused", [False, True], ids=["reencode_then_attend", "fused"])
 def test_cluster_launch(w, fused):
     shapes = []
     o, lse, o_ref, lse_ref = run_warm(w, B.BA_MODE_BLOCK, fused=fused, shape_out=shapes)
     items = sum(-(-n // (256 // _hpt(w))) for n in w.final_lens()) * (w.n_q_heads // _hpt(w))
-    assert shapes[0]["partials"] == 1 and shapes[0]["ctas"] in [items * n for n in range(2, 9)]
+    assert shapes[0]["partials"] == 1 and shapes[0]["ctas"] in [items * n * m for n in range(2, 9) for m in (1, 2)]
     check_attention(o, o_ref, lse, lse_ref)
     o, lse, _, _ = run_warm(w, B.BA_MODE_BLOCK, out_dtype=B.BA_OUT_BF16, fused=fused)
     check_attention(o, o_ref, lse, lse_ref, bf16_store=True)
