@@ -519,7 +519,7 @@ def run_ours(args):
             ev1.record(stream)
             torch.cuda.synchronize()
             fused[key] = ev0.elapsed_time(ev1) * 1e3 / reps / L
-        fused["k_out"] = "re-encoded keys written back by the same call: the re-encoding kernel runs on the context's side stream beside the attention launch (65.5 MB per layer)"
+        fused["k_out"] = "re-encoded keys written back by the same call: the cached keys are re-encoded into k_out and attended from there (65.5 MB per layer)"
         # short final block: 32 x 1000 cached + 64 final tokens, one layer's tensors reused over 4 buffers
         Ts = 64
         lens_s = np.asarray([1000] * 32 + [Ts], dtype=np.int32)
