@@ -332,6 +332,8 @@ ba_status ba_final_attend(ba_ctx *ctx, const void *q_f, const void *k_f, const v
  *                   rows cache_cu[c] .. when src_off is NULL (cache packing)
  *   n_cache_rows    total cached rows of the batch (= cache_cu[Bc])
  *   k_out           NULL, or bf16 [n_cache_rows, n_kv_heads, head_dim] (cache packing), not k_src
+ *                   A source row outside [0, n_src_rows) counts as zeros; with k_out it is written as
+ *                   zeros there and reported through ba_last_device_status() as BA_ERR_INVALID_ARG.
  *   seg             tables of ba_segment(); its cache_rope table holds the rotations
  * A queued ba_reencode_k_deferred job is run as a stand-alone launch first.
  */
@@ -372,7 +374,8 @@ ba_status ba_block_prefill_bwd(ba_ctx *ctx, const void *q, const void *k, const 
  *   page_rows   a power of two, 16 .. 65536
  *   page_cu     device int32 [n_blocks + 1], page_idx device int32 [page_cu[n_blocks]]
  * A page number outside [0, n_pages) is never read: ba_reencode_k_paged skips the row and reports
- * BA_ERR_INVALID_ARG through ba_last_device_status(); the attention calls read zeros in its place.
+ * BA_ERR_INVALID_ARG through ba_last_device_status(); the attention calls read zeros in its place
+ * (ba_final_attend_fused_paged with k_out writes them there and reports as well).
  */
 typedef struct {
   int32_t page_rows;

@@ -1660,6 +1660,9 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
     b.k_cache = (const __nv_bfloat16 *)keys;
     ba_reencode_job job = ba_make_reencode_job(ctx, a.k_cache, a.k_src_off, a.n_k_rows, keys, seg->cache_cu, seg->cache_delta,
                                                seg->n_cached_blocks, a.n_cache_rows, reinterpret_cast<const float2 *>(seg->cache_rope));
+    // A row outside the source is a row of zeros for the attention, as the fused kernel's loads have it; nothing that k_out or
+    // the workspace held before may show.  Only written keys are reported: those are ba_reencode_k's.
+    job.outside = a.k_out ? BA_ROWS_ZERO_REPORTED : BA_ROWS_ZERO;
     if (a.page_rows > 0) {
       job.src_off = nullptr; job.page_cu = a.page_cu; job.page_idx = a.page_idx;
       while ((1 << job.page_lg) < a.page_rows) ++job.page_lg;

@@ -74,7 +74,11 @@ struct ba_reencode_job {
   // 1 << page_lg rows each (src_off is ignored)
   const int32_t *page_cu, *page_idx;
   int32_t page_lg;
+  // a row whose source lies outside `src`: skipped and reported (BA_ROWS_SKIPPED), or written as zeros, as an attention call
+  // that reads it in place would see it
+  int32_t outside;
 };
+constexpr int32_t BA_ROWS_SKIPPED = 0, BA_ROWS_ZERO = 1, BA_ROWS_ZERO_REPORTED = 2;
 
 // Source row of row `t` (0-based inside its block) of a job's block `c`; negative when the page number is bad.
 __device__ __forceinline__ long long ba_job_source_row(const ba_reencode_job &job, int c, int c_begin, int t) {

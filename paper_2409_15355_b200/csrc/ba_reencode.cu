@@ -105,7 +105,7 @@ ba_reencode_job ba_make_reencode_job(const ba_ctx *ctx, const void *k_src, const
   job.head_dim = ctx->cfg.head_dim; job.row_vecs = ctx->cfg.n_kv_heads * ctx->cfg.head_dim / 8;
   job.layout = ctx->cfg.rope_layout;
   job.gen = nullptr; job.gen_expected = 0;
-  job.page_cu = nullptr; job.page_idx = nullptr; job.page_lg = 0;
+  job.page_cu = nullptr; job.page_idx = nullptr; job.page_lg = 0; job.outside = BA_ROWS_SKIPPED;
   return job;
 }
 

@@ -92,6 +92,14 @@ __device__ __forceinline__ void ba_reencode_rotate(const float4 (&tcs)[4], uint4
   }
 }
 
+// A row whose source lies outside the job's: is it written, and as what (a rotated zero is a zero)?
+__device__ __forceinline__ bool ba_reencode_outside_row(const ba_reencode_job &job, uint4 &x, uint4 &y, int32_t *status) {
+  x = y = make_uint4(0u, 0u, 0u, 0u);
+  if (job.outside == BA_ROWS_ZERO) return true;
+  ba_record_status(status, BA_ERR_INVALID_ARG);
+  return job.outside != BA_ROWS_SKIPPED;
+}
+
 // Rows row0, row0 + row_step, ... (kRows of them, those below total_rows), all loads first.
 template <int kLayout, int kRows>
 __device__ __forceinline__ void ba_reencode_rows(const ba_reencode_job &job, ba_reencode_state &st, int row0,
@@ -134,8 +142,7 @@ __device__ __forceinline__ void ba_reencode_rows(const ba_reencode_job &job, ba_
         sr = page < 0 ? -1 : ((long long)page << job.page_lg) + (t & ((1 << job.page_lg) - 1));
       }
       if (sr < 0 || sr >= n_src_rows) {
-        ba_record_status(status, BA_ERR_INVALID_ARG);
-        live[i] = false;
+        live[i] = ba_reencode_outside_row(job, x[i], y[i], status);
       } else {
         const uint4 *p = src + sr * row_vecs;
         x[i] = __ldcs(p + vec_x);
@@ -180,8 +187,7 @@ __device__ __forceinline__ void ba_reencode_block_rows(const ba_reencode_job &jo
       sr = page < 0 ? -1 : ((long long)page << job.page_lg) + (t & ((1 << job.page_lg) - 1));
     }
     if (sr < 0 || sr >= job.n_src_rows) {
-      ba_record_status(status, BA_ERR_INVALID_ARG);
-      live[i] = false;
+      live[i] = ba_reencode_outside_row(job, x[i], y[i], status);
     } else {
       x[i] = __ldcs(job.src + sr * row_vecs + st.vec_x);
       if (kLayout == BA_ROPE_HALF) y[i] = __ldcs(job.src + sr * row_vecs + st.vec_y);

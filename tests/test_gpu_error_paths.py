@@ -1,0 +1,74 @@
+"""What the calls do with indexes that point outside their source, tables that do not hold and shapes at the edge of what a
+step takes: reported, bounded and reproducible, as include/ba.h states.  Tolerances are those of the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import block_attention as ob
+from paper_2409_15355_b200 import binding as B
+from paper_2409_15355_b200 import runtime as R
+from paper_2409_15355_b200 import workloads as W
+from tests.test_gpu_parity import check_attention, check_reencoded, dev
+
+pytestmark = pytest.mark.gpu
+
+
+# ------------------------------------------------------------------ cached rows that point outside their source
+def _fused(c, seg, x, ks, vs, source, Tc, Tf, w, k_out):
+    """One fused call over rows at offsets (`source` an int32 tensor) or pages (a page table)."""
+    o = torch.full((Tf, w.n_q_heads, w.head_dim), float("nan"), device="cuda")
+    lse = torch.full((Tf, w.n_q_heads), float("nan"), device="cuda")
+    q, k, v = (dev(x[n]) for n in ("q_f", "k_f", "v_f"))
+    if isinstance(source, B.ba_page_table):
+        B.ba_final_attend_fused_paged(c.ctx, q, k, v, Tf, ks, vs, source, Tc, o, lse, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32, k_out=k_out)
+    else:
+        B.ba_final_attend_fused(c.ctx, q, k, v, Tf, ks, vs, len(ks), source, Tc, o, lse, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32, k_out=k_out)
+    return o, lse
+
+
+@pytest.mark.parametrize("layout", [B.BA_ROPE_ADJACENT, B.BA_ROPE_HALF], ids=["adjacent", "half"])
+@pytest.mark.parametrize("paged", [False, True], ids=["offsets", "pages"])
+@pytest.mark.parametrize("with_k_out", [False, True], ids=["workspace", "k_out"])
+def test_fused_call_reads_zeros_for_rows_outside_the_source(layout, paged, with_k_out):
+    """Rows whose offset or page lies outside the source count as zeros in the fused call, whichever way it takes: nothing
+    of an earlier call (here NaN keys and values) shows in the result, and it is the same from run to run."""
+    w = W.Workload("outside", 8, 2, 128, 1e4, [64, 33, 100, 64, 40], [5], seed=141)
+    lens, t, x = w.block_lens[:4], ob.segment_tables(w.block_lens, w.seq_nblocks), W.warm_inputs(w)
+    Tc, Tf, f64 = t["n_cached_tokens"], t["n_final_tokens"], W.bf16_bits_to_f64
+    c = R.Context(8, 2, 128, 1e4, rope_layout=layout)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    if paged:
+        (kp, page_cu, page_idx, n_pages), vp = W.scatter_into_pages(x["k_cache"], lens, 16, 3), W.scatter_into_pages(x["v_cache"], lens, 16, 3)[0]
+        bad_idx = page_idx.copy()
+        bad_idx[2], bad_idx[5], bad_idx[-1] = 10 ** 6, -2, n_pages
+        keep = [torch.from_numpy(a).cuda() for a in (page_cu, page_idx, bad_idx)]
+        good, bad = (B.make_page_table(16, n_pages, keep[0], i) for i in keep[1:])
+        rows = np.concatenate([bad_idx[page_cu[i] + np.arange(n) // 16] * 16 + np.arange(n) % 16 for i, n in enumerate(lens)])
+    else:
+        kp, vp = x["k_cache"], x["v_cache"]
+        off = np.asarray([0, -5, Tc - 30, 1 << 30], dtype=np.int32)        # in place, partly in front, partly behind, far outside
+        keep = [torch.from_numpy(a).cuda() for a in (t["cache_cu"][:-1].astype(np.int32), off)]
+        good, bad = keep
+        rows = np.concatenate([o.astype(np.int64) + np.arange(n) for o, n in zip(off, lens)])
+    inside = (rows >= 0) & (rows < len(kp))
+    assert inside.any() and not inside.all()
+    k64, v64 = (np.where(inside[:, None, None], f64(p)[np.where(inside, rows, 0)], 0.0) for p in (kp, vp))
+    k_ref = ob.reencode_blocks(k64, None, t["cache_cu"], t["cache_delta"], 1e4, layout)
+    o_ref, lse_ref = ob.final_attend(f64(x["q_f"]), f64(x["k_f"]), f64(x["v_f"]), k_ref, v64, w.block_lens, w.seq_nblocks)
+    k, v = dev(kp), dev(vp)
+    nan = torch.full_like(k, float("nan"))
+    k_out = torch.empty(Tc, 2, 128, dtype=torch.bfloat16, device="cuda") if with_k_out else None
+    got = []
+    for _ in range(2):
+        if with_k_out:
+            k_out.fill_(float("nan"))
+        _fused(c, seg, x, nan, nan, good, Tc, Tf, w, k_out)                # an earlier call with other contents
+        got.append(_fused(c, seg, x, k, v, bad, Tc, Tf, w, k_out))
+        # written keys are ba_reencode_k's, which reports such rows; a call that only attends reads zeros and says nothing
+        assert c.device_status() == (B.BA_ERR_INVALID_ARG if with_k_out else B.BA_OK)
+        check_attention(got[-1][0].cpu().numpy(), o_ref, got[-1][1].cpu().numpy(), lse_ref)
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    if with_k_out:
+        check_reencoded(R.device_to_bits(k_out), k_ref)
+        assert not k_out[torch.from_numpy(~inside).cuda()].any()
+    c.close()
