@@ -1638,10 +1638,11 @@ int ba_heads_per_tile(const ba_config &c) {
 //    64 / 101 / 256 tokens: fused 81 / 121 / 244 us, two steps 74 / 95 / 163);
 //  * for caches a re-encoding pass takes only a few microseconds over (10 x 128-384 and 32: 23.5 and 19.9).
 // What is left to the fused kernel: short final blocks over long caches (32 x 1000 and 1 / 32 / 64: 53 / 55 / 66 us, two steps
-// 67 / 68 / 73).
+// 67 / 68 / 73), and rows wider than the re-encoding kernel takes.
 static bool fused_in_two_steps(const ba_ctx *ctx, const ba_attend_args &a, const ba_segments *seg, size_t *scratch) {
   if (!a.fused || !a.final_only || a.n_cache_rows < 1 || !seg->cache_rope) return false;
   if (a.k_out) return true;
+  if (ba_reencode_units(ctx->cfg.rope_layout, ctx->cfg.n_kv_heads * ctx->cfg.head_dim / 8) > kBaReencodeMaxUnits) return false;
   *scratch = ba_align_up((size_t)a.n_cache_rows * ctx->cfg.n_kv_heads * ctx->cfg.head_dim * 2, 256);
   if (*scratch > (16u << 20) && (seg->n_final_items < 1 || 2LL * seg->n_final_items < 3LL * seg->batch)) return false;
   return ctx->workspace && ctx->workspace_bytes > ba_scratch_offset(ctx) && *scratch <= (ctx->workspace_bytes - ba_scratch_offset(ctx)) / 2;

@@ -252,6 +252,10 @@ ba_status ba_segment_launch(ba_ctx *ctx, const int32_t *block_lens, const int32_
 ba_status ba_reencode_table_launch(ba_ctx *ctx, const int32_t *delta, int32_t n_blocks, float2 *table,
                                    cudaStream_t stream);
 ba_status ba_reencode_main_launch(ba_ctx *ctx, const ba_reencode_job &job, cudaStream_t stream);
+// Units of a row (a thread moves one: a 16-byte vector, or a pair of them in the half layout).  The re-encoding kernel takes
+// rows of up to kBaReencodeMaxUnits: 4096 elements, 8192 in the half layout.
+constexpr int kBaReencodeMaxUnits = 512;
+static inline int ba_reencode_units(int layout, int row_vecs) { return layout == BA_ROPE_ADJACENT ? row_vecs : row_vecs / 2; }
 ba_status ba_reencode_launch(ba_ctx *ctx, const void *k_src, const int32_t *src_off,
                              int32_t n_src_rows, void *k_dst, const int32_t *cu,
                              const int32_t *delta, int32_t n_blocks, int32_t n_rows, float2 *table,

@@ -37,7 +37,7 @@ ba_rope_table_kernel(const int32_t *__restrict__ delta, int n_blocks, int half_d
 // rows, kRows loads in flight each, so the per-thread set-up (column arithmetic, block search, table
 // fetch) is paid once per kPasses * kRows rows.  A CTA whose rows all lie in one block looks nothing up on the way.
 template <int kLayout, int kRows, int kPasses>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(kBaReencodeMaxUnits)
 ba_reencode_kernel(const ba_reencode_job job, int units_shift, int32_t *status) {
   ba_pdl_wait();
   ba_pdl_trigger();
@@ -115,12 +115,12 @@ ba_status ba_reencode_main_launch(ba_ctx *ctx, const ba_reencode_job &job, cudaS
   // longer than a small job can afford (2400 rows: 5.1 us, 7.6 us with eight).
   constexpr int kRows = 2;
   const bool adjacent = job.layout == BA_ROPE_ADJACENT;
-  const int units = adjacent ? job.row_vecs : job.row_vecs / 2;
+  const int units = ba_reencode_units(job.layout, job.row_vecs);
+  if (units > kBaReencodeMaxUnits) return BA_ERR_UNSUPPORTED;
   // threads per CTA: a multiple of the units per row, close to 128
   int threads = units >= 128 ? units : (128 / units) * units;
   int units_shift = -1;                       // log2(units) when it is a power of two
   for (int k = 0; k < 12; ++k) if ((1 << k) == units) units_shift = k;
-  if (threads > 512) return BA_ERR_UNSUPPORTED;   // more than 4096 bf16 per row
   constexpr int kPasses = 2;                // consecutive row groups per CTA
   const int rows_per_cta = (threads / units) * kRows * kPasses;
   const int grid = (job.n_rows + rows_per_cta - 1) / rows_per_cta;

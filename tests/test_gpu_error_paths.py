@@ -72,3 +72,35 @@ def test_fused_call_reads_zeros_for_rows_outside_the_source(layout, paged, with_
         check_reencoded(R.device_to_bits(k_out), k_ref)
         assert not k_out[torch.from_numpy(~inside).cuda()].any()
     c.close()
+
+
+# ------------------------------------------------------------------ more KV heads than a re-encoding row has threads for
+@pytest.mark.parametrize("heads,layout,wide", [((40, 40, 128), B.BA_ROPE_ADJACENT, True), ((32, 32, 128), B.BA_ROPE_ADJACENT, False),
+                                               ((40, 40, 128), B.BA_ROPE_HALF, False), ((65, 65, 128), B.BA_ROPE_HALF, True),
+                                               ((66, 66, 64), B.BA_ROPE_ADJACENT, True)], ids=str)
+def test_fused_call_takes_rows_wider_than_the_reencoding_kernel(heads, layout, wide):
+    """n_kv_heads * head_dim above what ba_reencode_k takes (it says so): the fused call without k_out still works, as the
+    rotation is then applied to the queries; with k_out it is refused like ba_reencode_k."""
+    w = W.Workload("wide", *heads, 1e4, [70, 33, 20], [3], seed=151)
+    t, x, f64 = ob.segment_tables(w.block_lens, w.seq_nblocks), W.warm_inputs(w), W.bf16_bits_to_f64
+    Tc, Tf = t["n_cached_tokens"], t["n_final_tokens"]
+    c = R.Context(*heads, 1e4, rope_layout=layout, max_q_rows=4096)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    k, v = dev(x["k_cache"]), dev(x["v_cache"])
+    k_ref = ob.reencode_blocks(f64(x["k_cache"]), None, t["cache_cu"], t["cache_delta"], 1e4, layout)
+    o_ref, lse_ref = ob.final_attend(f64(x["q_f"]), f64(x["k_f"]), f64(x["v_f"]), k_ref, f64(x["v_cache"]), w.block_lens, w.seq_nblocks)
+    (kp, page_cu, page_idx, n_pages), vp = W.scatter_into_pages(x["k_cache"], w.block_lens[:2], 16, 3), W.scatter_into_pages(x["v_cache"], w.block_lens[:2], 16, 3)[0]
+    d_cu, d_idx = torch.from_numpy(page_cu).cuda(), torch.from_numpy(page_idx).cuda()
+    for ks, vs, source in ((k, v, None), (dev(kp), dev(vp), B.make_page_table(16, n_pages, d_cu, d_idx))):
+        o, lse = _fused(c, seg, x, ks, vs, source, Tc, Tf, w, None)
+        assert c.device_status() == B.BA_OK
+        check_attention(o.cpu().numpy(), o_ref, lse.cpu().numpy(), lse_ref)
+        k_out = torch.empty_like(k)
+        if wide:
+            with pytest.raises(B.BaError) as e:
+                _fused(c, seg, x, ks, vs, source, Tc, Tf, w, k_out)
+            assert e.value.status == B.BA_ERR_UNSUPPORTED
+        else:
+            _fused(c, seg, x, ks, vs, source, Tc, Tf, w, k_out)
+            check_reencoded(R.device_to_bits(k_out), k_ref)
+    c.close()
