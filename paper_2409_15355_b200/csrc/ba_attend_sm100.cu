@@ -1440,7 +1440,7 @@ ba_combine_splits_kernel(const CombineParams p) {
   ba_pdl_wait();
   ba_pdl_trigger();
   const int n_final = __ldg(p.totals + 3);
-  if ((int)blockIdx.y >= n_final) return;
+  if (__ldg(p.totals + 7) != BA_TABLES_VALID || (int)blockIdx.y >= n_final) return;    // (nothing was attended either)
   const int32_t *line = p.items + 8 * ((p.final_only ? 0 : __ldg(p.totals + 2) - n_final) + blockIdx.y);
   const int q_row0 = __ldg(line), q_rows = min(__ldg(line + 1), p.n_q_rows - q_row0);
   const int part0 = p.final_only ? q_row0 : __ldg(line + 5), head0 = (blockIdx.x >> p.parts_log2) * p.hpt;

@@ -104,3 +104,37 @@ def test_fused_call_takes_rows_wider_than_the_reencoding_kernel(heads, layout, w
             _fused(c, seg, x, ks, vs, source, Tc, Tf, w, k_out)
             check_reencoded(R.device_to_bits(k_out), k_ref)
     c.close()
+
+
+# ------------------------------------------------------------------ tables of lengths that do not add up
+@pytest.mark.parametrize("fault", ["tokens", "zero_length", "block_counts"])
+def test_split_keys_over_inconsistent_tables_leave_the_output_alone(fault):
+    """Lengths on the device that do not add up leave the item tables as they were (here: those of an earlier call).  The keys of a
+    short final block are split over several CTAs, whose results a second kernel merges: neither touches the output."""
+    w = W.Workload("tables", 8, 2, 64, 1e4, [64, 33, 300, 40], [4], seed=161)
+    x = W.warm_inputs(w)
+    Tf, Tc = 40, w.n_tokens - 40
+    c = R.Context(8, 2, 64, 1e4)
+    q, k, v, kc, vc = (dev(x[n]) for n in ("q_f", "k_f", "v_f", "k_cache", "v_cache"))
+    o = torch.full((Tf, 8, 64), 7.0, device="cuda")
+    lse = torch.full((Tf, 8), 7.0, device="cuda")
+    lens, nb = torch.tensor(w.block_lens, dtype=torch.int32, device="cuda"), torch.tensor([4], dtype=torch.int32, device="cuda")
+    buf = torch.zeros(B.ba_segments_bytes(1, 4, w.n_tokens), dtype=torch.uint8, device="cuda")
+    seg = B.ba_segment(c.ctx, lens, nb, 1, 4, w.n_tokens, B.BA_MODE_BLOCK, buf)
+    B.ba_final_attend(c.ctx, q, k, v, Tf, kc, vc, Tc, None, 0, o, lse, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    assert c.device_status() == B.BA_OK and c.last_attend_shape()["partials"] > 1
+    assert torch.isfinite(o).all() and not (o == 7.0).any()
+    o.fill_(7.0); lse.fill_(7.0)
+    if fault == "tokens":
+        lens[1] += 1
+    elif fault == "zero_length":
+        lens[1] = 0
+    else:
+        nb[0] = 3
+    seg = B.ba_segment(c.ctx, lens, nb, 1, 4, w.n_tokens, B.BA_MODE_BLOCK, buf)
+    assert c.device_status() == B.BA_ERR_INVALID_ARG
+    B.ba_final_attend(c.ctx, q, k, v, Tf, kc, vc, Tc, None, 0, o, lse, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    torch.cuda.synchronize()
+    assert c.last_attend_shape()["partials"] > 1
+    assert (o == 7.0).all() and (lse == 7.0).all()
+    c.close()
