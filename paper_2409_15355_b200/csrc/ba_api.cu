@@ -139,7 +139,7 @@ ba_status ba_create(ba_ctx **out, const ba_config *cfg, int device, size_t works
   ctx->pending_table_bytes = 0;
   ctx->pending_stream = nullptr;
   ctx->seg_delta = nullptr; ctx->seg_rope = nullptr; ctx->seg_rope_blocks = 0;
-  ctx->seg_gen = nullptr; ctx->seg_gen_value = 0; ctx->seg_counter = 0;
+  ctx->seg_totals = nullptr; ctx->seg_stamp = 0; ctx->seg_counter = 0;
   ctx->maps = nullptr;
   ctx->workspace = nullptr;
   ctx->dev_status = nullptr;
@@ -304,7 +304,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
   out->totals = next();
   out->cache_rope = (float *)next();
   out->prompt_items = next(); out->final_items = next(); out->cu_stream = next(); out->cache_tile_block = next();
-  ctx->seg_delta = nullptr; ctx->seg_rope = nullptr; ctx->seg_rope_blocks = 0; ctx->seg_gen = nullptr;
+  ctx->seg_delta = nullptr; ctx->seg_rope = nullptr; ctx->seg_rope_blocks = 0; ctx->seg_totals = nullptr;
   // Every call stamps its tables (totals[6]) with a value that differs from call to call and from
   // context to context: a later re-encoding that wants to reuse the rotation table stored with the
   // tables can tell on the device whether the buffer still holds this call's tables.
@@ -316,7 +316,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
   if (st == BA_OK && out->n_cached_blocks > 0) {
     ctx->seg_delta = out->cache_delta; ctx->seg_rope = (const float2 *)out->cache_rope;
     ctx->seg_rope_blocks = out->n_cached_blocks;
-    ctx->seg_gen = out->totals + 6; ctx->seg_gen_value = gen;
+    ctx->seg_totals = out->totals; ctx->seg_stamp = gen;
   }
   return st;
 }
@@ -354,7 +354,7 @@ ba_status ba_reencode_k(ba_ctx *ctx, const void *k_src, const int32_t *src_off, 
   if (delta == ctx->seg_delta && n_blocks == ctx->seg_rope_blocks) {   // the table ba_segment built is for these deltas
     ba_reencode_job job =
         ba_make_reencode_job(ctx, k_src, src_off, n_src_rows, k_dst, cu, delta, n_blocks, n_rows, ctx->seg_rope);
-    job.gen = ctx->seg_gen; job.gen_expected = ctx->seg_gen_value;
+    job.totals = ctx->seg_totals; job.stamp = ctx->seg_stamp;
     return ba_reencode_main_launch(ctx, job, (cudaStream_t)stream);
   }
   float2 *table; size_t bytes;
@@ -386,7 +386,7 @@ ba_status ba_reencode_k_deferred(ba_ctx *ctx, const void *k_src, const int32_t *
     table_used = table;
   }
   ctx->pending = ba_make_reencode_job(ctx, k_src, src_off, n_src_rows, k_dst, cu, delta, n_blocks, n_rows, table_used);
-  if (table_used == ctx->seg_rope) { ctx->pending.gen = ctx->seg_gen; ctx->pending.gen_expected = ctx->seg_gen_value; }
+  if (table_used == ctx->seg_rope) { ctx->pending.totals = ctx->seg_totals; ctx->pending.stamp = ctx->seg_stamp; }
   ctx->has_pending = 1;
   ctx->pending_table_bytes = bytes;
   ctx->pending_stream = (cudaStream_t)stream;
@@ -527,7 +527,7 @@ ba_status ba_reencode_k_paged(ba_ctx *ctx, const void *k_pool, const ba_page_tab
   }
   ba_reencode_job job = ba_make_reencode_job(ctx, k_pool, nullptr, n_src_rows, k_dst, cu, delta, n_blocks, n_rows,
                                              reuse ? ctx->seg_rope : table);
-  if (reuse) { job.gen = ctx->seg_gen; job.gen_expected = ctx->seg_gen_value; }
+  if (reuse) { job.totals = ctx->seg_totals; job.stamp = ctx->seg_stamp; }
   job.page_cu = pages->page_cu; job.page_idx = pages->page_idx;
   job.page_lg = 0;
   while ((1 << job.page_lg) < pages->page_rows) ++job.page_lg;

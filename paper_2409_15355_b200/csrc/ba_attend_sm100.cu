@@ -1663,6 +1663,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
                                                seg->n_cached_blocks, a.n_cache_rows, reinterpret_cast<const float2 *>(seg->cache_rope));
     // A row outside the source is a row of zeros for the attention, as the fused kernel's loads have it; nothing that k_out or
     // the workspace held before may show.  Only written keys are reported: those are ba_reencode_k's.
+    job.totals = seg->totals;
     job.outside = a.k_out ? BA_ROWS_ZERO_REPORTED : BA_ROWS_ZERO;
     if (a.page_rows > 0) {
       job.src_off = nullptr; job.page_cu = a.page_cu; job.page_idx = a.page_idx;

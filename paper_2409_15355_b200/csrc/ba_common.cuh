@@ -65,11 +65,11 @@ struct ba_reencode_job {
   const float2 *table;      // [n_blocks][head_dim / 2] (cos, sin)
   int32_t n_src_rows, n_blocks, n_rows;
   int32_t head_dim, row_vecs /* uint4 per row */, layout;
-  // non-null: `table` is the rotation table ba_segment() stored with its tables; *gen must still hold
-  // gen_expected (the stamp that call wrote), else the tables were rebuilt or overwritten since and
-  // the job reports BA_ERR_INVALID_ARG instead of rotating with a foreign table
-  const int32_t *gen;
-  int32_t gen_expected;
+  // non-null: the totals of the ba_segment() tables that `cu`, `delta` or `table` belong to.  They must be valid -- of tables
+  // whose lengths did not add up nothing but the totals is written -- and, with stamp != 0 (`table` is the rotation table
+  // stored with them), still those of the call that stamped them; else the job reports BA_ERR_INVALID_ARG and moves nothing.
+  const int32_t *totals;
+  int32_t stamp;
   // non-null: the source is a paged pool -- block c owns pages page_idx[page_cu[c] .. page_cu[c+1]) of
   // 1 << page_lg rows each (src_off is ignored)
   const int32_t *page_cu, *page_idx;
@@ -80,14 +80,19 @@ struct ba_reencode_job {
 };
 constexpr int32_t BA_ROWS_SKIPPED = 0, BA_ROWS_ZERO = 1, BA_ROWS_ZERO_REPORTED = 2;
 
-// Source row of row `t` (0-based inside its block) of a job's block `c`; negative when the page number is bad.
+// Source row of row `t` (0-based inside its block) of a job's block `c`; negative when its page list has no good entry for it.
 __device__ __forceinline__ long long ba_job_source_row(const ba_reencode_job &job, int c, int c_begin, int t) {
   if (job.page_cu) {
-    const int page = __ldg(job.page_idx + __ldg(job.page_cu + c) + (t >> job.page_lg));
+    const int page0 = __ldg(job.page_cu + c), k = t >> job.page_lg;
+    const int page = k >= 0 && k < __ldg(job.page_cu + c + 1) - page0 ? __ldg(job.page_idx + page0 + k) : -1;
     if (page < 0) return -1;
     return ((long long)page << job.page_lg) + (t & ((1 << job.page_lg) - 1));
   }
   return (job.src_off ? (long long)__ldg(job.src_off + c) : (long long)c_begin) + t;
+}
+
+__device__ __forceinline__ bool ba_job_tables_hold(const ba_reencode_job &job) {
+  return !job.totals || (__ldg(job.totals + 7) == BA_TABLES_VALID && (job.stamp == 0 || __ldg(job.totals + 6) == job.stamp));
 }
 
 // Context: configuration, workspace and the device status word.
@@ -112,8 +117,8 @@ struct ba_ctx {
   const int32_t *seg_delta;
   const float2 *seg_rope;
   int32_t seg_rope_blocks;
-  const int32_t *seg_gen;   // device word the same ba_segment stamped with seg_gen_value (totals[6])
-  int32_t seg_gen_value;
+  const int32_t *seg_totals;   // totals of the same ba_segment, which stamped them with seg_stamp ([6])
+  int32_t seg_stamp;
   int32_t seg_counter;      // ba_segment calls so far on this context
   // tensor maps of recently used tensors (attention launches re-use a handful of buffers)
   struct ba_map_cache *maps;

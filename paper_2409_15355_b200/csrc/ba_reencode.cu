@@ -48,7 +48,7 @@ ba_reencode_kernel(const ba_reencode_job job, int units_shift, int32_t *status) 
   const int rsub = units_shift >= 0 ? (int)(threadIdx.x >> units_shift) : (int)(threadIdx.x / units_per_row);
   const int total_rows = min(job.n_rows, __ldg(job.cu + job.n_blocks));
   const int cta_row0 = blockIdx.x * (row_step * kRows * kPasses);
-  if (job.gen && __ldg(job.gen) != job.gen_expected) {     // the rotation table is not the one this job was given
+  if (!ba_job_tables_hold(job)) {
     if (threadIdx.x == 0) ba_record_status(status, BA_ERR_INVALID_ARG);
     return;
   }
@@ -67,7 +67,7 @@ ba_reencode_kernel(const ba_reencode_job job, int units_shift, int32_t *status) 
   st.c_begin = __ldg(job.cu + st.c);
   st.c_end = __ldg(job.cu + st.c + 1);
   st.shift = job.src_off ? (long long)__ldg(job.src_off + st.c) - st.c_begin : 0;
-  st.page0 = job.page_cu ? __ldg(job.page_cu + st.c) : 0;
+  if (job.page_cu) { st.page0 = __ldg(job.page_cu + st.c); st.n_pages = max(0, __ldg(job.page_cu + st.c + 1) - st.page0); }
   const int cta_end = min(cta_row0 + row_step * kRows * kPasses, total_rows);
   if (cta_end <= st.c_end) {                               // the usual case: one block, looked up above
     st.t_delta = __ldg(job.delta + st.c);
@@ -104,7 +104,7 @@ ba_reencode_job ba_make_reencode_job(const ba_ctx *ctx, const void *k_src, const
   job.table = table; job.n_src_rows = n_src_rows; job.n_blocks = n_blocks; job.n_rows = n_rows;
   job.head_dim = ctx->cfg.head_dim; job.row_vecs = ctx->cfg.n_kv_heads * ctx->cfg.head_dim / 8;
   job.layout = ctx->cfg.rope_layout;
-  job.gen = nullptr; job.gen_expected = 0;
+  job.totals = nullptr; job.stamp = 0;
   job.page_cu = nullptr; job.page_idx = nullptr; job.page_lg = 0; job.outside = BA_ROWS_SKIPPED;
   return job;
 }
@@ -215,7 +215,7 @@ extern "C" ba_status ba_reencode_k_noalloc(const ba_config *cfg, int device, con
   tmp.pending_table_bytes = 0;
   tmp.pending_stream = nullptr;
   tmp.seg_delta = nullptr; tmp.seg_rope = nullptr; tmp.seg_rope_blocks = 0;
-  tmp.seg_gen = nullptr; tmp.seg_gen_value = 0; tmp.seg_counter = 0; tmp.maps = nullptr;
+  tmp.seg_totals = nullptr; tmp.seg_stamp = 0; tmp.seg_counter = 0; tmp.maps = nullptr;
   return ba_reencode_launch(&tmp, k_src, src_off, n_src_rows, k_dst, cu, delta, n_blocks, n_rows,
                             g_noalloc_table[device], (cudaStream_t)stream);
 }

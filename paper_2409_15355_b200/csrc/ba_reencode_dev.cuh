@@ -38,7 +38,7 @@ struct ba_reencode_state {
   int vec_x, vec_y, m0;              // the thread's vector column(s) and first rotary pair
   int c, c_begin, c_end;             // block of the last row and its row range
   long long shift;                   // source row = row + shift (contiguous source)
-  int page0;                         // first entry of the block's page list (paged source)
+  int page0, n_pages;                // the block's page list (paged source): first entry, entries
   int t_blk, t_delta;                // block whose (cos, sin) values are loaded, and its delta
   float4 tcs[4];
 };
@@ -56,7 +56,7 @@ __device__ __forceinline__ void ba_reencode_state_init(const ba_reencode_job &jo
     st.vec_y = st.vec_x + hv;
     st.m0 = v * 8;
   }
-  st.c = 0; st.c_begin = 0; st.c_end = -1; st.shift = 0; st.page0 = 0;
+  st.c = 0; st.c_begin = 0; st.c_end = -1; st.shift = 0; st.page0 = 0; st.n_pages = 0;
   st.t_blk = -1; st.t_delta = 0;
 }
 
@@ -90,6 +90,13 @@ __device__ __forceinline__ void ba_reencode_rotate(const float4 (&tcs)[4], uint4
     x = make_uint4(ox[0], ox[1], ox[2], ox[3]);
     y = make_uint4(oy[0], oy[1], oy[2], oy[3]);
   }
+}
+
+// Source row of row t of the block in a paged pool; negative when the block's page list has no good entry for it.
+__device__ __forceinline__ long long ba_reencode_page_row(const ba_reencode_job &job, const ba_reencode_state &st, int t) {
+  const int k = t >> job.page_lg;
+  const int page = (unsigned)k < (unsigned)st.n_pages ? __ldg(job.page_idx + st.page0 + k) : -1;
+  return page < 0 ? -1 : ((long long)page << job.page_lg) + (t & ((1 << job.page_lg) - 1));
 }
 
 // A row whose source lies outside the job's: is it written, and as what (a rotated zero is a zero)?
@@ -132,14 +139,12 @@ __device__ __forceinline__ void ba_reencode_rows(const ba_reencode_job &job, ba_
         st.c_begin = __ldg(cu + c);
         st.c_end = __ldg(cu + c + 1);
         st.shift = src_off ? (long long)__ldg(src_off + c) - st.c_begin : 0;
-        st.page0 = job.page_cu ? __ldg(job.page_cu + c) : 0;
+        if (job.page_cu) { st.page0 = __ldg(job.page_cu + c); st.n_pages = max(0, __ldg(job.page_cu + c + 1) - st.page0); }
       }
       blk[i] = st.c;
       long long sr = r + st.shift;
       if (job.page_cu) {
-        const int t = r - st.c_begin;
-        const int page = __ldg(job.page_idx + st.page0 + (t >> job.page_lg));
-        sr = page < 0 ? -1 : ((long long)page << job.page_lg) + (t & ((1 << job.page_lg) - 1));
+        sr = ba_reencode_page_row(job, st, r - st.c_begin);
       }
       if (sr < 0 || sr >= n_src_rows) {
         live[i] = ba_reencode_outside_row(job, x[i], y[i], status);
@@ -183,8 +188,7 @@ __device__ __forceinline__ void ba_reencode_block_rows(const ba_reencode_job &jo
     if (!live[i]) continue;
     long long sr = r + st.shift;
     if (job.page_cu) {
-      const int t = r - st.c_begin, page = __ldg(job.page_idx + st.page0 + (t >> job.page_lg));
-      sr = page < 0 ? -1 : ((long long)page << job.page_lg) + (t & ((1 << job.page_lg) - 1));
+      sr = ba_reencode_page_row(job, st, r - st.c_begin);
     }
     if (sr < 0 || sr >= job.n_src_rows) {
       live[i] = ba_reencode_outside_row(job, x[i], y[i], status);
@@ -236,7 +240,7 @@ __device__ __forceinline__ void ba_reencode_background(const ba_reencode_job &jo
   const int total_rows = min(job.n_rows, __ldg(job.cu + job.n_blocks));
   const int n_chunks = (total_rows + rows_per_chunk - 1) / rows_per_chunk;
   const bool adjacent = job.layout == BA_ROPE_ADJACENT;
-  if (job.gen && __ldg(job.gen) != job.gen_expected) {     // the rotation table is not the one this job was given
+  if (!ba_job_tables_hold(job)) {
     if (lane == 0) ba_record_status(status, BA_ERR_INVALID_ARG);
     return;
   }

@@ -106,7 +106,7 @@ def test_fused_call_takes_rows_wider_than_the_reencoding_kernel(heads, layout, w
     c.close()
 
 
-# ------------------------------------------------------------------ tables of lengths that do not add up
+# ------------------------------------------------------------------ tables of lengths that do not add up, page lists too short
 @pytest.mark.parametrize("fault", ["tokens", "zero_length", "block_counts"])
 def test_split_keys_over_inconsistent_tables_leave_the_output_alone(fault):
     """Lengths on the device that do not add up leave the item tables as they were (here: those of an earlier call).  The keys of a
@@ -137,4 +137,75 @@ def test_split_keys_over_inconsistent_tables_leave_the_output_alone(fault):
     torch.cuda.synchronize()
     assert c.last_attend_shape()["partials"] > 1
     assert (o == 7.0).all() and (lse == 7.0).all()
+    c.close()
+
+
+def _paged_request():
+    w = W.Workload("tables", 8, 2, 64, 1e4, [64, 33, 100, 40], [4], seed=161)
+    t, x = ob.segment_tables(w.block_lens, w.seq_nblocks), W.warm_inputs(w)
+    (kp, page_cu, page_idx, n_pages), vp = W.scatter_into_pages(x["k_cache"], w.block_lens[:3], 16, 3), W.scatter_into_pages(x["v_cache"], w.block_lens[:3], 16, 3)[0]
+    d_cu, d_idx = torch.from_numpy(page_cu).cuda(), torch.from_numpy(page_idx).cuda()
+    return w, t, x, dev(kp), dev(vp), d_cu, d_idx, n_pages
+
+
+@pytest.mark.parametrize("fault", ["tokens", "zero_length", "block_counts"])
+def test_calls_over_inconsistent_tables_report_and_move_nothing(fault):
+    """Lengths on the device that do not add up: ba_segment leaves the tables unwritten (here: a buffer of a large pattern).
+    Every call that walks them reports it and touches none of its outputs, the re-encoding step of a fused call among them."""
+    w, t, x, kp, vp, d_cu, d_idx, n_pages = _paged_request()
+    Tc, Tf = t["n_cached_tokens"], t["n_final_tokens"]
+    c = R.Context(8, 2, 64, 1e4)
+    lens, nb, T = torch.tensor(w.block_lens, dtype=torch.int32, device="cuda"), torch.tensor([4], dtype=torch.int32, device="cuda"), w.n_tokens
+    buf = torch.full((B.ba_segments_bytes(1, 4, T),), 0x3f, dtype=torch.uint8, device="cuda")
+    if fault == "tokens":
+        lens[1] += 1
+    elif fault == "zero_length":
+        lens[1] = 0
+    else:
+        nb[0] = 3
+    seg = B.ba_segment(c.ctx, lens, nb, 1, 4, T, B.BA_MODE_BLOCK, buf)
+    assert c.device_status() == B.BA_ERR_INVALID_ARG
+    pages = B.make_page_table(16, n_pages, d_cu, d_idx)
+    q, k, v = (dev(x[n]) for n in ("q_f", "k_f", "v_f"))
+    k_src, v_src = dev(x["k_cache"]), dev(x["v_cache"])
+    o = torch.full((Tf, 8, 64), 7.0, device="cuda")
+    for with_k_out in (False, True):
+        for call in ("fused", "paged", "reencode_paged", "reencode", "deferred"):
+            if call in ("reencode_paged", "reencode", "deferred") and not with_k_out:
+                continue
+            keys = torch.full((Tc, 2, 64), 7.0, dtype=torch.bfloat16, device="cuda")
+            k_out = keys if with_k_out else None
+            if call == "fused":
+                B.ba_final_attend_fused(c.ctx, q, k, v, Tf, k_src, v_src, Tc, None, Tc, o, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32, k_out=k_out)
+            elif call == "paged":
+                B.ba_final_attend_fused_paged(c.ctx, q, k, v, Tf, kp, vp, pages, Tc, o, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32, k_out=k_out)
+            elif call == "reencode_paged":
+                B.ba_reencode_k_paged(c.ctx, kp, pages, keys, seg.cache_cu, seg.cache_delta, 3, Tc)
+            elif call == "reencode":
+                B.ba_reencode_k(c.ctx, k_src, None, Tc, keys, seg.cache_cu, seg.cache_delta, 3, Tc)
+            else:
+                B.ba_reencode_k_deferred(c.ctx, k_src, None, Tc, keys, seg.cache_cu, seg.cache_delta, 3, Tc)
+                B.ba_final_attend(c.ctx, q, k, v, Tf, k_src, v_src, Tc, None, 0, o, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+            assert c.device_status() == B.BA_ERR_INVALID_ARG, call
+            assert (o == 7.0).all() and (keys == 7.0).all(), call
+    c.close()
+
+
+def test_page_list_shorter_than_its_block():
+    """Rows past the end of their block's page list are rows outside the source; the next list's entries are not theirs."""
+    w, t, x, kp, vp, d_cu, d_idx, n_pages = _paged_request()
+    Tc = t["n_cached_tokens"]
+    c = R.Context(8, 2, 64, 1e4)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    want, got = (torch.zeros(Tc, 2, 64, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    B.ba_reencode_k_paged(c.ctx, kp, B.make_page_table(16, n_pages, d_cu, d_idx), want, seg.cache_cu, seg.cache_delta, 3, Tc)
+    assert c.device_status() == B.BA_OK
+    short = d_cu.clone()
+    short[-1] -= 2                                                         # the last block: rows 80 .. 99 have no page
+    for call in range(2):
+        got.zero_()
+        own = torch.from_numpy(t["cache_delta"].astype(np.int32)).cuda()   # (the tables' own array, then a caller's)
+        B.ba_reencode_k_paged(c.ctx, kp, B.make_page_table(16, n_pages, short, d_idx), got, seg.cache_cu, own if call else seg.cache_delta, 3, Tc)
+        assert c.device_status() == B.BA_ERR_INVALID_ARG
+        assert torch.equal(got[:Tc - 20], want[:Tc - 20]) and not got[Tc - 20:].any()
     c.close()
