@@ -217,6 +217,12 @@ __device__ __forceinline__ int count_items(const AttnParams &p) {
   return __ldg(p.seg.totals + (p.final_only ? 3 : 2));
 }
 
+// Partial results of a prefill are indexed by the row's place among the rows of final blocks, of which the host made room for
+// n_part_rows; the tables may have been rebuilt in their buffer since.  (Those of a final attend are indexed by the query row.)
+__device__ __forceinline__ bool partials_fit(const int32_t *totals, int final_only, int n_splits, int n_part_rows) {
+  return final_only || n_splits <= 1 || __ldg(totals + 1) <= n_part_rows;
+}
+
 // Item `idx`: independent loads of one line of the table ba_segment built, instead of a search for the item's sequence or
 // block and look-ups that depend on it.  (Four-byte loads: 16-byte ones tie up groups of four registers, and the softmax
 // loop of the fused path spills.)
@@ -593,6 +599,10 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   WorkEntry first = {-1, 0, 0, 0, -1, 0};
   if (warp == 8) {
     n_items = count_items(p);
+    if (kVariant == kPlain && n_items > 0 && !partials_fit(p.seg.totals, p.final_only, p.n_splits, p.n_part_rows)) {
+      ba_record_status(p.status, BA_ERR_SHAPE);            // the tables describe another launch than the host sized
+      n_items = 0;
+    }
     if (kClustered) first = cluster_entry(p, n_items);
     else if (!balanced && !stream) first = list_entry(p, n_items, (int)blockIdx.x);
   }
@@ -1440,7 +1450,9 @@ ba_combine_splits_kernel(const CombineParams p) {
   ba_pdl_wait();
   ba_pdl_trigger();
   const int n_final = __ldg(p.totals + 3);
-  if (__ldg(p.totals + 7) != BA_TABLES_VALID || (int)blockIdx.y >= n_final) return;    // (nothing was attended either)
+  if (__ldg(p.totals + 7) != BA_TABLES_VALID || (int)blockIdx.y >= n_final ||
+      !partials_fit(p.totals, p.final_only, p.n_splits, p.n_part_rows))
+    return;                                                // (nothing was attended either)
   const int32_t *line = p.items + 8 * ((p.final_only ? 0 : __ldg(p.totals + 2) - n_final) + blockIdx.y);
   const int q_row0 = __ldg(line), q_rows = min(__ldg(line + 1), p.n_q_rows - q_row0);
   const int part0 = p.final_only ? q_row0 : __ldg(line + 5), head0 = (blockIdx.x >> p.parts_log2) * p.hpt;

@@ -209,3 +209,22 @@ def test_page_list_shorter_than_its_block():
         assert c.device_status() == B.BA_ERR_INVALID_ARG
         assert torch.equal(got[:Tc - 20], want[:Tc - 20]) and not got[Tc - 20:].any()
     c.close()
+
+
+def test_prefill_over_tables_rebuilt_with_longer_final_blocks():
+    """A prefill keeps partial results of the final blocks' rows, in room for as many as its ba_segments says.  When the buffer has
+    been rebuilt since with more of them, the call reports it and writes nothing."""
+    a, b = [300] * 9 + [65], [100] * 9 + [1865]
+    w = W.Workload("rebuilt", 32, 8, 128, 1e4, a, [10], seed=171)
+    x = [dev(v) for v in W.prefill_inputs(w)]
+    c = R.Context.for_workload(w)
+    seg, buf = c.segment(a, [10], B.BA_MODE_BLOCK)
+    o = torch.full((w.n_tokens, 32, 128), 7.0, device="cuda")
+    B.ba_block_prefill(c.ctx, *x, o, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    assert c.device_status() == B.BA_OK and c.last_attend_shape()["partials"] > 1
+    o.fill_(7.0)
+    B.ba_segment(c.ctx, np.asarray(b, dtype=np.int32), np.asarray([10], dtype=np.int32), 1, 10, w.n_tokens, B.BA_MODE_BLOCK, buf)
+    B.ba_block_prefill(c.ctx, *x, o, None, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    assert c.device_status() == B.BA_ERR_SHAPE
+    assert (o == 7.0).all()
+    c.close()
