@@ -111,10 +111,11 @@ __device__ __forceinline__ bool segment_blocks(const SegmentArgs &a, const int32
 
   // --- first block of every sequence
   int carry = 0;
+  bool seq_bad = false;
   for (int base = 0; base < batch; base += (int)blockDim.x) {
     const int s = base + tid;
     int v[1] = {s < batch ? seq_nblocks[s] : 0}, total[1];
-    if (s < batch && v[0] < 1) { *bad = 1; v[0] = 0; }
+    if (s < batch && v[0] < 1) { seq_bad = true; v[0] = 0; }
     cta_exclusive_scan<1>(v, total, scan_smem);
     if (s < batch) {
       t.cu_seq_block[s] = carry + v[0];
@@ -126,8 +127,8 @@ __device__ __forceinline__ bool segment_blocks(const SegmentArgs &a, const int32
     t.cu_seq_block[batch] = carry;
     if (kShared && writer) seg.cu_seq_block[batch] = carry;
   }
-  __syncthreads();
-  if (carry != B || *bad) return false;  // uniform: every thread holds the same carry and reads the same flag
+  // (one decision for all threads, made before any of them can raise the flag for a block's length)
+  if (__syncthreads_or(carry != B || seq_bad)) return false;
 
   // --- per-block prefix sums: rows, rows of final blocks, query tiles, 128-key tiles (all / final blocks), query tiles of
   // the final blocks
