@@ -354,6 +354,7 @@ ba_status ba_final_attend_fused(ba_ctx *ctx, const void *q_f, const void *k_f, c
  *   lse                  fp32 [T, n_q_heads]: the forward call's log-sum-exp (required)
  *   d_o                  bf16 [T, n_q_heads, head_dim]: gradient of the loss with respect to o
  *   dq                   [T, n_q_heads, head_dim];  dk, dv  [T, n_kv_heads, head_dim]; bf16 or fp32
+ *                        dq in bf16 may take the place of q or d_o; no other output may overlap an input
  * Uses T * n_q_heads * 4 bytes of workspace (BA_ERR_WORKSPACE when the context has less).  No
  * atomics: results are run-to-run identical.
  */

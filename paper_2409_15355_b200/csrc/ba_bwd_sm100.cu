@@ -486,7 +486,7 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
   const int tid = threadIdx.x, warp = tid >> 5;
   const ba_segments &sg = p.seg;
   // This kernel needs dO . O, which was complete before the dK/dV kernel triggered, and nothing of the dK/dV kernel itself:
-  // it starts on the SMs that one leaves and waits for it only before it ends.
+  // it starts on the SMs that one leaves (unless dq takes the place of an input) and waits for it only before it ends.
   struct WaitAtExit { __device__ ~WaitAtExit() { ba_pdl_wait(); } } wait_at_exit;
   if (__ldg(sg.totals + 7) != BA_TABLES_VALID) return;
 
@@ -711,15 +711,22 @@ bool bwd_make_map(CUtensorMap *m, const void *ptr, int D, int heads, long long r
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool overlap(const void *a, size_t a_bytes, const void *b, size_t b_bytes) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+  return x < y + b_bytes && y < x + a_bytes;
+}
+
+// dq_in_place: dq takes the place of q or d_o.  A CTA of the dQ kernel has its own rows of both in shared memory before it writes
+// them, but the dK/dV kernel reads all of them: the dQ kernel must not start before that one has ended.
 template <int D>
-ba_status launch_bwd(ba_ctx *ctx, const BwdParams &p, const CUtensorMap &tq, const CUtensorMap &tdo, const CUtensorMap &tk,
+ba_status launch_bwd(ba_ctx *ctx, const BwdParams &p, bool dq_in_place, const CUtensorMap &tq, const CUtensorMap &tdo, const CUtensorMap &tk,
                      const CUtensorMap &tv, const CUtensorMap &tk64, const CUtensorMap &tv64, int n_ktiles_upper, int n_pairs_upper,
                      cudaStream_t stream) {
   BA_CUDA_TRY(ba_launch(ba_bwd_dkv_kernel<D>, dim3((unsigned)n_ktiles_upper, (unsigned)p.Hkv), kDkvThreads, DkvLayout<D>::kBytes + 1024,
                         stream, true, tq, tdo, tk, tv, p));
   const int n_head_chunks = p.Hq / p.hpt;
   BA_CUDA_TRY(ba_launch(ba_bwd_dq_kernel<D>, dim3((unsigned)(2 * n_pairs_upper) * n_head_chunks), kDqThreads, DqLayout<D>::kBytes, stream,
-                        true, tq, tdo, tk64, tv64, p, 2 * n_pairs_upper, n_head_chunks));
+                        !dq_in_place, tq, tdo, tk64, tv64, p, 2 * n_pairs_upper, n_head_chunks));
   ctx->launches += 2;
   return BA_OK;
 }
@@ -767,6 +774,8 @@ ba_status ba_bwd_sm100_launch(ba_ctx *ctx, const void *q, const void *k, const v
     return BA_ERR_CUDA;
   const int n_ktiles_upper = T / kTile + seg->n_blocks;
   const int n_pairs_upper = seg->n_prompt_items > 0 ? seg->n_prompt_items : T / (2 * p.tok) + seg->n_blocks;
-  if (D == 128) return launch_bwd<128>(ctx, p, tq, tdo, tk, tv, tk64, tv64, n_ktiles_upper, n_pairs_upper, stream);
-  return launch_bwd<64>(ctx, p, tq, tdo, tk, tv, tk64, tv64, n_ktiles_upper, n_pairs_upper, stream);
+  const size_t q_bytes = (size_t)T * Hq * D * 2, dq_bytes = out_f32 ? 2 * q_bytes : q_bytes;
+  const bool dq_in_place = overlap(dq, dq_bytes, q, q_bytes) || overlap(dq, dq_bytes, d_o, q_bytes);
+  if (D == 128) return launch_bwd<128>(ctx, p, dq_in_place, tq, tdo, tk, tv, tk64, tv64, n_ktiles_upper, n_pairs_upper, stream);
+  return launch_bwd<64>(ctx, p, dq_in_place, tq, tdo, tk, tv, tk64, tv64, n_ktiles_upper, n_pairs_upper, stream);
 }

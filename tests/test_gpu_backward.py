@@ -136,3 +136,29 @@ def test_backward_rejects_missing_arguments():
     assert e.value.status == B.BA_ERR_WORKSPACE
     B.ba_destroy(small)
     c.close()
+
+
+@pytest.mark.parametrize("place", ["q", "d_o"])
+@pytest.mark.parametrize("heads", [(6, 2, 64), (8, 2, 128)], ids=str)
+def test_backward_writes_dq_in_the_place_of_an_input(place, heads):
+    """dQ over q or d_o gives the bits of separate tensors, call after call: the dK/dV kernel reads both to its end."""
+    rng = np.random.default_rng(91)
+    lens = [int(v) for v in rng.integers(1, 400, 14)]
+    w = W.Workload("in_place", *heads, 1e4, lens, [6, 8], seed=91)
+    c = R.Context.for_workload(w)
+    T = w.n_tokens
+    q, k, v = (R.bits_to_device(x) for x in W.prefill_inputs(w))
+    g = R.bits_to_device(W.normal_bf16(92, (T, heads[0], heads[2])))
+    for mode in (B.BA_MODE_BLOCK, B.BA_MODE_FULL):
+        seg, buf = c.segment(w.block_lens, w.seq_nblocks, mode)
+        o, lse = torch.empty_like(q), torch.empty(T, heads[0], device="cuda")
+        B.ba_block_prefill(c.ctx, q, k, v, o, lse, seg, mode, B.BA_OUT_BF16)
+        want = [torch.empty_like(q), torch.empty_like(k), torch.empty_like(v)]
+        B.ba_block_prefill_bwd(c.ctx, q, k, v, o, lse, g, *want, seg, mode, B.BA_OUT_BF16)
+        for _ in range(4):
+            q2, g2, dk, dv = q.clone(), g.clone(), torch.empty_like(k), torch.empty_like(v)
+            dq = q2 if place == "q" else g2
+            B.ba_block_prefill_bwd(c.ctx, q2, k, v, o, lse, g2, dq, dk, dv, seg, mode, B.BA_OUT_BF16)
+            assert all(torch.equal(a, b) for a, b in zip((dq, dk, dv), want))
+    assert c.device_status() == B.BA_OK
+    c.close()
