@@ -116,7 +116,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
-__device__ __forceinline__ void row_warps_barrier() { __syncwarp(); asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void row_warps_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 __device__ __forceinline__ int upper_bound_dev(const int32_t *a, int n, int x) {
   int lo = 0, hi = n;
@@ -401,14 +401,14 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     };
     if (tid < 128 && n_iter > 0) fetch_stats(0);
     bool ok = true;
-    for (int it = 0; it < n_iter; ++it) {
+    int it = 0;
+    for (; it < n_iter; ++it) {
       float *st = stats + (it & 1) * 3 * 128;
       if (tid < 128) {
         st[tid] = n_lse * -1.4426950408889634f; st[128 + tid] = -n_dls * p.scale; reinterpret_cast<int *>(st)[256 + tid] = n_lim;
         if (it + 1 < n_iter) fetch_stats(it + 1);
       }
-      row_warps_barrier();                               // (which has no limit: a warp that gave up a wait still comes to each)
-      if (!ok) continue;
+      row_warps_barrier();
       int row0, row_end, head0; bool causal;
       iter_rows(it, row0, row_end, causal, head0);
       // every pair of this thread's half visible?  (all 128 keys exist, the rows exist and, in the causal range,
@@ -420,7 +420,7 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       const int *lim = reinterpret_cast<const int *>(st) + 256 + h * 64;
       uint32_t s[64], w[16];
       ok = mbar_wait(&ctrl->s_full, it & 1, abort_flag);
-      if (!ok) continue;
+      if (!ok) break;
       tc_fence_after();
       // P^T as bf16 over the S^T columns the thread has read, two per column: the A operand of dV
       auto form_p = [&](auto masked) {
@@ -440,7 +440,7 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       tc_fence_before();
       mbar_arrive(&ctrl->p_done);
       ok = mbar_wait(&ctrl->dp_full, it & 1, abort_flag);
-      if (!ok) continue;
+      if (!ok) break;
       tc_fence_after();
       uint32_t d0[32], d1[32];
       tmem_ld_32x32b_x32(d, d0);
@@ -455,6 +455,9 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       tc_fence_before();
       mbar_arrive(&ctrl->ds_done);
     }
+    // a warp that gave up a wait still comes to the barriers the others may be on their way to: those have no limit
+    __syncwarp();
+    for (++it; it < n_iter; ++it) row_warps_barrier();
     // accumulators: lane = key row of the tile; one thread of a key writes dV, the other dK
     if (ok && n_iter > 0) ok = mbar_wait(&ctrl->fin, 0, abort_flag);
     if (ok && n_iter > 0) {
