@@ -148,7 +148,7 @@ ba_status ba_create(ba_ctx **out, const ba_config *cfg, int device, size_t works
       (workspace_bytes && cudaMalloc(&ctx->workspace, workspace_bytes) != cudaSuccess) ||
       // launch counters of the attention kernels (below the scratch area): zero once, every launch leaves them zero
       (workspace_bytes >= ba_scratch_offset(ctx) &&
-       cudaMemset((char *)ctx->workspace + ba_scratch_offset(ctx) - 256, 0, 256) != cudaSuccess) ||
+       cudaMemset(ba_counters(ctx), 0, 256) != cudaSuccess) ||
       ba_attend_sm100_setup(ctx) != BA_OK || ba_bwd_sm100_setup(ctx) != BA_OK) {
     cudaGetLastError();
     ba_attend_sm100_teardown(ctx);
@@ -183,7 +183,7 @@ ba_status ba_last_device_status(ba_ctx *ctx) {
     BA_CUDA_TRY(cudaMemset(ctx->dev_status, 0, 4));
     // a launch that gave up may have left its work counters half-way: back to zero for the next one
     if (ctx->workspace && ctx->workspace_bytes >= ba_scratch_offset(ctx))
-      BA_CUDA_TRY(cudaMemset((char *)ctx->workspace + ba_scratch_offset(ctx) - 256, 0, 256));
+      BA_CUDA_TRY(cudaMemset(ba_counters(ctx), 0, 256));
   }
   return (ba_status)h;
 }

@@ -1774,7 +1774,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   // the counters live in the last 256 bytes below the scratch area: zeroed by ba_create, left at zero by every launch
   int32_t *counters = nullptr;
   if (ctx->workspace && ctx->workspace_bytes >= ba_scratch_offset(ctx))
-    counters = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(ctx->workspace) + ba_scratch_offset(ctx) - 256);
+    counters = ba_counters(ctx);
   p.counters = nullptr;
   if (p.persistent && !counters) p.persistent = 0;   // a context without workspace: one CTA per entry, however many
   if (p.persistent) p.counters = counters;

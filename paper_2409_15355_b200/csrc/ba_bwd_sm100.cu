@@ -49,6 +49,8 @@ constexpr int kStep = 64;              // keys a step of the dQ kernel works on
 struct BwdParams {
   const float *lse;          // [T, Hq] natural-log softmax denominators of the forward pass
   const float *delta;        // [T, Hq] dO . O
+  int32_t *started;          // 0 until the dK/dV kernel of this call has seen all that was written before it; then 1 + the query
+                             // tile pairs of the tables, or -1 when they are not valid
   void *dq, *dk, *dv;
   int out_f32;
   int32_t *status;
@@ -125,6 +127,32 @@ __device__ __forceinline__ int upper_bound_dev(const int32_t *a, int n, int x) {
     if (__ldg(a + mid) <= x) lo = mid + 1; else hi = mid;
   }
   return lo;
+}
+// The dQ kernel reads what other kernels wrote behind an acquire, not behind a wait: with ordinary loads, as the read-only path
+// (which the compiler may also take by itself) need not see it.
+template <class T>
+__device__ __forceinline__ T ld_plain(const T *p) {
+  static_assert(sizeof(T) == 4, "one word");
+  uint32_t v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return *reinterpret_cast<T *>(&v);
+}
+__device__ __forceinline__ int upper_bound_plain(const int32_t *a, int n, int x) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    int mid = (lo + hi) >> 1;
+    if (ld_plain(a + mid) <= x) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+// BwdParams::started, once it is not zero; 0 when that takes a second (it is set before the kernel that asks can start).
+__device__ __forceinline__ int32_t wait_started(const int32_t *started) {
+  int32_t v = ld_acquire(started);
+  if (v == 0) {
+    const unsigned long long t0 = global_ns();
+    while ((v = ld_acquire(started)) == 0 && global_ns() - t0 <= kWaitLimitNs) __nanosleep(kSleepNs);
+  }
+  return v;
 }
 
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
@@ -254,6 +282,10 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
   const int tid = threadIdx.x, warp = tid >> 5;
   const ba_segments &sg = p.seg;
   ba_pdl_wait();
+  if (blockIdx.x == gridDim.x - 1) {                       // a CTA without keys: off the way of those the dQ kernel waits for
+    if (tid == 0 && blockIdx.y == 0) st_release(p.started, __ldg(sg.totals + 7) == BA_TABLES_VALID ? __ldg(sg.totals + 2) + 1 : -1);
+    return;
+  }
   if (__ldg(sg.totals + 7) != BA_TABLES_VALID) return;
 
   // which keys: tile `kt` of the batch (a tile never spans two blocks), KV head `g`
@@ -488,22 +520,28 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
   DqCtrl *ctrl = reinterpret_cast<DqCtrl *>(smem + L::kCtrl);
   const int tid = threadIdx.x, warp = tid >> 5;
   const ba_segments &sg = p.seg;
-  // This kernel needs dO . O, which was complete before the dK/dV kernel triggered, and nothing of the dK/dV kernel itself:
-  // it starts on the SMs that one leaves (unless dq takes the place of an input) and waits for it only before it ends.
+  // This kernel needs nothing of the dK/dV kernel but what that one had to wait for itself (dO . O, the tables, the inputs): it
+  // starts on the SMs that one leaves (unless dq takes the place of an input) and waits for it only before it ends.  Until then
+  // nothing makes the earlier kernels' writes visible here but the word that the dK/dV kernel released after its own wait, so
+  // every thread acquires it first (the copy engine's reads: behind a proxy fence).
   struct WaitAtExit { __device__ ~WaitAtExit() { ba_pdl_wait(); } } wait_at_exit;
-  if (__ldg(sg.totals + 7) != BA_TABLES_VALID) return;
+  const int32_t n_pairs_1 = wait_started(p.started);
+  if (!__syncthreads_and(n_pairs_1 != 0)) {
+    if (tid == 0) ba_record_status(p.status, BA_ERR_TIMEOUT);
+    return;
+  }
 
   // query tile: one half of a query-tile pair of the forward kernel.  Tiles are taken from the end of the list (within a
   // sequence the last ones see the most keys), all head chunks of a tile side by side.
   const int qt = n_tiles_upper - 1 - (int)blockIdx.x / n_head_chunks;
   const int pair = qt >> 1, half = qt & 1;
-  if (pair >= __ldg(sg.totals + 2)) return;
-  const int b = upper_bound_dev(sg.cu_qtile, sg.n_blocks + 1, pair) - 1;
-  const int blk0 = __ldg(sg.cu_block + b), blk1 = __ldg(sg.cu_block + b + 1);
-  const int q0 = blk0 + (pair - __ldg(sg.cu_qtile + b)) * 2 * p.tok + half * p.tok;
+  if (pair + 1 >= n_pairs_1) return;                      // (no tables, or no such pair)
+  const int b = upper_bound_plain(sg.cu_qtile, sg.n_blocks + 1, pair) - 1;
+  const int blk0 = ld_plain(sg.cu_block + b), blk1 = ld_plain(sg.cu_block + b + 1);
+  const int q0 = blk0 + (pair - ld_plain(sg.cu_qtile + b)) * 2 * p.tok + half * p.tok;
   if (q0 >= blk1) return;
   const int q_end = min(q0 + p.tok, blk1);                // rows q0 .. q_end - 1
-  const int kv0 = __ldg(sg.block_kv_begin + b);           // row i sees keys kv0 .. i
+  const int kv0 = ld_plain(sg.block_kv_begin + b);           // row i sees keys kv0 .. i
   const int head0 = ((int)blockIdx.x % n_head_chunks) * p.hpt, g = head0 / p.G;
   const int n_steps = (q_end - kv0 + kStep - 1) / kStep;  // step i: keys kv0 + 64 i .. + 63
 
@@ -526,6 +564,7 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
 
   if (warp == kDqLoadWarp) {
     if (elect_one()) {
+      fence_proxy_async_global();
       mbar_arrive_expect_tx(&ctrl->fix_full, 2 * L::kTileBytes);
       for (int c = 0; c < L::kChunks; ++c) {
         tma_load_3d(smem + L::kQ + c * L::kRegion, &tmap_q, &ctrl->fix_full, c * 64, head0, q0);
@@ -618,8 +657,8 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     const bool row_ok = tok_i < q_end;
     float nlse = 0.f, ndl = 0.f;
     if (row_ok) {
-      nlse = __ldg(p.lse + (size_t)tok_i * p.Hq + head) * -1.4426950408889634f;
-      ndl = -__ldg(p.delta + (size_t)tok_i * p.Hq + head) * p.scale;
+      nlse = ld_plain(p.lse + (size_t)tok_i * p.Hq + head) * -1.4426950408889634f;
+      ndl = -ld_plain(p.delta + (size_t)tok_i * p.Hq + head) * p.scale;
     }
     bool ok = true;
     for (int i = 0; i < n_steps; ++i) {
@@ -668,9 +707,10 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
 template <int D>
 __global__ void __launch_bounds__(256)
 ba_bwd_delta_kernel(const __nv_bfloat16 *__restrict__ o, const __nv_bfloat16 *__restrict__ d_o, float *__restrict__ delta,
-                    int n_rows_heads) {
+                    int n_rows_heads, int32_t *started) {
   ba_pdl_wait();
   ba_pdl_trigger();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *started = 0;
   constexpr int kLanes = D / 8;                          // 8 or 16 threads per row
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long rh = t / kLanes;
@@ -725,7 +765,7 @@ template <int D>
 ba_status launch_bwd(ba_ctx *ctx, const BwdParams &p, bool dq_in_place, const CUtensorMap &tq, const CUtensorMap &tdo, const CUtensorMap &tk,
                      const CUtensorMap &tv, const CUtensorMap &tk64, const CUtensorMap &tv64, int n_ktiles_upper, int n_pairs_upper,
                      cudaStream_t stream) {
-  BA_CUDA_TRY(ba_launch(ba_bwd_dkv_kernel<D>, dim3((unsigned)n_ktiles_upper, (unsigned)p.Hkv), kDkvThreads, DkvLayout<D>::kBytes + 1024,
+  BA_CUDA_TRY(ba_launch(ba_bwd_dkv_kernel<D>, dim3((unsigned)n_ktiles_upper + 1, (unsigned)p.Hkv), kDkvThreads, DkvLayout<D>::kBytes + 1024,
                         stream, true, tq, tdo, tk, tv, p));
   const int n_head_chunks = p.Hq / p.hpt;
   BA_CUDA_TRY(ba_launch(ba_bwd_dq_kernel<D>, dim3((unsigned)(2 * n_pairs_upper) * n_head_chunks), kDqThreads, DqLayout<D>::kBytes, stream,
@@ -765,10 +805,11 @@ ba_status ba_bwd_sm100_launch(ba_ctx *ctx, const void *q, const void *k, const v
   if (!ctx->workspace || ctx->workspace_bytes < ba_scratch_offset(ctx) + need) return BA_ERR_WORKSPACE;
   float *delta = reinterpret_cast<float *>(reinterpret_cast<char *>(ctx->workspace) + ba_scratch_offset(ctx));
   p.delta = delta;
+  p.started = ba_backward_flag(ctx);
   const int n_rh = T * Hq;
   const long long threads = (long long)n_rh * (D / 8);
   BA_CUDA_TRY(ba_launch(D == 128 ? ba_bwd_delta_kernel<128> : ba_bwd_delta_kernel<64>, dim3((unsigned)((threads + 255) / 256)), 256, 0,
-                        stream, true, (const __nv_bfloat16 *)o, (const __nv_bfloat16 *)d_o, delta, n_rh));
+                        stream, true, (const __nv_bfloat16 *)o, (const __nv_bfloat16 *)d_o, delta, n_rh, p.started));
   ctx->launches += 1;
   CUtensorMap tq, tdo, tk, tv, tk64, tv64;
   if (!bwd_make_map(&tq, q, D, Hq, T, p.hpt, p.tok) || !bwd_make_map(&tdo, d_o, D, Hq, T, p.hpt, p.tok) ||

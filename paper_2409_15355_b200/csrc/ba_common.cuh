@@ -131,6 +131,10 @@ static inline size_t ba_align_up(size_t x, size_t a) { return (x + a - 1) / a * 
 // of the workspace, the angle table (re-encode).  Calls on one context are stream-ordered,
 // so the regions may be reused from call to call.
 static inline size_t ba_scratch_offset(const ba_ctx *) { return 64 * 1024; }
+// The last 256 bytes below the scratch area: three words of launch counters (attention) and, 128 bytes on, a word of the
+// backward pass.
+static inline int32_t *ba_counters(const ba_ctx *ctx) { return (int32_t *)((char *)ctx->workspace + ba_scratch_offset(ctx) - 256); }
+static inline int32_t *ba_backward_flag(const ba_ctx *ctx) { return ba_counters(ctx) + 32; }
 
 // How ba_final_attend divides the key tiles of its work items among CTAs (pure host arithmetic, also reachable
 // through ba_plan_final_attend).  Inputs: SMs; work items (query tile pairs x head chunks); pairs and head chunks;
