@@ -116,9 +116,10 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
             raise RuntimeError(f"{name}: prototype not declared")
         if name not in ("ba_status_string", "ba_launch_count"):
             getattr(lib, name).restype = C.c_int
-    _marshal = _load_marshal()
-    _marshal.bind(lib._handle)
+    marshal = _load_marshal()
+    marshal.bind(lib._handle, _through_ctypes, vp, ba_segments, ba_page_table)
     _lib = lib
+    _marshal = marshal
     return lib
 
 
@@ -129,6 +130,15 @@ def _load_marshal():
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
     return mod
+
+
+def _through_ctypes(name, *args):
+    """A hot call whose arguments the extension does not take: through ctypes, like every other function of the library."""
+    fn = getattr(load_library(), name)
+    given = [args[0]]
+    for a, t in zip(args[1:], fn.argtypes[1:]):
+        given.append(_ptr(a) if t is C.c_void_p else C.byref(a) if issubclass(t, C._Pointer) else a)
+    return fn(*given)
 
 
 def _calls():
