@@ -10,6 +10,7 @@ import os
 import subprocess
 import sys
 import sysconfig
+import threading
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -40,6 +41,24 @@ def _digest() -> str:
     return h.hexdigest()
 
 
+def _compile(cmd, out: str, digest: str, failed: str) -> str:
+    """Runs the compiler with `out` as its output, whole: a process that loads `out` meanwhile, or builds it as well, finds the old
+    file or the new one.  Returns the compiler's messages."""
+    own = f"{out}.{os.getpid()}.{threading.get_ident()}"
+    try:
+        res = subprocess.run(cmd + ["-o", own], capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError(failed + res.stdout + res.stderr)
+        os.replace(own, out)
+        with open(own, "w") as fh:
+            fh.write(digest)
+        os.replace(own, out + ".hash")
+    finally:
+        if os.path.exists(own):
+            os.remove(own)
+    return res.stderr
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile csrc/*.cu into libba.so (if needed) and return its path."""
     digest = _digest()
@@ -48,34 +67,27 @@ def build(force: bool = False, verbose: bool = False) -> str:
             if fh.read().strip() == digest:
                 return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
-    cmd = [nvcc] + NVCC_FLAGS + ["-I", INCLUDE, "-I", CSRC] + _sources() + ["-o", LIB]
+    cmd = [nvcc] + NVCC_FLAGS + ["-I", INCLUDE, "-I", CSRC] + _sources()
     if verbose:
         cmd.insert(1, "-Xptxas=-v")
         print(" ".join(cmd), file=sys.stderr)
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+    messages = _compile(cmd, LIB, digest, "nvcc failed:\n")
     if verbose:
-        print(res.stderr, file=sys.stderr)
-    with open(STAMP, "w") as fh:
-        fh.write(digest)
+        print(messages, file=sys.stderr)
     return LIB
 
 
 def build_marshal(force: bool = False) -> str:
     """Compile csrc/ba_marshal.c into ba_marshal.so (if needed) and return its path."""
     out, src, header = os.path.join(HERE, "ba_marshal.so"), os.path.join(CSRC, "ba_marshal.c"), os.path.join(INCLUDE, "ba.h")
-    cmd = [os.environ.get("CC", "gcc"), "-O2", "-fPIC", "-shared", "-Wall", "-Werror",
-           "-I", sysconfig.get_paths()["include"], "-I", INCLUDE, src, "-o", out]
-    digest = hashlib.sha256(" ".join(cmd + [sys.version]).encode() + open(src, "rb").read() + open(header, "rb").read()).hexdigest()
+    flags = ["-O2", "-fPIC", "-shared", "-Wall", "-Werror"]
+    # (what goes into it, not where it lies: a tree that was copied elsewhere keeps its build)
+    digest = hashlib.sha256(" ".join(flags + [sys.version]).encode() + open(src, "rb").read() + open(header, "rb").read()).hexdigest()
     stamp = out + ".hash"
     if not force and os.path.exists(out) and os.path.exists(stamp) and open(stamp).read().strip() == digest:
         return out
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("the argument marshalling extension failed to build:\n" + res.stdout + res.stderr)
-    with open(stamp, "w") as fh:
-        fh.write(digest)
+    _compile([os.environ.get("CC", "gcc")] + flags + ["-I", sysconfig.get_paths()["include"], "-I", INCLUDE, src], out, digest,
+             "the argument marshalling extension failed to build:\n")
     return out
 
 
