@@ -9,7 +9,9 @@ when no sm_100 device is present.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
+import warnings
 from typing import Optional
 
 from . import build as _build
@@ -117,19 +119,27 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
         if name not in ("ba_status_string", "ba_launch_count"):
             getattr(lib, name).restype = C.c_int
     marshal = _load_marshal()
-    marshal.bind(lib._handle, _through_ctypes, vp, ba_segments, ba_page_table)
+    if marshal is not None:
+        marshal.bind(lib._handle, _through_ctypes, vp, ba_segments, ba_page_table)
+    else:
+        marshal = _CtypesCalls()
     _lib = lib
     _marshal = marshal
     return lib
 
 
 def _load_marshal():
-    """The extension that marshals the arguments of the hot calls (csrc/ba_marshal.c)."""
+    """The extension that marshals the arguments of the hot calls (csrc/ba_marshal.c).  None where there is no build of it and no
+    compiler, Python headers or room to make one: the library itself needs none of these."""
     import importlib.util
-    spec = importlib.util.spec_from_file_location("ba_marshal", _build.build_marshal())
-    mod = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(mod)
-    return mod
+    try:
+        spec = importlib.util.spec_from_file_location("ba_marshal", _build.build_marshal())
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        return mod
+    except (OSError, RuntimeError, ImportError) as e:
+        warnings.warn("calls go through ctypes, 2-3 us each: " + str(e).strip().split("\n")[0], RuntimeWarning, stacklevel=3)
+        return None
 
 
 def _through_ctypes(name, *args):
@@ -139,6 +149,13 @@ def _through_ctypes(name, *args):
     for a, t in zip(args[1:], fn.argtypes[1:]):
         given.append(_ptr(a) if t is C.c_void_p else C.byref(a) if issubclass(t, C._Pointer) else a)
     return fn(*given)
+
+
+class _CtypesCalls:
+    """The extension's functions without it."""
+
+    def __getattr__(self, name):
+        return functools.partial(_through_ctypes, "ba_" + name)
 
 
 def _calls():

@@ -56,3 +56,26 @@ def test_a_copied_tree_keeps_its_builds(tmp_path):
     got = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, env=env, capture_output=True, text=True)
     assert got.returncode == 0, got.stderr
     assert got.stdout.split() == [str(tmp_path / "paper_2409_15355_b200" / n) for n in ("libba.so", "ba_marshal.so")]
+
+
+@pytest.mark.parametrize("found", ["no_build", "stale_build"])
+def test_a_prebuilt_library_loads_without_a_compiler(tmp_path, found):
+    """BA_LIBRARY names a library to use as it is: neither a compiler nor a writable folder is needed beside it."""
+    lib = b.build()
+    for d in ("paper_2409_15355_b200", "include"):
+        shutil.copytree(os.path.join(ROOT, d), tmp_path / d, ignore=shutil.ignore_patterns("*.so", "*.hash", "__pycache__"))
+    if found == "stale_build":
+        (tmp_path / "paper_2409_15355_b200" / "ba_marshal.so").write_text("of other sources")
+        (tmp_path / "paper_2409_15355_b200" / "ba_marshal.so.hash").write_text("of other sources")
+    code = ("import types, warnings\nfrom paper_2409_15355_b200 import binding as B\n"
+            "with warnings.catch_warnings(record=True) as w:\n    warnings.simplefilter('always')\n    B.load_library()\n"
+            "assert len(w) == 1 and issubclass(w[0].category, RuntimeWarning), w\n"
+            "s = types.SimpleNamespace(cuda_stream=0)\n"
+            "try:\n    B.ba_block_prefill(None, None, None, None, None, None, B.ba_segments(), 0, 0, s)\n"
+            "except B.BaError as e:\n    assert e.status == B.BA_ERR_INVALID_ARG\n"
+            "else:\n    raise SystemExit('no error')\n"
+            "try:\n    B.ba_block_prefill(None, None, None, None, None, None, None, 0, 0, s)\n"
+            "except TypeError:\n    print('loaded')\n")
+    env = dict(os.environ, NVCC="/nonexistent/nvcc", CC="/nonexistent/cc", PYTHONPATH=str(tmp_path), BA_LIBRARY=lib)
+    got = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, env=env, capture_output=True, text=True)
+    assert got.returncode == 0 and got.stdout.strip() == "loaded", got.stderr
