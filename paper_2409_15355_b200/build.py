@@ -82,10 +82,15 @@ def build_marshal(force: bool = False) -> str:
     out, src, header = os.path.join(HERE, "ba_marshal.so"), os.path.join(CSRC, "ba_marshal.c"), os.path.join(INCLUDE, "ba.h")
     flags = ["-O2", "-fPIC", "-shared", "-Wall", "-Werror"]
     # (what goes into it, not where it lies: a tree that was copied elsewhere keeps its build)
-    digest = hashlib.sha256(" ".join(flags + [sys.version]).encode() + open(src, "rb").read() + open(header, "rb").read()).hexdigest()
-    stamp = out + ".hash"
-    if not force and os.path.exists(out) and os.path.exists(stamp) and open(stamp).read().strip() == digest:
-        return out
+    h = hashlib.sha256(" ".join(flags + [sys.version]).encode())
+    for f in (src, header):
+        with open(f, "rb") as fh:
+            h.update(fh.read())
+    digest = h.hexdigest()
+    if not force and os.path.exists(out) and os.path.exists(out + ".hash"):
+        with open(out + ".hash") as fh:
+            if fh.read().strip() == digest:
+                return out
     _compile([os.environ.get("CC", "gcc")] + flags + ["-I", sysconfig.get_paths()["include"], "-I", INCLUDE, src], out, digest,
              "the argument marshalling extension failed to build:\n")
     return out

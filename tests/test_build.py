@@ -69,7 +69,7 @@ def test_a_prebuilt_library_loads_without_a_compiler(tmp_path, found):
         (tmp_path / "paper_2409_15355_b200" / "ba_marshal.so.hash").write_text("of other sources")
     code = ("import types, warnings\nfrom paper_2409_15355_b200 import binding as B\n"
             "with warnings.catch_warnings(record=True) as w:\n    warnings.simplefilter('always')\n    B.load_library()\n"
-            "assert len(w) == 1 and issubclass(w[0].category, RuntimeWarning), w\n"
+            "assert [x.category for x in w if x.category is not ResourceWarning] == [RuntimeWarning], [str(x) for x in w]\n"
             "s = types.SimpleNamespace(cuda_stream=0)\n"
             "try:\n    B.ba_block_prefill(None, None, None, None, None, None, B.ba_segments(), 0, 0, s)\n"
             "except B.BaError as e:\n    assert e.status == B.BA_ERR_INVALID_ARG\n"
