@@ -11,6 +11,7 @@ from __future__ import annotations
 import ctypes as C
 import functools
 import os
+import threading
 import warnings
 from typing import Optional
 
@@ -69,7 +70,8 @@ class BaError(RuntimeError):
 
 _lib = None
 _marshal = None
-_raw_stream = _raw_device = None
+_loading = threading.RLock()
+_raw = None
 
 
 def load_library(path: Optional[str] = None) -> C.CDLL:
@@ -77,6 +79,15 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     global _lib, _marshal
     if _lib is not None and path is None:
         return _lib
+    with _loading:
+        if _lib is None or path is not None:
+            lib, _marshal = _open_library(path)
+            _lib = lib                                     # last: with it, other threads go ahead
+        return _lib
+
+
+def _open_library(path: Optional[str]):
+    """The library with its prototypes declared, and the extension bound to it."""
     if path is None:
         path = os.environ.get("BA_LIBRARY") or _build.build()   # BA_LIBRARY: use this prebuilt library as it is
     if not os.path.exists(path):
@@ -123,9 +134,7 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
         marshal.bind(lib._handle, _through_ctypes, vp, ba_segments, ba_page_table)
     else:
         marshal = _CtypesCalls()
-    _lib = lib
-    _marshal = marshal
-    return lib
+    return lib, marshal
 
 
 def _load_marshal():
@@ -198,12 +207,13 @@ def _stream_ptr(stream) -> Optional[int]:
 def _current_raw_stream() -> Optional[int]:
     """Handle of torch's current stream.  torch.cuda.current_stream() builds a stream object, 3.4 us a call; the raw query
     takes 0.1 us."""
-    global _raw_stream, _raw_device
-    if _raw_stream is None:
+    global _raw
+    if _raw is None:
         import torch
         torch.cuda.current_stream()                        # initialises CUDA in torch
-        _raw_stream, _raw_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-    return _raw_stream(_raw_device()) or None
+        _raw = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    stream_of, device = _raw
+    return stream_of(device()) or None
 
 
 # ---------------------------------------------------------------------------

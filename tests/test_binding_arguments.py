@@ -2,6 +2,7 @@
 refused.  No device is needed: a stand-in library records what it is given."""
 import ctypes as C
 import subprocess
+import threading
 import types
 
 import numpy as np
@@ -125,3 +126,22 @@ def test_calls_without_a_context_reach_the_library(name, number):
     with pytest.raises(B.BaError) as e:
         _calls(B.ba_segments(), B.ba_page_table(page_rows=16), lambda: np.zeros(8, dtype=np.int32), lambda: number)[name]()
     assert e.value.status in (B.BA_ERR_INVALID_ARG, B.BA_ERR_UNSUPPORTED)
+
+
+def test_no_thread_sees_the_extension_before_it_is_bound(monkeypatch):
+    """A second thread's first call while one loads the library: it waits for what is complete."""
+    seen, bound = [], []
+
+    class Extension:
+        def bind(self, *args):
+            other = threading.Thread(target=lambda: seen.append((B._calls(), list(bound))))
+            other.start()
+            other.join(0.3)
+            bound.append(1)
+            self.other = other
+    e = Extension()
+    for name, value in (("_lib", None), ("_marshal", None), ("_load_marshal", lambda: e)):
+        monkeypatch.setattr(B, name, value)
+    B.load_library()
+    e.other.join()
+    assert seen == [(e, [1])]
