@@ -598,8 +598,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   int n_items = 0;
   WorkEntry first = {-1, 0, 0, 0, -1, 0};
   if (warp == 8) {
+    const bool fit = kVariant != kPlain || partials_fit(p.seg.totals, p.final_only, p.n_splits, p.n_part_rows);
     n_items = count_items(p);
-    if (kVariant == kPlain && n_items > 0 && !partials_fit(p.seg.totals, p.final_only, p.n_splits, p.n_part_rows)) {
+    if (!fit && n_items > 0) {
       ba_record_status(p.status, BA_ERR_SHAPE);            // the tables describe another launch than the host sized
       n_items = 0;
     }
@@ -1449,10 +1450,9 @@ ba_combine_splits_kernel(const CombineParams p) {
   constexpr int kVec = D / 4, kBatch = kMax < 8 ? kMax : 8;
   ba_pdl_wait();
   ba_pdl_trigger();
-  const int n_final = __ldg(p.totals + 3);
-  if (__ldg(p.totals + 7) != BA_TABLES_VALID || (int)blockIdx.y >= n_final ||
-      !partials_fit(p.totals, p.final_only, p.n_splits, p.n_part_rows))
-    return;                                                // (nothing was attended either)
+  const int n_final = __ldg(p.totals + 3), valid = __ldg(p.totals + 7);
+  const bool fit = partials_fit(p.totals, p.final_only, p.n_splits, p.n_part_rows);
+  if (valid != BA_TABLES_VALID || (int)blockIdx.y >= n_final || !fit) return;    // (not valid, no room: nothing was attended either)
   const int32_t *line = p.items + 8 * ((p.final_only ? 0 : __ldg(p.totals + 2) - n_final) + blockIdx.y);
   const int q_row0 = __ldg(line), q_rows = min(__ldg(line + 1), p.n_q_rows - q_row0);
   const int part0 = p.final_only ? q_row0 : __ldg(line + 5), head0 = (blockIdx.x >> p.parts_log2) * p.hpt;
