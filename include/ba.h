@@ -168,10 +168,14 @@ int64_t ba_launch_count(const ba_ctx *ctx);
 
 /* Diagnostic: how the last attention launch through `ctx` was laid out.  out[0] = CTAs, out[1] = partial
  * results per row that a second kernel merges (1: none), out[2] = CTAs that each took the tail of one work
- * item in a balanced launch (0: not balanced), out[3] = key tiles of such a tail. */
+ * item in a balanced launch (0: not balanced), out[3] = key tiles of such a tail.  The other layouts are told by the
+ * counts alone: equal splits (CTAs = items x partial results, or one per SM), a stream launch (at most one CTA per SM,
+ * more than one partial result), a cluster launch (items x 2 .. 8 CTAs, or twice that, one result per row). */
 ba_status ba_last_attend_shape(const ba_ctx *ctx, int32_t out[4]);
 
-/* Diagnostic, no device needed: the planning step of ba_final_attend as a function of its inputs.  n_sms SMs,
+/* Diagnostic, no device needed: the first planning step of ba_final_attend, which weighs equal splits against a
+ * balanced launch, as a function of its inputs.  (Where it does not choose a balanced launch, ba_final_attend goes on to weigh
+ * its equal splits against a stream and a cluster launch, whose plans this call does not give.)  n_sms SMs,
  * n_pairs work items per head chunk (ba_segments.n_final_items), n_head_chunks head chunks, avg_key_tiles 128-key
  * tiles of an average item, key_tiles = {sum, minimum, maximum} of the key tiles over the n_pairs items (zeros:
  * unknown), max_partials = the most partial results per row the workspace has room for.  out[0] = partial results
@@ -193,7 +197,8 @@ ba_status ba_segments_bytes(int32_t batch, int32_t n_blocks, int32_t n_tokens, s
  *   table_buf               device buffer of at least ba_segments_bytes() bytes, 16-byte aligned
  *   out                     host struct, filled with pointers into table_buf
  * With host arrays the lengths are checked before launching (BA_ERR_INVALID_ARG
- * for a length < 1 or sums that do not match); with device arrays the same
+ * for a length < 1 or sums that do not match) and, up to 960 values of both together, taken with the
+ * call (a captured launch keeps them); longer ones are copied on `stream`.  With device arrays the same
  * check runs on the device and is reported by ba_last_device_status().
  */
 ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_nblocks,
@@ -315,17 +320,19 @@ ba_status ba_final_attend(ba_ctx *ctx, const void *q_f, const void *k_f, const v
                           ba_out_dtype out_dtype, void *stream);
 
 /*
- * Section 2.5, steps 2 and 3 in one launch: the final block of every sequence attends that
+ * Section 2.5, steps 2 and 3 in one call: the final block of every sequence attends that
  * sequence's cached blocks and itself, with the cached keys still at their CACHE-TIME positions
- * (token t of a block rotated to position t, as Section 2.3 stores them).  The position
- * re-encoding of Eq. 3 after Eq. 2 -- one rotation by the block's delta -- is applied to the
- * other side of the dot product: (R(p) q) . (R(delta + t) k) = (R(-delta) R(p) q) . (R(t) k),
- * so the query tiles are rotated once per cached block on chip and the cached keys are neither
- * rewritten nor read twice.  The result equals ba_reencode_k followed by ba_final_attend up to
- * the rounding of the rotated operand to bf16 (queries here, keys there).  The re-encoded keys
- * themselves -- what the rest of generation reads -- are written as well when k_out is given, bit-identical to
- * ba_reencode_k's output.  Where the two steps are quicker (k_out given, final blocks of several query tiles, small caches) the
- * call takes them one after the other, the keys going to k_out or the workspace.
+ * (token t of a block rotated to position t, as Section 2.3 stores them).  The call takes one of two ways:
+ *  - The position re-encoding of Eq. 3 after Eq. 2 -- one rotation by the block's delta -- is applied to the
+ *    other side of the dot product: (R(p) q) . (R(delta + t) k) = (R(-delta) R(p) q) . (R(t) k),
+ *    so the query tiles are rotated once per cached block on chip and the cached keys are neither
+ *    rewritten nor read twice.  This way without k_out where final blocks are short and the cache is large, where the
+ *    workspace has no room for the keys, and where ba_reencode_k does not take their rows.
+ *  - Otherwise the keys are re-encoded into k_out or the workspace and attended from there: quicker with
+ *    k_out, with final blocks of several query tiles, and over small caches.
+ * The result equals ba_reencode_k followed by ba_final_attend up to the rounding of the rotated operand to bf16
+ * (queries the first way, keys the second).  The re-encoded keys themselves -- what the rest of generation reads --
+ * are written when k_out is given, bit-identical to ba_reencode_k's output.
  *   q_f, k_f, v_f   as for ba_final_attend
  *   k_src, v_src    bf16 [n_src_rows, n_kv_heads, head_dim]: cached block c (cache order, as in
  *                   seg->cache_cu) occupies rows src_off[c] .. src_off[c] + length - 1 of both, or

@@ -245,7 +245,8 @@ def ba_launch_count(ctx) -> int:
 
 
 def ba_last_attend_shape(ctx) -> dict:
-    """Layout of the last attention launch: CTAs, partial results per row, balanced tails and their key tiles."""
+    """Layout of the last attention launch: CTAs, partial results per row, balanced tails and their key tiles (ba.h: how the
+    other layouts show in the counts)."""
     out = (C.c_int32 * 4)()
     _check(load_library().ba_last_attend_shape(ctx, C.byref(out)), "ba_last_attend_shape")
     return {"ctas": out[0], "partials": out[1], "balanced_tails": out[2], "tail_tiles": out[3]}
@@ -253,7 +254,7 @@ def ba_last_attend_shape(ctx) -> dict:
 
 def ba_plan_final_attend(n_sms: int, n_pairs: int, n_head_chunks: int, avg_key_tiles: int, key_tiles,
                          max_partials: int) -> dict:
-    """The planning step of ba_final_attend (host arithmetic only)."""
+    """The first planning step of ba_final_attend, equal splits against a balanced launch (host arithmetic only)."""
     kt = (C.c_int32 * 3)(*[int(v) for v in key_tiles])
     out = (C.c_int32 * 3)()
     _check(load_library().ba_plan_final_attend(n_sms, n_pairs, n_head_chunks, avg_key_tiles, C.byref(kt), max_partials,
