@@ -137,14 +137,6 @@ __device__ __forceinline__ T ld_plain(const T *p) {
   asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return *reinterpret_cast<T *>(&v);
 }
-__device__ __forceinline__ int upper_bound_plain(const int32_t *a, int n, int x) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (ld_plain(a + mid) <= x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
 // BwdParams::started, once it is not zero; 0 when that takes a second (it is set before the kernel that asks can start).
 __device__ __forceinline__ int32_t wait_started(const int32_t *started) {
   int32_t v = ld_acquire(started);
@@ -526,22 +518,19 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
   // every thread acquires it first (the copy engine's reads: behind a proxy fence).
   struct WaitAtExit { __device__ ~WaitAtExit() { ba_pdl_wait(); } } wait_at_exit;
   const int32_t n_pairs_1 = wait_started(p.started);
-  if (!__syncthreads_and(n_pairs_1 != 0)) {
-    if (tid == 0) ba_record_status(p.status, BA_ERR_TIMEOUT);
-    return;
-  }
+  if (n_pairs_1 == 0) ba_record_status(p.status, BA_ERR_TIMEOUT);
 
-  // query tile: one half of a query-tile pair of the forward kernel.  Tiles are taken from the end of the list (within a
-  // sequence the last ones see the most keys), all head chunks of a tile side by side.
+  // query tile: one half of a query-tile pair of the forward kernel, an item of ba_segment's list (one line of it: behind the
+  // acquire nothing is in L1).  Tiles are taken from the end of the list (final blocks, then within a sequence the last ones: those
+  // see the most keys), all head chunks of a tile side by side.
   const int qt = n_tiles_upper - 1 - (int)blockIdx.x / n_head_chunks;
   const int pair = qt >> 1, half = qt & 1;
   if (pair + 1 >= n_pairs_1) return;                      // (no tables, or no such pair)
-  const int b = upper_bound_plain(sg.cu_qtile, sg.n_blocks + 1, pair) - 1;
-  const int blk0 = ld_plain(sg.cu_block + b), blk1 = ld_plain(sg.cu_block + b + 1);
-  const int q0 = blk0 + (pair - ld_plain(sg.cu_qtile + b)) * 2 * p.tok + half * p.tok;
-  if (q0 >= blk1) return;
-  const int q_end = min(q0 + p.tok, blk1);                // rows q0 .. q_end - 1
-  const int kv0 = ld_plain(sg.block_kv_begin + b);           // row i sees keys kv0 .. i
+  const int32_t *item = sg.prompt_items + 8 * (size_t)pair;
+  const int row0 = ld_plain(item), n_rows = ld_plain(item + 1), kv0 = ld_plain(item + 2);   // row i sees keys kv0 .. i
+  const int q0 = row0 + half * p.tok;
+  if (q0 >= row0 + n_rows) return;
+  const int q_end = min(q0 + p.tok, row0 + n_rows);       // rows q0 .. q_end - 1
   const int head0 = ((int)blockIdx.x % n_head_chunks) * p.hpt, g = head0 / p.G;
   const int n_steps = (q_end - kv0 + kStep - 1) / kStep;  // step i: keys kv0 + 64 i .. + 63
 
@@ -799,7 +788,7 @@ ba_status ba_bwd_sm100_launch(ba_ctx *ctx, const void *q, const void *k, const v
   p.scale = ctx->scale;
   p.scale_log2 = ctx->scale * 1.4426950408889634f;
   p.mode = mode; p.n_rows = T; p.seg = *seg;
-  if (seg->q_tile_tokens != 2 * p.tok || !seg->cu_ktile) return BA_ERR_INVALID_ARG;
+  if (seg->q_tile_tokens != 2 * p.tok || !seg->cu_ktile || !seg->prompt_items) return BA_ERR_INVALID_ARG;
   // delta = dO . O sits in the scratch area of the workspace
   const size_t need = (size_t)T * Hq * sizeof(float);
   if (!ctx->workspace || ctx->workspace_bytes < ba_scratch_offset(ctx) + need) return BA_ERR_WORKSPACE;

@@ -93,7 +93,9 @@ __device__ __forceinline__ long long ba_job_source_row(const ba_reencode_job &jo
 }
 
 __device__ __forceinline__ bool ba_job_tables_hold(const ba_reencode_job &job) {
-  return !job.totals || (__ldg(job.totals + 7) == BA_TABLES_VALID && (job.stamp == 0 || __ldg(job.totals + 6) == job.stamp));
+  if (!job.totals) return true;
+  const int2 w = __ldg(reinterpret_cast<const int2 *>(job.totals + 6));    // stamp, validity (the totals are 16-byte aligned)
+  return w.y == BA_TABLES_VALID && (job.stamp == 0 || w.x == job.stamp);
 }
 
 // Context: configuration, workspace and the device status word.
