@@ -22,7 +22,8 @@
 // prompts: 91 -> 66 us).  Kernels launched with ba_launch may be scheduled as soon as every CTA of the kernel
 // before them in the stream has said ba_pdl_trigger() or exited: their set-up runs beside that kernel's tail.
 //  * ba_pdl_wait() returns when the kernel before has completed and its writes are visible; every thread calls it before it
-//    touches global memory, on every path to an exit, so that a kernel's completion implies that of all before it.
+//    touches global memory, on every path to an exit, so that a kernel's completion implies that of all before it.  (The dQ
+//    kernel of the backward pass reads beside its predecessor: it acquires a word that one released, and waits at its exit.)
 //  * A kernel that allocates tensor memory triggers after its allocation: a CTA of the next kernel on the same SM must
 //    never hold columns that a CTA of this one still waits for.
 // A kernel launched in the ordinary way, before or after, behaves as usual.

@@ -111,8 +111,9 @@ ba_reencode_job ba_make_reencode_job(const ba_ctx *ctx, const void *k_src, const
 
 ba_status ba_reencode_main_launch(ba_ctx *ctx, const ba_reencode_job &job, cudaStream_t stream) {
   // Two rows in flight per thread and four per CTA: one in flight leaves the memory system short of requests (32000 rows of
-  // 2 KB 27.0 us = 4.9 TB/s, 23.9 us = 5.5 TB/s with two; 87000 gathered rows 71 -> 65.5 us), more rows per CTA make its life
-  // longer than a small job can afford (2400 rows: 5.1 us, 7.6 us with eight).
+  // 2 KB, back to back: 27.0 us = 4.9 TB/s, 23.9 us = 5.5 TB/s with two; 87000 gathered rows 71 -> 65.5 us; one call between two
+  // attention launches takes 25-27 us), more rows per CTA make its life longer than a small job can afford (2400 rows: 5.1 us,
+  // 7.6 us with eight).
   constexpr int kRows = 2;
   const bool adjacent = job.layout == BA_ROPE_ADJACENT;
   const int units = ba_reencode_units(job.layout, job.row_vecs);
