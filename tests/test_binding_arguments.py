@@ -1,6 +1,7 @@
 """The calls that a layer makes go through a small extension: it passes what ctypes would pass, and what ctypes refuses stays
 refused.  No device is needed: a stand-in library records what it is given."""
 import ctypes as C
+import shutil
 import subprocess
 import threading
 import types
@@ -40,6 +41,8 @@ NAMES = sorted(_calls(None, None, None, None))
 def recorder(tmp_path):
     """A library with the prototypes of the hot calls that keeps every argument (of a structure: its first words)."""
     lib = B.load_library()
+    if shutil.which("gcc") is None or isinstance(B._calls(), B._CtypesCalls):
+        pytest.skip("no C compiler")
     src = ["#include <string.h>", "long long rec[64]; int n_rec;", "#define A(x) rec[n_rec++] = (long long)(x);"]
     for name in NAMES:
         types_ = getattr(lib, name).argtypes
