@@ -1166,7 +1166,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               const float alpha = (m_new == -INFINITY) ? 1.f : ex2((m_used - m_new) * sl);
               m_used = m_new;
               l *= alpha;
-#pragma unroll
+#pragma unroll 1
               for (int c = 0; c < D / 32; ++c) {
                 uint32_t o[32];
                 tmem_ld_32x32b_x32(tO + c * 32, o);
@@ -1246,6 +1246,10 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         // Rows leave through shared memory -- the warp's quarter of the entry's own query tile, which every product has
         // read by now -- so that a store instruction writes whole rows: stores straight from the row each thread owns touch
         // 32 rows at a time and took 5000-7000 cycles a tile (seven edited blocks, 312 entries: 34.9 -> 27 us a layer).
+        // Its loops stay loops: the code is passed once an entry and has been displaced by the softmax loop since, so that its
+        // length is what it costs (unrolled over the columns a tile took 2700-4000 cycles from the last product; rolled, a cold
+        // prompt of 7200 tokens, us over eight layers: 842 -> 782; seven edited blocks 224 -> 213; 8 x 16384 tokens 3105 -> 3000;
+        // 64 queries over 32000 cached tokens 592 -> 577).
         const int thread = thread_index_anew();
         const int lane = thread & 31, quarter = (thread >> 5) & 3;
         const int q_last = q_row0 + q_rows - 1, out_head0 = e.chunk * p.hpt;
@@ -1284,7 +1288,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (whole_tile) {
           uint8_t *tile = smem + ((p.q_double && (n_loaded & 1)) ? L::kBg + t * L::kTileBytes : (t ? L::kQ1 : L::kQ0));
           uint8_t *row = tile + (thread & 127) * 128;
-#pragma unroll
+#pragma unroll 1
           for (int c = 0; c < D / 32; ++c) {
             uint32_t o[32];
             tmem_ld_32x32b_x32(tO + c * 32, o);
@@ -1320,7 +1324,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           // product that reads them has completed)
           if (n_tiles > 0) {
             uint8_t *row = smem + (t ? L::kRing : L::kQ0) + (thread & 127) * (D * 4);
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {
               uint32_t o[32];
               tmem_ld_32x32b_x32(tO + c * 32, o);
@@ -1337,9 +1341,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           if (partial || p.out_f32) {
             uint8_t *base = partial ? reinterpret_cast<uint8_t *>(p.o_part + (size_t)e.split * p.n_part_rows * p.Hq * D)
                                     : reinterpret_cast<uint8_t *>(p.o);
-#pragma unroll
+#pragma unroll 1
             for (int h = 0; h < 4 * D / kStageRow; ++h) {            // kStageRow bytes of every row at a time
-#pragma unroll
+#pragma unroll 1
               for (int q = 0; q < kStageRow / 128; ++q) {
                 uint32_t o[32];
                 tmem_ld_32x32b_x32(tO + h * (kStageRow / 4) + q * 32, o);
@@ -1353,9 +1357,9 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               store_rows(base + out_row0 * D * 4 + h * kStageRow, D * 4);
             }
           } else {
-#pragma unroll
+#pragma unroll 1
             for (int h = 0; h < 2 * D / kStageRow; ++h) {
-#pragma unroll
+#pragma unroll 1
               for (int c = 0; c < kStageRow / 64; ++c) {
                 uint32_t o[32];
                 tmem_ld_32x32b_x32(tO + h * (kStageRow / 2) + c * 32, o);
