@@ -172,6 +172,7 @@ struct Ctrl {
   uint64_t o_done[2];
   uint64_t o_free[2];             // the softmax warps have read O_t out of tensor memory
   uint64_t out_staged[2];         // every row of the output tile is in shared memory
+  uint64_t solo_full;             // one query tile, both softmax groups: group 1's maxima and sums are in shared memory
   int n_staged_out[2];            // output tiles handed to the copy engine so far
   uint64_t work_full[kWorkSlots];  // work entry published by the scheduler (producer thread)
   uint64_t work_empty[kWorkSlots]; // entry read by the MMA thread and the 8 softmax warps
@@ -251,6 +252,16 @@ struct Work {
   int head0, kv_head;
   int tile0, n_tiles;   // key tiles [tile0, tile0 + n_tiles) of the item (split-KV share)
 };
+
+// Cluster launch, an entry of one query tile: the two softmax groups share its key tiles.  Group 0 takes tiles 0, 2, .. and group
+// 1 tiles 1, 3, .. with maxima, sums and an accumulator of its own (O_1), which group 0 merges when it writes the rows out.  One
+// group alone leaves the tensor core idle while it exponentiates and the exponentials idle while the products run.  The ring then
+// holds the keys one tile further ahead of the values: K_0, K_1, V_0, K_2, V_1, ..  (2500 cached tokens and a question of 64, 32
+// layers: 706 -> 664 us.  In the other kernels the test for it cost more than it gave: the thread that issues the products
+// is on every tile's path, 16 pooled requests with two query tiles each +5 %; and at twice the keys per unit of time
+// a ring of three stages runs dry, cold prompt of 7200 tokens 785 -> 890 us.)
+template <bool kAllowed>
+__device__ __forceinline__ bool is_solo(const Work &wk) { return kAllowed && wk.it.n_qt == 1 && wk.n_tiles > 1; }
 
 // Entry w of the global work list (equal shares of every item's key tiles).  pair < 0 past the end.
 //  Prefill: items heaviest-first (descending index: the table ends with the items of the final blocks, and within a
@@ -559,6 +570,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   // (four layers).  Not on the fused path: the flags cost its product thread more than the halves save.
   constexpr bool kWalks = kDeep;
   constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster;
+  constexpr bool kSolo = kVariant == kDeepCluster;
   // (layouts a variant is never launched with are not in its code: a short launch pays for every instruction it passes; a 32-layer
   // prompt of 2500 cached tokens 824 -> 795 us)
   const int balanced = kClustered || kDeep ? 0 : p.balanced, stream = kClustered ? 0 : p.stream, persistent = kClustered ? 0 : p.persistent;
@@ -583,6 +595,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       mbar_init(&ctrl->qr_full[t][0], 4); mbar_init(&ctrl->qr_full[t][1], 4); mbar_init(&ctrl->cs_full[t], D / 2);
       mbar_init(&ctrl->qraw_full[t], 1);
     }
+    mbar_init(&ctrl->solo_full, 128);
     for (int k = 0; k < kWorkSlots; ++k) { mbar_init(&ctrl->work_full[k], 1); mbar_init(&ctrl->work_empty[k], 9); }
     if (kClustered) ctrl->work_ring[0].pair = -1;
     ctrl->abort_flag = 0; ctrl->n_staged_out[0] = 0; ctrl->n_staged_out[1] = 0;
@@ -782,42 +795,99 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               tma_load_3d(dst + c * L::kRegionBytes + sb * sub_rows * 128, m, bar, c * 64, wk.kv_head, row);
           }
         };
-        for (int j = 0; j < wk.n_tiles && ok; ++j) {
-          const int jt = wk.tile0 + j;
-          const bool cached = jt < it.n_cache_tiles;
-          int k_row, v_row, t_off = 0, t_len = 0, t_kbase = 0, t_vbase = 0;
-          bool k_pg = false, v_pg = false;
-          if (!cached) {
-            k_row = v_row = it.own_row0 + (jt - it.n_cache_tiles) * kBlockN;
-          } else if (!p.walk) {
-            k_row = v_row = it.cache_row0 + jt * kBlockN;
-          } else {
-            k_row = k_base + poff;
-            v_row = v_base + poff;
-            k_pg = p.k_paged; v_pg = p.v_paged;
-            t_off = poff; t_len = c_len; t_kbase = k_base; t_vbase = v_base;
-            ctrl->tile_valid[(gidx >> 1) & 7] = min(kBlockN, c_len - poff);   // read by the softmax warps
-            poff += kBlockN;
-            if (poff >= c_len) {
-              ++pc; poff = 0;
-              c_len = n_len; k_base = n_kbase; v_base = n_vbase;
-              load_block(pc + 1, n_len, n_kbase, n_vbase);
+        // (one loop for both orders, with a tile's rows kept for its values, cost the kernels that have one order 1-2 %: cold prompt of
+        // 7200 tokens 783 -> 798 us)
+        if constexpr (!kSolo) {
+          for (int j = 0; j < wk.n_tiles && ok; ++j) {
+            const int jt = wk.tile0 + j;
+            const bool cached = jt < it.n_cache_tiles;
+            int k_row, v_row, t_off = 0, t_len = 0, t_kbase = 0, t_vbase = 0;
+            bool k_pg = false, v_pg = false;
+            if (!cached) {
+              k_row = v_row = it.own_row0 + (jt - it.n_cache_tiles) * kBlockN;
+            } else if (!p.walk) {
+              k_row = v_row = it.cache_row0 + jt * kBlockN;
+            } else {
+              k_row = k_base + poff;
+              v_row = v_base + poff;
+              k_pg = p.k_paged; v_pg = p.v_paged;
+              t_off = poff; t_len = c_len; t_kbase = k_base; t_vbase = v_base;
+              ctrl->tile_valid[(gidx >> 1) & 7] = min(kBlockN, c_len - poff);   // read by the softmax warps
+              poff += kBlockN;
+              if (poff >= c_len) {
+                ++pc; poff = 0;
+                c_len = n_len; k_base = n_kbase; v_base = n_vbase;
+                load_block(pc + 1, n_len, n_kbase, n_vbase);
+              }
+            }
+            for (int kv = 0; kv < 2; ++kv) {
+              const int stage = gidx % kStages;
+              ok = mbar_wait(&ctrl->kv_empty[stage], ((gidx / kStages) & 1) ^ 1, abort_flag);
+              if (!ok) break;
+              const CUtensorMap *m = cached ? (kv ? &tmap_vc : &tmap_kc) : (kv ? &tmap_v : &tmap_k);
+              uint8_t *dst = smem + L::kRing + stage * L::kTileBytes;
+              mbar_arrive_expect_tx(&ctrl->kv_full[stage], L::kTileBytes);
+              if (kv ? v_pg : k_pg) {
+                load_paged_tile(dst, m, &ctrl->kv_full[stage], kv ? t_vbase : t_kbase, t_off, t_len);
+              } else {
+                for (int c = 0; c < L::kChunks; ++c)
+                  tma_load_3d(dst + c * L::kRegionBytes, m, &ctrl->kv_full[stage], c * 64, wk.kv_head, kv ? v_row : k_row);
+              }
+              ++gidx;
             }
           }
-          for (int kv = 0; kv < 2; ++kv) {
+        } else {
+          // one tile of K (kv = 0) or V into the next stage of the ring
+          struct TileRows { int k_row, v_row, off, len, kbase, vbase; bool cached, k_pg, v_pg; };
+          auto load_tile = [&](const TileRows &x, int kv) {
             const int stage = gidx % kStages;
             ok = mbar_wait(&ctrl->kv_empty[stage], ((gidx / kStages) & 1) ^ 1, abort_flag);
-            if (!ok) break;
-            const CUtensorMap *m = cached ? (kv ? &tmap_vc : &tmap_kc) : (kv ? &tmap_v : &tmap_k);
+            if (!ok) return;
+            const CUtensorMap *m = x.cached ? (kv ? &tmap_vc : &tmap_kc) : (kv ? &tmap_v : &tmap_k);
             uint8_t *dst = smem + L::kRing + stage * L::kTileBytes;
             mbar_arrive_expect_tx(&ctrl->kv_full[stage], L::kTileBytes);
-            if (kv ? v_pg : k_pg) {
-              load_paged_tile(dst, m, &ctrl->kv_full[stage], kv ? t_vbase : t_kbase, t_off, t_len);
+            if (kv ? x.v_pg : x.k_pg) {
+              load_paged_tile(dst, m, &ctrl->kv_full[stage], kv ? x.vbase : x.kbase, x.off, x.len);
             } else {
               for (int c = 0; c < L::kChunks; ++c)
-                tma_load_3d(dst + c * L::kRegionBytes, m, &ctrl->kv_full[stage], c * 64, wk.kv_head, kv ? v_row : k_row);
+                tma_load_3d(dst + c * L::kRegionBytes, m, &ctrl->kv_full[stage], c * 64, wk.kv_head, kv ? x.v_row : x.k_row);
             }
             ++gidx;
+          };
+          const bool solo = is_solo<kSolo>(wk);
+          const int first_tile = gidx >> 1;   // tiles of all earlier entries (the other roles count the same way)
+          TileRows x = {}, before = {};
+          for (int j = 0; j < wk.n_tiles + (solo ? 1 : 0) && ok; ++j) {
+            if (j < wk.n_tiles) {
+              const int jt = wk.tile0 + j;
+              x = {};
+              x.cached = jt < it.n_cache_tiles;
+              if (!x.cached) {
+                x.k_row = x.v_row = it.own_row0 + (jt - it.n_cache_tiles) * kBlockN;
+              } else if (!p.walk) {
+                x.k_row = x.v_row = it.cache_row0 + jt * kBlockN;
+              } else {
+                x.k_row = k_base + poff;
+                x.v_row = v_base + poff;
+                x.k_pg = p.k_paged; x.v_pg = p.v_paged;
+                x.off = poff; x.len = c_len; x.kbase = k_base; x.vbase = v_base;
+                ctrl->tile_valid[(first_tile + j) & 7] = min(kBlockN, c_len - poff);   // read by the softmax warps
+                poff += kBlockN;
+                if (poff >= c_len) {
+                  ++pc; poff = 0;
+                  c_len = n_len; k_base = n_kbase; v_base = n_vbase;
+                  load_block(pc + 1, n_len, n_kbase, n_vbase);
+                }
+              }
+              load_tile(x, 0);
+            }
+            if (!ok) break;
+            if (!solo) {
+              load_tile(x, 1);
+            } else {
+              if (j > 0) load_tile(before, 1);
+              before = x;
+            }
           }
         }
         if (kClustered) break;
@@ -851,12 +921,13 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       bool half_last = false;              // the entry's last key tile is used in its first 64 keys only
       int entry_tiles = 0;
       // a cached tile whose block ends in its first 64 keys (walk mode; the producer's word comes with the tile)
-      auto cached_half = [&](int jrel, int idx) -> bool {
-        return kWalks && p.walk && wk.tile0 + jrel < wk.it.n_cache_tiles && ctrl->tile_valid[(idx >> 1) & 7] <= kBlockN / 2;
+      int first_tile = 0;                  // tiles of all earlier entries
+      auto cached_half = [&](int jrel) -> bool {
+        return kWalks && p.walk && wk.tile0 + jrel < wk.it.n_cache_tiles && ctrl->tile_valid[(first_tile + jrel) & 7] <= kBlockN / 2;
       };
       auto issue_qk_with = [&](int t, int jrel, int idx, uint64_t qd) {
         const uint64_t kd = k_desc0 + (uint64_t)(((idx % kStages) * L::kTileBytes) >> 4);
-        const uint32_t idesc = ((half_last && jrel + 1 == entry_tiles) || cached_half(jrel, idx)) ? idesc_qk_half : idesc_qk;
+        const uint32_t idesc = ((half_last && jrel + 1 == entry_tiles) || cached_half(jrel)) ? idesc_qk_half : idesc_qk;
 #pragma unroll
         for (int k = 0; k < D / 16; ++k) {
           const uint64_t off = (uint64_t)(((k >> 2) * L::kRegionBytes + (k & 3) * 32) >> 4);
@@ -887,9 +958,10 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       int walk_pc = 0, walk_end = -1;      // block of the current cached tile and the tile index where it ends
       int cached_end = 0;                  // tiles [tile0, cached_end) of the entry are cached keys
       int q_buf = 0;                       // plain path: buffer pair that holds the entry's query tiles
+      bool solo = false;                   // one query tile, key tiles shared by the softmax groups (is_solo)
       // S_t = Q_t K^T for tile `jrel` of the entry, whose keys sit at ring position idx
       auto issue_qk = [&](int t, int jrel, int idx) -> bool {
-        if (!kFused) { issue_qk_with(t, jrel, idx, q_buf ? qb_desc[t] : q_desc[t]); return true; }
+        if (!kFused) { const int q = solo ? 0 : t; issue_qk_with(t, jrel, idx, q_buf ? qb_desc[q] : q_desc[q]); return true; }
         const int jt = wk.tile0 + jrel;
         bool change = false;
         if (jt < cached_end) {
@@ -926,6 +998,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (n_tiles == 0) continue;
         half_last = last_tile_is_half(wk);
         entry_tiles = n_tiles;
+        first_tile = gidx >> 1;
+        solo = is_solo<kSolo>(wk);
         walk_end = -1; ver_end[0] = ver_end[1] = -1;
         cached_end = min(wk.tile0 + n_tiles, wk.it.n_cache_tiles);
         if (!kFused) {
@@ -944,50 +1018,67 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           if (t < n_qt && ok) ok = issue_qk(t, 0, gidx);
         if (!ok) break;
         mma_commit(&ctrl->kv_empty[gidx % kStages]);
-        if (kDeep && n_tiles == 1) mma_commit(&ctrl->q_empty[0][0]);
-        for (int j = 0; j < n_tiles && ok; ++j) {
-          const bool last = j + 1 == n_tiles;
-          const int iv = gidx + 2 * j + 1, ik = gidx + 2 * j + 2;   // ring positions of V_j and K_(j+1)
-          BA_TR(3, j, 0);
-          ok = wait_kv(iv);
-          BA_TR(3, j, 1);
+        if (solo) {
+          ok = wait_kv(gidx + 1);
+          if (!ok) break;
+          tc_fence_after();
+          issue_qk(1, 1, gidx + 1);
+          mma_commit(&ctrl->kv_empty[(gidx + 1) % kStages]);
+        }
+        if (kDeep && n_tiles <= (solo ? 2 : 1)) mma_commit(&ctrl->q_empty[0][0]);
+        // Round i: tile i for every query tile, or (solo) tiles 2 i and 2 i + 1.
+        for (int i = 0; solo ? 2 * i < n_tiles : i < n_tiles; ++i) {
+          int iv = gidx + 2 * i + 1, ik = gidx + 2 * i + 2;         // ring positions of V_j and of K of the tile S_t takes next
+          BA_TR(3, i, 0);
+          if (!solo) ok = wait_kv(iv);
+          BA_TR(3, i, 1);
 #pragma unroll
           for (int t = 0; t < 2; ++t) {
-            if (t >= n_qt || !ok) continue;
-            BA_TR(2, j, t * 4 + 0);
+            const int j = solo ? 2 * i + t : i, jn = j + (solo ? 2 : 1);
+            if (!ok || (solo ? j >= n_tiles : t >= n_qt)) continue;
+            const bool last = jn >= n_tiles;
+            if (solo) {                                    // K_0, K_1, V_0, K_2, V_1, .., K_(n-1), V_(n-2), V_(n-1)
+              iv = gidx + 2 * j + (j + 1 < n_tiles ? 2 : 1);
+              ik = gidx + 2 * j + 3;
+              ok = wait_kv(iv);
+              if (!ok) continue;
+            }
+            BA_TR(2, i, t * 4 + 0);
             // the first PV of an item overwrites O_t: the previous item's rows must have been read out
-            if (j == 0) { ok = mbar_wait(&ctrl->o_free[t], (q_uses[t] & 1) ^ 1, abort_flag); if (!ok) continue; }
+            if (i == 0) { ok = mbar_wait(&ctrl->o_free[t], (q_uses[t] & 1) ^ 1, abort_flag); if (!ok) continue; }
             ok = mbar_wait(&ctrl->p_full[t][0], p_uses[t] & 1, abort_flag);
             if (!ok) continue;
             tc_fence_after();
-            BA_TR(2, j, t * 4 + 1);
-            issue_pv(t, iv, j == 0, 0);
-            // K_(j+1) is needed right after the second half of PV: make sure of it while P is still
+            BA_TR(2, i, t * 4 + 1);
+            issue_pv(t, iv, i == 0, 0);
+            // the next K is needed right after the second half of PV: make sure of it while P is still
             // being finished, off the critical path
-            if (t == 0 && !last) { BA_TR(3, j, 2); ok = wait_kv(ik); if (!ok) continue; BA_TR(3, j, 3); }
+            if ((t == 0 || solo) && !last) { BA_TR(3, i, 2); ok = wait_kv(ik); if (!ok) continue; BA_TR(3, i, 3); }
             ok = mbar_wait(&ctrl->p_full[t][1], p_uses[t] & 1, abort_flag);
             if (!ok) continue;
             tc_fence_after();
-            if (!(last && half_last) && !cached_half(j, iv)) issue_pv(t, iv, j == 0, 1);
+            if (!(j + 1 == n_tiles && half_last) && !cached_half(j)) issue_pv(t, iv, i == 0, 1);
             ++p_uses[t];
-            BA_TR(2, j, t * 4 + 2);
+            BA_TR(2, i, t * 4 + 2);
             if (last) mma_commit(&ctrl->o_done[t]);
-            if (t + 1 == n_qt) mma_commit(&ctrl->kv_empty[iv % kStages]);
+            if (solo || t + 1 == n_qt) mma_commit(&ctrl->kv_empty[iv % kStages]);
             if (!last) {
-              ok = issue_qk(t, j + 1, ik);
+              ok = issue_qk(t, jn, ik);
               if (!ok) continue;
-              BA_TR(2, j, t * 4 + 3);
-              if (t + 1 == n_qt) {
+              BA_TR(2, i, t * 4 + 3);
+              if (solo || t + 1 == n_qt) {
                 mma_commit(&ctrl->kv_empty[ik % kStages]);
-                if (kDeep && j + 2 == n_tiles) mma_commit(&ctrl->q_empty[0][0]);   // that was the entry's last QK^T
+                if (kDeep && jn + 1 == n_tiles) mma_commit(&ctrl->q_empty[0][0]);   // that was the entry's last QK^T
               }
             }
           }
+          if (!ok) break;
         }
+        if (!ok) break;
         gidx += 2 * n_tiles;
 #pragma unroll
         for (int t = 0; t < 2; ++t)
-          if (t < n_qt) ++q_uses[t];
+          if (t < n_qt || solo) ++q_uses[t];
         if (kClustered) break;                             // (one entry)
       }
     }
@@ -1016,7 +1107,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     const uint32_t tO = tmem + 256 + t * 128 + lane_off;
     const float sl = p.scale_log2;
     int s_uses = 0;                       // S tiles of this query tile consumed so far
-    int o_uses = 0;                       // items in which this query tile was active
+    int o_uses = 0;                       // entries that used this group's accumulator so far
     int n_staged = 0;                     // fused: (cos, sin) rows staged so far by this group
     int n_made = 0;                       // fused: versions of this query tile prepared so far
     int tiles_before = 0;                 // key tiles of all earlier items (the producer counts the same way)
@@ -1046,9 +1137,12 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       const int n_tiles = wk.n_tiles, tile0 = wk.tile0, head0 = wk.head0;
       const bool half_last = last_tile_is_half(wk);
       release_out();
-      if (t < it.n_qt) {
+      const bool solo = is_solo<kSolo>(wk);
+      const int j0 = solo ? t : 0;         // this group's key tiles: j0, j0 + 1 (solo: j0 + 2), ..
+      if (t < it.n_qt || solo) {
+      const int tq = solo ? 0 : t;
       // rows past the block behave like its last row
-      const int tok_c = min(it.q_row0 + t * p.tok + (r >> p.hpt_log2), it.q_row0 + it.q_rows - 1);
+      const int tok_c = min(it.q_row0 + tq * p.tok + (r >> p.hpt_log2), it.q_row0 + it.q_rows - 1);
       float m_used = -INFINITY, l = 0.f;
 
       // fused path: this thread prepares row r of every version of query tile t (see the MMA warp):
@@ -1110,7 +1204,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         plan_next(first_cached ? f_pc : -1);
       }
 
-      for (int j = 0; j < n_tiles; ++j) {
+      for (int j = j0; j < n_tiles; j += solo ? 2 : 1) {
         if (r == 0) BA_TR(t, j, 0);
         ok = mbar_wait(&ctrl->s_full[t], s_uses & 1, abort_flag);
         if (!ok) break;
@@ -1157,7 +1251,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
           for (int i = 1; i < n3; ++i) mx = fmaxf(mx, l3[i]);
           const float m_new = fmaxf(m_used, mx);
           if (r == 0) BA_TR(t, j, 3);
-          if (j == 0) {
+          if (j == j0) {
             m_used = m_new;
           } else {
             const bool grow = (m_new - m_used) * sl > kRescaleThreshold;
@@ -1237,10 +1331,26 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       asm volatile("ld.global.nc.v2.s32 {%0, %1}, [%3];\n\tld.global.nc.s32 %2, [%3 + 20];"
                    : "=&r"(q_row0), "=&r"(q_rows), "=r"(part_row0) : "l"(p.items + 8 * (size_t)e.pair));
       if (kClustered && e.fill == 2) { q_row0 += p.tok; q_rows -= p.tok; }
-      if (ok && n_tiles > 0) { ok = mbar_wait(&ctrl->o_done[t], o_uses & 1, abort_flag); ++o_uses; }
-      if (ok) {
+      if (ok && n_tiles > 0 && !(solo && t == 1)) { ok = mbar_wait(&ctrl->o_done[t], o_uses & 1, abort_flag); ++o_uses; }
+      float weight = 1.f, inv1 = 0.f;      // (solo) what O_0 and O_1 count for
+      if (kSolo && solo) {                 // (a cluster's CTA has one entry)
+        // group 1's maximum and sum of every row, where the other deep-ring kernel stages its output
+        float2 *other = reinterpret_cast<float2 *>(smem + L::kBg + L::kTileBytes) + r;
+        if (t == 1) {
+          if (ok) { *other = make_float2(m_used, l); mbar_arrive(&ctrl->solo_full); }
+        } else if (ok) {
+          ok = mbar_wait(&ctrl->solo_full, 0, abort_flag) && mbar_wait(&ctrl->o_done[1], 0, abort_flag);
+          const float2 x = *other;
+          const float m = fmaxf(m_used, x.x);
+          if (m != -INFINITY) { weight = ex2((m_used - m) * sl); inv1 = ex2((x.x - m) * sl); }
+          l = weight * l + inv1 * x.y;
+          m_used = m;
+        }
+      }
+      if (ok && !(solo && t == 1)) {
         tc_fence_after();
-        const float inv = l > 0.f ? 1.f / l : 0.f;
+        const float inv_l = l > 0.f ? 1.f / l : 0.f, inv = weight * inv_l;
+        inv1 *= inv_l;
         const float lse_val = l > 0.f ? (m_used * sl + log2f(l)) * 0.6931471805599453f : -INFINITY;
         const bool partial = !kClustered && e.split >= 0;
         // Rows leave through shared memory -- the warp's quarter of the entry's own query tile, which every product has
@@ -1255,7 +1365,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         const int q_last = q_row0 + q_rows - 1, out_head0 = e.chunk * p.hpt;
         // a row is stored only if it belongs to the item and lies inside the caller's tensors; tables that
         // describe more rows than the caller gave are reported, nothing is written past the end
-        const int row_tok = q_row0 + t * p.tok + ((quarter * 32 + lane) >> p.hpt_log2), head = out_head0 + (lane & (p.hpt - 1));
+        const int row_tok = q_row0 + tq * p.tok + ((quarter * 32 + lane) >> p.hpt_log2), head = out_head0 + (lane & (p.hpt - 1));
         const bool row_valid = row_tok <= q_last && row_tok < p.n_q_rows;
         if (row_tok <= q_last && row_tok >= p.n_q_rows) ba_record_status(p.status, BA_ERR_SHAPE);
         // (kDeepRing: through rows of its own, 128 bytes at a time)
@@ -1266,7 +1376,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
                          quarter * (32 * kStageRow);
         // partial results of a prefill are indexed by the row's place among the rows of final blocks
         const int part_shift = partial && !p.final_only ? part_row0 - q_row0 : 0;
-        const int tile_row0 = q_row0 + t * p.tok, tile_rows = min(q_last + 1, p.n_q_rows) - tile_row0;   // tokens stored
+        const int tile_row0 = q_row0 + tq * p.tok, tile_rows = min(q_last + 1, p.n_q_rows) - tile_row0;   // tokens stored
         const size_t out_row0 = (size_t)(tile_row0 + part_shift) * p.Hq + out_head0;
         // dst: where the staged bytes of the tile's first row go; row_bytes: from one (token, head) row to the next
         auto store_rows = [&](uint8_t *dst, int row_bytes) {
@@ -1326,14 +1436,21 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
             uint8_t *row = smem + (t ? L::kRing : L::kQ0) + (thread & 127) * (D * 4);
 #pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {
-              uint32_t o[32];
-              tmem_ld_32x32b_x32(tO + c * 32, o);
+              uint32_t a[32];
+              float o[32];
+              tmem_ld_32x32b_x32(tO + c * 32, a);
               tmem_wait_ld();
 #pragma unroll
+              for (int i = 0; i < 32; ++i) o[i] = __uint_as_float(a[i]) * inv;
+              if (kSolo && solo) {
+                tmem_ld_32x32b_x32(tO + 128 + c * 32, a);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = fmaf(__uint_as_float(a[i]), inv1, o[i]);
+              }
+#pragma unroll
               for (int i = 0; i < 8; ++i)
-                *reinterpret_cast<float4 *>(row + (((c * 8 + i) ^ (lane & 7)) << 4)) =
-                    make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
-                                __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
+                *reinterpret_cast<float4 *>(row + (((c * 8 + i) ^ (lane & 7)) << 4)) = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
             }
           }
           reinterpret_cast<float *>(smem + L::kCtrl + 1024)[t * 128 + (thread & 127)] = lse_val;

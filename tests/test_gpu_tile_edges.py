@@ -174,6 +174,24 @@ def test_cluster_launch(w, fused):
     check_attention(o, o_ref, lse, lse_ref, bf16_store=True)
 
 
+# Items of one query tile, whose key tiles both softmax groups of a CTA share: one, two, three and more key tiles a CTA (an odd number
+# leaves the groups unequal, one leaves the second idle), CTAs of a cluster with unequal numbers, a last tile used in half, values
+# walked in a pool.
+@pytest.mark.parametrize("w", [_requests("one_each", 1, 141, (2, 64, 100), (32, 32), heads=(8, 2, 128)),
+                               _requests("ragged", 4, 142, (9, 40, 300), (1, 32), heads=(32, 8, 128)),
+                               _requests("many_tiles", 4, 143, (20, 300, 400), (5, 32), heads=(32, 8, 128)),
+                               _requests("narrow_heads", 6, 144, (7, 100, 400), (100, 128), heads=(6, 2, 64)),
+                               _requests("pool", 3, 145, (9, 20, 290), (1, 30), heads=(8, 2, 128), pool=True)], ids=lambda w: w.name)
+def test_cluster_launch_one_query_tile(w):
+    shapes = []
+    o, lse, o_ref, lse_ref = run_warm(w, B.BA_MODE_BLOCK, shape_out=shapes)
+    items = w.n_q_heads // _hpt(w) * w.batch
+    assert shapes[0]["partials"] == 1 and shapes[0]["ctas"] in [items * m for m in range(2, 9)]
+    check_attention(o, o_ref, lse, lse_ref)
+    again, lse_again, _, _ = run_warm(w, B.BA_MODE_BLOCK)
+    assert np.array_equal(o, again) and np.array_equal(lse, lse_again)
+
+
 def _hpt(w):
     g = w.n_q_heads // w.n_kv_heads
     return 4 if g % 4 == 0 else 2 if g % 2 == 0 else 1
