@@ -253,6 +253,22 @@ struct Work {
   int tile0, n_tiles;   // key tiles [tile0, tile0 + n_tiles) of the item (split-KV share)
 };
 
+// The item of a published entry, decoded by the producer a few tiles ahead, for the roles whose wait for the item's line would stand
+// between two entries (seven edited blocks, 312 entries, us over eight layers: 213 -> 209.5; cold prompt of 7200 tokens 784 -> 778).
+struct ReadyItem { int q_row0, q_rows, own_row0, cache_len, n_cache_tiles, n_tiles, ctile0, pad; };
+constexpr int kReadyOff = 1600;          // [kWorkSlots], in the control area behind the spare warps' barriers
+static_assert(kReadyOff >= 1024 + 2 * (int)sizeof(ba_bg_smem) && kReadyOff + kWorkSlots * (int)sizeof(ReadyItem) <= 2048, "control area layout");
+__device__ __forceinline__ bool ready_work(const AttnParams &p, const WorkEntry &e, const ReadyItem &x, Work &wk) {
+  if (e.pair < 0) return false;
+  wk.it.q_row0 = x.q_row0; wk.it.q_rows = x.q_rows; wk.it.own_row0 = x.own_row0; wk.it.cache_len = x.cache_len;
+  wk.it.n_cache_tiles = x.n_cache_tiles; wk.it.n_tiles = x.n_tiles; wk.it.ctile0 = x.ctile0;
+  wk.it.n_qt = x.q_rows > p.tok ? 2 : 1;
+  wk.head0 = e.chunk * p.hpt;
+  wk.tile0 = e.tile0;
+  wk.n_tiles = e.n_tiles;
+  return true;
+}
+
 // Cluster launch, an entry of one query tile: the two softmax groups share its key tiles.  Group 0 takes tiles 0, 2, .. and group
 // 1 tiles 1, 3, .. with maxima, sums and an accumulator of its own (O_1), which group 0 merges when it writes the rows out.  One
 // group alone leaves the tensor core idle while it exponentiates and the exponentials idle while the products run.  The ring then
@@ -571,6 +587,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   constexpr bool kWalks = kDeep;
   constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster;
   constexpr bool kSolo = kVariant == kDeepCluster;
+  constexpr bool kReady = kVariant == kPlain || kVariant == kDeepRing;
   // (layouts a variant is never launched with are not in its code: a short launch pays for every instruction it passes; a 32-layer
   // prompt of 2500 cached tokens 824 -> 795 us)
   const int balanced = kClustered || kDeep ? 0 : p.balanced, stream = kClustered ? 0 : p.stream, persistent = kClustered ? 0 : p.persistent;
@@ -625,6 +642,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   tc_fence_after();
   const uint32_t tmem = ctrl->tmem_base;
   volatile int *abort_flag = &ctrl->abort_flag;
+  ReadyItem *ready = reinterpret_cast<ReadyItem *>(smem + L::kCtrl + kReadyOff);
   ba_pdl_trigger();
 
   // The CTA is persistent: its producer thread draws entries of the global work list from an
@@ -736,6 +754,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         const bool more = load_work<kClustered>(p, e, wk);
         if (!more) e.pair = -1;
         ctrl->work_ring[slot] = e;
+        if (kReady && more)
+          ready[slot] = {wk.it.q_row0, wk.it.q_rows, wk.it.own_row0, wk.it.cache_len, wk.it.n_cache_tiles, wk.it.n_tiles, wk.it.ctile0, 0};
         mbar_arrive(&ctrl->work_full[slot]);
         ++n_work;
         if (!more) break;
@@ -992,7 +1012,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (!ok) break;
         const WorkEntry e = ctrl->work_ring[slot];
         ++n_work;
-        if (!load_work<kClustered>(p, e, wk)) break;
+        if (!(kReady ? ready_work(p, e, ready[slot], wk) : load_work<kClustered>(p, e, wk))) break;
         mbar_arrive(&ctrl->work_empty[slot]);          // the entry has been decoded into registers
         const int n_tiles = wk.n_tiles, n_qt = wk.it.n_qt;
         if (n_tiles == 0) continue;
@@ -1130,7 +1150,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       if (!ok) break;
       const WorkEntry e = ctrl->work_ring[slot];
       ++n_work;
-      if (!load_work<kClustered>(p, e, wk)) break;
+      if (!(kReady ? ready_work(p, e, ready[slot], wk) : load_work<kClustered>(p, e, wk))) break;
       __syncwarp();
       if ((tid & 31) == 0) mbar_arrive(&ctrl->work_empty[slot]);   // one arrival per softmax warp
       const Item &it = wk.it;
