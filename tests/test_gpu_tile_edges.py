@@ -27,6 +27,18 @@ def test_backward_tile_edges(lens, heads):
         rq, rk, rv = ob.block_prefill_backward(q, k, v, g, w.block_lens, w.seq_nblocks, mode)
         check_grad("dq", dq, rq); check_grad("dk", dk, rk); check_grad("dv", dv, rv)
 
+# The search for a key tile's block, 32 places a round: one round, two, three; gradients stored as bf16 and fp32 rows.
+@pytest.mark.parametrize("n_blocks", [31, 32, 33, 1024, 1025])
+@pytest.mark.parametrize("dtype", [B.BA_OUT_F32, B.BA_OUT_BF16], ids=["f32", "bf16"])
+def test_backward_many_blocks(n_blocks, dtype):
+    lens = [1 + i * 7 % 4 for i in range(n_blocks)]
+    lens[0] = lens[-1] = 130
+    w = W.Workload("many_blocks", 2, 1, 64, 1e4, lens, [n_blocks // 8] * 8 + ([n_blocks % 8] if n_blocks % 8 else []), seed=82)
+    dq, dk, dv, q, k, v, g = run_forward_backward(w, B.BA_MODE_BLOCK, grad_dtype=dtype)
+    rq, rk, rv = ob.block_prefill_backward(q, k, v, g, w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    check_grad("dq", dq, rq); check_grad("dk", dk, rk); check_grad("dv", dv, rv)
+
+
 def _ragged_lens(n_blocks, seed):
     return [int(v) for v in np.random.default_rng(seed).integers(1, 9, n_blocks)]
 
