@@ -9,7 +9,7 @@
 //
 // Structure of a CTA (384 threads, one CTA per SM):
 //   warps 0-3   softmax of query tile 0      (one thread per tile row = TMEM lane)
-//   warps 4-7   softmax of query tile 1
+//   warps 4-7   softmax of query tile 1 (in a cluster, where there is one query tile only: of every second key tile)
 //   warp  8     TMA producer: Q tiles once, then K_j, V_j, K_j+1, ... into a ring of stages
 //   warp  9     MMA issuer (one elected thread): S = Q K^T and O += P V with tcgen05.mma,
 //               accumulators in tensor memory (S0, S1, O0, O1 = 4 x 128 columns)
