@@ -96,7 +96,7 @@ typedef struct {
   int32_t final_key_tiles[6];
   int32_t prompt_key_tiles; /* sum over the work items of ba_block_prefill in block mode, lengths on the host (else 0) */
   int32_t final_key_tiles_odd[2]; /* final_key_tiles[0] and [3] over every second item (1, 3, ..) of a sequence only */
-  int32_t reserved;
+  int32_t final_rows_max;  /* rows of the longest final block, lengths on the host (else 0) */
   /* per sequence, [batch + 1] */
   int32_t *cu_seq;         /* first row of the sequence, prompt packing */
   int32_t *cu_cache_seq;   /* first row of the sequence, cache packing */

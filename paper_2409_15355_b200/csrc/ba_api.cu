@@ -277,6 +277,7 @@ ba_status ba_segment(ba_ctx *ctx, const int32_t *block_lens, const int32_t *seq_
       b += seq_nblocks[q];
       const long long ct[2] = {(cached + 127) / 128, walked};
       const int fin = block_lens[b - 1];
+      out->final_rows_max = std::max(out->final_rows_max, fin);
       for (int r0 = 0; r0 < fin; r0 += tt) {
         const long long own = (std::min(fin, r0 + tt) + 127) / 128;
         for (int k = 0; k < 2; ++k) {

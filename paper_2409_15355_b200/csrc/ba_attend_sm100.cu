@@ -9,8 +9,9 @@
 //
 // Structure of a CTA (384 threads, one CTA per SM):
 //   warps 0-3   softmax of query tile 0      (one thread per tile row = TMEM lane)
-//   warps 4-7   softmax of query tile 1 (in a cluster, where there is one query tile only: of every second key tile)
-//   warp  8     TMA producer: Q tiles once, then K_j, V_j, K_j+1, ... into a ring of stages
+//   warps 4-7   softmax of query tile 1 (kSharedCluster, where there is one query tile only: of every second key tile)
+//   warp  8     TMA producer: Q tiles once, then K_j, V_j, K_j+1, ... into a ring of stages (key tiles shared by both softmax
+//               groups: K_0, K_1, V_0, K_2, V_1, ...)
 //   warp  9     MMA issuer (one elected thread): S = Q K^T and O += P V with tcgen05.mma,
 //               accumulators in tensor memory (S0, S1, O0, O1 = 4 x 128 columns)
 // A query tile is 128 rows = (128 / HPT) tokens x HPT query heads of one KV group,
@@ -66,10 +67,11 @@ constexpr int kBlockN = 128;      // keys per tile
 // takes 2000-4500 cycles, three stages cover 2700 (64-token query over 32K cached keys: 800-1900 cycles of waiting in a
 // period of 4000-4900), and with the write-out elsewhere the one pair of query buffers is reloaded as soon as its last
 // product is done.
-// The cluster forms of the last two merge the results of a cluster's CTAs in shared memory.
-constexpr int kPlain = 0, kFusedPath = 1, kDeepRing = 2, kFusedCluster = 3, kDeepCluster = 4;
+// The cluster forms of the last two merge the results of a cluster's CTAs in shared memory; kSharedCluster is kDeepCluster for
+// launches whose CTAs have one query tile (is_solo).
+constexpr int kPlain = 0, kFusedPath = 1, kDeepRing = 2, kFusedCluster = 3, kDeepCluster = 4, kSharedCluster = 5;
 constexpr bool is_fused(int variant) { return variant == kFusedPath || variant == kFusedCluster; }
-constexpr bool is_deep(int variant) { return variant == kDeepRing || variant == kDeepCluster; }
+constexpr bool is_deep(int variant) { return variant == kDeepRing || variant == kDeepCluster || variant == kSharedCluster; }
 constexpr int kMaxStages = 4;
 constexpr float kRescaleThreshold = 8.0f;
 constexpr int kBgStageBytes = 16384; // two spare warps x two stages of source rows
@@ -273,9 +275,9 @@ __device__ __forceinline__ bool ready_work(const AttnParams &p, const WorkEntry 
 // 1 tiles 1, 3, .. with maxima, sums and an accumulator of its own (O_1), which group 0 merges when it writes the rows out.  One
 // group alone leaves the tensor core idle while it exponentiates and the exponentials idle while the products run.  The ring then
 // holds the keys one tile further ahead of the values: K_0, K_1, V_0, K_2, V_1, ..  (2500 cached tokens and a question of 64, 32
-// layers: 706 -> 664 us.  In the other kernels the test for it cost more than it gave: the thread that issues the products
-// is on every tile's path, 16 pooled requests with two query tiles each +5 %; and at twice the keys per unit of time
-// a ring of three stages runs dry, cold prompt of 7200 tokens 785 -> 890 us.)
+// layers: 706 -> 664 us.)  The test for it costs where there are two query tiles, as the thread that issues the products is on every
+// tile's path: 16 pooled requests +5 %; clusters of whole items +1-3 % (ba_cluster_plan::shared: a kernel of their own without
+// it).  At twice the keys per unit of time a ring of three stages runs dry: cold prompt of 7200 tokens 785 -> 890 us.
 template <bool kAllowed>
 __device__ __forceinline__ bool is_solo(const Work &wk) { return kAllowed && wk.it.n_qt == 1 && wk.n_tiles > 1; }
 
@@ -585,8 +587,8 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   // Half tiles at the ends of cached blocks, values walked in a pool: 16 requests over 20 blocks of 50-500 tokens 1401 -> 1377 us
   // (four layers).  Not on the fused path: the flags cost its product thread more than the halves save.
   constexpr bool kWalks = kDeep;
-  constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster;
-  constexpr bool kSolo = kVariant == kDeepCluster;
+  constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster || kVariant == kSharedCluster;
+  constexpr bool kSolo = kVariant == kSharedCluster;
   constexpr bool kReady = kVariant == kPlain || kVariant == kDeepRing;
   // (layouts a variant is never launched with are not in its code: a short launch pays for every instruction it passes; a 32-layer
   // prompt of 2500 cached tokens 824 -> 795 us)
@@ -1720,11 +1722,13 @@ ba_status ba_attend_sm100_setup(ba_ctx *ctx) {
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedCluster>, attend_smem_bytes<128>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepCluster>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kSharedCluster>, attend_smem_bytes<128>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedPath>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedCluster>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepCluster>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kSharedCluster>, attend_smem_bytes<64>()));
   ctx->maps = new (std::nothrow) ba_map_cache();
   if (!ctx->maps) return BA_ERR_CUDA;
   for (auto &sl : ctx->maps->slot) sl.ptr = nullptr;
@@ -1868,7 +1872,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   const unsigned pairs_upper = pairs_known > 0 ? (unsigned)pairs_known : (unsigned)(a.n_q_rows / pair_tok + n_units);
   const long long items = (a.final_only && seg->n_final_items > 0 ? (long long)seg->n_final_items
                                                                   : (long long)((a.n_q_rows + pair_tok - 1) / pair_tok)) * (Hq / p.hpt);
-  int n_splits = 1, stream_ctas = 0;
+  int n_splits = 1, stream_ctas = 0, cluster_shared = 0;
   p.stream = 0; p.n_odd = 0; p.cluster = 0; p.single = 0;
   if (a.final_only) {
     // key tiles of an average item: counted by ba_segment() when it saw the lengths, else estimated
@@ -1892,8 +1896,9 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
         p.stream = 1; stream_ctas = stream.n_ctas; p.n_odd = stream.n_odd; n_splits = stream.n_slots;
       }
       if (a.n_cache_rows > 0 && !ctx->has_pending) {
-        const ba_cluster_plan cl = ba_plan_cluster(items, a.n_q_rows > (long long)p.tok * seg->n_final_items, ft[2], [&](int n) { return max_clusters(ctx, n); });
-        if (cl.size > 0 && cl.cost < (double)(p.stream ? stream.cost : equal_cost)) { p.cluster = cl.size; p.single = cl.single; p.stream = 0; n_splits = 1; }
+        const ba_cluster_plan cl = ba_plan_cluster(items, a.n_q_rows > (long long)p.tok * seg->n_final_items,
+                                                   seg->final_rows_max > 0 && seg->final_rows_max <= p.tok, ft[2], [&](int n) { return max_clusters(ctx, n); });
+        if (cl.size > 0 && cl.cost < (double)(p.stream ? stream.cost : equal_cost)) { p.cluster = cl.size; p.single = cl.single; cluster_shared = cl.shared; p.stream = 0; n_splits = 1; }
       }
     }
   } else if (!a.final_only && a.mode == BA_MODE_BLOCK && seg->n_final_items > 0 && seg->prompt_key_tiles > 0) {
@@ -1967,7 +1972,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
   const bool early = !p.balanced;
   cudaError_t launched = cudaSuccess;
   auto launch_attend = [&](auto kern, int smem) { launched = ba_launch_clusters(kern, p.cluster, grid, kThreads, smem, stream, early, tq, tk, tv, tkc, tvc, to, p); };
-  const int variant = p.fused ? (p.cluster > 1 ? kFusedCluster : kFusedPath) : deep_ring ? (p.cluster > 1 ? kDeepCluster : kDeepRing) : kPlain;
+  const int variant = p.fused ? (p.cluster > 1 ? kFusedCluster : kFusedPath) : deep_ring ? (p.cluster > 1 ? (cluster_shared ? kSharedCluster : kDeepCluster) : kDeepRing) : kPlain;
   auto pick = [&](auto d_tag) {
     constexpr int kD = decltype(d_tag)::value, kSmem = attend_smem_bytes<kD>();
     switch (variant) {
@@ -1975,6 +1980,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
       case kFusedCluster: launch_attend(ba_attend_sm100_kernel<kD, kFusedCluster>, kSmem); break;
       case kDeepRing: launch_attend(ba_attend_sm100_kernel<kD, kDeepRing>, kSmem); break;
       case kDeepCluster: launch_attend(ba_attend_sm100_kernel<kD, kDeepCluster>, kSmem); break;
+      case kSharedCluster: launch_attend(ba_attend_sm100_kernel<kD, kSharedCluster>, kSmem); break;
       default: launch_attend(ba_attend_sm100_kernel<kD, kPlain>, kSmem);
     }
   };

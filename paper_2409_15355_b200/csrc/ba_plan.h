@@ -88,12 +88,15 @@ static inline ba_stream_plan ba_plan_stream(int sm_count, int n_chunks, const in
 // tile costs a little less and a CTA has half the rows to fetch, write out and collect from the others.  (32/8 heads of 128, us a
 // layer, whole items and single tiles, CTAs: 2500 cached tokens and 64 final ones, 56 and 80 CTAs: 23.9, 22.1; 6000, 64 and 96:
 // 32.7, 31.3; 128 final ones, 96 and 128 CTAs, 1000: 26.8, 27.3; 6000: 36.7, 37.7.)  fits(size): clusters of that size the GPU
-// runs at a time (0: none).
+// runs at a time (0: none).  shared: every CTA has one query tile, and the kernel is taken in which both softmax groups share its
+// key tiles (32/8 heads, 6000 cached tokens and 64 final ones: 31.4 -> 28.3 us a layer).  Where a CTA has two that kernel is the
+// slower one: 6000 cached tokens and 65 / 128 / 256 final ones 35.8 and 36.5, 36.9 and 37.6, 45.7 and 47.0; four requests of 2000
+// and 128 final ones 43.0 and 43.8, of 6000 and 8, 8, 8 and 60 final ones 55.2 and 56.4 (one_tile: no item has two).
 constexpr int kMaxCluster = 8;
-struct ba_cluster_plan { int size, single; double cost; };
+struct ba_cluster_plan { int size, single, shared; double cost; };
 template <class Fits>
-static inline ba_cluster_plan ba_plan_cluster(long long items, bool two_tiles, long long max_tiles, Fits fits) {
-  ba_cluster_plan plan = {0, 0, 0.};
+static inline ba_cluster_plan ba_plan_cluster(long long items, bool two_tiles, bool one_tile, long long max_tiles, Fits fits) {
+  ba_cluster_plan plan = {0, 0, 0, 0.};
   for (int single = 0; single <= (two_tiles ? 1 : 0); ++single)
     for (int n = 2; n <= kMaxCluster && n <= max_tiles; ++n) {
       const long long units = items << single, at_a_time = units == 1 ? 1 : fits(n);
@@ -102,6 +105,7 @@ static inline ba_cluster_plan ba_plan_cluster(long long items, bool two_tiles, l
       const double cost = (double)((units + at_a_time - 1) / at_a_time) * ((max_tiles + n - 1) / n * tile + 3) + merge;
       if (!plan.size || cost < plan.cost) { plan.size = n; plan.single = single; plan.cost = cost; }
     }
+  plan.shared = plan.size > 0 && (plan.single || one_tile);
   return plan;
 }
 

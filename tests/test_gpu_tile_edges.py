@@ -204,6 +204,17 @@ def test_cluster_launch_one_query_tile(w):
     assert np.array_equal(o, again) and np.array_equal(lse, lse_again)
 
 
+# Rows of the longest final block, which decide whether CTAs of whole items share key tiles: counted from lengths on the host only
+@pytest.mark.parametrize("w", [_requests("one", 1, 146, (2, 10, 40), (33, 33)), _requests("mixed", 4, 147, (2, 10, 40), (1, 70))], ids=lambda w: w.name)
+def test_longest_final_block(w):
+    c = R.Context.for_workload(w)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    assert seg.final_rows_max == max(w.final_lens())
+    lens, counts = (torch.tensor(v, dtype=torch.int32, device="cuda") for v in (w.block_lens, w.seq_nblocks))
+    assert c.segment(lens, counts, B.BA_MODE_BLOCK, n_tokens=w.n_tokens)[0].final_rows_max == 0
+    c.close()
+
+
 def _hpt(w):
     g = w.n_q_heads // w.n_kv_heads
     return 4 if g % 4 == 0 else 2 if g % 2 == 0 else 1

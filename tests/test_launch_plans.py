@@ -18,9 +18,9 @@ extern "C" void stream_plan(int sms, int chunks, const int32_t *tiles, int odd, 
   const ba_stream_plan p = ba_plan_stream(sms, chunks, tiles, odd, cap);
   out[0] = p.n_ctas; out[1] = p.n_odd; out[2] = p.n_slots; out[3] = p.cost;
 }
-extern "C" void cluster_plan(long long items, int two, long long tiles, const int32_t *at_a_time, double *out) {
-  const ba_cluster_plan p = ba_plan_cluster(items, two != 0, tiles, [&](int n) { return at_a_time[n]; });
-  out[0] = p.size; out[1] = p.single; out[2] = p.cost;
+extern "C" void cluster_plan(long long items, int two, int one, long long tiles, const int32_t *at_a_time, double *out) {
+  const ba_cluster_plan p = ba_plan_cluster(items, two != 0, one != 0, tiles, [&](int n) { return at_a_time[n]; });
+  out[0] = p.size; out[1] = p.single; out[2] = p.cost; out[3] = p.shared;
 }
 extern "C" int final_splits(int sms, int chunks, int items, int tiles, int longest, int cap) {
   return ba_plan_final_splits(sms, chunks, items, tiles, longest, cap);
@@ -38,7 +38,7 @@ def plans(tmp_path_factory):
     subprocess.run([gxx, "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2409_15355_b200", "csrc"), str(d / "plans.cc"),
                     "-o", str(d / "plans.so")], check=True)
     lib = C.CDLL(str(d / "plans.so"))
-    lib.cluster_plan.argtypes = [C.c_longlong, C.c_int, C.c_longlong, C.POINTER(C.c_int32 * 9), C.POINTER(C.c_double * 3)]
+    lib.cluster_plan.argtypes = [C.c_longlong, C.c_int, C.c_int, C.c_longlong, C.POINTER(C.c_int32 * 9), C.POINTER(C.c_double * 4)]
     return lib
 
 
@@ -145,9 +145,10 @@ def test_cluster_plans_take_the_cheapest_size_that_fits(plans):
     for _ in range(3000):
         items, two, tiles = int(rng.integers(1, 200)), bool(rng.integers(2)), int(rng.integers(1, 120))
         fits = (C.c_int32 * 9)(*[0, 0] + [int(rng.choice([0, 148 // n])) for n in range(2, 9)])
-        out = (C.c_double * 3)()
-        plans.cluster_plan(items, two, tiles, C.byref(fits), C.byref(out))
-        size, single, cost = int(out[0]), int(out[1]), out[2]
+        out = (C.c_double * 4)()
+        one = not two and bool(rng.integers(2))                           # (two: on average more than one query tile an item)
+        plans.cluster_plan(items, two, one, tiles, C.byref(fits), C.byref(out))
+        size, single, cost, shared = int(out[0]), int(out[1]), out[2], int(out[3])
         want = {}
         for s in (0, 1)[:2 if two else 1]:
             for n in range(2, min(8, tiles) + 1):
@@ -157,9 +158,10 @@ def test_cluster_plans_take_the_cheapest_size_that_fits(plans):
                 rounds = -(-units // (1 if units == 1 else fits[n]))
                 want[n, s] = rounds * (-(-tiles // n) * (0.85 if s else 1.0) + 3) + (0.25 if s else 1.5)
         if not want:
-            assert size == 0
+            assert size == 0 and not shared
             continue
         chosen += 1
+        assert shared == (single or one)                                 # a CTA with two query tiles: the kernel without sharing
         assert 2 <= size <= min(8, tiles) and (not single or two)
         assert cost == pytest.approx(min(want.values())) and want[size, single] == pytest.approx(cost)
         cuts = [tiles * k // size for k in range(size + 1)]                # every CTA has a share, none is empty
