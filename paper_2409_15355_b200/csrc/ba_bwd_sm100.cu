@@ -233,14 +233,17 @@ __device__ __forceinline__ void dkv_ds(const uint32_t *p, const uint32_t *dp, ui
   }
 }
 
-// Writes a warp's 32 accumulator rows (D fp32 columns of tensor memory, lane = row) to global memory.  row_at(r): element offset of
-// row r in dst, negative where the row is not stored.  The rows go through shared memory (`stage`: 32 rows of 2 D bytes, 16-byte
-// chunk c of row r at chunk position c ^ (r & 7)), so that a store instruction writes whole rows: 16 bytes each of 32 rows
-// fill no sector.  The loops stay loops: the code is passed once, and fetching it costs more than running it.  (8 x 16384 ragged
-// tokens, forward and backward: 13580 -> 13464 us; three small prompts 63.8 -> 63.0.)
+// Writes the first n_rows of a warp's 32 accumulator rows (D fp32 columns of tensor memory, lane = row) to global memory.  row_at(r):
+// element offset of row r in dst.  The rows go through shared memory (`stage`: 32 rows of 2 D bytes, 16-byte chunk c of row r at
+// chunk position c ^ (r & 7)), so that a store instruction writes whole bf16 rows or halves of fp32 rows, 2 D bytes in a run: 16
+// bytes each of 32 rows fill no sector.  The loops stay loops: the code is passed once, and fetching it costs more than running it.
+// (8 x 16384 ragged tokens, forward and backward: 13580 -> 13464 us; three small prompts 63.8 -> 63.0.)  Only rows that exist are
+// gone through: blocks of 1-20 tokens leave most of a tile's rows empty (2 x 8192 tokens of them: 1582 us with stores from the
+// threads' own rows, 1634 with all 32 rows passed, 1572; 4/4 heads, blocks of 50-500: 389, 393, 382).
 template <int D, class RowAt>
-__device__ __forceinline__ void store_acc_rows(uint32_t tAcc, uint8_t *stage, void *dst, int out_f32, RowAt row_at) {
+__device__ __forceinline__ void store_acc_rows(uint32_t tAcc, uint8_t *stage, void *dst, int out_f32, int n_rows, RowAt row_at) {
   constexpr int kRowBytes = 2 * D, kChunks = kRowBytes / 16;
+  if (n_rows <= 0) return;
   const int lane = threadIdx.x & 31, c = lane % kChunks;
   uint8_t *own = stage + lane * kRowBytes;
 #pragma unroll 1
@@ -266,11 +269,9 @@ __device__ __forceinline__ void store_acc_rows(uint32_t tAcc, uint8_t *stage, vo
     }
     __syncwarp();
 #pragma unroll 4
-    for (int i = 0; i < kChunks; ++i) {
-      const int r = i * (32 / kChunks) + lane / kChunks;
+    for (int r = lane / kChunks; r < n_rows; r += 32 / kChunks) {
       const uint4 x = *reinterpret_cast<const uint4 *>(stage + r * kRowBytes + ((c ^ (r & 7)) << 4));
-      const long long at = row_at(r);
-      if (at >= 0) *reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(dst) + at * (out_f32 ? 4 : 2) + h * kRowBytes + c * 16) = x;
+      *reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(dst) + row_at(r) * (out_f32 ? 4 : 2) + h * kRowBytes + c * 16) = x;
     }
     __syncwarp();
   }
@@ -505,9 +506,8 @@ ba_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     if (ok && n_iter > 0) {
       tc_fence_after();
       const int j0 = (warp & 3) * 32;
-      store_acc_rows<D>((h ? tDK : tDV) + lane_off, smem + (h ? L::kFix1 : L::kFix0) + j0 * (2 * D), h ? p.dk : p.dv, p.out_f32, [&](int r) {
-        return j0 + r < n_keys ? ((long long)(k0 + j0 + r) * p.Hkv + g) * D : -1LL;
-      });
+      store_acc_rows<D>((h ? tDK : tDV) + lane_off, smem + (h ? L::kFix1 : L::kFix0) + j0 * (2 * D), h ? p.dk : p.dv, p.out_f32, min(32, n_keys - j0),
+                        [&](int r) { return ((size_t)(k0 + j0 + r) * p.Hkv + g) * D; });
     }
   }
   tc_fence_before();
@@ -704,9 +704,10 @@ ba_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     if (ok && n_steps > 0) ok = mbar_wait(&ctrl->fin, 0, abort_flag);
     if (ok && n_steps > 0) {
       tc_fence_after();
-      store_acc_rows<D>(tDQ + lane_off, smem + L::kQ + warp * 32 * (2 * D), p.dq, p.out_f32, [&](int i) {
+      store_acc_rows<D>(tDQ + lane_off, smem + L::kQ + warp * 32 * (2 * D), p.dq, p.out_f32, min(32, ((q_end - q0) << p.hpt_log2) - warp * 32),
+                        [&](int i) {
         const int row = warp * 32 + i, tk = q0 + (row >> p.hpt_log2);
-        return tk < q_end ? ((long long)tk * p.Hq + head0 + (row & (p.hpt - 1))) * D : -1LL;
+        return ((size_t)tk * p.Hq + head0 + (row & (p.hpt - 1))) * D;
       });
     }
   }

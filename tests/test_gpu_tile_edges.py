@@ -27,6 +27,17 @@ def test_backward_tile_edges(lens, heads):
         rq, rk, rv = ob.block_prefill_backward(q, k, v, g, w.block_lens, w.seq_nblocks, mode)
         check_grad("dq", dq, rq); check_grad("dk", dk, rk); check_grad("dv", dv, rv)
 
+# Gradients leave as whole rows of the tiles' rows that exist: blocks that end in any of a warp's rows, next to rows of other blocks
+@pytest.mark.parametrize("heads", [(8, 2, 128), (6, 2, 64), (2, 2, 128)], ids=str)
+@pytest.mark.parametrize("dtype", [B.BA_OUT_F32, B.BA_OUT_BF16], ids=["f32", "bf16"])
+def test_backward_row_counts(heads, dtype):
+    lens = [1, 2, 3, 4, 5, 7, 8, 9, 15, 17, 31, 32, 33, 34, 36, 95, 97, 1]
+    w = W.Workload("row_counts", *heads, 1e4, lens + lens[::-1], [len(lens)] * 2, seed=83)
+    dq, dk, dv, q, k, v, g = run_forward_backward(w, B.BA_MODE_BLOCK, grad_dtype=dtype)
+    rq, rk, rv = ob.block_prefill_backward(q, k, v, g, w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    check_grad("dq", dq, rq); check_grad("dk", dk, rk); check_grad("dv", dv, rv)      # (a row not written is NaN)
+
+
 # The search for a key tile's block, 32 places a round: one round, two, three; gradients stored as bf16 and fp32 rows.
 @pytest.mark.parametrize("n_blocks", [31, 32, 33, 1024, 1025])
 @pytest.mark.parametrize("dtype", [B.BA_OUT_F32, B.BA_OUT_BF16], ids=["f32", "bf16"])
