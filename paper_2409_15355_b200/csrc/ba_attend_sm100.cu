@@ -590,6 +590,10 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   constexpr bool kClustered = kVariant == kFusedCluster || kVariant == kDeepCluster || kVariant == kSharedCluster;
   constexpr bool kSolo = kVariant == kSharedCluster;
   constexpr bool kReady = kVariant == kPlain || kVariant == kDeepRing;
+  // The rescaling of O stays a loop (kFusedCluster, eight requests of 12 cached blocks of 37-611 and 32 final tokens: 262 -> 255 us),
+  // but not in kFusedPath: with one query tile nothing else runs meanwhile, and the loop takes longer (32 x 1000 cached tokens and
+  // 1 / 32 final ones, eight layers, as a loop and unrolled: 439 and 421, 452 and 439 us; two query tiles: 519 and 521).
+  constexpr int kRescaleUnroll = kVariant == kFusedPath ? D / 32 : 1;
   // (layouts a variant is never launched with are not in its code: a short launch pays for every instruction it passes; a 32-layer
   // prompt of 2500 cached tokens 824 -> 795 us)
   const int balanced = kClustered || kDeep ? 0 : p.balanced, stream = kClustered ? 0 : p.stream, persistent = kClustered ? 0 : p.persistent;
@@ -1282,7 +1286,7 @@ ba_attend_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
               const float alpha = (m_new == -INFINITY) ? 1.f : ex2((m_used - m_new) * sl);
               m_used = m_new;
               l *= alpha;
-#pragma unroll 1
+#pragma unroll(kRescaleUnroll)
               for (int c = 0; c < D / 32; ++c) {
                 uint32_t o[32];
                 tmem_ld_32x32b_x32(tO + c * 32, o);

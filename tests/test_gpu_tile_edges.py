@@ -332,6 +332,75 @@ def test_fused_kernel(w, layout):
     B.ba_destroy(ctx)
 
 
+# Magnitudes of the cached keys that make a row's maximum grow from tile to tile, fall, or differ between the tiles that the two softmax
+# groups of a CTA take, by far more than the factor the reference maximum may lag behind.
+RAMPS = {"rising": lambda i, n, top: 1 + (top - 1) * i / n, "falling": lambda i, n, top: 1 + (top - 1) * (n - i) / n,
+         "every_second_tile": lambda i, n, top: np.where(i // 128 % 2, top, 1.0)}
+
+
+def _ramped_keys(w, x, ramp, top):
+    n = len(x["k_cache"])
+    return W.f32_to_bf16_bits(W.bf16_bits_to_f32(x["k_cache"]) * RAMPS[ramp](np.arange(n), n, top).astype(np.float32)[:, None, None])
+
+
+# Clusters of one query tile (shared by both groups) and of whole items.  The oracle attends the keys as the GPU re-encoded them: at
+# logits of hundreds their rounding to bf16 would weigh more than the attention's own error.  Bounds: those of the prefill's test.
+@pytest.mark.parametrize("w", [_requests("one_query_tile", 2, 151, (9, 200, 340), (20, 32)),
+                               _requests("whole_items", 1, 152, (20, 280, 320), (128, 128), heads=(32, 8, 128))], ids=lambda w: w.name)
+@pytest.mark.parametrize("ramp", RAMPS)
+def test_cluster_running_maximum(w, ramp):
+    x, t, f64 = W.warm_inputs(w), ob.segment_tables(w.block_lens, w.seq_nblocks), W.bf16_bits_to_f64
+    c = R.Context.for_workload(w)
+    seg, buf = c.segment(w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    keys = R.bits_to_device(_ramped_keys(w, x, ramp, 60.0))
+    q, k, v, vc = (R.bits_to_device(x[n]) for n in ("q_f", "k_f", "v_f", "v_cache"))
+    Tc, Tf = t["n_cached_tokens"], t["n_final_tokens"]
+    k_re = torch.empty_like(keys)
+    B.ba_reencode_k(c.ctx, keys, None, Tc, k_re, seg.cache_cu, seg.cache_delta, seg.n_cached_blocks, Tc)
+    o, lse = torch.empty(Tf, w.n_q_heads, w.head_dim, device="cuda"), torch.empty(Tf, w.n_q_heads, device="cuda")
+    B.ba_final_attend(c.ctx, q, k, v, Tf, k_re, vc, Tc, None, 0, o, lse, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    assert c.device_status() == B.BA_OK
+    assert c.last_attend_shape()["partials"] == 1 and c.last_attend_shape()["balanced_tails"] == 0
+    o_ref, lse_ref = ob.final_attend(f64(x["q_f"]), f64(x["k_f"]), f64(x["v_f"]), f64(R.device_to_bits(k_re)), f64(x["v_cache"]),
+                                     w.block_lens, w.seq_nblocks, B.BA_MODE_BLOCK)
+    d = np.abs(o.cpu().numpy() - o_ref)
+    assert d.max() <= 2e-2 and d.mean() <= 1e-3 and np.linalg.norm(d) / np.linalg.norm(o_ref) <= 5e-3
+    assert (np.abs(lse.cpu().numpy() - lse_ref) <= 2e-3 + 1e-5 * np.abs(lse_ref)).all()
+    c.close()
+
+
+# The fused kernel, on its own and in clusters, one and two query tiles.  It rounds the queries to bf16 once more after each block's
+# rotation: a logit of standard deviation s is off by about s 2^-9 / sqrt(3) rms, 0.005 at s = 4, and a weight by as much of itself;
+# five of those for the largest of 1e4 logits times values of up to 4 bound an element, twice the rms the whole.
+@pytest.mark.parametrize("w", [_requests("short", 1, 153, (24, 250, 330), (9, 9), heads=(32, 8, 128)),
+                               _requests("two_tiles", 1, 154, (24, 250, 330), (64, 64), heads=(32, 8, 128)),
+                               _requests("cluster", 1, 155, (9, 200, 340), (30, 30), heads=(8, 2, 128))], ids=lambda w: w.name)
+@pytest.mark.parametrize("ramp", RAMPS)
+def test_fused_kernel_running_maximum(w, ramp):
+    x, t, f64 = W.warm_inputs(w), ob.segment_tables(w.block_lens, w.seq_nblocks), W.bf16_bits_to_f64
+    Tc, Tf = t["n_cached_tokens"], t["n_final_tokens"]
+    bits = _ramped_keys(w, x, ramp, 4.0)
+    k_ref = ob.reencode_blocks(f64(bits), None, t["cache_cu"], t["cache_delta"], w.rope_theta)
+    o_ref, lse_ref = ob.final_attend(f64(x["q_f"]), f64(x["k_f"]), f64(x["v_f"]), k_ref, f64(x["v_cache"]), w.block_lens, w.seq_nblocks,
+                                     B.BA_MODE_BLOCK)
+    cfg = B.ba_config(w.n_q_heads, w.n_kv_heads, w.head_dim, 0, w.rope_theta, 0.0, 0)
+    # (partial results have room, re-encoded keys have not)
+    ctx = B.ba_create(cfg, 0, 64 * 1024 + Tc * w.n_kv_heads * w.head_dim * 3)
+    tb = torch.empty(B.ba_segments_bytes(w.batch, w.n_blocks, w.n_tokens), dtype=torch.uint8, device="cuda")
+    seg = B.ba_segment(ctx, np.asarray(w.block_lens, dtype=np.int32), np.asarray(w.seq_nblocks, dtype=np.int32), w.batch, w.n_blocks, w.n_tokens,
+                       B.BA_MODE_BLOCK, tb)
+    n0 = B.ba_launch_count(ctx)
+    q, k, v, ks, vs = (R.bits_to_device(b) for b in (x["q_f"], x["k_f"], x["v_f"], bits, x["v_cache"]))
+    o, lse = torch.empty(Tf, w.n_q_heads, w.head_dim, device="cuda"), torch.empty(Tf, w.n_q_heads, device="cuda")
+    B.ba_final_attend_fused(ctx, q, k, v, Tf, ks, vs, Tc, None, Tc, o, lse, seg, B.BA_MODE_BLOCK, B.BA_OUT_F32)
+    assert B.ba_last_device_status(ctx) == B.BA_OK
+    assert B.ba_launch_count(ctx) - n0 == (1 if B.ba_last_attend_shape(ctx)["partials"] == 1 else 2)     # no re-encoding pass
+    d = np.abs(o.cpu().numpy() - o_ref)
+    assert d.max() <= 1e-1 and np.linalg.norm(d) / np.linalg.norm(o_ref) <= 1e-2
+    assert np.abs(lse.cpu().numpy() - lse_ref).max() <= 2.5e-2
+    B.ba_destroy(ctx)
+
+
 # Tensors of one call whose cached tensor maps fall on the same slot of the context's 512: with the keys at 4096 places the
 # map of the queries or of the values is met about 16 times.
 def test_tensor_maps_that_share_a_slot():
