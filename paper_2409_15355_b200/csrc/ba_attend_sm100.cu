@@ -1903,7 +1903,7 @@ ba_status ba_attend_sm100_launch(ba_ctx *ctx, const ba_attend_args &a, const ba_
       }
       if (a.n_cache_rows > 0 && !ctx->has_pending) {
         const ba_cluster_plan cl = ba_plan_cluster(items, a.n_q_rows > (long long)p.tok * seg->n_final_items,
-                                                   seg->final_rows_max > 0 && seg->final_rows_max <= p.tok, ft[2], [&](int n) { return max_clusters(ctx, n); });
+                                                   seg->final_rows_max > 0 && seg->final_rows_max <= p.tok, p.fused, ft[2], [&](int n) { return max_clusters(ctx, n); });
         if (cl.size > 0 && cl.cost < (double)(p.stream ? stream.cost : equal_cost)) { p.cluster = cl.size; p.single = cl.single; cluster_shared = cl.shared; p.stream = 0; n_splits = 1; }
       }
     }

@@ -83,29 +83,35 @@ static inline ba_stream_plan ba_plan_stream(int sm_count, int n_chunks, const in
 }
 
 // Cluster launch of ba_final_attend: the `size` CTAs of a cluster share one item's key tiles and merge their results in
-// shared memory, which costs about as much as 1.5 tiles and saves the partial results' way through memory and the merging
-// kernel.  single: a cluster takes one query tile of an item instead of two, where most items have two (`two_tiles`): a key
-// tile costs a little less and a CTA has half the rows to fetch, write out and collect from the others.  (32/8 heads of 128, us a
-// layer, whole items and single tiles, CTAs: 2500 cached tokens and 64 final ones, 56 and 80 CTAs: 23.9, 22.1; 6000, 64 and 96:
-// 32.7, 31.3; 128 final ones, 96 and 128 CTAs, 1000: 26.8, 27.3; 6000: 36.7, 37.7.)  fits(size): clusters of that size the GPU
-// runs at a time (0: none).  shared: every CTA has one query tile, and the kernel is taken in which both softmax groups share its
-// key tiles (32/8 heads, 6000 cached tokens and 64 final ones: 31.4 -> 28.3 us a layer).  Where a CTA has two that kernel is the
-// slower one: 6000 cached tokens and 65 / 128 / 256 final ones 35.8 and 36.5, 36.9 and 37.6, 45.7 and 47.0; four requests of 2000
-// and 128 final ones 43.0 and 43.8, of 6000 and 8, 8, 8 and 60 final ones 55.2 and 56.4 (one_tile: no item has two).
+// shared memory, which saves the partial results' way through memory and the merging kernel.  single: a cluster takes one query
+// tile of an item instead of two, where most items have two (`two_tiles`): a CTA has half the rows to fetch, write out and collect
+// from the others.  shared: every CTA has one query tile (one_tile: no item has two), and unless the call is the fused one both softmax
+// groups share its key tiles.  A CTA's time in key tiles of two query tiles, its start and write-out, and the merge:
+//   two query tiles, or one of a whole item     1    a tile, 3,   1.5
+//   one query tile, fused                       0.85 a tile, 3,   0.25
+//   one query tile, shared by both groups       0.6  a tile, 3.5, 0.25
+// The last row was fitted to 240 shapes of 1-8 requests, 16-256 final and 250-9000 cached tokens, six shapes of heads, every layout and
+// cluster size timed (32/8 heads, us a launch, whole items, single tiles, no cluster: 6000 cached tokens and 64 final ones 24.6, 19.8, 23.1;
+// 128 final ones 28.5, 23.8, 25.8; 1000 and 256 20.1, 18.5, 20.1).  With the prices from before the groups shared tiles (the second row and,
+// for items of one tile, the first) 30 of them took a layout that is 0.6-19 % slower (6000 and 128: whole items; two requests
+// of 9000 and 20: 28.9 us without a cluster, 23.5 with), none a faster one.  Sharing is not for CTAs with two query tiles, where that
+// kernel is the slower one: with a re-encoding pass, 6000 cached tokens and 65 / 128 / 256 final ones 35.8 and 36.5, 36.9 and 37.6,
+// 45.7 and 47.0; four requests of 6000 and 8, 8, 8 and 60 55.2 and 56.4.  fits(size): clusters of that size the GPU runs at a time
+// (0: none).
 constexpr int kMaxCluster = 8;
 struct ba_cluster_plan { int size, single, shared; double cost; };
 template <class Fits>
-static inline ba_cluster_plan ba_plan_cluster(long long items, bool two_tiles, bool one_tile, long long max_tiles, Fits fits) {
+static inline ba_cluster_plan ba_plan_cluster(long long items, bool two_tiles, bool one_tile, bool fused, long long max_tiles, Fits fits) {
   ba_cluster_plan plan = {0, 0, 0, 0.};
   for (int single = 0; single <= (two_tiles ? 1 : 0); ++single)
     for (int n = 2; n <= kMaxCluster && n <= max_tiles; ++n) {
       const long long units = items << single, at_a_time = units == 1 ? 1 : fits(n);
       if (at_a_time < 1) continue;
-      const double tile = single ? 0.85 : 1.0, merge = single ? 0.25 : 1.5;
-      const double cost = (double)((units + at_a_time - 1) / at_a_time) * ((max_tiles + n - 1) / n * tile + 3) + merge;
-      if (!plan.size || cost < plan.cost) { plan.size = n; plan.single = single; plan.cost = cost; }
+      const bool shared = !fused && (single || one_tile);
+      const double tile = shared ? 0.6 : single ? 0.85 : 1.0, start = shared ? 3.5 : 3.0, merge = shared || single ? 0.25 : 1.5;
+      const double cost = (double)((units + at_a_time - 1) / at_a_time) * ((max_tiles + n - 1) / n * tile + start) + merge;
+      if (!plan.size || cost < plan.cost) { plan.size = n; plan.single = single; plan.shared = shared; plan.cost = cost; }
     }
-  plan.shared = plan.size > 0 && (plan.single || one_tile);
   return plan;
 }
 

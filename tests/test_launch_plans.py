@@ -18,8 +18,8 @@ extern "C" void stream_plan(int sms, int chunks, const int32_t *tiles, int odd, 
   const ba_stream_plan p = ba_plan_stream(sms, chunks, tiles, odd, cap);
   out[0] = p.n_ctas; out[1] = p.n_odd; out[2] = p.n_slots; out[3] = p.cost;
 }
-extern "C" void cluster_plan(long long items, int two, int one, long long tiles, const int32_t *at_a_time, double *out) {
-  const ba_cluster_plan p = ba_plan_cluster(items, two != 0, one != 0, tiles, [&](int n) { return at_a_time[n]; });
+extern "C" void cluster_plan(long long items, int two, int one, int fused, long long tiles, const int32_t *at_a_time, double *out) {
+  const ba_cluster_plan p = ba_plan_cluster(items, two != 0, one != 0, fused != 0, tiles, [&](int n) { return at_a_time[n]; });
   out[0] = p.size; out[1] = p.single; out[2] = p.cost; out[3] = p.shared;
 }
 extern "C" int final_splits(int sms, int chunks, int items, int tiles, int longest, int cap) {
@@ -38,7 +38,7 @@ def plans(tmp_path_factory):
     subprocess.run([gxx, "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2409_15355_b200", "csrc"), str(d / "plans.cc"),
                     "-o", str(d / "plans.so")], check=True)
     lib = C.CDLL(str(d / "plans.so"))
-    lib.cluster_plan.argtypes = [C.c_longlong, C.c_int, C.c_int, C.c_longlong, C.POINTER(C.c_int32 * 9), C.POINTER(C.c_double * 4)]
+    lib.cluster_plan.argtypes = [C.c_longlong, C.c_int, C.c_int, C.c_int, C.c_longlong, C.POINTER(C.c_int32 * 9), C.POINTER(C.c_double * 4)]
     return lib
 
 
@@ -147,7 +147,8 @@ def test_cluster_plans_take_the_cheapest_size_that_fits(plans):
         fits = (C.c_int32 * 9)(*[0, 0] + [int(rng.choice([0, 148 // n])) for n in range(2, 9)])
         out = (C.c_double * 4)()
         one = not two and bool(rng.integers(2))                           # (two: on average more than one query tile an item)
-        plans.cluster_plan(items, two, one, tiles, C.byref(fits), C.byref(out))
+        fused = bool(rng.integers(2))
+        plans.cluster_plan(items, two, one, fused, tiles, C.byref(fits), C.byref(out))
         size, single, cost, shared = int(out[0]), int(out[1]), out[2], int(out[3])
         want = {}
         for s in (0, 1)[:2 if two else 1]:
@@ -156,17 +157,28 @@ def test_cluster_plans_take_the_cheapest_size_that_fits(plans):
                 if units > 1 and fits[n] < 1:
                     continue
                 rounds = -(-units // (1 if units == 1 else fits[n]))
-                want[n, s] = rounds * (-(-tiles // n) * (0.85 if s else 1.0) + 3) + (0.25 if s else 1.5)
+                tile, start, merge = (0.6, 3.5, 0.25) if not fused and (s or one) else (0.85, 3, 0.25) if s else (1.0, 3, 1.5)
+                want[n, s] = rounds * (-(-tiles // n) * tile + start) + merge
         if not want:
             assert size == 0 and not shared
             continue
         chosen += 1
-        assert shared == (single or one)                                 # a CTA with two query tiles: the kernel without sharing
+        assert shared == (not fused and (single or one))                 # a CTA with two query tiles: the kernel without sharing
         assert 2 <= size <= min(8, tiles) and (not single or two)
         assert cost == pytest.approx(min(want.values())) and want[size, single] == pytest.approx(cost)
         cuts = [tiles * k // size for k in range(size + 1)]                # every CTA has a share, none is empty
         assert cuts[0] == 0 and cuts[-1] == tiles and all(b > a for a, b in zip(cuts, cuts[1:]))
     assert chosen > 2000
+
+
+# Shapes whose layouts were all timed: items, more than one query tile an item, all of one, key tiles, the fastest (size, single) and the
+# price of the best layout without a cluster.  148 SMs, clusters at a time as the driver gives them.
+@pytest.mark.parametrize("items,two,one,tiles,best,without", [(16, True, False, 48, (4, 1), 14), (32, True, False, 9, (2, 1), 11),
+                                                              (8, True, False, 48, (6, 1), 11), (16, False, True, 71, (6, 0), 16)])
+def test_cluster_plans_where_every_layout_was_timed(plans, items, two, one, tiles, best, without):
+    fits, out = (C.c_int32 * 9)(0, 0, 74, 45, 33, 26, 22, 15, 15), (C.c_double * 4)()
+    plans.cluster_plan(items, two, one, 0, tiles, C.byref(fits), C.byref(out))
+    assert (int(out[0]), int(out[1])) == best and out[3] == 1 and out[2] < without
 
 
 def test_final_blocks_of_a_prefill_are_cut_only_where_they_would_end_the_launch(plans):
