@@ -61,12 +61,12 @@ namespace {
 
 constexpr int kThreads = 384;
 constexpr int kBlockN = 128;      // keys per tile
-// Variants of the kernel, so that each carries only its own code.  The ring of K/V tiles (K_j, V_j, K_j+1, ...) has three
-// stages; the rest of the shared memory is a second pair of query buffers (or the background job's staging area).  In
-// kDeepRing it is a fourth stage and a staging area for the write-out: a tile that comes from HBM while every SM streams
-// takes 2000-4500 cycles, three stages cover 2700 (64-token query over 32K cached keys: 800-1900 cycles of waiting in a
-// period of 4000-4900), and with the write-out elsewhere the one pair of query buffers is reloaded as soon as its last
-// product is done.
+// Variants of the kernel, so that each carries only its own code.  The ring of K/V tiles (K_j, V_j, K_j+1, ...; in kSharedCluster
+// K_0, K_1, V_0, K_2, V_1, ...) has three stages; the rest of the shared memory is a second pair of query buffers (or the
+// background job's staging area).  In kDeepRing it is a fourth stage and a staging area for the write-out: a tile that comes from
+// HBM while every SM streams takes 2000-4500 cycles, three stages cover 2700 (64-token query over 32K cached keys: 800-1900 cycles
+// of waiting in a period of 4000-4900; with four the product thread finds every tile there), and with the write-out elsewhere the
+// one pair of query buffers is reloaded as soon as its last product is done.
 // The cluster forms of the last two merge the results of a cluster's CTAs in shared memory; kSharedCluster is kDeepCluster for
 // launches whose CTAs have one query tile (is_solo).
 constexpr int kPlain = 0, kFusedPath = 1, kDeepRing = 2, kFusedCluster = 3, kDeepCluster = 4, kSharedCluster = 5;
