@@ -1721,20 +1721,21 @@ constexpr int attend_smem_bytes() {
 // limit is raised once here instead of on every launch, and the tensor-map table is created.
 ba_status ba_attend_sm100_setup(ba_ctx *ctx) {
   auto raise = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
-  // (The kernels lie in memory in the reverse of this order.  A kernel that moves with another one's length gains or loses up to 1 %: with
-  // kFusedPath second, its unrolled rescaling moved kPlain: cold prompt of 7200 tokens 765 -> 767 us, 4096 in blocks of 300 145 -> 147.)
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kPlain>, attend_smem_bytes<128>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepCluster>, attend_smem_bytes<128>()));
+  // (The kernels lie in memory in the reverse of this order, and one that moves gains or loses up to 1 % with the same code: five
+  // orders, us a pass, cold prompt of 7200 tokens 767-772, 32 x 1000 cached tokens and one final token 479-490; 765 and 489 without
+  // kSharedCluster, 767 and 483 with it last in memory, where it moves no other kernel.)
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kSharedCluster>, attend_smem_bytes<128>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedCluster>, attend_smem_bytes<128>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepCluster>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kSharedCluster>, attend_smem_bytes<64>()));
-  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedCluster>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kPlain>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedPath>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepRing>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kFusedCluster>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<128, kDeepCluster>, attend_smem_bytes<128>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kPlain>, attend_smem_bytes<64>()));
   BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedPath>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepRing>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kFusedCluster>, attend_smem_bytes<64>()));
+  BA_CUDA_TRY(raise(ba_attend_sm100_kernel<64, kDeepCluster>, attend_smem_bytes<64>()));
   ctx->maps = new (std::nothrow) ba_map_cache();
   if (!ctx->maps) return BA_ERR_CUDA;
   for (auto &sl : ctx->maps->slot) sl.ptr = nullptr;
